@@ -63,7 +63,9 @@ struct BigWorkspace {
   int* kwarm;    // nblocks: how many of them (0 = none)
   size_t ystride;
   // blocks wider than 256 (k_block_huge.cu): G is a full square there
-  float* H;      // nblocks * nn * nn: certificate matrix, factored in place
+  void* Ma;      // nblocks * np * np FP16, np = nn rounded up to 64: certificate matrices
+  void* Mb;
+  double* fpart; // nblocks * tiles: their F-norm partials
   float* tstat;  // nblocks * ntiles * 2: per-tile diagonal sums, sums of squares
   float* V;      // nblocks * nn * 32: subspace basis (kept across calls)
   float* Wv;     // nblocks * nn * 32: G V
@@ -85,7 +87,7 @@ enum KernelKind {
   KK_MISC,
   KK_EIG_FALLBACK,
   KK_SUBSPACE,  // wide blocks over 256: G V, orthonormalisation, Rayleigh-Ritz
-  KK_CERT,      // wide blocks over 256: the tiled Cholesky certificate
+  KK_CERT,      // wide blocks over 256: the certificate
   KK_COUNT
 };
 

@@ -15,6 +15,7 @@
 #include <stdlib.h>
 
 #include "common.cuh"
+#include "huge.cuh"
 #include "internal.h"
 #include "lanczos.cuh"
 #include "symeig.cuh"
@@ -671,6 +672,7 @@ cudaError_t configure_big_kernels() {
   sm_count();  // cache the SM count outside any stream capture
   gram_fp32_forced();
   if (cudaError_t e0 = configure_gram_tc()) return e0;
+  if (cudaError_t e1 = configure_cert()) return e1;
   cudaError_t e = cudaFuncSetAttribute(eig_big_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)eig_smem_bytes(kEigMax));
   if (e != cudaSuccess) return e;

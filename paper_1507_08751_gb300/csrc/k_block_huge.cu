@@ -14,11 +14,10 @@
 //   3. Rayleigh-Ritz on V^T G V (32 x 32, the tridiagonal solver of
 //      symeig.cuh) for the pairs above tau^2, their residuals and a
 //      convergence test; unconverged blocks get further rounds of steps;
-//   4. certificate: lambda_max(P G P) < tau^2 with P = I - U U^T over the
-//      kept Ritz vectors, proved by a tiled Cholesky factorisation of
-//      c I - P G P (Golub & Van Loan Sec. 4.2), a panel launch and a
-//      trailing-update launch per 64 columns; by Cauchy interlacing G then
-//      has no eigenvalue above tau^2 besides the kept ones;
+//   4. certificate: ||P G P||_2 < tau^2 with P = I - U U^T over the kept
+//      Ritz vectors, by repeated squaring on the tensor cores
+//      (k_cert_tc.cu); by Cauchy interlacing G then has no eigenvalue above
+//      tau^2 besides the kept ones;
 //   5. rebuild: Z'_b = (C_b V_f) V_f^T with V_f = U diag(sqrt(1 - tau/sigma))
 //      over the pairs above tau, scattered through Shift_{-s}, with the fused
 //      dual update W' = 2 Z' - A of eq:admm.
@@ -28,6 +27,7 @@
 
 #include "../../include/msllr.h"
 #include "common.cuh"
+#include "huge.cuh"
 #include "internal.h"
 #include "symeig.cuh"
 
@@ -35,27 +35,10 @@ namespace msllr {
 
 namespace {
 
-constexpr int kHT = 64;          // Gram and Cholesky tile
-constexpr int kHP = 32;          // subspace width
-constexpr int kHK = 16;          // most Ritz pairs kept per block
+constexpr int kHT = 64;          // Gram tile
 constexpr int kHThreads = 256;   // tile kernels
 constexpr int kHBlockThreads = 512;  // per-block kernels
 constexpr int kHGvRows = 8;      // rows of W per CTA in W = G V
-
-// per-block state of the wide path
-struct HugeBlock {
-  float trace;   // trace(G) (>= lambda_max)
-  float gF;      // ||G||_F
-  float c;       // certificate shift (valid when status == kHsCert)
-  float theta[kHK];
-  int status;    // kHs*
-  int ku;        // kept Ritz pairs
-  int k;         // pairs above tau
-  int conv;      // Rayleigh-Ritz residual test passed
-  int chol_fail; // the tiled Cholesky met a non-positive pivot
-  int orth_fail; // a CholQR factorisation broke down (basis restarted)
-};
-enum : int { kHsSkip = 1, kHsIter = 2, kHsCert = 3, kHsNoCert = 4 };
 
 struct HugeDims {
   int mm, nn, nblocks, T, ntiles, chunk_rows, chunks;
@@ -87,14 +70,6 @@ __device__ __forceinline__ float huge_load(const ScaleLaunch& a, size_t off) {
   float v = a.A1[off];
   if (a.A2) v += a.A2[off];
   return v;
-}
-
-__device__ __forceinline__ void tile_of(int t, int* ta, int* tc) {
-  int i = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
-  while (((i + 1) * (i + 2)) / 2 <= t) ++i;
-  while ((i * (i + 1)) / 2 > t) --i;
-  *ta = i;
-  *tc = t - (i * (i + 1)) / 2;
 }
 
 // deterministic pseudo-random value in [-1, 1)
@@ -252,7 +227,8 @@ huge_prep_kernel(const float* __restrict__ tstat, int ntiles, HugeBlock* __restr
     h.ku = 0;
     h.k = 0;
     h.conv = 0;
-    h.chol_fail = 0;
+    h.cert = kCertOpen;
+    h.arrived = 0;
     h.orth_fail = 0;
     h.c = 0.f;
   }
@@ -674,204 +650,17 @@ huge_rr_kernel(const float* __restrict__ V, const float* __restrict__ W, float* 
       trb += Bm[q * kHK + q];
       if (rq[q] > fmaxf(3e-4f * thr, 4e-6f * th0)) conv = 0;
     }
-    // Certificate shift: lambda_max(P G P) < c proves, by Cauchy interlacing,
-    // that G has at most ku eigenvalues above c (and the ku Ritz values above
+    // Certificate bound: ||P G P||_2 < c proves, by Cauchy interlacing, that
+    // G has at most ku eigenvalues above c (and the ku Ritz values above
     // tau^2 are lower bounds of ku eigenvalues), so exactly the kept pairs
-    // lie above tau^2.  c = tau^2 less the rounding margins: the tiled
-    // Cholesky of H = c I - X succeeds only if H + E is positive definite
-    // with ||E||_2 <= gamma_d trace(H) (Higham, Thm. 10.3, with inner-product
-    // depth d <= 2 * 64 + nn / 64 + 2), trace(H) = nn c - trace(G) + sum
-    // theta; and forming X costs (2 ku + 4) eps (||G||_F + 2 sqrt(ku) ||What||_F).
-    const float depth = (float)(2 * kHT + nn / kHT + 2);
-    const float trh = fmaxf((float)nn * thr - (h.trace - trb), 0.f);
+    // lie above tau^2.  c = tau^2 less the rounding of forming X = P G P,
+    // (2 ku + 4) eps (||G||_F + 2 sqrt(ku) ||What||_F); the certificate
+    // accounts for its own rounding.
     const float xf = h.gF + 2.f * sqrtf((float)ku) * sqrtf(wsum);
-    const float margin =
-        1.1f * FLT_EPSILON * (depth * trh + (float)(2 * ku + 4) * xf);
-    h.c = thr - margin;
+    h.c = thr - 1.1f * FLT_EPSILON * (float)(2 * ku + 4) * xf;
     h.ku = ku;
     h.k = k;
     h.conv = conv;
-  }
-}
-
-
-// ---------------------------------------------------------------------------
-// 4. Certificate.  H = c I - X, X = G - U What^T - What U^T = P G P (the
-// deflated Gram matrix), lower 64x64 tiles; then H = L L^T tile by tile.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kHThreads)
-huge_form_kernel(const float* __restrict__ G, const float* __restrict__ U,
-                 const float* __restrict__ Wh, float* __restrict__ H, int nn,
-                 HugeBlock* __restrict__ hb) {
-  __shared__ float Ui[kHT][kHK + 1], Wi[kHT][kHK + 1], Uj[kHT][kHK + 1], Wj[kHT][kHK + 1];
-  const int t = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
-  const HugeBlock& h = hb[b];
-  if (h.status != kHsIter) return;
-  const float c = h.c;
-  if (!(c > 0.f)) {
-    if (t == 0 && tid == 0) hb[b].chol_fail = 1;
-    return;
-  }
-  const int ku = h.ku;
-  int ta, tc;
-  tile_of(t, &ta, &tc);
-  const float* Ub = U + (size_t)b * nn * kHK;
-  const float* Wb = Wh + (size_t)b * nn * kHK;
-  for (int e = tid; e < kHT * kHK; e += kHThreads) {
-    const int x = e / kHK, q = e - x * kHK;
-    const int gi = ta * kHT + x, gj = tc * kHT + x;
-    const bool qi = q < ku && gi < nn, qj = q < ku && gj < nn;
-    Ui[x][q] = qi ? Ub[(size_t)gi * kHK + q] : 0.f;
-    Wi[x][q] = qi ? Wb[(size_t)gi * kHK + q] : 0.f;
-    Uj[x][q] = qj ? Ub[(size_t)gj * kHK + q] : 0.f;
-    Wj[x][q] = qj ? Wb[(size_t)gj * kHK + q] : 0.f;
-  }
-  __syncthreads();
-  const float* Gb = G + (size_t)b * nn * nn;
-  float* Hb = H + (size_t)b * nn * nn;
-  for (int e = tid; e < kHT * kHT; e += kHThreads) {
-    const int x = e / kHT, y = e - x * kHT;
-    const int i = ta * kHT + x, j = tc * kHT + y;
-    if (i >= nn || j >= nn || j > i) continue;
-    float v = Gb[(size_t)i * nn + j];
-    for (int q = 0; q < ku; ++q) {
-      v = fmaf(-Ui[x][q], Wj[y][q], v);
-      v = fmaf(-Wi[x][q], Uj[y][q], v);
-    }
-    Hb[(size_t)i * nn + j] = (i == j ? c : 0.f) - v;
-  }
-}
-
-// Panel j: every CTA factors the diagonal tile (j, j) in shared memory (all
-// get the same factor); CTA i > 0 solves tile (j + i, j): L_ij = H_ij
-// L_jj^{-T}.  A non-positive pivot marks the block.
-__global__ void __launch_bounds__(kHThreads)
-huge_chol_panel_kernel(float* __restrict__ H, int nn, int j, HugeBlock* __restrict__ hb) {
-  __shared__ float Ld[kHT][kHT + 1];
-  __shared__ float Xs[kHT][kHT + 1];
-  const int b = blockIdx.y, tid = threadIdx.x;
-  {
-    const HugeBlock& h = hb[b];
-    if (h.status != kHsIter || h.chol_fail) return;
-  }
-  const int i = j + blockIdx.x;
-  float* Hb = H + (size_t)b * nn * nn;
-  const int j0 = j * kHT, i0 = i * kHT;
-  for (int e = tid; e < kHT * kHT; e += kHThreads) {
-    const int x = e / kHT, y = e - x * kHT;
-    const int gi = j0 + x, gj = j0 + y;
-    float v;
-    if (gi < nn && gj < nn) v = (y <= x) ? Hb[(size_t)gi * nn + gj] : 0.f;
-    else v = (x == y) ? 1.f : 0.f;  // identity padding keeps definiteness
-    Ld[x][y] = v;
-  }
-  __syncthreads();
-  // the 64 x 64 diagonal factor, column by column (Crout form, Golub & Van
-  // Loan Sec. 4.2): thread (r, part) = (tid / 4, tid mod 4) forms a quarter
-  // of row r's inner product with row c, the four quarters are added by
-  // shuffles inside the warp; two CTA barriers per column
-  __shared__ int bad_s;
-  if (tid == 0) bad_s = 0;
-  const int r = tid >> 2, part = tid & 3;
-  for (int c = 0; c < kHT; ++c) {
-    float sdot = 0.f;
-    if (r >= c)
-      for (int k = part; k < c; k += 4) sdot = fmaf(Ld[r][k], Ld[c][k], sdot);
-    sdot += __shfl_xor_sync(0xffffffffu, sdot, 1);
-    sdot += __shfl_xor_sync(0xffffffffu, sdot, 2);
-    const float t = r >= c ? Ld[r][c] - sdot : 0.f;
-    if (r == c && part == 0) {
-      const bool ok = t > 0.f && isfinite(t);
-      if (!ok) bad_s = 1;
-      Ld[c][c] = sqrtf(ok ? t : 1.f);
-    }
-    __syncthreads();
-    if (r > c && part == 0) Ld[r][c] = t / Ld[c][c];
-    __syncthreads();
-  }
-  const bool bad = bad_s != 0;
-  if (bad) {
-    if (blockIdx.x == 0 && tid == 0) hb[b].chol_fail = 1;
-    return;
-  }
-  // the diagonal factor is needed only inside this launch (every CTA has
-  // it); tile (j, j) stays as it is, so no CTA can read a half-written one
-  if (i == j) return;
-  for (int e = tid; e < kHT * kHT; e += kHThreads) {
-    const int x = e / kHT, y = e - x * kHT;
-    const int gi = i0 + x, gj = j0 + y;
-    Xs[x][y] = (gi < nn && gj < nn) ? Hb[(size_t)gi * nn + gj] : 0.f;
-  }
-  __syncthreads();
-  {
-    // rows of X L^T = A: thread (x, part) = (tid / 4, tid mod 4) forms a
-    // quarter of each inner product, the row's four threads (one warp) add
-    // them by shuffles; no CTA barrier between columns
-    const int x = tid >> 2;
-    for (int c = 0; c < kHT; ++c) {
-      float sdot = 0.f;
-      for (int l = part; l < c; l += 4) sdot = fmaf(Xs[x][l], Ld[c][l], sdot);
-      sdot += __shfl_xor_sync(0xffffffffu, sdot, 1);
-      sdot += __shfl_xor_sync(0xffffffffu, sdot, 2);
-      if (part == 0) Xs[x][c] = (Xs[x][c] - sdot) / Ld[c][c];
-      __syncwarp();
-    }
-  }
-  __syncthreads();
-  for (int e = tid; e < kHT * kHT; e += kHThreads) {
-    const int x = e / kHT, y = e - x * kHT;
-    const int gi = i0 + x, gj = j0 + y;
-    if (gi < nn && gj < nn) Hb[(size_t)gi * nn + gj] = Xs[x][y];
-  }
-}
-
-// Trailing update after panel j: H_il -= L_ij L_lj^T for j < l <= i.
-__global__ void __launch_bounds__(kHThreads)
-huge_chol_update_kernel(float* __restrict__ H, int nn, int j, HugeBlock* __restrict__ hb) {
-  __shared__ __align__(16) float Ai[kHT][kHT + 4];
-  __shared__ __align__(16) float Al[kHT][kHT + 4];
-  const int b = blockIdx.y, tid = threadIdx.x;
-  {
-    const HugeBlock& h = hb[b];
-    if (h.status != kHsIter || h.chol_fail) return;
-  }
-  int ta, tc;
-  tile_of(blockIdx.x, &ta, &tc);
-  const int i = j + 1 + ta, l = j + 1 + tc;
-  float* Hb = H + (size_t)b * nn * nn;
-  const int i0 = i * kHT, l0 = l * kHT, j0 = j * kHT;
-  for (int e = tid; e < kHT * kHT; e += kHThreads) {
-    const int x = e / kHT, kk = e - x * kHT;
-    const bool kin = j0 + kk < nn;
-    Ai[kk][x] = (kin && i0 + x < nn) ? Hb[(size_t)(i0 + x) * nn + j0 + kk] : 0.f;
-    Al[kk][x] = (kin && l0 + x < nn) ? Hb[(size_t)(l0 + x) * nn + j0 + kk] : 0.f;
-  }
-  __syncthreads();
-  const int tx = tid & 15, ty = tid >> 4;
-  float acc[4][4];
-#pragma unroll
-  for (int x = 0; x < 4; ++x)
-#pragma unroll
-    for (int y = 0; y < 4; ++y) acc[x][y] = 0.f;
-#pragma unroll 8
-  for (int kk = 0; kk < kHT; ++kk) {
-    const float4 a4 = *reinterpret_cast<const float4*>(&Ai[kk][ty * 4]);
-    const float4 b4 = *reinterpret_cast<const float4*>(&Al[kk][tx * 4]);
-    const float av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
-#pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-      for (int y = 0; y < 4; ++y) acc[x][y] = fmaf(av[x], bv[y], acc[x][y]);
-  }
-#pragma unroll
-  for (int x = 0; x < 4; ++x) {
-    const int gi = i0 + ty * 4 + x;
-    if (gi >= nn) continue;
-#pragma unroll
-    for (int y = 0; y < 4; ++y) {
-      const int gl = l0 + tx * 4 + y;
-      if (gl < nn && gl <= gi) Hb[(size_t)gi * nn + gl] -= acc[x][y];
-    }
   }
 }
 
@@ -902,7 +691,7 @@ huge_final_kernel(ScaleLaunch a, const float* __restrict__ U, float* __restrict_
     }
     ks = k;
     const bool skipped = h.status == kHsSkip;
-    const bool cert = skipped || (h.status == kHsIter && h.c > 0.f && !h.chol_fail);
+    const bool cert = skipped || (h.status == kHsIter && h.cert == kCertYes);
     kout[b] = k;
     if (a.rank_out) a.rank_out[b] = k;
     if (a.cnt) {
@@ -997,7 +786,9 @@ size_t huge_workspace_bytes(int M, int N, int m, int n) {
   const size_t B = (size_t)d.nblocks, nn = (size_t)d.nn;
   size_t bytes = 0;
   bytes += sizeof(float) * B * d.chunks * d.ntiles * kHT * kHT;  // Gram partials
-  bytes += 2 * sizeof(float) * B * nn * nn;                      // G, H
+  bytes += sizeof(float) * B * nn * nn;                          // G
+  bytes += 2 * B * cert_matrix_bytes(d.nn);                      // certificate matrices
+  bytes += sizeof(double) * B * cert_fpart_count(d.nn);
   bytes += 2 * sizeof(float) * B * d.ntiles;                     // tile sums
   bytes += 2 * sizeof(float) * B * nn * kHP;                     // V, W
   bytes += 3 * sizeof(float) * B * nn * kHK;                     // U, What, V_f
@@ -1019,7 +810,9 @@ BigWorkspace carve_huge_workspace(void* base, int M, int N, int m, int n) {
   };
   w.part = (float*)take(sizeof(float) * B * d.chunks * d.ntiles * kHT * kHT);
   w.G = (float*)take(sizeof(float) * B * nn * nn);
-  w.H = (float*)take(sizeof(float) * B * nn * nn);
+  w.Ma = take(B * cert_matrix_bytes(d.nn));
+  w.Mb = take(B * cert_matrix_bytes(d.nn));
+  w.fpart = (double*)take(sizeof(double) * B * cert_fpart_count(d.nn));
   w.tstat = (float*)take(2 * sizeof(float) * B * d.ntiles);
   w.V = (float*)take(sizeof(float) * B * nn * kHP);
   w.Wv = (float*)take(sizeof(float) * B * nn * kHP);
@@ -1109,21 +902,9 @@ cudaError_t launch_huge(const ScaleLaunch& s, const BigWorkspace& ws, cudaStream
     huge_rr_kernel<<<B, kHBlockThreads, 0, st>>>(ws.V, ws.Wv, ws.U, ws.GU, nn, thr, hb);
     PROF_AFTER()
   }
-  // certificate
-  PROF_BEFORE(KK_CERT)
-  huge_form_kernel<<<dim3(d.ntiles, B), kHThreads, 0, st>>>(ws.G, ws.U, ws.GU, ws.H, nn, hb);
-  PROF_AFTER()
-  for (int j = 0; j < d.T; ++j) {
-    PROF_BEFORE(KK_CERT)
-    huge_chol_panel_kernel<<<dim3(d.T - j, B), kHThreads, 0, st>>>(ws.H, nn, j, hb);
-    PROF_AFTER()
-    const int rem = d.T - j - 1;
-    if (rem > 0) {
-      PROF_BEFORE(KK_CERT)
-      huge_chol_update_kernel<<<dim3(rem * (rem + 1) / 2, B), kHThreads, 0, st>>>(ws.H, nn, j, hb);
-      PROF_AFTER()
-    }
-  }
+  if (cudaError_t e_ = launch_cert(ws.G, ws.U, ws.GU, ws.Ma, ws.Mb, ws.fpart, hb, nn, B, s.err, st,
+                                   prof))
+    return e_;
   PROF_BEFORE(KK_EIG)
   huge_final_kernel<<<B, kHThreads, 0, st>>>(s, ws.U, ws.Y, ws.k, nn, hb);
   PROF_AFTER()
