@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <float.h>
 #include <stddef.h>
 
 #include "internal.h"
@@ -41,6 +42,36 @@ __device__ __forceinline__ void tile_of(int t, int* ta, int* tc) {
   *ta = i;
   *tc = t - (i * (i + 1)) / 2;
 }
+
+// The bound the certificate has to prove: ||P G P||_2 < c shows, by Cauchy
+// interlacing, that G has at most ku eigenvalues above c (and the ku Ritz
+// values above tau^2 are lower bounds of ku eigenvalues), so exactly the kept
+// pairs lie above tau^2.  c = tau^2 less the rounding of forming X = P G P,
+// (2 ku + 4) eps (||G||_F + 2 sqrt(ku) ||What||_F), wsum = ||What||_F^2; the
+// certificate accounts for its own rounding.
+__device__ __forceinline__ float cert_bound(float thr, float gF, int ku, float wsum) {
+  const float xf = gF + 2.f * sqrtf((float)ku) * sqrtf(wsum);
+  return thr - 1.1f * FLT_EPSILON * (float)(2 * ku + 4) * xf;
+}
+
+// deterministic pseudo-random value in [-1, 1)
+__device__ __forceinline__ float huge_hash(uint32_t a, uint32_t b) {
+  uint32_t h = a * 0x9E3779B1u ^ (b + 0x7F4A7C15u) * 0x85EBCA77u;
+  h ^= h >> 15;
+  h *= 0x2C1B3C6Du;
+  h ^= h >> 12;
+  h *= 0x297A2D39u;
+  h ^= h >> 15;
+  return (float)(h >> 8) * (2.f / 16777216.f) - 1.f;
+}
+
+// The subspace iteration in one cluster per block (k_subspace.cu): the
+// padded orders it takes, kernel attributes, and the launch (first: steps of
+// the first round).
+bool subspace_cluster_path(int np);
+cudaError_t configure_subspace();
+cudaError_t launch_subspace(const float* G, float* V, float* U, float* GU, int nn, int np, float thr,
+                            int first, HugeBlock* hb, int B, cudaStream_t st);
 
 // Certificate workspace per block (bytes of one of the two FP16 matrices,
 // F-norm partials) and its launches: form plus kCertLevels squarings.

@@ -673,6 +673,7 @@ cudaError_t configure_big_kernels() {
   gram_fp32_forced();
   if (cudaError_t e0 = configure_gram_tc()) return e0;
   if (cudaError_t e1 = configure_cert()) return e1;
+  if (cudaError_t e2 = configure_subspace()) return e2;
   cudaError_t e = cudaFuncSetAttribute(eig_big_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)eig_smem_bytes(kEigMax));
   if (e != cudaSuccess) return e;

@@ -72,17 +72,6 @@ __device__ __forceinline__ float huge_load(const ScaleLaunch& a, size_t off) {
   return v;
 }
 
-// deterministic pseudo-random value in [-1, 1)
-__device__ __forceinline__ float huge_hash(uint32_t a, uint32_t b) {
-  uint32_t h = a * 0x9E3779B1u ^ (b + 0x7F4A7C15u) * 0x85EBCA77u;
-  h ^= h >> 15;
-  h *= 0x2C1B3C6Du;
-  h ^= h >> 12;
-  h *= 0x297A2D39u;
-  h ^= h >> 15;
-  return (float)(h >> 8) * (2.f / 16777216.f) - 1.f;
-}
-
 // ---------------------------------------------------------------------------
 // 1. Gram partial sums: tile t of the lower triangle over one row chunk.
 // ---------------------------------------------------------------------------
@@ -142,18 +131,19 @@ huge_gram_kernel(ScaleLaunch a, float* __restrict__ part, int chunk_rows, int ch
     for (int y = 0; y < 4; ++y) dst[(ty * 4 + x) * kHT + tx * 4 + y] = acc[x][y];
 }
 
-// Sum of the chunk partials in chunk order; G_b written as a full square,
+// Sum of the chunk partials in chunk order; G_b written as a full square of
+// order np (nn rounded up to the tile; the tiles are zero beyond nn),
 // and per tile: the diagonal sum and the sum of squares (off-diagonal tiles
 // twice), for trace(G) and ||G||_F.
 __global__ void __launch_bounds__(kHThreads)
 huge_gram_finish_kernel(const float* __restrict__ part, float* __restrict__ G,
-                        float* __restrict__ tstat, int nn, int chunks) {
+                        float* __restrict__ tstat, int np, int chunks) {
   __shared__ float red[2][kHThreads / 32];
   const int t = blockIdx.x, b = blockIdx.y, ntiles = gridDim.x;
   int ta, tc;
   tile_of(t, &ta, &tc);
   const int tid = threadIdx.x;
-  float* Gb = G + (size_t)b * nn * nn;
+  float* Gb = G + (size_t)b * np * np;
   float dsum = 0.f, sq = 0.f;
   for (int e = tid; e < kHT * kHT; e += kHThreads) {
     const int x = e / kHT, y = e - x * kHT;
@@ -161,18 +151,17 @@ huge_gram_finish_kernel(const float* __restrict__ part, float* __restrict__ G,
     float s = 0.f;
     for (int c = 0; c < chunks; ++c)
       s += part[(((size_t)b * chunks + c) * ntiles + t) * (kHT * kHT) + e];
-    if (i >= nn || j >= nn) continue;
     if (ta == tc) {
       // diagonal tile: the lower half is authoritative
       if (j <= i) {
-        Gb[(size_t)i * nn + j] = s;
-        Gb[(size_t)j * nn + i] = s;
+        Gb[(size_t)i * np + j] = s;
+        Gb[(size_t)j * np + i] = s;
         sq += (i == j ? 1.f : 2.f) * s * s;
         if (i == j) dsum += s;
       }
     } else {
-      Gb[(size_t)i * nn + j] = s;
-      Gb[(size_t)j * nn + i] = s;
+      Gb[(size_t)i * np + j] = s;
+      Gb[(size_t)j * np + i] = s;
       sq += 2.f * s * s;
     }
   }
@@ -236,12 +225,14 @@ huge_prep_kernel(const float* __restrict__ tstat, int ntiles, HugeBlock* __restr
 
 // Start basis: deterministic pseudo-random columns (any full-rank start
 // serves subspace iteration), the same for every block (rows r of a block
-// at V + (b nn + r) kHP), so that a block's start does not depend on its
+// at V + (b np + r) kHP, zero beyond nn), so that a block's start does not depend on its
 // index.
-__global__ void huge_init_basis_kernel(float* __restrict__ V, size_t total, int nn) {
+__global__ void huge_init_basis_kernel(float* __restrict__ V, size_t total, int nn, int np) {
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
-       e += (size_t)gridDim.x * blockDim.x)
-    V[e] = huge_hash((uint32_t)((e / kHP) % nn), (uint32_t)(e % kHP) + 0x51EDu);
+       e += (size_t)gridDim.x * blockDim.x) {
+    const int r = (int)((e / kHP) % np);
+    V[e] = r < nn ? huge_hash((uint32_t)r, (uint32_t)(e % kHP) + 0x51EDu) : 0.f;
+  }
 }
 
 __device__ __forceinline__ bool huge_active(const HugeBlock& h) {
@@ -386,7 +377,8 @@ __device__ bool huge_chol32(float* Sm, float shift, float* Rm, float* Ri, int* f
 constexpr int kHOrthRows = 32;
 __global__ void __launch_bounds__(kHThreads)
 huge_orth_sweep_kernel(float* __restrict__ V, float* __restrict__ W, const float* __restrict__ pin,
-                       float* __restrict__ pout, int nn, int pass, HugeBlock* __restrict__ hb) {
+                       float* __restrict__ pout, int nn, int order, int pass,
+                       HugeBlock* __restrict__ hb) {
   constexpr int NT = kHThreads, PER = kHOrthRows * kHP / NT;
   __shared__ float Xin[kHOrthRows * 33];
   __shared__ float Sm[kHP * 33];
@@ -429,7 +421,7 @@ huge_orth_sweep_kernel(float* __restrict__ V, float* __restrict__ W, const float
     if (pass == 1) {
       float tr = 0.f;
       for (int i = 0; i < kHP; ++i) tr += Sm[i * 33 + i];
-      shift = 11.f * (float)((double)nn * kHP + kHP * (kHP + 1)) * FLT_EPSILON * tr;
+      shift = 11.f * (float)((double)order * kHP + kHP * (kHP + 1)) * FLT_EPSILON * tr;
     }
     ok = huge_chol32(Sm, shift, Rm, Ri, &flag);
   }
@@ -437,7 +429,7 @@ huge_orth_sweep_kernel(float* __restrict__ V, float* __restrict__ W, const float
     for (int j = 0; j < PER; ++j) {
       const int e = tid + j * NT;
       const int r = r0 + (e >> 5), cc = e & 31;
-      if (r < nn) Vb[(size_t)r * kHP + cc] = huge_hash((uint32_t)r + 977u * b, (uint32_t)cc + 0xB0Bu);
+      if (r < order) Vb[(size_t)r * kHP + cc] = huge_hash((uint32_t)r + 977u * b, (uint32_t)cc + 0xB0Bu);
     }
     if (chunk == 0 && tid == 0) hb[b].orth_fail = 1;
     return;
@@ -644,20 +636,12 @@ huge_rr_kernel(const float* __restrict__ V, const float* __restrict__ W, float* 
     // above tau converge slowly; they need this accuracy all the same, since
     // the consensus step carries their error into every scale.
     int conv = 1;
-    float trb = 0.f, th0 = 0.f;
+    float th0 = 0.f;
     for (int q = 0; q < ku; ++q) th0 = fmaxf(th0, Bm[q * kHK + q]);
     for (int q = 0; q < ku; ++q) {
-      trb += Bm[q * kHK + q];
       if (rq[q] > fmaxf(3e-4f * thr, 4e-6f * th0)) conv = 0;
     }
-    // Certificate bound: ||P G P||_2 < c proves, by Cauchy interlacing, that
-    // G has at most ku eigenvalues above c (and the ku Ritz values above
-    // tau^2 are lower bounds of ku eigenvalues), so exactly the kept pairs
-    // lie above tau^2.  c = tau^2 less the rounding of forming X = P G P,
-    // (2 ku + 4) eps (||G||_F + 2 sqrt(ku) ||What||_F); the certificate
-    // accounts for its own rounding.
-    const float xf = h.gF + 2.f * sqrtf((float)ku) * sqrtf(wsum);
-    h.c = thr - 1.1f * FLT_EPSILON * (float)(2 * ku + 4) * xf;
+    h.c = cert_bound(thr, h.gF, ku, wsum);
     h.ku = ku;
     h.k = k;
     h.conv = conv;
@@ -670,7 +654,7 @@ huge_rr_kernel(const float* __restrict__ V, const float* __restrict__ W, float* 
 // and the nuclear-norm sum.
 __global__ void __launch_bounds__(kHThreads)
 huge_final_kernel(ScaleLaunch a, const float* __restrict__ U, float* __restrict__ Y, int* kout,
-                  int nn, const HugeBlock* __restrict__ hb) {
+                  int np, const HugeBlock* __restrict__ hb) {
   __shared__ int sel[kHK];
   __shared__ float fs[kHK];
   __shared__ int ks;
@@ -710,9 +694,9 @@ huge_final_kernel(ScaleLaunch a, const float* __restrict__ U, float* __restrict_
   __syncthreads();
   const int k = ks;
   if (k == 0) return;
-  const float* Ub = U + (size_t)b * nn * kHK;
-  float* Yb = Y + (size_t)b * nn * kHK;
-  for (int e = tid; e < nn * kHK; e += kHThreads) {
+  const float* Ub = U + (size_t)b * np * kHK;
+  float* Yb = Y + (size_t)b * np * kHK;
+  for (int e = tid; e < np * kHK; e += kHThreads) {
     const int r = e / kHK, c = e - r * kHK;
     Yb[e] = c < k ? Ub[(size_t)r * kHK + sel[c]] * fs[c] : 0.f;
   }
@@ -725,14 +709,14 @@ huge_final_kernel(ScaleLaunch a, const float* __restrict__ U, float* __restrict_
 constexpr int kHRebRows = 32;
 template <bool ST>
 __global__ void __launch_bounds__(kHThreads)
-huge_rebuild_kernel(ScaleLaunch a, const float* __restrict__ Y, const int* __restrict__ kin) {
+huge_rebuild_kernel(ScaleLaunch a, const float* __restrict__ Y, int np, const int* __restrict__ kin) {
   const int b = blockIdx.y;
   const int k = kin[b];
   const BlockGeom g = block_geom_t<ST>(a, b);
   const int mm = g.mm(), nn = g.nn();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int RPW = kHRebRows / (kHThreads / 32);
-  const float* Yb = Y + (size_t)b * nn * kHK;
+  const float* Yb = Y + (size_t)b * np * kHK;
   for (int rr = 0; rr < RPW; ++rr) {
     const int i = blockIdx.x * kHRebRows + warp * RPW + rr;
     if (i >= mm) break;
@@ -783,15 +767,15 @@ static char* halign(char* p) { return (char*)(((uintptr_t)p + 255) & ~(uintptr_t
 
 size_t huge_workspace_bytes(int M, int N, int m, int n) {
   const HugeDims d = huge_dims(M, N, m, n);
-  const size_t B = (size_t)d.nblocks, nn = (size_t)d.nn;
+  const size_t B = (size_t)d.nblocks, np = (size_t)d.T * kHT;
   size_t bytes = 0;
   bytes += sizeof(float) * B * d.chunks * d.ntiles * kHT * kHT;  // Gram partials
-  bytes += sizeof(float) * B * nn * nn;                          // G
+  bytes += sizeof(float) * B * np * np;                          // G
   bytes += 2 * B * cert_matrix_bytes(d.nn);                      // certificate matrices
   bytes += sizeof(double) * B * cert_fpart_count(d.nn);
   bytes += 2 * sizeof(float) * B * d.ntiles;                     // tile sums
-  bytes += 2 * sizeof(float) * B * nn * kHP;                     // V, W
-  bytes += 3 * sizeof(float) * B * nn * kHK;                     // U, What, V_f
+  bytes += 2 * sizeof(float) * B * np * kHP;                     // V, W
+  bytes += 3 * sizeof(float) * B * np * kHK;                     // U, What, V_f
   bytes += sizeof(HugeBlock) * B + sizeof(int) * B;
   bytes += 16 * 256;
   return bytes;
@@ -801,7 +785,7 @@ BigWorkspace carve_huge_workspace(void* base, int M, int N, int m, int n) {
   BigWorkspace w{};
   if (!base) return w;
   const HugeDims d = huge_dims(M, N, m, n);
-  const size_t B = (size_t)d.nblocks, nn = (size_t)d.nn;
+  const size_t B = (size_t)d.nblocks, np = (size_t)d.T * kHT;
   char* p = halign((char*)base);
   auto take = [&](size_t bytes) {
     char* q = p;
@@ -809,17 +793,17 @@ BigWorkspace carve_huge_workspace(void* base, int M, int N, int m, int n) {
     return q;
   };
   w.part = (float*)take(sizeof(float) * B * d.chunks * d.ntiles * kHT * kHT);
-  w.G = (float*)take(sizeof(float) * B * nn * nn);
+  w.G = (float*)take(sizeof(float) * B * np * np);
   w.Ma = take(B * cert_matrix_bytes(d.nn));
   w.Mb = take(B * cert_matrix_bytes(d.nn));
   w.fpart = (double*)take(sizeof(double) * B * cert_fpart_count(d.nn));
   w.tstat = (float*)take(2 * sizeof(float) * B * d.ntiles);
-  w.V = (float*)take(sizeof(float) * B * nn * kHP);
-  w.Wv = (float*)take(sizeof(float) * B * nn * kHP);
-  w.U = (float*)take(sizeof(float) * B * nn * kHK);
-  w.GU = (float*)take(sizeof(float) * B * nn * kHK);
-  w.Y = (float*)take(sizeof(float) * B * nn * kHK);
-  w.ystride = nn * kHK;
+  w.V = (float*)take(sizeof(float) * B * np * kHP);
+  w.Wv = (float*)take(sizeof(float) * B * np * kHP);
+  w.U = (float*)take(sizeof(float) * B * np * kHK);
+  w.GU = (float*)take(sizeof(float) * B * np * kHK);
+  w.Y = (float*)take(sizeof(float) * B * np * kHK);
+  w.ystride = np * kHK;
   w.hb = take(sizeof(HugeBlock) * B);
   w.k = (int*)take(sizeof(int) * B);
   return w;
@@ -829,9 +813,9 @@ BigWorkspace carve_huge_workspace(void* base, int M, int N, int m, int n) {
 cudaError_t reset_huge_basis(const BigWorkspace& w, int M, int N, int m, int n, cudaStream_t st) {
   if (!w.V) return cudaSuccess;
   const HugeDims d = huge_dims(M, N, m, n);
-  const size_t total = (size_t)d.nblocks * d.nn * kHP;
+  const size_t total = (size_t)d.nblocks * d.T * kHT * kHP;
   const int grid = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
-  huge_init_basis_kernel<<<grid, 256, 0, st>>>(w.V, total, d.nn);
+  huge_init_basis_kernel<<<grid, 256, 0, st>>>(w.V, total, d.nn, d.T * kHT);
   return cudaGetLastError();
 }
 
@@ -847,7 +831,7 @@ cudaError_t launch_huge(const ScaleLaunch& s, const BigWorkspace& ws, cudaStream
     if (cudaError_t e_ = prof->after(st)) return e_;
   HugeBlock* hb = (HugeBlock*)ws.hb;
   const float thr = s.tau * s.tau;
-  const int B = d.nblocks, nn = d.nn;
+  const int B = d.nblocks, nn = d.nn, np = d.T * kHT;
   PROF_BEFORE(KK_GRAM)
   if (gram_tc_eligible(s) && !gram_fp32_forced()) {
     // tensor-core Gram (k_gram_tc.cu), partial sums in the same 64 x 64 tile
@@ -863,7 +847,7 @@ cudaError_t launch_huge(const ScaleLaunch& s, const BigWorkspace& ws, cudaStream
                                                                       d.chunks, hb);
   PROF_AFTER()
   PROF_BEFORE(KK_GRAM_REDUCE)
-  huge_gram_finish_kernel<<<dim3(d.ntiles, B), kHThreads, 0, st>>>(ws.part, ws.G, ws.tstat, nn,
+  huge_gram_finish_kernel<<<dim3(d.ntiles, B), kHThreads, 0, st>>>(ws.part, ws.G, ws.tstat, np,
                                                                    d.chunks);
   PROF_AFTER()
   if (after_gram)
@@ -876,45 +860,52 @@ cudaError_t launch_huge(const ScaleLaunch& s, const BigWorkspace& ws, cudaStream
   // blocks whose Ritz residuals are still large
   const bool full = (s.m == launch_rows(s) && s.n == s.N);
   const bool warm = s.warm_start && (full || !s.shift);
-  const int rounds[3] = {warm ? 2 : 6, 4, 8};
-  const dim3 gv_grid((nn + kHGvRows - 1) / kHGvRows, B);
-  const int orth_chunks = (nn + kHOrthRows - 1) / kHOrthRows;
-  for (int r = 0; r < 3; ++r) {
-    for (int st_i = 0; st_i < rounds[r]; ++st_i) {
-      PROF_BEFORE(KK_SUBSPACE)
-      huge_gv_kernel<<<gv_grid, kHThreads, 0, st>>>(ws.G, ws.V, ws.Wv, nn, hb);
-      PROF_AFTER()
-      for (int pass = 0; pass < 4; ++pass) {
-        // S partials alternate between the two halves of the Gram partial
-        // buffer (free once G is formed)
-        float* pa = ws.part;
-        float* pb = ws.part + (size_t)B * orth_chunks * (kHP * kHP);
+  if (subspace_cluster_path(np)) {
+    PROF_BEFORE(KK_SUBSPACE)
+    if (cudaError_t e_ = launch_subspace(ws.G, ws.V, ws.U, ws.GU, nn, np, thr, warm ? 2 : 6, hb, B, st))
+      return e_;
+    PROF_AFTER()
+  } else {
+    const int rounds[3] = {warm ? 2 : 6, 4, 8};
+    const dim3 gv_grid((np + kHGvRows - 1) / kHGvRows, B);
+    const int orth_chunks = (np + kHOrthRows - 1) / kHOrthRows;
+    for (int r = 0; r < 3; ++r) {
+      for (int st_i = 0; st_i < rounds[r]; ++st_i) {
         PROF_BEFORE(KK_SUBSPACE)
-        huge_orth_sweep_kernel<<<dim3(orth_chunks, B), kHThreads, 0, st>>>(
-            ws.V, ws.Wv, (pass & 1) ? pa : pb, (pass & 1) ? pb : pa, nn, pass, hb);
+        huge_gv_kernel<<<gv_grid, kHThreads, 0, st>>>(ws.G, ws.V, ws.Wv, np, hb);
         PROF_AFTER()
+        for (int pass = 0; pass < 4; ++pass) {
+          // S partials alternate between the two halves of the Gram partial
+          // buffer (free once G is formed)
+          float* pa = ws.part;
+          float* pb = ws.part + (size_t)B * orth_chunks * (kHP * kHP);
+          PROF_BEFORE(KK_SUBSPACE)
+          huge_orth_sweep_kernel<<<dim3(orth_chunks, B), kHThreads, 0, st>>>(
+              ws.V, ws.Wv, (pass & 1) ? pa : pb, (pass & 1) ? pb : pa, np, nn, pass, hb);
+          PROF_AFTER()
+        }
       }
+      PROF_BEFORE(KK_SUBSPACE)
+      huge_gv_kernel<<<gv_grid, kHThreads, 0, st>>>(ws.G, ws.V, ws.Wv, np, hb);
+      PROF_AFTER()
+      PROF_BEFORE(KK_SUBSPACE)
+      huge_rr_kernel<<<B, kHBlockThreads, 0, st>>>(ws.V, ws.Wv, ws.U, ws.GU, np, thr, hb);
+      PROF_AFTER()
     }
-    PROF_BEFORE(KK_SUBSPACE)
-    huge_gv_kernel<<<gv_grid, kHThreads, 0, st>>>(ws.G, ws.V, ws.Wv, nn, hb);
-    PROF_AFTER()
-    PROF_BEFORE(KK_SUBSPACE)
-    huge_rr_kernel<<<B, kHBlockThreads, 0, st>>>(ws.V, ws.Wv, ws.U, ws.GU, nn, thr, hb);
-    PROF_AFTER()
   }
   if (cudaError_t e_ = launch_cert(ws.G, ws.U, ws.GU, ws.Ma, ws.Mb, ws.fpart, hb, nn, B, s.err, st,
                                    prof))
     return e_;
   PROF_BEFORE(KK_EIG)
-  huge_final_kernel<<<B, kHThreads, 0, st>>>(s, ws.U, ws.Y, ws.k, nn, hb);
+  huge_final_kernel<<<B, kHThreads, 0, st>>>(s, ws.U, ws.Y, ws.k, np, hb);
   PROF_AFTER()
   PROF_BEFORE(KK_REBUILD)
   if (s.fw || s.rows)
-    huge_rebuild_kernel<true><<<dim3((d.mm + kHRebRows - 1) / kHRebRows, B), kHThreads, 0, st>>>(s, ws.Y,
-                                                                                         ws.k);
+    huge_rebuild_kernel<true><<<dim3((d.mm + kHRebRows - 1) / kHRebRows, B), kHThreads, 0, st>>>(
+        s, ws.Y, np, ws.k);
   else
-    huge_rebuild_kernel<false><<<dim3((d.mm + kHRebRows - 1) / kHRebRows, B), kHThreads, 0, st>>>(s, ws.Y,
-                                                                                         ws.k);
+    huge_rebuild_kernel<false><<<dim3((d.mm + kHRebRows - 1) / kHRebRows, B), kHThreads, 0, st>>>(
+        s, ws.Y, np, ws.k);
   PROF_AFTER()
 #undef PROF_BEFORE
 #undef PROF_AFTER

@@ -170,8 +170,8 @@ cert_form_kernel(const float* __restrict__ G, const float* __restrict__ U,
   const int ku = h.ku;
   int ta, tc;
   tile_of(t, &ta, &tc);
-  const float* Ub = U + (size_t)b * nn * kHK;
-  const float* Wb = Wh + (size_t)b * nn * kHK;
+  const float* Ub = U + (size_t)b * np * kHK;
+  const float* Wb = Wh + (size_t)b * np * kHK;
   for (int e = tid; e < kFT * kHK; e += kFThreads) {
     const int x = e / kHK, q = e - x * kHK;
     const int gi = ta * kFT + x, gj = tc * kFT + x;
@@ -182,7 +182,7 @@ cert_form_kernel(const float* __restrict__ G, const float* __restrict__ U,
     Wj[x][q] = qj ? Wb[(size_t)gj * kHK + q] : 0.f;
   }
   __syncthreads();
-  const float* Gb = G + (size_t)b * nn * nn;
+  const float* Gb = G + (size_t)b * np * np;
   __half* Mb = M0 + (size_t)b * np * np;
   float f2 = 0.f;
 #pragma unroll 4
@@ -191,7 +191,7 @@ cert_form_kernel(const float* __restrict__ G, const float* __restrict__ U,
     const int i = ta * kFT + x, j = tc * kFT + y;
     float v = 0.f;
     if (i < nn && j < nn) {
-      v = Gb[(size_t)i * nn + j];
+      v = Gb[(size_t)i * np + j];
       for (int q = 0; q < ku; ++q) {
         v = fmaf(-Ui[x][q], Wj[y][q], v);
         v = fmaf(-Wi[x][q], Uj[y][q], v);
