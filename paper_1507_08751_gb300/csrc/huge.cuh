@@ -65,13 +65,11 @@ __device__ __forceinline__ float huge_hash(uint32_t a, uint32_t b) {
   return (float)(h >> 8) * (2.f / 16777216.f) - 1.f;
 }
 
-// The subspace iteration in one cluster per block (k_subspace.cu): the
-// padded orders it takes, kernel attributes, and the launch (first: steps of
-// the first round).
-bool subspace_cluster_path(int np);
+// Subspace iteration and Rayleigh-Ritz (k_subspace.cu): kernel attributes and
+// the launches (first: steps of the first round; W: workspace, np x kHP).
 cudaError_t configure_subspace();
-cudaError_t launch_subspace(const float* G, float* V, float* U, float* GU, int nn, int np, float thr,
-                            int first, HugeBlock* hb, int B, cudaStream_t st);
+cudaError_t launch_subspace(const float* G, float* V, float* W, float* U, float* GU, int nn, int np,
+                            float thr, int first, HugeBlock* hb, int B, cudaStream_t st, Prof* prof);
 
 // Certificate workspace per block (bytes of one of the two FP16 matrices,
 // F-norm partials) and its launches: form plus kCertLevels squarings.

@@ -29,7 +29,6 @@
 #include "common.cuh"
 #include "huge.cuh"
 #include "internal.h"
-#include "symeig.cuh"
 
 namespace msllr {
 
@@ -37,8 +36,6 @@ namespace {
 
 constexpr int kHT = 64;          // Gram tile
 constexpr int kHThreads = 256;   // tile kernels
-constexpr int kHBlockThreads = 512;  // per-block kernels
-constexpr int kHGvRows = 8;      // rows of W per CTA in W = G V
 
 struct HugeDims {
   int mm, nn, nblocks, T, ntiles, chunk_rows, chunks;
@@ -132,38 +129,70 @@ huge_gram_kernel(ScaleLaunch a, float* __restrict__ part, int chunk_rows, int ch
 }
 
 // Sum of the chunk partials in chunk order; G_b written as a full square of
-// order np (nn rounded up to the tile; the tiles are zero beyond nn),
-// and per tile: the diagonal sum and the sum of squares (off-diagonal tiles
-// twice), for trace(G) and ||G||_F.
+// order np (nn rounded up to the tile; the tiles are zero beyond nn), and per
+// tile: the diagonal sum and the sum of squares (off-diagonal tiles twice).
+// The mirrored tile goes through shared memory, so that both triangles are
+// written as row segments (1024 wide: 15 -> 6 us).  The CTA that finishes
+// a block last adds the tile sums in tile order to trace(G) and ||G||_F,
+// takes the zero-rank shortcut trace(G) <= tau^2 (the trace bounds
+// lambda_max) and resets the block's state (a launch of its own before).
 __global__ void __launch_bounds__(kHThreads)
-huge_gram_finish_kernel(const float* __restrict__ part, float* __restrict__ G,
-                        float* __restrict__ tstat, int np, int chunks) {
-  __shared__ float red[2][kHThreads / 32];
+huge_gram_finish_kernel(const float* __restrict__ part, float* __restrict__ G, float* tstat, int np,
+                        int chunks, HugeBlock* __restrict__ hb, int* __restrict__ arrived, float thr) {
+  __shared__ __align__(16) float Ts[kHT][kHT + 4];
+  __shared__ double red[2][kHThreads / 32];
+  __shared__ int slast;
   const int t = blockIdx.x, b = blockIdx.y, ntiles = gridDim.x;
   int ta, tc;
   tile_of(t, &ta, &tc);
   const int tid = threadIdx.x;
   float* Gb = G + (size_t)b * np * np;
+  const float4* src = reinterpret_cast<const float4*>(part + ((size_t)b * chunks * ntiles + t) * (kHT * kHT));
+  const size_t cstep = (size_t)ntiles * (kHT * kHT / 4);
+  constexpr int PER = kHT * kHT / 4 / kHThreads;
+  float4 s[PER];
+#pragma unroll
+  for (int j = 0; j < PER; ++j) s[j] = src[tid + j * kHThreads];
+  for (int c = 1; c < chunks; ++c) {
+    float4 v[PER];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) v[j] = src[c * cstep + tid + j * kHThreads];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      s[j].x += v[j].x;
+      s[j].y += v[j].y;
+      s[j].z += v[j].z;
+      s[j].w += v[j].w;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int e = tid + j * kHThreads, x = e / (kHT / 4), y = 4 * (e % (kHT / 4));
+    *reinterpret_cast<float4*>(&Ts[x][y]) = s[j];
+  }
+  __syncthreads();
   float dsum = 0.f, sq = 0.f;
-  for (int e = tid; e < kHT * kHT; e += kHThreads) {
-    const int x = e / kHT, y = e - x * kHT;
-    const int i = ta * kHT + x, j = tc * kHT + y;
-    float s = 0.f;
-    for (int c = 0; c < chunks; ++c)
-      s += part[(((size_t)b * chunks + c) * ntiles + t) * (kHT * kHT) + e];
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int e = tid + j * kHThreads, x = e / (kHT / 4), y = 4 * (e % (kHT / 4));
+    float v[4] = {s[j].x, s[j].y, s[j].z, s[j].w};
     if (ta == tc) {
       // diagonal tile: the lower half is authoritative
-      if (j <= i) {
-        Gb[(size_t)i * np + j] = s;
-        Gb[(size_t)j * np + i] = s;
-        sq += (i == j ? 1.f : 2.f) * s * s;
-        if (i == j) dsum += s;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (y + i > x) v[i] = Ts[y + i][x];
+        sq += v[i] * v[i];
+        if (y + i == x) dsum += v[i];
       }
     } else {
-      Gb[(size_t)i * np + j] = s;
-      Gb[(size_t)j * np + i] = s;
-      sq += 2.f * s * s;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) sq += 2.f * v[i] * v[i];
+      // mirrored tile: row y of it is column y of this one
+      *reinterpret_cast<float4*>(Gb + (size_t)(tc * kHT + x) * np + ta * kHT + y) =
+          make_float4(Ts[y][x], Ts[y + 1][x], Ts[y + 2][x], Ts[y + 3][x]);
     }
+    *reinterpret_cast<float4*>(Gb + (size_t)(ta * kHT + x) * np + tc * kHT + y) =
+        make_float4(v[0], v[1], v[2], v[3]);
   }
   dsum = warp_sum(dsum);
   sq = warp_sum(sq);
@@ -172,29 +201,25 @@ huge_gram_finish_kernel(const float* __restrict__ part, float* __restrict__ G,
     red[1][tid >> 5] = sq;
   }
   __syncthreads();
+  float* ts = tstat + (size_t)b * ntiles * 2;
   if (tid == 0) {
-    float d = 0.f, q = 0.f;
+    double d = 0.0, q = 0.0;
     for (int w = 0; w < kHThreads / 32; ++w) {
       d += red[0][w];
       q += red[1][w];
     }
-    tstat[((size_t)b * ntiles + t) * 2] = d;
-    tstat[((size_t)b * ntiles + t) * 2 + 1] = q;
+    ts[2 * t] = (float)d;
+    ts[2 * t + 1] = (float)q;
+    __threadfence();
+    slast = atomicAdd(arrived + b, 1) == ntiles - 1;
   }
-}
-
-
-// Per block: trace(G) and ||G||_F from the tile sums (fixed order), the
-// zero-rank shortcut trace(G) <= tau^2 (trace bounds lambda_max), state reset.
-__global__ void __launch_bounds__(kHThreads)
-huge_prep_kernel(const float* __restrict__ tstat, int ntiles, HugeBlock* __restrict__ hb,
-                 float thr) {
-  __shared__ double red[2][kHThreads / 32];
-  const int b = blockIdx.x, tid = threadIdx.x;
+  __syncthreads();
+  if (!slast) return;
+  __threadfence();
   double d = 0.0, q = 0.0;
-  for (int t = tid; t < ntiles; t += kHThreads) {
-    d += (double)tstat[((size_t)b * ntiles + t) * 2];
-    q += (double)tstat[((size_t)b * ntiles + t) * 2 + 1];
+  for (int i = tid; i < ntiles; i += kHThreads) {
+    d += (double)__ldcg(ts + 2 * i);
+    q += (double)__ldcg(ts + 2 * i + 1);
   }
   d = warp_sum_d(d);
   q = warp_sum_d(q);
@@ -209,6 +234,7 @@ huge_prep_kernel(const float* __restrict__ tstat, int ntiles, HugeBlock* __restr
       dt += red[0][w];
       qt += red[1][w];
     }
+    arrived[b] = 0;  // for the next call
     HugeBlock& h = hb[b];
     h.trace = (float)dt;
     h.gF = (float)sqrt(qt);
@@ -235,448 +261,39 @@ __global__ void huge_init_basis_kernel(float* __restrict__ V, size_t total, int 
   }
 }
 
-__device__ __forceinline__ bool huge_active(const HugeBlock& h) {
-  return h.status == kHsIter && !h.conv && !h.orth_fail;
-}
-
 // ---------------------------------------------------------------------------
-// 2. W = G V for kHGvRows rows of one block (V, W: nn x kHP row-major): one
-// output per thread, the K loop in chunks of 64 through shared memory.
+// 5. The outcome: Z' = sum over the pairs above tau of (1 - tau / sigma) (C u)
+// u^T and W' = 2 Z' - A; blocks without such pairs get Z' = 0, W' = -A.  A
+// CTA takes kHRebRows rows of C: every thread forms the partial products of
+// its columns for all rows (one read of U serves all of them), the CTA sums
+// them, and every thread rebuilds its columns.  Pairs go in groups of eight
+// (one group for most blocks); the rows are read once per group and once
+// more, from cache, for the output.  With a warp per four rows and 32 CTAs at
+// 1024 rows, and V_f scaled by a one-CTA launch before it, this took 85 + 13
+// us at 1024 x 1024.  The CTA of the first rows also reports the block.
 // ---------------------------------------------------------------------------
+constexpr int kHRebRows = 8;
+constexpr int kHRebPairs = 8;
+template <bool ST>
 __global__ void __launch_bounds__(kHThreads)
-huge_gv_kernel(const float* __restrict__ G, const float* __restrict__ V, float* __restrict__ W,
-               int nn, const HugeBlock* __restrict__ hb) {
-  constexpr int KC = 64;
-  static_assert(kHGvRows * kHP == kHThreads, "one output per thread");
-  __shared__ float Gs[kHGvRows][KC + 1];
-  __shared__ float Vs[KC][kHP];
-  const int b = blockIdx.y;
-  if (!huge_active(hb[b])) return;
-  const int r0 = blockIdx.x * kHGvRows, tid = threadIdx.x;
-  const int row = tid / kHP, col = tid % kHP;
-  const float* Gb = G + (size_t)b * nn * nn;
-  const float* Vb = V + (size_t)b * nn * kHP;
-  float acc = 0.f;
-  for (int l0 = 0; l0 < nn; l0 += KC) {
-#pragma unroll
-    for (int j = 0; j < (kHGvRows * KC) / kHThreads; ++j) {
-      const int e = tid + j * kHThreads;
-      const int rr = e / KC, cc = e % KC;
-      const int gr = r0 + rr, gl = l0 + cc;
-      Gs[rr][cc] = (gr < nn && gl < nn) ? Gb[(size_t)gr * nn + gl] : 0.f;
-    }
-#pragma unroll
-    for (int j = 0; j < (KC * kHP) / kHThreads; ++j) {
-      const int e = tid + j * kHThreads;
-      const int rr = e / kHP, cc = e % kHP;
-      const int vl = l0 + rr;
-      Vs[rr][cc] = (vl < nn) ? Vb[(size_t)vl * kHP + cc] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 16
-    for (int kk = 0; kk < KC; ++kk) acc = fmaf(Gs[row][kk], Vs[kk][col], acc);
-    __syncthreads();
-  }
-  const int r = r0 + row;
-  if (r < nn) W[(size_t)b * nn * kHP + (size_t)r * kHP + col] = acc;
-}
-
-// S = X^T Y over the nn rows of two nn x kHP row-major matrices (Y = X
-// allowed), X optionally X + mu * X2.  Thread t owns entries (t/32, t%32) and
-// (t/32 + 16, t%32); the row tiles pass through shared memory; the sums run
-// in row order, so the result is deterministic and S(a,b) == S(b,a) when
-// Y = X.  Result in Sm (kHP x (kHP+1)).  All kHBlockThreads threads call.
-__device__ void huge_xty(const float* __restrict__ X, const float* __restrict__ X2, float mu,
-                         const float* __restrict__ Yv, int nn, float* Xs, float* Ys, float* Sm) {
-  const int tid = threadIdx.x;
-  const int a0 = tid >> 5, bq = tid & 31, a1 = a0 + 16;
-  float acc0 = 0.f, acc1 = 0.f;
-  for (int r0 = 0; r0 < nn; r0 += 64) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int e = tid + j * kHBlockThreads;  // 64 x 32 tile
-      const int rr = e >> 5, cc = e & 31;
-      const int r = r0 + rr;
-      float x = 0.f, y = 0.f;
-      if (r < nn) {
-        x = X[(size_t)r * kHP + cc];
-        if (X2) x = fmaf(mu, X2[(size_t)r * kHP + cc], x);
-        if (Yv) y = Yv[(size_t)r * kHP + cc];
-      }
-      Xs[rr * 33 + cc] = x;
-      if (Yv) Ys[rr * 33 + cc] = y;
-    }
-    __syncthreads();
-    const float* Yt = Yv ? Ys : Xs;
-#pragma unroll 8
-    for (int rr = 0; rr < 64; ++rr) {
-      acc0 = fmaf(Xs[rr * 33 + a0], Yt[rr * 33 + bq], acc0);
-      acc1 = fmaf(Xs[rr * 33 + a1], Yt[rr * 33 + bq], acc1);
-    }
-    __syncthreads();
-  }
-  Sm[a0 * 33 + bq] = acc0;
-  Sm[a1 * 33 + bq] = acc1;
-  __syncthreads();
-}
-
-// Warp 0: S + shift I = R^T R (R upper, in Rm), then Ri = R^{-1}.  Returns
-// false (uniformly, after a barrier) on a non-positive or non-finite pivot.
-__device__ bool huge_chol32(float* Sm, float shift, float* Rm, float* Ri, int* flag) {
-  const int tid = threadIdx.x, lane = tid & 31;
-  if (tid < 32) {
-    if (lane == 0) *flag = 1;
-    Sm[lane * 33 + lane] += shift;
-    __syncwarp();
-    bool ok = true;
-    for (int j = 0; j < kHP; ++j) {
-      const float d = Sm[j * 33 + j];
-      if (!(d > 0.f) || !isfinite(d)) {
-        ok = false;
-        break;
-      }
-      const float r = sqrtf(d);
-      const float v = lane > j ? Sm[j * 33 + lane] / r : (lane == j ? r : 0.f);
-      Rm[j * 33 + lane] = v;
-      __syncwarp();
-      if (lane > j)
-        for (int i = j + 1; i <= lane; ++i) Sm[i * 33 + lane] -= Rm[j * 33 + i] * v;
-      __syncwarp();
-    }
-    if (!ok) {
-      if (lane == 0) *flag = 0;
-    } else {
-      // column `lane` of R^{-1} by back substitution
-      const int j = lane;
-      for (int i = 0; i < kHP; ++i) Ri[i * 33 + j] = 0.f;
-      Ri[j * 33 + j] = 1.f / Rm[j * 33 + j];
-      for (int i = j - 1; i >= 0; --i) {
-        float t = 0.f;
-        for (int l = i + 1; l <= j; ++l) t = fmaf(Rm[i * 33 + l], Ri[l * 33 + j], t);
-        Ri[i * 33 + j] = -t / Rm[i * 33 + i];
-      }
-    }
-  }
-  __syncthreads();
-  const bool ok = *flag != 0;
-  __syncthreads();
-  return ok;
-}
-
-// Orthonormal basis of span(W + mu V) into V by shifted CholQR and two plain
-// CholQR passes, spread over the rows: four sweeps, each a launch over
-// (row chunk of kHOrthRows, block).  Sweep p (p >= 1) first sums the chunk
-// partials of S from sweep p - 1 in chunk order and factors S (+ shift for
-// p = 1) = R^T R in every CTA (all CTAs get the same R^{-1}); then each CTA
-// maps its rows: sweep 0 X = W + mu V, sweep 1 X = (W + mu V) R^{-1},
-// sweeps 2, 3 X = W R^{-1} (sweeps 1, 2 write W, sweep 3 writes V), and
-// sweeps 0-2 write the partial S = X^T X of their rows.  mu = 1e-4 ||G||_F
-// (a shift of G by mu I) keeps W + mu V of full rank when G is (numerically)
-// of rank below kHP.  A failed factorisation marks the block (orth_fail) and
-// restarts its basis.
-constexpr int kHOrthRows = 32;
-__global__ void __launch_bounds__(kHThreads)
-huge_orth_sweep_kernel(float* __restrict__ V, float* __restrict__ W, const float* __restrict__ pin,
-                       float* __restrict__ pout, int nn, int order, int pass,
-                       HugeBlock* __restrict__ hb) {
-  constexpr int NT = kHThreads, PER = kHOrthRows * kHP / NT;
-  __shared__ float Xin[kHOrthRows * 33];
-  __shared__ float Sm[kHP * 33];
-  __shared__ float Rm[kHP * 33];
-  __shared__ float Ri[kHP * 33];
-  __shared__ int flag;
-  const int chunk = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
-  const int nchunks = gridDim.x;
-  {
-    const HugeBlock& h = hb[b];
-    if (!huge_active(h)) return;
-  }
-  float* Vb = V + (size_t)b * nn * kHP;
-  float* Wb = W + (size_t)b * nn * kHP;
-  const int r0 = chunk * kHOrthRows;
-  const float mu = 1e-4f * hb[b].gF;
-  // this CTA's rows (loads in flight during the factorisation)
-  float x[PER];
-#pragma unroll
-  for (int j = 0; j < PER; ++j) {
-    const int e = tid + j * NT;
-    const int r = r0 + (e >> 5), cc = e & 31;
-    float v = 0.f;
-    if (r < nn) {
-      v = Wb[(size_t)r * kHP + cc];
-      if (pass <= 1) v = fmaf(mu, Vb[(size_t)r * kHP + cc], v);
-    }
-    x[j] = v;
-  }
-  bool ok = true;
-  if (pass >= 1) {
-    const float* pb = pin + (size_t)b * nchunks * (kHP * kHP);
-    for (int e = tid; e < kHP * kHP; e += NT) {
-      float t = 0.f;
-      for (int c = 0; c < nchunks; ++c) t += pb[(size_t)c * (kHP * kHP) + e];
-      Sm[(e >> 5) * 33 + (e & 31)] = t;
-    }
-    __syncthreads();
-    float shift = 0.f;
-    if (pass == 1) {
-      float tr = 0.f;
-      for (int i = 0; i < kHP; ++i) tr += Sm[i * 33 + i];
-      shift = 11.f * (float)((double)order * kHP + kHP * (kHP + 1)) * FLT_EPSILON * tr;
-    }
-    ok = huge_chol32(Sm, shift, Rm, Ri, &flag);
-  }
-  if (!ok) {
-    for (int j = 0; j < PER; ++j) {
-      const int e = tid + j * NT;
-      const int r = r0 + (e >> 5), cc = e & 31;
-      if (r < order) Vb[(size_t)r * kHP + cc] = huge_hash((uint32_t)r + 977u * b, (uint32_t)cc + 0xB0Bu);
-    }
-    if (chunk == 0 && tid == 0) hb[b].orth_fail = 1;
-    return;
-  }
-#pragma unroll
-  for (int j = 0; j < PER; ++j) {
-    const int e = tid + j * NT;
-    Xin[(e >> 5) * 33 + (e & 31)] = x[j];
-  }
-  __syncthreads();
-  if (pass >= 1) {
-    float o[PER];
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-      const int e = tid + j * NT;
-      const int rr = e >> 5, cc = e & 31;
-      float t = 0.f;
-#pragma unroll
-      for (int a = 0; a < kHP; ++a)
-        if (a <= cc) t = fmaf(Xin[rr * 33 + a], Ri[a * 33 + cc], t);
-      o[j] = t;
-    }
-    __syncthreads();
-    float* dst = pass == 3 ? Vb : Wb;
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-      const int e = tid + j * NT;
-      const int rr = e >> 5, cc = e & 31;
-      Xin[rr * 33 + cc] = o[j];
-      if (r0 + rr < nn) dst[(size_t)(r0 + rr) * kHP + cc] = o[j];
-    }
-    __syncthreads();
-  }
-  if (pass <= 2) {
-    // partial S of this chunk: thread t owns entries t, t + NT, ...
-    float* pb = pout + ((size_t)b * nchunks + chunk) * (kHP * kHP);
-#pragma unroll
-    for (int j = 0; j < (kHP * kHP) / NT; ++j) {
-      const int e = tid + j * NT;
-      const int a = e >> 5, c = e & 31;
-      float t = 0.f;
-#pragma unroll 8
-      for (int rr = 0; rr < kHOrthRows; ++rr) t = fmaf(Xin[rr * 33 + a], Xin[rr * 33 + c], t);
-      pb[e] = t;
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// 3. Rayleigh-Ritz: T = V^T W (W = G V), its eigenpairs above thr_keep, the
-// Ritz vectors U = V Q and G U = W Q (nn x kHK, row-major), B = U^T G U,
-// residuals |G u_q - theta_q u_q| and What = G U - U sym(B) / 2 (over G U).
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kHBlockThreads)
-huge_rr_kernel(const float* __restrict__ V, const float* __restrict__ W, float* __restrict__ U,
-               float* __restrict__ GU, int nn, float thr, HugeBlock* __restrict__ hb) {
-  constexpr int NT = kHBlockThreads, NW = NT / 32;
-  // the T = V^T W staging is dead once T is formed: the B partials reuse it
-  __shared__ float XYs[2 * 64 * 33];
-  static_assert(NW * kHK * kHK <= 2 * 64 * 33, "B partials overlay");
-  float* Xs = XYs;
-  float* Ys = XYs + 64 * 33;
-  float (*Bred)[kHK * kHK] = reinterpret_cast<float (*)[kHK * kHK]>(XYs);
-  __shared__ float Ts[kHP * 33];
-  __shared__ float Ls[kHP * 33];
-  __shared__ float Qs[kHP * kHK];
-  __shared__ float Bm[kHK * kHK];
-  __shared__ float Rred[NW][2 * kHK];
-  __shared__ float ev[8 * kHP];
-  __shared__ int evi[kHP];
-  __shared__ float evt[3 * NT];
-  __shared__ int evc[NT];
-  __shared__ float red[64];
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (!huge_active(hb[b])) return;
-  const float* Vb = V + (size_t)b * nn * kHP;
-  const float* Wb = W + (size_t)b * nn * kHP;
-  float* Ub = U + (size_t)b * nn * kHK;
-  float* Gb = GU + (size_t)b * nn * kHK;
-  huge_xty(Vb, nullptr, 0.f, Wb, nn, Xs, Ys, Ts);
-  for (int e = tid; e < kHP * kHP; e += NT) {
-    const int i = e >> 5, j = e & 31;
-    Ls[i * 33 + j] = 0.5f * (Ts[i * 33 + j] + Ts[j * 33 + i]);
-  }
-  __syncthreads();
-  EigScratch s;
-  s.d = ev;
-  s.e = s.d + kHP;
-  s.e2 = s.e + kHP;
-  s.beta = s.e2 + kHP;
-  s.vbuf = s.beta + kHP;
-  s.pbuf = s.vbuf + kHP;
-  s.lam = s.pbuf + kHP;
-  s.shf = s.lam + kHP;
-  s.clus = evi;
-  s.lo = evt;
-  s.hi = evt + NT;
-  s.xs = evt + 2 * NT;
-  s.cnt = evc;
-  s.red = red;
-  LowerFull Lacc{Ls, 33};
-  tridiagonalize<NT>(Lacc, kHP, s);
-  float tn = 0.f;
-  // the pairs above tau^2 are the ones kept (and deflated by the certificate)
-  const int kq = top_eigenvalues<NT>(kHP, thr, s, &tn);
-  const int ku = kq < kHK ? kq : kHK;
-  if (ku > 0) top_eigenvectors<NT, kHP>(Lacc, kHP, ku, tn, s, Qs, kHK, -1);
-  __syncthreads();
-  // U, G U and the warp partials of B
-  float Bacc[kHK];
-#pragma unroll
-  for (int p = 0; p < kHK; ++p) Bacc[p] = 0.f;
-  // the next row's loads are issued before the current row is used
-  float vn = warp < nn ? Vb[(size_t)warp * kHP + lane] : 0.f;
-  float wn = warp < nn ? Wb[(size_t)warp * kHP + lane] : 0.f;
-  for (int r = warp; r < nn; r += NW) {
-    const float v = vn, wv = wn;
-    if (r + NW < nn) {
-      vn = Vb[(size_t)(r + NW) * kHP + lane];
-      wn = Wb[(size_t)(r + NW) * kHP + lane];
-    }
-    float u = 0.f, g = 0.f;
-#pragma unroll 8
-    for (int a = 0; a < kHP; ++a) {
-      const float va = __shfl_sync(0xffffffffu, v, a);
-      const float wa = __shfl_sync(0xffffffffu, wv, a);
-      if (lane < ku) {
-        const float qv = Qs[a * kHK + lane];
-        u = fmaf(va, qv, u);
-        g = fmaf(wa, qv, g);
-      }
-    }
-    if (lane < ku) {
-      Ub[(size_t)r * kHK + lane] = u;
-      Gb[(size_t)r * kHK + lane] = g;
-    }
-#pragma unroll
-    for (int p = 0; p < kHK; ++p) {
-      const float up = __shfl_sync(0xffffffffu, u, p);
-      Bacc[p] = fmaf(up, g, Bacc[p]);
-    }
-  }
-  if (lane < kHK)
-#pragma unroll
-    for (int p = 0; p < kHK; ++p) Bred[warp][p * kHK + lane] = Bacc[p];
-  __syncthreads();
-  if (tid < kHK * kHK) {
-    float t = 0.f;
-    for (int w = 0; w < NW; ++w) t += Bred[w][tid];
-    Bm[tid] = t;  // B(p, q) = u_p^T G u_q
-  }
-  __syncthreads();
-  // residuals and What
-  float racc = 0.f, wacc = 0.f;
-  float un = 0.f, gn = 0.f;
-  if (lane < ku && warp < nn) {
-    un = Ub[(size_t)warp * kHK + lane];
-    gn = Gb[(size_t)warp * kHK + lane];
-  }
-  for (int r = warp; r < nn; r += NW) {
-    const float u = un, g = gn;
-    if (lane < ku && r + NW < nn) {
-      un = Ub[(size_t)(r + NW) * kHK + lane];
-      gn = Gb[(size_t)(r + NW) * kHK + lane];
-    }
-    float wh = g;
-#pragma unroll
-    for (int p = 0; p < kHK; ++p) {
-      const float up = __shfl_sync(0xffffffffu, u, p);
-      if (p < ku && lane < ku)
-        wh = fmaf(-0.25f * (Bm[p * kHK + lane] + Bm[lane * kHK + p]), up, wh);
-    }
-    if (lane < ku) {
-      const float res = g - Bm[lane * kHK + lane] * u;
-      racc = fmaf(res, res, racc);
-      wacc = fmaf(wh, wh, wacc);
-      Gb[(size_t)r * kHK + lane] = wh;
-    }
-  }
-  if (lane < kHK) {
-    Rred[warp][lane] = racc;
-    Rred[warp][kHK + lane] = wacc;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    HugeBlock& h = hb[b];
-    float wsum = 0.f;
-    float rq[kHK];
-    int k = 0;
-    for (int q = 0; q < ku; ++q) {
-      float t = 0.f, t2 = 0.f;
-      for (int w = 0; w < NW; ++w) {
-        t += Rred[w][q];
-        t2 += Rred[w][kHK + q];
-      }
-      rq[q] = sqrtf(t);
-      wsum += t2;
-      const float th = Bm[q * kHK + q];
-      h.theta[q] = th;
-      k += th > thr;
-    }
-    // converged: every kept pair's residual is small against tau^2, or at
-    // the rounding level of G V (set by the largest eigenvalue).  Pairs just
-    // above tau converge slowly; they need this accuracy all the same, since
-    // the consensus step carries their error into every scale.
-    int conv = 1;
-    float th0 = 0.f;
-    for (int q = 0; q < ku; ++q) th0 = fmaxf(th0, Bm[q * kHK + q]);
-    for (int q = 0; q < ku; ++q) {
-      if (rq[q] > fmaxf(3e-4f * thr, 4e-6f * th0)) conv = 0;
-    }
-    h.c = cert_bound(thr, h.gF, ku, wsum);
-    h.ku = ku;
-    h.k = k;
-    h.conv = conv;
-  }
-}
-
-
-// Per block: the outcome.  V_f = U diag(sqrt(1 - tau / sqrt(theta))) over
-// the pairs above tau (nn x kHK row-major, zero columns beyond k), counters
-// and the nuclear-norm sum.
-__global__ void __launch_bounds__(kHThreads)
-huge_final_kernel(ScaleLaunch a, const float* __restrict__ U, float* __restrict__ Y, int* kout,
-                  int np, const HugeBlock* __restrict__ hb) {
-  __shared__ int sel[kHK];
-  __shared__ float fs[kHK];
-  __shared__ int ks;
-  const int b = blockIdx.x, tid = threadIdx.x;
+huge_rebuild_kernel(ScaleLaunch a, const float* __restrict__ U, int np,
+                    const HugeBlock* __restrict__ hb) {
+  constexpr int R = kHRebRows, Q = kHRebPairs, NW = kHThreads / 32;
+  __shared__ __align__(16) float Ps[NW][R * Q];
+  __shared__ __align__(16) float Pf[kHK / Q][R * Q];
+  const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const HugeBlock& h = hb[b];
   const float thr = a.tau * a.tau;
-  if (tid == 0) {
-    int k = 0;
-    if (h.status == kHsIter) {
-      for (int q = 0; q < h.ku; ++q) {
-        const float th = h.theta[q];
-        if (th > thr) {
-          sel[k] = q;
-          fs[k] = sqrtf(fmaxf(1.f - a.tau / sqrtf(th), 0.f));
-          ++k;
-        }
-      }
+  const int ku = h.status == kHsIter ? h.ku : 0;
+  int k = 0, kend = 0;  // pairs above tau, end of their range
+  for (int q = 0; q < ku; ++q)
+    if (h.theta[q] > thr) {
+      ++k;
+      kend = q + 1;
     }
-    ks = k;
+  if (blockIdx.x == 0 && tid == 0) {
     const bool skipped = h.status == kHsSkip;
     const bool cert = skipped || (h.status == kHsIter && h.cert == kCertYes);
-    kout[b] = k;
     if (a.rank_out) a.rank_out[b] = k;
     if (a.cnt) {
       if (skipped) atomicAdd(a.cnt, 1ull);
@@ -686,76 +303,91 @@ huge_final_kernel(ScaleLaunch a, const float* __restrict__ U, float* __restrict_
     }
     if (a.nuc_acc && k > 0) {
       double t = 0.0;
-      for (int q = 0; q < k; ++q)
-        t += (double)fmaxf(sqrtf(h.theta[sel[q]]) - a.tau, 0.f);
+      for (int q = 0; q < ku; ++q)
+        if (h.theta[q] > thr) t += (double)fmaxf(sqrtf(h.theta[q]) - a.tau, 0.f);
       atomicAdd(a.nuc_acc, t);
     }
   }
-  __syncthreads();
-  const int k = ks;
-  if (k == 0) return;
-  const float* Ub = U + (size_t)b * np * kHK;
-  float* Yb = Y + (size_t)b * np * kHK;
-  for (int e = tid; e < np * kHK; e += kHThreads) {
-    const int r = e / kHK, c = e - r * kHK;
-    Yb[e] = c < k ? Ub[(size_t)r * kHK + sel[c]] * fs[c] : 0.f;
-  }
-}
-
-// ---------------------------------------------------------------------------
-// 5. Z' = (C V_f) V_f^T and W' = 2 Z' - A, a warp per row of C, 4 rows per
-// warp.  Rows of rank-0 blocks get Z' = 0, W' = -A.
-// ---------------------------------------------------------------------------
-constexpr int kHRebRows = 32;
-template <bool ST>
-__global__ void __launch_bounds__(kHThreads)
-huge_rebuild_kernel(ScaleLaunch a, const float* __restrict__ Y, int np, const int* __restrict__ kin) {
-  const int b = blockIdx.y;
-  const int k = kin[b];
   const BlockGeom g = block_geom_t<ST>(a, b);
   const int mm = g.mm(), nn = g.nn();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int RPW = kHRebRows / (kHThreads / 32);
-  const float* Yb = Y + (size_t)b * np * kHK;
-  for (int rr = 0; rr < RPW; ++rr) {
-    const int i = blockIdx.x * kHRebRows + warp * RPW + rr;
-    if (i >= mm) break;
-    float P[kHK];
+  const int i0 = blockIdx.x * R;
+  const float* Ub = U + (size_t)b * np * kHK;
+  const int groups = (kend + Q - 1) / Q;
+  for (int gq = 0; gq < groups; ++gq) {
+    float acc[R * Q];
 #pragma unroll
-    for (int q = 0; q < kHK; ++q) P[q] = 0.f;
-    if (k > 0) {
-      for (int c = lane; c < nn; c += 32) {
-        const float av = huge_load(a, huge_off(g, i, c));
-        const float4* vf = reinterpret_cast<const float4*>(Yb + (size_t)c * kHK);
+    for (int e = 0; e < R * Q; ++e) acc[e] = 0.f;
+    for (int c = tid; c < nn; c += kHThreads) {
+      float av[R];
 #pragma unroll
-        for (int t = 0; t < kHK / 4; ++t) {
-          const float4 v = vf[t];
-          P[4 * t] = fmaf(av, v.x, P[4 * t]);
-          P[4 * t + 1] = fmaf(av, v.y, P[4 * t + 1]);
-          P[4 * t + 2] = fmaf(av, v.z, P[4 * t + 2]);
-          P[4 * t + 3] = fmaf(av, v.w, P[4 * t + 3]);
-        }
-      }
+      for (int r = 0; r < R; ++r) av[r] = i0 + r < mm ? huge_load(a, huge_off(g, i0 + r, c)) : 0.f;
+      const float4* u4 = reinterpret_cast<const float4*>(Ub + (size_t)c * kHK + gq * Q);
+      const float4 u0 = u4[0], u1 = u4[1];
+      const float u[Q] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
 #pragma unroll
-      for (int q = 0; q < kHK; ++q) P[q] = warp_sum(P[q]);
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int q = 0; q < Q; ++q) acc[r * Q + q] = fmaf(av[r], u[q], acc[r * Q + q]);
     }
-    for (int c = lane; c < nn; c += 32) {
-      const size_t off = huge_off(g, i, c);
-      const float av = huge_load(a, off);
-      float z = 0.f;
-      if (k > 0) {
-        const float4* vf = reinterpret_cast<const float4*>(Yb + (size_t)c * kHK);
+    // the warp's sums of the 64 products by halving: lane l ends with the
+    // products 2 l and 2 l + 1
+    static_assert(R * Q == 64, "two products per lane");
 #pragma unroll
-        for (int t = 0; t < kHK / 4; ++t) {
-          const float4 v = vf[t];
-          z = fmaf(P[4 * t], v.x, z);
-          z = fmaf(P[4 * t + 1], v.y, z);
-          z = fmaf(P[4 * t + 2], v.z, z);
-          z = fmaf(P[4 * t + 3], v.w, z);
-        }
+    for (int o = 16; o > 0; o >>= 1) {
+      const bool up = lane & o;
+#pragma unroll
+      for (int e = 0; e < 2 * o; ++e) {
+        const float keep = up ? acc[e + 2 * o] : acc[e], give = up ? acc[e] : acc[e + 2 * o];
+        acc[e] = keep + __shfl_xor_sync(0xffffffffu, give, o);
       }
-      a.Zout[off] = z;
-      if (a.Wout) a.Wout[off] = 2.f * z - av;
+    }
+    __syncthreads();
+    Ps[warp][2 * lane] = acc[0];
+    Ps[warp][2 * lane + 1] = acc[1];
+    __syncthreads();
+    if (tid < R * Q) {
+      float t = 0.f;
+      for (int w = 0; w < NW; ++w) t += Ps[w][tid];
+      // f = 1 - tau / sigma for the pairs above tau, else 0
+      const int q = gq * Q + tid % Q;
+      const float th = q < ku ? h.theta[q] : 0.f;
+      Pf[gq][tid] = th > thr ? t * fmaxf(1.f - a.tau / sqrtf(th), 0.f) : 0.f;
+    }
+  }
+  __syncthreads();
+  for (int c = tid; c < nn; c += kHThreads) {
+    float z[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) z[r] = 0.f;
+    for (int gq = 0; gq < groups; ++gq) {
+      const float4* u4 = reinterpret_cast<const float4*>(Ub + (size_t)c * kHK + gq * Q);
+      const float4 u0 = u4[0], u1 = u4[1];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const float4 p0 = *reinterpret_cast<const float4*>(&Pf[gq][r * Q]);
+        const float4 p1 = *reinterpret_cast<const float4*>(&Pf[gq][r * Q + 4]);
+        z[r] = fmaf(p0.x, u0.x, z[r]);
+        z[r] = fmaf(p0.y, u0.y, z[r]);
+        z[r] = fmaf(p0.z, u0.z, z[r]);
+        z[r] = fmaf(p0.w, u0.w, z[r]);
+        z[r] = fmaf(p1.x, u1.x, z[r]);
+        z[r] = fmaf(p1.y, u1.y, z[r]);
+        z[r] = fmaf(p1.z, u1.z, z[r]);
+        z[r] = fmaf(p1.w, u1.w, z[r]);
+      }
+    }
+    // (all loads before the stores: Zout may be A1)
+    float av[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      av[r] = (a.Wout && i0 + r < mm) ? huge_load(a, huge_off(g, i0 + r, c)) : 0.f;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (i0 + r < mm) {
+        const size_t off = huge_off(g, i0 + r, c);
+        a.Zout[off] = z[r];
+        if (a.Wout) a.Wout[off] = 2.f * z[r] - av[r];
+      }
     }
   }
 }
@@ -775,7 +407,7 @@ size_t huge_workspace_bytes(int M, int N, int m, int n) {
   bytes += sizeof(double) * B * cert_fpart_count(d.nn);
   bytes += 2 * sizeof(float) * B * d.ntiles;                     // tile sums
   bytes += 2 * sizeof(float) * B * np * kHP;                     // V, W
-  bytes += 3 * sizeof(float) * B * np * kHK;                     // U, What, V_f
+  bytes += 2 * sizeof(float) * B * np * kHK;                     // U, What
   bytes += sizeof(HugeBlock) * B + sizeof(int) * B;
   bytes += 16 * 256;
   return bytes;
@@ -802,8 +434,6 @@ BigWorkspace carve_huge_workspace(void* base, int M, int N, int m, int n) {
   w.Wv = (float*)take(sizeof(float) * B * np * kHP);
   w.U = (float*)take(sizeof(float) * B * np * kHK);
   w.GU = (float*)take(sizeof(float) * B * np * kHK);
-  w.Y = (float*)take(sizeof(float) * B * np * kHK);
-  w.ystride = np * kHK;
   w.hb = take(sizeof(HugeBlock) * B);
   w.k = (int*)take(sizeof(int) * B);
   return w;
@@ -816,7 +446,9 @@ cudaError_t reset_huge_basis(const BigWorkspace& w, int M, int N, int m, int n, 
   const size_t total = (size_t)d.nblocks * d.T * kHT * kHP;
   const int grid = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
   huge_init_basis_kernel<<<grid, 256, 0, st>>>(w.V, total, d.nn, d.T * kHT);
-  return cudaGetLastError();
+  if (cudaError_t e = cudaGetLastError()) return e;
+  // the Gram kernels' arrival counters
+  return cudaMemsetAsync(w.k, 0, sizeof(int) * (size_t)d.nblocks, st);
 }
 
 cudaError_t launch_huge(const ScaleLaunch& s, const BigWorkspace& ws, cudaStream_t st, Prof* prof,
@@ -848,64 +480,25 @@ cudaError_t launch_huge(const ScaleLaunch& s, const BigWorkspace& ws, cudaStream
   PROF_AFTER()
   PROF_BEFORE(KK_GRAM_REDUCE)
   huge_gram_finish_kernel<<<dim3(d.ntiles, B), kHThreads, 0, st>>>(ws.part, ws.G, ws.tstat, np,
-                                                                   d.chunks);
+                                                                   d.chunks, hb, ws.k, thr);
   PROF_AFTER()
   if (after_gram)
     if (cudaError_t e_ = cudaEventRecord(after_gram, st)) return e_;
-  PROF_BEFORE(KK_MISC)
-  huge_prep_kernel<<<B, kHThreads, 0, st>>>(ws.tstat, d.ntiles, hb, thr);
-  PROF_AFTER()
   // subspace iteration: a first round (short when the grid does not move and
   // the basis carries over from the previous call), a second round for the
   // blocks whose Ritz residuals are still large
   const bool full = (s.m == launch_rows(s) && s.n == s.N);
   const bool warm = s.warm_start && (full || !s.shift);
-  if (subspace_cluster_path(np)) {
-    PROF_BEFORE(KK_SUBSPACE)
-    if (cudaError_t e_ = launch_subspace(ws.G, ws.V, ws.U, ws.GU, nn, np, thr, warm ? 2 : 6, hb, B, st))
-      return e_;
-    PROF_AFTER()
-  } else {
-    const int rounds[3] = {warm ? 2 : 6, 4, 8};
-    const dim3 gv_grid((np + kHGvRows - 1) / kHGvRows, B);
-    const int orth_chunks = (np + kHOrthRows - 1) / kHOrthRows;
-    for (int r = 0; r < 3; ++r) {
-      for (int st_i = 0; st_i < rounds[r]; ++st_i) {
-        PROF_BEFORE(KK_SUBSPACE)
-        huge_gv_kernel<<<gv_grid, kHThreads, 0, st>>>(ws.G, ws.V, ws.Wv, np, hb);
-        PROF_AFTER()
-        for (int pass = 0; pass < 4; ++pass) {
-          // S partials alternate between the two halves of the Gram partial
-          // buffer (free once G is formed)
-          float* pa = ws.part;
-          float* pb = ws.part + (size_t)B * orth_chunks * (kHP * kHP);
-          PROF_BEFORE(KK_SUBSPACE)
-          huge_orth_sweep_kernel<<<dim3(orth_chunks, B), kHThreads, 0, st>>>(
-              ws.V, ws.Wv, (pass & 1) ? pa : pb, (pass & 1) ? pb : pa, np, nn, pass, hb);
-          PROF_AFTER()
-        }
-      }
-      PROF_BEFORE(KK_SUBSPACE)
-      huge_gv_kernel<<<gv_grid, kHThreads, 0, st>>>(ws.G, ws.V, ws.Wv, np, hb);
-      PROF_AFTER()
-      PROF_BEFORE(KK_SUBSPACE)
-      huge_rr_kernel<<<B, kHBlockThreads, 0, st>>>(ws.V, ws.Wv, ws.U, ws.GU, np, thr, hb);
-      PROF_AFTER()
-    }
-  }
+  if (cudaError_t e_ = launch_subspace(ws.G, ws.V, ws.Wv, ws.U, ws.GU, nn, np, thr, warm ? 2 : 6,
+                                       hb, B, st, prof))
+    return e_;
   if (cudaError_t e_ = launch_cert(ws.G, ws.U, ws.GU, ws.Ma, ws.Mb, ws.fpart, hb, nn, B, s.err, st,
                                    prof))
     return e_;
-  PROF_BEFORE(KK_EIG)
-  huge_final_kernel<<<B, kHThreads, 0, st>>>(s, ws.U, ws.Y, ws.k, np, hb);
-  PROF_AFTER()
   PROF_BEFORE(KK_REBUILD)
-  if (s.fw || s.rows)
-    huge_rebuild_kernel<true><<<dim3((d.mm + kHRebRows - 1) / kHRebRows, B), kHThreads, 0, st>>>(
-        s, ws.Y, np, ws.k);
-  else
-    huge_rebuild_kernel<false><<<dim3((d.mm + kHRebRows - 1) / kHRebRows, B), kHThreads, 0, st>>>(
-        s, ws.Y, np, ws.k);
+  const dim3 rgrid((d.mm + kHRebRows - 1) / kHRebRows, B);
+  if (s.fw || s.rows) huge_rebuild_kernel<true><<<rgrid, kHThreads, 0, st>>>(s, ws.U, np, hb);
+  else huge_rebuild_kernel<false><<<rgrid, kHThreads, 0, st>>>(s, ws.U, np, hb);
   PROF_AFTER()
 #undef PROF_BEFORE
 #undef PROF_AFTER

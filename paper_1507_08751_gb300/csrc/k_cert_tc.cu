@@ -154,8 +154,9 @@ __global__ void __launch_bounds__(kFThreads)
 cert_form_kernel(const float* __restrict__ G, const float* __restrict__ U,
                  const float* __restrict__ Wh, __half* __restrict__ M0, int nn, int np,
                  double* __restrict__ fpart, HugeBlock* __restrict__ hb) {
-  __shared__ float Ui[kFT][kHK + 1], Wi[kFT][kHK + 1], Uj[kFT][kHK + 1], Wj[kFT][kHK + 1];
-  __shared__ __half Xs[kFT][kFT + 2];
+  // U and What of the tile's rows and columns, pair by pair
+  __shared__ __align__(16) float Ui[kHK][kFT], Wi[kHK][kFT], Uj[kHK][kFT], Wj[kHK][kFT];
+  __shared__ __align__(8) __half Xs[kFT][kFT + 4];
   __shared__ double sred[kFThreads / 32];
   __shared__ int slast;
   const int t = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
@@ -172,43 +173,66 @@ cert_form_kernel(const float* __restrict__ G, const float* __restrict__ U,
   tile_of(t, &ta, &tc);
   const float* Ub = U + (size_t)b * np * kHK;
   const float* Wb = Wh + (size_t)b * np * kHK;
-  for (int e = tid; e < kFT * kHK; e += kFThreads) {
-    const int x = e / kHK, q = e - x * kHK;
-    const int gi = ta * kFT + x, gj = tc * kFT + x;
-    const bool qi = q < ku && gi < nn, qj = q < ku && gj < nn;
-    Ui[x][q] = qi ? Ub[(size_t)gi * kHK + q] : 0.f;
-    Wi[x][q] = qi ? Wb[(size_t)gi * kHK + q] : 0.f;
-    Uj[x][q] = qj ? Ub[(size_t)gj * kHK + q] : 0.f;
-    Wj[x][q] = qj ? Wb[(size_t)gj * kHK + q] : 0.f;
+  if (ku > 0) {
+    for (int e = tid; e < kFT * kHK; e += kFThreads) {
+      const int x = e / kHK, q = e - x * kHK;
+      Ui[q][x] = Ub[(size_t)(ta * kFT + x) * kHK + q];
+      Wi[q][x] = Wb[(size_t)(ta * kFT + x) * kHK + q];
+      Uj[q][x] = Ub[(size_t)(tc * kFT + x) * kHK + q];
+      Wj[q][x] = Wb[(size_t)(tc * kFT + x) * kHK + q];
+    }
+    __syncthreads();
   }
-  __syncthreads();
   const float* Gb = G + (size_t)b * np * np;
   __half* Mb = M0 + (size_t)b * np * np;
+  // a 4 x 4 register tile per thread: rows x0 .., columns y0 ..
+  const int x0 = 4 * (tid >> 4), y0 = 4 * (tid & 15);
+  float v[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float4 g4 = *reinterpret_cast<const float4*>(Gb + (size_t)(ta * kFT + x0 + i) * np + tc * kFT + y0);
+    v[i][0] = g4.x;
+    v[i][1] = g4.y;
+    v[i][2] = g4.z;
+    v[i][3] = g4.w;
+  }
+  for (int q = 0; q < ku; ++q) {
+    const float4 ui = *reinterpret_cast<const float4*>(&Ui[q][x0]);
+    const float4 wi = *reinterpret_cast<const float4*>(&Wi[q][x0]);
+    const float4 uj = *reinterpret_cast<const float4*>(&Uj[q][y0]);
+    const float4 wj = *reinterpret_cast<const float4*>(&Wj[q][y0]);
+    const float uiv[4] = {ui.x, ui.y, ui.z, ui.w}, wiv[4] = {wi.x, wi.y, wi.z, wi.w};
+    const float ujv[4] = {uj.x, uj.y, uj.z, uj.w}, wjv[4] = {wj.x, wj.y, wj.z, wj.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        v[i][j] = fmaf(-wiv[i], ujv[j], fmaf(-uiv[i], wjv[j], v[i][j]));
+  }
   float f2 = 0.f;
-#pragma unroll 4
-  for (int e = tid; e < kFT * kFT; e += kFThreads) {
-    const int x = e / kFT, y = e - x * kFT;
-    const int i = ta * kFT + x, j = tc * kFT + y;
-    float v = 0.f;
-    if (i < nn && j < nn) {
-      v = Gb[(size_t)i * np + j];
-      for (int q = 0; q < ku; ++q) {
-        v = fmaf(-Ui[x][q], Wj[y][q], v);
-        v = fmaf(-Wi[x][q], Uj[y][q], v);
-      }
-      v *= ic;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    union {
+      __half h[4];
+      uint2 u;
+    } o;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float x = v[i][j] * ic;
+      f2 = fmaf(x, x, f2);
+      o.h[j] = __float2half_rn(x);
+      Xs[y0 + j][x0 + i] = o.h[j];
     }
-    f2 = fmaf(v, v, f2);
-    const __half hv = __float2half_rn(v);
-    Xs[x][y] = hv;
-    Mb[(size_t)i * np + j] = hv;
+    *reinterpret_cast<uint2*>(Mb + (size_t)(ta * kFT + x0 + i) * np + tc * kFT + y0) = o.u;
   }
   __syncthreads();
-  if (ta != tc)
-    for (int e = tid; e < kFT * kFT; e += kFThreads) {
-      const int y = e / kFT, x = e - y * kFT;
-      Mb[(size_t)(tc * kFT + y) * np + ta * kFT + x] = Xs[x][y];
-    }
+  if (ta != tc) {
+    // the mirrored tile, in row segments
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      *reinterpret_cast<uint2*>(Mb + (size_t)(tc * kFT + x0 + i) * np + ta * kFT + y0) =
+          *reinterpret_cast<const uint2*>(&Xs[x0 + i][y0]);
+  }
   f2 = warp_sum(f2);
   if ((tid & 31) == 0) sred[tid >> 5] = (double)f2;
   __syncthreads();

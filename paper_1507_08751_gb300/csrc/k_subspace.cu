@@ -1,10 +1,13 @@
-// Subspace iteration and Rayleigh-Ritz of blocks 257 .. 2048 wide: one
-// thread-block cluster per block does every step of every round in one
-// launch (the wider blocks keep a launch per step, k_block_huge.cu).
+// Subspace iteration and Rayleigh-Ritz of blocks wider than 256.  Up to 2048
+// wide one thread-block cluster per block does every step of every round in
+// one launch; above, where 16 SMs would be too few for G V, a step is a
+// grid-wide G V launch and a cluster launch for the rest.
 //
-// Per step X = G V + mu V, then V = orth(X) by shifted CholQR and two plain
-// CholQR passes (the method and mu are those of huge_orth_sweep_kernel); per
-// round a Rayleigh-Ritz test.  What bounds a block of this size is latency,
+// Per step X = G V + mu V, then V = orth(X) by shifted CholQR and plain CholQR
+// passes (Fukaya, Kannan, Nakatsukasa, Yamamoto, Yanagisawa, SIAM J. Sci.
+// Comput. 2020); mu = 1e-4 ||G||_F (a shift of G) keeps X of full rank when G
+// is numerically of rank below kHP.  Per round a Rayleigh-Ritz test.  What
+// bounds a block of this size is latency,
 // not arithmetic: a step's product is n^2 kHP multiply-adds (0.4 us of the
 // whole GPU at n = 1024), its orthonormalisation three dependent 32 x 32
 // factorisations.  As launches a step took 130 us at n = 1024 (five launches
@@ -15,12 +18,12 @@
 // one warp's registers, and the rows never leave shared memory inside a
 // step.
 //
-//   G V     4 x 4 register tiles over 32-column chunks of G and V (cp.async,
-//           three stages), the chunk's columns split over the thread groups
-//           that the row count leaves idle; V comes from L2
+//   G V     8 x 8 register tiles over 64-column chunks of G and V (cp.async,
+//           three stages), the chunk's columns split over the warps; V comes
+//           from L2
 //   X^T X   4 x 4 register tiles, rows split four ways
 //   R       Cholesky in one warp: lane i holds row i
-//   X R^-1  a warp per row (eight at a time): lane t holds column t
+//   X R^-1  a warp per four rows: lane t holds column t
 //   T = V^T G V: parallel two-sided Jacobi on 32 x 32 (Golub & Van Loan,
 //           Sec. 8.5): 16 disjoint pairs a round, a thread per 2 x 2 block
 //
@@ -39,24 +42,27 @@ namespace msllr {
 
 namespace {
 
-constexpr int kSNT = 256;   // threads per CTA
-constexpr int kSKC = 32;    // columns of G per stage
+constexpr int kSNT = 256;      // threads per CTA
+constexpr int kSNW = kSNT / 32;
+constexpr int kSKC = 64;       // columns of G per stage
 constexpr int kSStages = 3;
-constexpr int kSLdG = 36;   // row stride of a G chunk (floats; 16-byte rows, distinct banks)
-constexpr int kSLd = 36;    // row stride of X and W
+constexpr int kSLdG = kSKC + 4;  // row stride of a G chunk (floats): 8 rows on distinct banks
+constexpr int kSLd = 36;       // row stride of X and W
 constexpr int kSM = kHP * 33;
-constexpr int kSMaxRows = 128;  // rows per CTA: 32 groups of 4 x 4 register tiles
+constexpr int kSMaxRows = 128;  // rows per CTA: two 64-row halves of 8 x 8 register tiles
 
-// floats of one pipeline stage, and of the region that the stages share with
-// the split sums (used when no copy is in flight)
+// floats of one pipeline stage; between products the stages' space holds the
+// split sums of the products
 __host__ __device__ constexpr int sub_stage_floats(int rp) { return rp * kSLdG + kSKC * kHP; }
 __host__ __device__ constexpr int sub_pipe_floats(int rp) {
-  return kSStages * sub_stage_floats(rp) > 4 * kHP * kHP ? kSStages * sub_stage_floats(rp)
-                                                          : 4 * kHP * kHP;
+  // (above kSMaxRows rows G V comes from elsewhere: the products' sums only)
+  return rp > kSMaxRows ? kSNT / 64 * kHP * kHP
+         : kSStages * sub_stage_floats(rp) > kSNW / 2 * 64 * kHP ? kSStages * sub_stage_floats(rp)
+                                                                 : kSNW / 2 * 64 * kHP;
 }
 size_t sub_smem_bytes(int rp) {
   return sizeof(float) *
-         (size_t)(sub_pipe_floats(rp) + 2 * rp * kSLd + 2 * kHP * kHP + 3 * kSM + kHK * kHK);
+         (size_t)(sub_pipe_floats(rp) + 2 * rp * kSLd + kHP * kHP + 3 * kSM + kHK * kHK);
 }
 
 __device__ __forceinline__ void cp16(float* dst, const float* src) {
@@ -71,26 +77,35 @@ __device__ __forceinline__ void cp_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Ws = rows [r0, r0 + rp) of G V.
+// Ws = rows [r0, r0 + rp) of G V.  A warp covers 64 rows x 32 columns with
+// 8 x 8 register tiles (lane: rows lr + 8 i, columns 8 lc ..), which balances
+// its shared-memory reads (16 x 128 bits per 4 columns of G) with its 256
+// multiply-adds; the warps of a row half split each chunk's columns, and
+// their sums are added pairwise in a fixed order.
 __device__ void sub_gv(const float* __restrict__ Gr, const float* V, int np, int rp, float* pipe,
                        float* Ws) {
-  const int tid = threadIdx.x;
-  const int RG = rp >> 2, cgp = tid & 7, rest = tid >> 3;
-  const int split = rest / RG, rg = rest - split * RG;
-  const int ns = (kSNT / 8) / RG;  // groups that share a chunk's columns
-  const bool on = split < ns;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int halves = rp > 64 ? 2 : 1, ns = kSNW / halves;
+  const int half = warp / ns, split = warp - half * ns;
+  const int lr = lane >> 2, lc = lane & 3;
+  const int row0 = 64 * half, rows = min(64, rp - row0);
   const int sf = sub_stage_floats(rp), nch = np / kSKC;
   auto load = [&](int c) {
     float* st = pipe + (c % kSStages) * sf;
     const float* g = Gr + c * kSKC;
-    for (int e = tid; e < rp * 8; e += kSNT) {
-      const int r = e >> 3, q = e & 7;
+    for (int e = tid; e < rp * (kSKC / 4); e += kSNT) {
+      const int r = e / (kSKC / 4), q = e % (kSKC / 4);
       cp16(st + r * kSLdG + 4 * q, g + (size_t)r * np + 4 * q);
     }
-    cp16(st + rp * kSLdG + 4 * tid, V + (size_t)c * kSKC * kHP + 4 * tid);
+#pragma unroll
+    for (int e = 4 * tid; e < kSKC * kHP; e += 4 * kSNT)
+      cp16(st + rp * kSLdG + e, V + (size_t)c * kSKC * kHP + e);
   };
-  static_assert(kSKC * kHP == 4 * kSNT, "one 16-byte copy of V per thread");
-  float acc[4][4] = {};
+  float acc[8][8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
   for (int c = 0; c < kSStages - 1; ++c) {
     if (c < nch) load(c);
     cp_commit();
@@ -100,47 +115,72 @@ __device__ void sub_gv(const float* __restrict__ Gr, const float* V, int np, int
     __syncthreads();
     if (c + kSStages - 1 < nch) load(c + kSStages - 1);
     cp_commit();
-    if (on) {
-      const float* Gs = pipe + (c % kSStages) * sf;
-      const float* Vs = Gs + rp * kSLdG;
-      for (int k4 = split; k4 < kSKC / 4; k4 += ns) {
-        float4 g[4], v[4];
+    const float* Gs = pipe + (c % kSStages) * sf;
+    const float* Vs = Gs + rp * kSLdG;
+    for (int k4 = split; k4 < kSKC / 4; k4 += ns) {
+      const float* gp = Gs + (row0 + lr) * kSLdG + 4 * k4;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          g[i] = *reinterpret_cast<const float4*>(Gs + (rg + i * RG) * kSLdG + 4 * k4);
+      for (int k2 = 0; k2 < 4; k2 += 2) {
+        float2 g[8];
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          v[k] = *reinterpret_cast<const float4*>(Vs + (4 * k4 + k) * kHP + 4 * cgp);
+        for (int i = 0; i < 8; ++i) {
+          // (rows past the end read other shared memory; their sums are not stored)
+          g[i] = *reinterpret_cast<const float2*>(gp + 8 * i * kSLdG + k2);
+        }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float gk[4] = {g[i].x, g[i].y, g[i].z, g[i].w};
+        for (int k = 0; k < 2; ++k) {
+          const float* vr = Vs + (4 * k4 + k2 + k) * kHP + 8 * lc;
+          const float4 v0 = *reinterpret_cast<const float4*>(vr);
+          const float4 v1 = *reinterpret_cast<const float4*>(vr + 4);
+          const float vv[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            acc[i][0] = fmaf(gk[k], v[k].x, acc[i][0]);
-            acc[i][1] = fmaf(gk[k], v[k].y, acc[i][1]);
-            acc[i][2] = fmaf(gk[k], v[k].z, acc[i][2]);
-            acc[i][3] = fmaf(gk[k], v[k].w, acc[i][3]);
+          for (int i = 0; i < 8; ++i) {
+            const float gk = k == 0 ? g[i].x : g[i].y;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(gk, vv[j], acc[i][j]);
           }
         }
       }
     }
   }
   cp_wait<0>();
-  // the groups' sums are added in group order
-  for (int s = 0; s < ns; ++s) {
+  // pairwise sums of the splits through shared memory
+  for (int o = ns >> 1; o > 0; o >>= 1) {
     __syncthreads();
-    if (on && split == s) {
+    float* slot = pipe + (size_t)(half * (ns >> 1) + (split & (o - 1))) * 64 * kHP + 4 * lane;
+    if (split >= o && split < 2 * o) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        float4* d = reinterpret_cast<float4*>(Ws + (rg + i * RG) * kSLd + 4 * cgp);
-        float4 t = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-        if (s > 0) {
-          const float4 o = *d;
-          t = make_float4(o.x + t.x, o.y + t.y, o.z + t.z, o.w + t.w);
-        }
-        *d = t;
+      for (int i = 0; i < 8; ++i) {
+        *reinterpret_cast<float4*>(slot + i * 256) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+        *reinterpret_cast<float4*>(slot + i * 256 + 128) =
+            make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
       }
     }
+    __syncthreads();
+    if (split < o) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float4 x = *reinterpret_cast<const float4*>(slot + i * 256);
+        const float4 y = *reinterpret_cast<const float4*>(slot + i * 256 + 128);
+        acc[i][0] += x.x;
+        acc[i][1] += x.y;
+        acc[i][2] += x.z;
+        acc[i][3] += x.w;
+        acc[i][4] += y.x;
+        acc[i][5] += y.y;
+        acc[i][6] += y.z;
+        acc[i][7] += y.w;
+      }
+    }
+  }
+  if (split == 0) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (lr + 8 * i < rows) {
+        float* d = Ws + (row0 + lr + 8 * i) * kSLd + 8 * lc;
+        *reinterpret_cast<float4*>(d) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+        *reinterpret_cast<float4*>(d + 4) = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
+      }
   }
   __syncthreads();
 }
@@ -151,7 +191,7 @@ __device__ void sub_atb(const float* A, const float* B, int rp, float* tmp, floa
   const int tid = threadIdx.x, q = tid >> 6, t = tid & 63;
   const int a0 = 4 * (t >> 3), b0 = 4 * (t & 7);
   float acc[4][4] = {};
-  for (int r = q; r < rp; r += 4) {
+  for (int r = q; r < rp; r += kSNT / 64) {
     const float4 x = *reinterpret_cast<const float4*>(A + r * kSLd + a0);
     const float4 y = *reinterpret_cast<const float4*>(B + r * kSLd + b0);
     const float xv[4] = {x.x, x.y, x.z, x.w}, yv[4] = {y.x, y.y, y.z, y.w};
@@ -165,94 +205,109 @@ __device__ void sub_atb(const float* A, const float* B, int rp, float* tmp, floa
     *reinterpret_cast<float4*>(tmp + q * (kHP * kHP) + (a0 + i) * kHP + b0) =
         make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
   __syncthreads();
-  const float4 s0 = reinterpret_cast<const float4*>(tmp)[tid];
-  const float4 s1 = reinterpret_cast<const float4*>(tmp + kHP * kHP)[tid];
-  const float4 s2 = reinterpret_cast<const float4*>(tmp + 2 * kHP * kHP)[tid];
-  const float4 s3 = reinterpret_cast<const float4*>(tmp + 3 * kHP * kHP)[tid];
-  reinterpret_cast<float4*>(P)[tid] =
-      make_float4((s0.x + s1.x) + (s2.x + s3.x), (s0.y + s1.y) + (s2.y + s3.y),
-                  (s0.z + s1.z) + (s2.z + s3.z), (s0.w + s1.w) + (s2.w + s3.w));
+#pragma unroll
+  for (int e = tid; e < kHP * kHP; e += kSNT) {
+    float v = tmp[e];
+#pragma unroll
+    for (int s = 1; s < kSNT / 64; ++s) v += tmp[s * kHP * kHP + e];
+    P[e] = v;
+  }
 }
 
-// Sm (32 x 33) = the sum of P over the cluster's CTAs, in rank order (the
-// same in every CTA).  Contains the cluster barrier that publishes P.
+// Sm (32 x 33, in every CTA) = the sum of P over the cluster's CTAs: each CTA
+// sums one slice (a lane per rank, shuffle tree) and stores it to all.
+// Contains two cluster barriers.
 __device__ void sub_cluster_sum(const cg::cluster_group& cl, float* P, float* Sm) {
   cl.sync();
-  const int tid = threadIdx.x, n = (int)cl.num_blocks();
-  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 8
-  for (int r = 0; r < n; ++r) {
-    const float4 v = reinterpret_cast<const float4*>(cl.map_shared_rank(P, r))[tid];
-    s.x += v.x;
-    s.y += v.y;
-    s.z += v.z;
-    s.w += v.w;
+  const int tid = threadIdx.x, n = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  if (tid < kHP * kHP / 4) {
+    // n = 8 or 16 lanes share a slice entry of four floats
+    const int r = tid & (n - 1), e = 4 * (rank * (kHP * kHP / 4 / n) + tid / n);
+    float4 v = *reinterpret_cast<const float4*>(cl.map_shared_rank(P, r) + e);
+    for (int o = 1; o < n; o <<= 1) {
+      v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+      v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+      v.z += __shfl_xor_sync(0xffffffffu, v.z, o);
+      v.w += __shfl_xor_sync(0xffffffffu, v.w, o);
+    }
+    float* d = cl.map_shared_rank(Sm, r) + (e >> 5) * 33 + (e & 31);
+    d[0] = v.x;
+    d[1] = v.y;
+    d[2] = v.z;
+    d[3] = v.w;
   }
-  float* d = Sm + (tid >> 3) * 33 + 4 * (tid & 7);
-  d[0] = s.x;
-  d[1] = s.y;
-  d[2] = s.z;
-  d[3] = s.w;
-  __syncthreads();
+  cl.sync();
 }
 
-// Warp 0: Sm + shift I = R^T R (R upper, row j at Rm + 33 j, zero below the
+// 1 / sqrt(x) by the approximation and one Newton step
+__device__ __forceinline__ float sub_rsqrt(float x) {
+  const float r = rsqrtf(x);
+  return r * fmaf(-0.5f * x * r, r, 1.5f);
+}
+
+// Warp 0: Sm + rel_shift trace(Sm) I = R^T R (R upper, row j at Rm + 33 j, zero below the
 // diagonal; rinv[j] = 1 / R_jj).  Returns false in every thread on a
 // non-positive or non-finite pivot.
-__device__ bool sub_chol(const float* Sm, float shift, float* Rm, float* rinv) {
+__device__ bool sub_chol(const float* Sm, float rel_shift, float* Rm, float* rinv) {
   const int tid = threadIdx.x, lane = tid & 31;
   bool ok = true;
   if (tid < 32) {
-    float a[kHP];
+    float a[kHP], myinv = 0.f;
+    const float shift = rel_shift > 0.f ? rel_shift * warp_sum(Sm[lane * 33 + lane]) : 0.f;
 #pragma unroll
     for (int j = 0; j < kHP; ++j) a[j] = Sm[lane * 33 + j] + (j == lane ? shift : 0.f);
 #pragma unroll
     for (int j = 0; j < kHP; ++j) {
       const float d = __shfl_sync(0xffffffffu, a[j], j);
       ok = ok && d > 0.f && d <= FLT_MAX;
-      const float r = sqrtf(d), inv = 1.f / r;
-      a[j] = lane == j ? r : a[j] * inv;
-      if (lane == j) rinv[j] = inv;
+      const float inv = sub_rsqrt(d);
+      if (lane == j) myinv = inv;
+      a[j] *= inv;  // lane j: d / sqrt(d) = R_jj
 #pragma unroll
       for (int t = j + 1; t < kHP; ++t)
         a[t] = fmaf(-a[j], __shfl_sync(0xffffffffu, a[j], t), a[t]);
     }
 #pragma unroll
     for (int j = 0; j < kHP; ++j) Rm[j * 33 + lane] = lane >= j ? a[j] : 0.f;
+    rinv[lane] = myinv;
   }
   return __syncthreads_and(ok);
 }
 
-// X <- X R^{-1}, rp rows.
+// X <- X R^{-1}, rp rows: a warp per four rows, lane t holds column t.
 __device__ void sub_solve(float* X, int rp, const float* Rm, const float* rinv) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int r0 = 8 * warp; r0 < rp; r0 += kSNT / 4) {
-    float v[8];
+  for (int r0 = 4 * warp; r0 < rp; r0 += 4 * kSNW) {
+    float v[4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = r0 + i < rp ? X[(r0 + i) * kSLd + lane] : 0.f;
+    for (int i = 0; i < 4; ++i) v[i] = X[(r0 + i) * kSLd + lane];
 #pragma unroll 8
     for (int j = 0; j < kHP; ++j) {
       const float rj = Rm[j * 33 + lane], ij = rinv[j];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
+      for (int i = 0; i < 4; ++i) {
         const float x = __shfl_sync(0xffffffffu, v[i], j) * ij;
         v[i] = lane == j ? x : fmaf(-x, rj, v[i]);
       }
     }
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-      if (r0 + i < rp) X[(r0 + i) * kSLd + lane] = v[i];
+    for (int i = 0; i < 4; ++i) X[(r0 + i) * kSLd + lane] = v[i];
   }
   __syncthreads();
 }
 
-// Eigen-decomposition of the symmetric A (32 x 33): A becomes diagonal, the
-// columns of Q the eigenvectors.  Off-diagonal entries below 3e-8 of the
-// geometric mean of their diagonal entries (or of `floor`) stay.
-__device__ void sub_jacobi(float* A, float* Q, float floor_, float* cs, int* flag) {
+// Eigen-decomposition of the symmetric A (32 x 33, entries scaled to about
+// 1): on return the eigenvalues stand on A's diagonal and the eigenvectors in
+// the columns of Q.  Parallel two-sided Jacobi, 16 disjoint pairs a round:
+// half of warp 0 forms the rotations, then thread (bi, bj) applies both
+// rotations of its 2 x 2 block and rotates its part of Q.
+// Converged when every off-diagonal entry is below 3e-7 of the geometric
+// mean of its diagonal entries (or of `floor_`), a few ulp.
+__device__ void sub_jacobi(float* A, float* Q, float floor_, float2* cs) {
   const int tid = threadIdx.x;
   for (int e = tid; e < kHP * kHP; e += kSNT) Q[(e >> 5) * 33 + (e & 31)] = (e >> 5) == (e & 31);
-  const int bi = tid >> 4, bj = tid & 15;
+  __syncthreads();
+  const int bi = (tid >> 4) & 15, bj = tid & 15;
   // pair i of round rd (round robin): column 31 stays, the others turn
   auto pair = [](int rd, int i, int& p, int& q) {
     p = rd + i;
@@ -261,56 +316,256 @@ __device__ void sub_jacobi(float* A, float* Q, float floor_, float* cs, int* fla
     if (q < 0) q += 31;
   };
   for (int sweep = 0; sweep < 12; ++sweep) {
-    if (tid == 0) *flag = 0;
-    __syncthreads();
+    bool any = false;
     for (int rd = 0; rd < 31; ++rd) {
+      int pj, qj;
+      pair(rd, bj, pj, qj);
       if (tid < 16) {
-        int p, q;
-        pair(rd, tid, p, q);
-        const float app = A[p * 33 + p], aqq = A[q * 33 + q];
-        const float apq = 0.5f * (A[p * 33 + q] + A[q * 33 + p]);
+        // the rotation that zeroes a_pq: cos 2 phi = |D| / q, sin 2 phi =
+        // 2 a_pq sign(D) / q, q = sqrt(D^2 + 4 a_pq^2), |phi| <= pi / 4
+        const float app = A[pj * 33 + pj], aqq = A[qj * 33 + qj], apq = A[pj * 33 + qj];
         float c = 1.f, s = 0.f;
-        const float lim = 3e-8f * fmaxf(sqrtf(fabsf(app)) * sqrtf(fabsf(aqq)), floor_);
-        if (fabsf(apq) > lim) {
-          const float tau = (aqq - app) / (2.f * apq);
-          const float t = copysignf(1.f, tau) / (fabsf(tau) + sqrtf(fmaf(tau, tau, 1.f)));
-          c = 1.f / sqrtf(fmaf(t, t, 1.f));
-          s = t * c;
-          *flag = 1;
+        if (apq * apq > 9e-14f * fmaxf(fabsf(app * aqq), floor_ * floor_)) {
+          const float d = aqq - app, g = 2.f * apq;
+          const float r = sub_rsqrt(fmaf(d, d, g * g));
+          const float c2 = fmaf(0.5f * fabsf(d), r, 0.5f);
+          const float rc = sub_rsqrt(c2);
+          c = c2 * rc;
+          s = copysignf(0.5f, d) * g * r * rc;
+          any = true;
         }
-        cs[2 * tid] = c;
-        cs[2 * tid + 1] = s;
+        cs[tid] = make_float2(c, s);
       }
       __syncthreads();
-      int pi, qi, pj, qj;
-      pair(rd, bi, pi, qi);
-      pair(rd, bj, pj, qj);
-      const float ci = cs[2 * bi], si = cs[2 * bi + 1], cj = cs[2 * bj], sj = cs[2 * bj + 1];
-      const float b00 = A[pi * 33 + pj], b01 = A[pi * 33 + qj];
-      const float b10 = A[qi * 33 + pj], b11 = A[qi * 33 + qj];
-      const float x0 = ci * b00 - si * b10, x1 = ci * b01 - si * b11;
-      const float y0 = si * b00 + ci * b10, y1 = si * b01 + ci * b11;
-      float n01 = sj * x0 + cj * x1, n10 = cj * y0 - sj * y1;
-      if (bi == bj && si != 0.f) n01 = n10 = 0.f;
-      A[pi * 33 + pj] = cj * x0 - sj * x1;
-      A[pi * 33 + qj] = n01;
-      A[qi * 33 + pj] = n10;
-      A[qi * 33 + qj] = sj * y0 + cj * y1;
+      const float2 rj = cs[bj];
+      const float cj = rj.x, sj = rj.y;
+      {
+        int pi, qi;
+        pair(rd, bi, pi, qi);
+        const float2 ri = cs[bi];
+        const float ci = ri.x, si = ri.y;
+        const float b00 = A[pi * 33 + pj], b01 = A[pi * 33 + qj];
+        const float b10 = A[qi * 33 + pj], b11 = A[qi * 33 + qj];
+        const float x0 = ci * b00 - si * b10, x1 = ci * b01 - si * b11;
+        const float y0 = si * b00 + ci * b10, y1 = si * b01 + ci * b11;
+        const bool own = bi == bj && si != 0.f;
+        A[pi * 33 + pj] = cj * x0 - sj * x1;
+        A[pi * 33 + qj] = own ? 0.f : sj * x0 + cj * x1;
+        A[qi * 33 + pj] = own ? 0.f : cj * y0 - sj * y1;
+        A[qi * 33 + qj] = sj * y0 + cj * y1;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        float* row = Q + (bi + 16 * h) * 33;
-        const float vp = row[pj], vq = row[qj];
-        row[pj] = cj * vp - sj * vq;
-        row[qj] = sj * vp + cj * vq;
+        for (int h = 0; h < 2; ++h) {
+          float* row = Q + (bi + 16 * h) * 33;
+          const float vp = row[pj], vq = row[qj];
+          row[pj] = cj * vp - sj * vq;
+          row[qj] = sj * vp + cj * vq;
+        }
       }
       __syncthreads();
     }
-    if (!*flag) break;
-    __syncthreads();
+    if (!__syncthreads_or(any)) break;
   }
-  __syncthreads();
 }
 
+// The shared memory of a CTA that owns rp rows.
+struct SubSmem {
+  float *pipe, *Xs, *Ws, *P, *Sm, *Rm, *Qm, *Bm;
+  __device__ SubSmem(float* sm, int rp) {
+    pipe = sm;
+    Xs = pipe + sub_pipe_floats(rp);
+    Ws = Xs + rp * kSLd;
+    P = Ws + rp * kSLd;  // this CTA's partial sum
+    Sm = P + kHP * kHP;
+    Rm = Sm + kSM;
+    Qm = Rm + kSM;
+    Bm = Qm + kSM;  // kHK x kHK
+  }
+};
+
+// Xs = orth(Ws + mu Xs) by `passes` CholQR passes, the first one shifted.
+// False (in every CTA) when a factorisation breaks down: Xs is then a fresh
+// start basis.
+__device__ bool sub_orth(const cg::cluster_group& cl, const SubSmem& m, int rp, int r0, int nn, int b,
+                         float mu, int passes) {
+  const int tid = threadIdx.x;
+  for (int e = tid; e < rp * kHP; e += kSNT) {
+    const int o = (e >> 5) * kSLd + (e & 31);
+    m.Xs[o] = fmaf(mu, m.Xs[o], m.Ws[o]);
+  }
+  __syncthreads();
+  __shared__ float rinv[kHP];
+  for (int pass = 1; pass <= passes; ++pass) {
+    sub_atb(m.Xs, m.Xs, rp, m.pipe, m.P);
+    sub_cluster_sum(cl, m.P, m.Sm);
+    const float shift =
+        pass == 1 ? 11.f * (float)((double)nn * kHP + kHP * (kHP + 1)) * FLT_EPSILON : 0.f;
+    // the same sum in every CTA: all of them fail or none
+    if (!sub_chol(m.Sm, shift, m.Rm, rinv)) {
+      for (int e = tid; e < rp * kHP; e += kSNT) {
+        const int r = r0 + (e >> 5), c = e & 31;
+        m.Xs[(e >> 5) * kSLd + c] =
+            r < nn ? huge_hash((uint32_t)r + 977u * b, (uint32_t)c + 0xB0Bu) : 0.f;
+      }
+      __syncthreads();
+      return false;
+    }
+    sub_solve(m.Xs, rp, m.Rm, rinv);
+  }
+  return true;
+}
+
+// Rayleigh-Ritz with V in Xs and G V in Ws: T = V^T G V, its eigenpairs above
+// thr (at most kHK, largest first), the Ritz vectors U = V Q, G U, B = U^T G
+// U, the residuals and What = G U - U sym(B) / 2 (into GU).  Overwrites Xs.
+// Returns true (in every CTA) when the pairs have converged.
+__device__ bool sub_ritz(const cg::cluster_group& cl, const SubSmem& m, int rp, float* Ub, float* GUb,
+                         float thr, HugeBlock& h) {
+  const int tid = threadIdx.x, CL = (int)cl.num_blocks();
+  __shared__ float rq[2 * kHK], red[kSNW][2 * kHK];
+  __shared__ float2 cs[16];
+  __shared__ int sel[kHK], ku_s;
+  float *Xs = m.Xs, *Ws = m.Ws, *P = m.P, *Sm = m.Sm, *Rm = m.Rm, *Qm = m.Qm, *Bm = m.Bm;
+  const float gF = h.gF;
+  sub_atb(Xs, Ws, rp, m.pipe, P);
+  sub_cluster_sum(cl, P, Sm);
+  // scaled by its trace (a sum of Rayleigh quotients of a Gram matrix), so
+  // that the rotations' squares stay in range
+  const float tr = warp_sum(Sm[(tid & 31) * 33 + (tid & 31)]);
+  const float isc = tr > 0.f ? 1.f / tr : 1.f;
+  for (int e = tid; e < kHP * kHP; e += kSNT) {
+    const int i = e >> 5, j = e & 31;
+    Rm[i * 33 + j] = 0.5f * (Sm[i * 33 + j] + Sm[j * 33 + i]) * isc;
+  }
+  __syncthreads();
+  sub_jacobi(Rm, Qm, 1e-2f * thr * isc, cs);
+  // the pairs above tau^2, largest first, at most kHK
+  if (tid < 32) {
+    const float th = Rm[tid * 33 + tid] * (tr > 0.f ? tr : 1.f);
+    int rk = 0;
+    for (int j = 0; j < kHP; ++j) {
+      const float o = __shfl_sync(0xffffffffu, th, j);
+      rk += o > th || (o == th && j < tid);
+    }
+    const unsigned above = __ballot_sync(0xffffffffu, th > thr);
+    if (th > thr && rk < kHK) sel[rk] = tid;
+    if (tid == 0) ku_s = min(__popc(above), kHK);
+  }
+  __syncthreads();
+  const int ku = ku_s;
+  // U = V Q and G U = W Q, over V's rows in Xs: entries 0 .. 15 U, 16 .. 31 G
+  // U (the 16 threads of a row are in one warp)
+  {
+    const int q = tid & 15;
+    const int cq = q < ku ? sel[q] : 0;
+    for (int r = tid >> 4; r < rp; r += kSNT / 16) {
+      float u = 0.f, g = 0.f;
+#pragma unroll
+      for (int a = 0; a < kHP; a += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(Xs + r * kSLd + a);
+        const float4 w = *reinterpret_cast<const float4*>(Ws + r * kSLd + a);
+        const float xv[4] = {x.x, x.y, x.z, x.w}, wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float qv = Qm[(a + i) * 33 + cq];
+          u = fmaf(xv[i], qv, u);
+          g = fmaf(wv[i], qv, g);
+        }
+      }
+      __syncwarp();
+      Xs[r * kSLd + q] = q < ku ? u : 0.f;
+      Xs[r * kSLd + kHK + q] = q < ku ? g : 0.f;
+    }
+  }
+  __syncthreads();
+  // B = U^T G U: partial sums in rank order
+  if (tid < kHK * kHK) {
+    const int p = tid >> 4, q = tid & 15;
+    float t = 0.f;
+#pragma unroll 4
+    for (int r = 0; r < rp; ++r) t = fmaf(Xs[r * kSLd + p], Xs[r * kSLd + kHK + q], t);
+    P[tid] = t;
+  }
+  cl.sync();
+  if (tid < kHK * kHK) {
+    float s = 0.f;
+#pragma unroll 8
+    for (int c = 0; c < CL; ++c) s += cl.map_shared_rank(P, c)[tid];
+    Bm[tid] = s;
+  }
+  __syncthreads();
+  // residuals |G u_q - theta_q u_q|^2 and What = G U - U sym(B) / 2, |What_q|^2
+  {
+    const int q = tid & 15, rr = tid >> 4;
+    float ra = 0.f, wa = 0.f;
+    for (int r = rr; r < rp; r += kSNT / 16) {
+      const float u = Xs[r * kSLd + q], g = Xs[r * kSLd + kHK + q];
+      float wh = g;
+      for (int p = 0; p < ku; ++p)
+        wh = fmaf(-0.25f * (Bm[p * kHK + q] + Bm[q * kHK + p]), Xs[r * kSLd + p], wh);
+      if (q < ku) {
+        const float res = g - Bm[q * kHK + q] * u;
+        ra = fmaf(res, res, ra);
+        wa = fmaf(wh, wh, wa);
+      }
+      Ub[(size_t)r * kHK + q] = u;
+      GUb[(size_t)r * kHK + q] = q < ku ? wh : 0.f;
+    }
+    ra += __shfl_xor_sync(0xffffffffu, ra, 16);
+    wa += __shfl_xor_sync(0xffffffffu, wa, 16);
+    if ((tid & 31) < 16) {
+      red[tid >> 5][q] = ra;
+      red[tid >> 5][kHK + q] = wa;
+    }
+  }
+  __syncthreads();
+  // (the B partials in P's first 256 entries may still be read)
+  float* P2 = P + kHK * kHK;
+  if (tid < 2 * kHK) {
+    float t = 0.f;
+    for (int w = 0; w < kSNW; ++w) t += red[w][tid];
+    P2[tid] = t;
+  }
+  cl.sync();
+  if (tid < 2 * kHK) {
+    float t = 0.f;
+#pragma unroll 8
+    for (int c = 0; c < CL; ++c) t += cl.map_shared_rank(P2, c)[tid];
+    rq[tid] = t;
+  }
+  __syncthreads();
+  // converged: every kept pair's residual is small against tau^2, or at the
+  // rounding level of G V (set by the largest eigenvalue).  Pairs just above
+  // tau converge slowly; they need this accuracy all the same, since the
+  // consensus step carries their error into every scale.
+  bool conv = true;
+  float th0 = 0.f, wsum = 0.f;
+  for (int q = 0; q < ku; ++q) {
+    th0 = fmaxf(th0, Bm[q * kHK + q]);
+    wsum += rq[kHK + q];
+  }
+  for (int q = 0; q < ku; ++q)
+    if (sqrtf(rq[q]) > fmaxf(3e-4f * thr, 4e-6f * th0)) conv = false;
+  if (cl.block_rank() == 0 && tid == 0) {
+    int k = 0;
+    for (int q = 0; q < ku; ++q) {
+      const float th = Bm[q * kHK + q];
+      h.theta[q] = th;
+      k += th > thr;
+    }
+    h.c = cert_bound(thr, gF, ku, wsum);
+    h.ku = ku;
+    h.k = k;
+    h.conv = conv;
+  }
+  cl.sync();  // the partial sums have been read
+  return conv;
+}
+
+__device__ __forceinline__ bool sub_active(const HugeBlock& h) {
+  return h.status == kHsIter && !h.conv && !h.orth_fail;
+}
+
+// Every step of every round for the blocks of a scale, a cluster per block.
 // `first`: steps of the first round (later rounds: 4 and 8).
 __global__ void __launch_bounds__(kSNT)
 subspace_cluster_kernel(const float* __restrict__ G, float* V, float* __restrict__ U,
@@ -323,188 +578,87 @@ subspace_cluster_kernel(const float* __restrict__ G, float* V, float* __restrict
   const int rp = np / CL, r0 = rank * rp;
   HugeBlock& h = hb[b];
   if (h.status != kHsIter) return;  // the whole cluster leaves
-  float* pipe = sm;
-  float* Xs = pipe + sub_pipe_floats(rp);
-  float* Ws = Xs + rp * kSLd;
-  float* Sp = Ws + rp * kSLd;  // two 32 x 32 partial sums, used in turn
-  float* Sm = Sp + 2 * kHP * kHP;
-  float* Rm = Sm + kSM;
-  float* Qm = Rm + kSM;
-  float* Bm = Qm + kSM;  // kHK x kHK
-  __shared__ float rinv[kHP], cs[32], rq[2 * kHK], red[kSNT / 32][2 * kHK];
-  __shared__ int flag, sel[kHK], ku_s;
+  const SubSmem m(sm, rp);
   const float* Gr = G + (size_t)b * np * np + (size_t)r0 * np;
   float* Vb = V + (size_t)b * np * kHP;
-  const float gF = h.gF, mu = 1e-4f * gF;
-  for (int e = tid; e < rp * kHP; e += kSNT) Xs[(e >> 5) * kSLd + (e & 31)] = Vb[(size_t)r0 * kHP + e];
+  const size_t uo = ((size_t)b * np + r0) * kHK;
+  const float mu = 1e-4f * h.gF;
+  for (int e = tid; e < rp * kHP; e += kSNT) m.Xs[(e >> 5) * kSLd + (e & 31)] = Vb[(size_t)r0 * kHP + e];
   __syncthreads();
-  int turn = 0;
-  auto part = [&]() {
-    float* p = Sp + turn * kHP * kHP;
-    turn ^= 1;
-    return p;
-  };
   const int rounds[3] = {first, 4, 8};
   bool failed = false, conv = false;
   for (int rd = 0; rd < 3 && !conv && !failed; ++rd) {
     for (int st = 0; st < rounds[rd] && !failed; ++st) {
-      sub_gv(Gr, Vb, np, rp, pipe, Ws);
-      for (int e = tid; e < rp * kHP; e += kSNT) {
-        const int o = (e >> 5) * kSLd + (e & 31);
-        Xs[o] = fmaf(mu, Xs[o], Ws[o]);
-      }
-      __syncthreads();
-      for (int pass = 1; pass <= 3; ++pass) {
-        float* P = part();
-        sub_atb(Xs, Xs, rp, pipe, P);
-        sub_cluster_sum(cl, P, Sm);
-        float shift = 0.f;
-        if (pass == 1) {
-          float tr = 0.f;
-          for (int i = 0; i < kHP; ++i) tr += Sm[i * 33 + i];
-          shift = 11.f * (float)((double)nn * kHP + kHP * (kHP + 1)) * FLT_EPSILON * tr;
-        }
-        // the same sum in every CTA: all of them fail or none
-        if (!sub_chol(Sm, shift, Rm, rinv)) {
-          failed = true;
-          break;
-        }
-        sub_solve(Xs, rp, Rm, rinv);
-      }
-      if (failed)
-        for (int e = tid; e < rp * kHP; e += kSNT) {
-          const int r = r0 + (e >> 5), c = e & 31;
-          Xs[(e >> 5) * kSLd + c] =
-              r < nn ? huge_hash((uint32_t)r + 977u * b, (uint32_t)c + 0xB0Bu) : 0.f;
-        }
-      __syncthreads();
-      for (int e = tid; e < rp * kHP; e += kSNT) Vb[(size_t)r0 * kHP + e] = Xs[(e >> 5) * kSLd + (e & 31)];
+      sub_gv(Gr, Vb, np, rp, m.pipe, m.Ws);
+      // the third pass brings V to working precision for the Ritz problem;
+      // between steps a well-conditioned basis of the same span is enough
+      failed = !sub_orth(cl, m, rp, r0, nn, b, mu, st + 1 < rounds[rd] ? 2 : 3);
+      for (int e = tid; e < rp * kHP; e += kSNT)
+        Vb[(size_t)r0 * kHP + e] = m.Xs[(e >> 5) * kSLd + (e & 31)];
       cl.sync();  // the new V is visible to the cluster
     }
     if (failed) break;
-    // Rayleigh-Ritz on T = V^T G V
-    sub_gv(Gr, Vb, np, rp, pipe, Ws);
-    {
-      float* P = part();
-      sub_atb(Xs, Ws, rp, pipe, P);
-      sub_cluster_sum(cl, P, Sm);
+    sub_gv(Gr, Vb, np, rp, m.pipe, m.Ws);
+    conv = sub_ritz(cl, m, rp, U + uo, GU + uo, thr, h);
+    if (!conv) {
+      for (int e = tid; e < rp * kHP; e += kSNT)
+        m.Xs[(e >> 5) * kSLd + (e & 31)] = Vb[(size_t)r0 * kHP + e];
+      __syncthreads();
     }
-    for (int e = tid; e < kHP * kHP; e += kSNT) {
-      const int i = e >> 5, j = e & 31;
-      Rm[i * 33 + j] = 0.5f * (Sm[i * 33 + j] + Sm[j * 33 + i]);
-    }
-    __syncthreads();
-    sub_jacobi(Rm, Qm, 1e-2f * thr, cs, &flag);
-    // the pairs above tau^2, largest first, at most kHK
-    if (tid < 32) {
-      const float th = Rm[tid * 33 + tid];
-      int rk = 0;
-      for (int j = 0; j < kHP; ++j) {
-        const float o = __shfl_sync(0xffffffffu, th, j);
-        rk += o > th || (o == th && j < tid);
-      }
-      const unsigned above = __ballot_sync(0xffffffffu, th > thr);
-      if (th > thr && rk < kHK) sel[rk] = tid;
-      if (tid == 0) ku_s = min(__popc(above), kHK);
-    }
-    __syncthreads();
-    const int ku = ku_s;
-    // U = V Q and G U in the pipeline's space (row stride 2 kHK); V stays,
-    // it is the next round's start
-    float* Us = pipe;
-    for (int e = tid; e < rp * kHK; e += kSNT) {
-      const int r = e >> 4, q = e & 15;
-      float u = 0.f, g = 0.f;
-      if (q < ku) {
-        const int cq = sel[q];
-#pragma unroll 8
-        for (int a = 0; a < kHP; ++a) {
-          const float w = Qm[a * 33 + cq];
-          u = fmaf(Xs[r * kSLd + a], w, u);
-          g = fmaf(Ws[r * kSLd + a], w, g);
-        }
-      }
-      Us[r * 2 * kHK + q] = u;
-      Us[r * 2 * kHK + kHK + q] = g;
-    }
-    __syncthreads();
-    // B = U^T G U: partial sums in rank order
-    {
-      float* P = part();
-      const int p = tid >> 4, q = tid & 15;
-      float t = 0.f;
-      for (int r = 0; r < rp; ++r) t = fmaf(Us[r * 2 * kHK + p], Us[r * 2 * kHK + kHK + q], t);
-      P[tid] = t;
-      cl.sync();
-      float s = 0.f;
-      for (int c = 0; c < CL; ++c) s += cl.map_shared_rank(P, c)[tid];
-      Bm[tid] = s;
-    }
-    __syncthreads();
-    // residuals |G u_q - theta_q u_q|^2 and What = G U - U sym(B) / 2, |What_q|^2
-    {
-      const int q = tid & 15, rr = tid >> 4;
-      float ra = 0.f, wa = 0.f;
-      for (int r = rr; r < rp; r += kSNT / 16) {
-        const float u = Us[r * 2 * kHK + q], g = Us[r * 2 * kHK + kHK + q];
-        float wh = g;
-        for (int p = 0; p < ku; ++p)
-          wh = fmaf(-0.25f * (Bm[p * kHK + q] + Bm[q * kHK + p]), Us[r * 2 * kHK + p], wh);
-        if (q < ku) {
-          const float res = g - Bm[q * kHK + q] * u;
-          ra = fmaf(res, res, ra);
-          wa = fmaf(wh, wh, wa);
-        }
-        U[((size_t)b * np + r0 + r) * kHK + q] = u;
-        GU[((size_t)b * np + r0 + r) * kHK + q] = q < ku ? wh : 0.f;
-      }
-      ra += __shfl_xor_sync(0xffffffffu, ra, 16);
-      wa += __shfl_xor_sync(0xffffffffu, wa, 16);
-      if ((tid & 31) < 16) {
-        red[tid >> 5][q] = ra;
-        red[tid >> 5][kHK + q] = wa;
-      }
-    }
-    __syncthreads();
-    float* P = part();
-    if (tid < 2 * kHK) {
-      float t = 0.f;
-      for (int w = 0; w < kSNT / 32; ++w) t += red[w][tid];
-      P[tid] = t;
-    }
-    cl.sync();
-    if (tid < 2 * kHK) {
-      float t = 0.f;
-      for (int c = 0; c < CL; ++c) t += cl.map_shared_rank(P, c)[tid];
-      rq[tid] = t;
-    }
-    __syncthreads();
-    // converged: see huge_rr_kernel (the same test)
-    conv = true;
-    float th0 = 0.f, wsum = 0.f;
-    for (int q = 0; q < ku; ++q) {
-      th0 = fmaxf(th0, Bm[q * kHK + q]);
-      wsum += rq[kHK + q];
-    }
-    for (int q = 0; q < ku; ++q)
-      if (sqrtf(rq[q]) > fmaxf(3e-4f * thr, 4e-6f * th0)) conv = false;
-    if (rank == 0 && tid == 0) {
-      int k = 0;
-      for (int q = 0; q < ku; ++q) {
-        const float th = Bm[q * kHK + q];
-        h.theta[q] = th;
-        k += th > thr;
-      }
-      h.c = cert_bound(thr, gF, ku, wsum);
-      h.ku = ku;
-      h.k = k;
-      h.conv = conv;
-    }
-    __syncthreads();
   }
   if (failed && rank == 0 && tid == 0) h.orth_fail = 1;
   cl.sync();  // no CTA leaves while others read its shared memory
 }
+
+// Wider blocks, a launch per phase.  W = G V, 64 rows a CTA.
+__global__ void __launch_bounds__(kSNT)
+subspace_gv_kernel(const float* __restrict__ G, const float* __restrict__ V, float* __restrict__ W,
+                   int np, const HugeBlock* __restrict__ hb) {
+  extern __shared__ __align__(16) float sm[];
+  const int b = blockIdx.y, r0 = blockIdx.x * 64, tid = threadIdx.x;
+  if (!sub_active(hb[b])) return;
+  float* Ws = sm + sub_pipe_floats(64);
+  sub_gv(G + (size_t)b * np * np + (size_t)r0 * np, V + (size_t)b * np * kHP, np, 64, sm, Ws);
+  float* Wb = W + ((size_t)b * np + r0) * kHP;
+  for (int e = tid; e < 64 * kHP; e += kSNT) Wb[e] = Ws[(e >> 5) * kSLd + (e & 31)];
+}
+
+// V = orth(W + mu V) (passes > 0), or the Rayleigh-Ritz test on V and W
+// (passes = 0), in one cluster per block.
+__global__ void __launch_bounds__(kSNT)
+subspace_phase_kernel(float* V, const float* __restrict__ W, float* __restrict__ U,
+                      float* __restrict__ GU, int nn, int np, float thr, int passes,
+                      HugeBlock* __restrict__ hb) {
+  extern __shared__ __align__(16) float sm[];
+  const cg::cluster_group cl = cg::this_cluster();
+  const int CL = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int b = blockIdx.x / CL, tid = threadIdx.x;
+  const int rp = np / CL, r0 = rank * rp;
+  HugeBlock& h = hb[b];
+  // (the state is written only after a later cluster barrier)
+  if (!sub_active(h)) return;
+  const SubSmem m(sm, rp);
+  float* Vr = V + ((size_t)b * np + r0) * kHP;
+  const float* Wr = W + ((size_t)b * np + r0) * kHP;
+  for (int e = tid; e < rp * kHP; e += kSNT) {
+    const int o = (e >> 5) * kSLd + (e & 31);
+    m.Xs[o] = Vr[e];
+    m.Ws[o] = Wr[e];
+  }
+  __syncthreads();
+  if (passes > 0) {
+    const bool ok = sub_orth(cl, m, rp, r0, nn, b, 1e-4f * h.gF, passes);
+    for (int e = tid; e < rp * kHP; e += kSNT) Vr[e] = m.Xs[(e >> 5) * kSLd + (e & 31)];
+    cl.sync();
+    if (!ok && rank == 0 && tid == 0) h.orth_fail = 1;
+  } else {
+    const size_t uo = ((size_t)b * np + r0) * kHK;
+    sub_ritz(cl, m, rp, U + uo, GU + uo, thr, h);
+  }
+  cl.sync();  // no CTA leaves while others read its shared memory
+}
+
+constexpr int kSPhaseRows = 512;  // rows per CTA of subspace_phase_kernel, at most
 
 // the widest cluster the device runs at the largest shared-memory size
 int widest_cluster() {
@@ -517,11 +671,11 @@ int widest_cluster() {
     at[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(16);
     cfg.blockDim = dim3(kSNT);
-    cfg.dynamicSmemBytes = sub_smem_bytes(kSMaxRows);
+    cfg.dynamicSmemBytes = sub_smem_bytes(kSPhaseRows);
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, subspace_cluster_kernel, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, subspace_phase_kernel, &cfg) != cudaSuccess) {
       cudaGetLastError();
       n = 0;
     }
@@ -530,28 +684,16 @@ int widest_cluster() {
   return w;
 }
 
-// CTAs per block: 8 up to 512 wide, 16 above (32 to 128 rows a CTA)
-int cluster_size(int np) { return np <= 512 ? 8 : widest_cluster(); }
-
-}  // namespace
-
-cudaError_t configure_subspace() {
-  if (cudaError_t e = cudaFuncSetAttribute(subspace_cluster_kernel,
-                                           cudaFuncAttributeNonPortableClusterSizeAllowed, 1))
+template <class K>
+cudaError_t sub_attributes(K k, int rows) {
+  if (cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)sub_smem_bytes(rows)))
     return e;
-  if (cudaError_t e = cudaFuncSetAttribute(subspace_cluster_kernel,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)sub_smem_bytes(kSMaxRows)))
-    return e;
-  widest_cluster();
-  return cudaSuccess;
+  return cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
 
-bool subspace_cluster_path(int np) { return np / cluster_size(np) <= kSMaxRows; }
-
-cudaError_t launch_subspace(const float* G, float* V, float* U, float* GU, int nn, int np, float thr,
-                            int first, HugeBlock* hb, int B, cudaStream_t st) {
-  const int CL = cluster_size(np);
+template <class K, class... A>
+cudaError_t sub_launch(K k, int CL, int B, int rows, cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -560,11 +702,58 @@ cudaError_t launch_subspace(const float* G, float* V, float* U, float* GU, int n
   at[0].val.clusterDim.z = 1;
   cfg.gridDim = dim3(CL * B);
   cfg.blockDim = dim3(kSNT);
-  cfg.dynamicSmemBytes = sub_smem_bytes(np / CL);
+  cfg.dynamicSmemBytes = sub_smem_bytes(rows);
   cfg.stream = st;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, subspace_cluster_kernel, G, V, U, GU, nn, np, thr, first, hb);
+  return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
+}  // namespace
+
+cudaError_t configure_subspace() {
+  if (cudaError_t e = sub_attributes(subspace_cluster_kernel, kSMaxRows)) return e;
+  if (cudaError_t e = sub_attributes(subspace_phase_kernel, kSPhaseRows)) return e;
+  if (cudaError_t e = cudaFuncSetAttribute(subspace_gv_kernel,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)sub_smem_bytes(64)))
+    return e;
+  // 8192-wide blocks need the 16-CTA cluster
+  return widest_cluster() == 16 ? cudaSuccess : cudaErrorNotSupported;
+}
+
+cudaError_t launch_subspace(const float* G, float* V, float* W, float* U, float* GU, int nn, int np,
+                            float thr, int first, HugeBlock* hb, int B, cudaStream_t st, Prof* prof) {
+  auto timed = [&](auto&& launch) -> cudaError_t {
+    if (prof)
+      if (cudaError_t e = prof->before(st, KK_SUBSPACE)) return e;
+    if (cudaError_t e = launch()) return e;
+    return prof ? prof->after(st) : cudaSuccess;
+  };
+  // 8 CTAs up to 512 wide, 16 above; 32 to 128 rows a CTA
+  const int CL = np <= 512 ? 8 : 16;
+  if (np / CL <= kSMaxRows)
+    return timed([&] {
+      return sub_launch(subspace_cluster_kernel, CL, B, np / CL, st, G, V, U, GU, nn, np, thr, first,
+                        hb);
+    });
+  auto gv = [&] {
+    subspace_gv_kernel<<<dim3(np / 64, B), kSNT, sub_smem_bytes(64), st>>>(G, V, W, np, hb);
+    return cudaGetLastError();
+  };
+  const int rounds[3] = {first, 4, 8};
+  for (int r = 0; r < 3; ++r) {
+    for (int i = 0; i <= rounds[r]; ++i) {
+      if (cudaError_t e = timed(gv)) return e;
+      const int passes = i < rounds[r] ? (i + 1 < rounds[r] ? 2 : 3) : 0;
+      if (cudaError_t e = timed([&] {
+            return sub_launch(subspace_phase_kernel, 16, B, np / 16, st, V, W, U, GU, nn, np, thr,
+                              passes, hb);
+          }))
+        return e;
+    }
+  }
+  return cudaSuccess;
 }
 
 }  // namespace msllr
