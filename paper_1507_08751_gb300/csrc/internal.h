@@ -190,6 +190,13 @@ cudaError_t launch_gram_tc(const ScaleLaunch& s, float* G, float* part, int chun
 // MSLLR_GRAM_FP32=1: the FP32 CUDA-core Gram kernels instead (comparisons)
 bool gram_fp32_forced();
 
+// The Householder path of blocks up to 256 wide (k_tridiag.cu): kernel
+// attributes, and the launch over the blocks with ws.k < 0 (`groups` clusters
+// stride over them).
+cudaError_t configure_tridiag();
+cudaError_t launch_tridiag(const ScaleLaunch& s, const BigWorkspace& ws, int nblocks, int groups,
+                           cudaStream_t st);
+
 // Launchers (all asynchronous on `st`).  Return cudaGetLastError().
 cudaError_t launch_scale(const ScaleLaunch& s, const BigWorkspace& ws, cudaStream_t st,
                          Prof* prof, cudaEvent_t after_gram = nullptr);

@@ -6,7 +6,7 @@
 //   2. eig_big: one CTA per block -- skip bound (Sec. 8), certified zero
 //      rank or certified Lanczos eigenpairs of G_b (lanczos.cuh,
 //      regchol.cuh), output V_b diag(sqrt(f));
-//   3. eig_fallback: the Householder path (symeig.cuh) for the blocks step 2
+//   3. tridiag (k_tridiag.cu): the Householder path for the blocks step 2
 //      could not certify;
 //   4. rebuild: Z'_b = (C_b V_f) V_f^T, scattered through Shift_{-s}, with
 //      the fused dual update W' = 2 Z' - A of eq:admm (warp per row for
@@ -33,6 +33,7 @@ constexpr int kChunk = 256;     // rows of C per Gram partial sum
 constexpr int kGramThreads = 256;
 constexpr int kEigThreads = 512;
 constexpr int kEigMax = 256;
+constexpr int kEigK = lz_maxk(kEigMax);  // Ritz pairs kept per block
 constexpr int kRebThreads = 256;
 constexpr int kRebElems = 4096;  // rows-per-slab * nn
 constexpr int kKC = 16;          // eigenvectors per rebuild step
@@ -275,7 +276,7 @@ eig_big_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace ws) {
   const float gbound = fminf(tr, rs);
   double fl = nn + fl_symv(nn);  // trace, Gershgorin row sums
   const bool full = (a.m == launch_rows(a) && a.n == a.N);
-  const int kwarm = (a.warm_start && (full || !a.shift)) ? min(ws.kwarm[b], kLzMaxK) : 0;
+  const int kwarm = (a.warm_start && (full || !a.shift)) ? min(ws.kwarm[b], kEigK) : 0;
   bool skipped = false, lanczos_ok = false;
   int k = -1, ku = 0;
   // Two certificates share one Cholesky call site: attempt 0 tests
@@ -303,7 +304,7 @@ eig_big_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace ws) {
       PHASE(3, 6);
     } else {
       PHASE(3, 1);
-      const float* warm = ws.warm + (size_t)b * kLzMaxK * nn;
+      const float* warm = ws.warm + (size_t)b * kEigK * nn;
       int J = 0;
       kk = lanczos_candidates<NT, NMAX>(Gacc, nn, thr, gbound, Qs,
                                                         min(nn, kLzMaxJ), U, warm, kwarm,
@@ -315,8 +316,8 @@ eig_big_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace ws) {
       fl += fl_deflate(nn, ku);
     }
     fl += fl_chol(nn);
-    const bool pd = regchol_pd<NT, NMAX>(Gacc, nn, c0, attempt == 1, panel, panel + 8 * n8,
-                                         attempt == 1 ? ku : 0, panel + 16 * n8, s.red,
+    const bool pd = regchol_pd<NT, NMAX>(Gacc, nn, c0, attempt == 1, panel, panel + kEigK * n8,
+                                         attempt == 1 ? ku : 0, panel + 2 * kEigK * n8, s.red,
                                          3 + attempt);
     PHASE(3, 7 + attempt);
     if (pd) {
@@ -327,7 +328,7 @@ eig_big_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace ws) {
   }
   if (lanczos_ok) {
     // keep the Ritz vectors for the next call's warm start
-    float* wdst = ws.warm + (size_t)b * kLzMaxK * nn;
+    float* wdst = ws.warm + (size_t)b * kEigK * nn;
     for (int e = tid; e < nn * ku; e += NT) wdst[e] = U[e];
     if (tid == 0) ws.kwarm[b] = ku;
     // V_f (row-major, ld nn) for the rebuild, staged through shared memory
@@ -341,7 +342,7 @@ eig_big_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace ws) {
   }
   if (tid == 0) {
     if (a.cnt) atomicAdd(a.cnt + 5, (unsigned long long)fl);
-    // k < 0: not settled here; eig_fallback_kernel takes the block
+    // k < 0: not settled here; tridiag_kernel takes the block
     ws.k[b] = k;
     if (k < 0) {
       if (ws.kwarm) ws.kwarm[b] = 0;
@@ -359,84 +360,6 @@ eig_big_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace ws) {
       }
     }
   }
-}
-
-// Householder path for the blocks eig_big_kernel left unsettled (ws.k < 0):
-// tridiagonalisation, Sturm multisection and inverse iteration on the
-// packed G (symeig.cuh).  Kept out of eig_big_kernel so that the common
-// paths run from a smaller instruction footprint.
-__device__ __forceinline__ void eig_fallback_block(const ScaleLaunch& a, const float* __restrict__ Gall,
-                                                   const BigWorkspace& ws, int b) {
-  extern __shared__ float sm[];
-  constexpr int NT = kEigThreads, NMAX = kEigMax;
-  const int tid = threadIdx.x;
-  const int nn = a.m >= a.n ? a.n : a.m;
-  const float* Gg = Gall + (size_t)b * nn * nn;
-  float* Y = ws.Y + (size_t)b * ws.ystride;
-  float* Gp = sm;
-  float* scr = Gp + (((nn * (nn + 1)) / 2 + 3) & ~3);
-  EigScratch s;
-  s.d = scr;
-  s.e = s.d + NMAX;
-  s.e2 = s.e + NMAX;
-  s.beta = s.e2 + NMAX;
-  s.vbuf = s.beta + NMAX;
-  s.pbuf = s.vbuf + NMAX;
-  s.lam = s.pbuf + NMAX;
-  s.shf = s.lam + NMAX;
-  s.clus = reinterpret_cast<int*>(s.shf + NMAX);
-  s.lo = reinterpret_cast<float*>(s.clus + NMAX);
-  s.hi = s.lo + NT;
-  s.xs = s.hi + NT;
-  s.cnt = reinterpret_cast<int*>(s.xs + NT);
-  s.red = reinterpret_cast<float*>(s.cnt + NT);
-  const int ntri = nn * (nn + 1) / 2;
-  for (int e = tid; e < ntri; e += NT) Gp[e] = Gg[e];
-  __syncthreads();
-  LowerPacked Gacc{Gp};
-  const float thr = a.tau * a.tau;
-  tridiagonalize<NT>(Gacc, nn, s);
-  float tn = 0.f;
-  const int k = top_eigenvalues<NT>(nn, thr, s, &tn);
-  if (k > 0) {
-    top_eigenvectors<NT, NMAX>(Gacc, nn, k, tn, s, Y, nn, -1);
-    // V_f = V diag(sqrt(f)), f = 1 - tau/sigma
-    for (int e = tid; e < nn * k; e += NT) {
-      const int i = e / k, q = e - i * k;
-      const float sig = sqrtf(s.lam[q]);
-      Y[(size_t)i * nn + q] *= sqrtf(fmaxf(1.f - a.tau / sig, 0.f));
-    }
-  }
-  if (tid == 0) {
-    ws.k[b] = k;
-    if (a.rank_out) a.rank_out[b] = k;
-    if (a.cnt) {
-      if (k == 0) atomicAdd(a.cnt + 1, 1ull);
-      atomicAdd(a.cnt + 3, 1ull);
-      atomicAdd(a.cnt + 6, (unsigned long long)fl_householder(nn, k));
-    }
-    if (a.nuc_acc && k > 0) {
-      double t = 0.0;
-      for (int q = 0; q < k; ++q) t += (double)fmaxf(sqrtf(s.lam[q]) - a.tau, 0.f);
-      atomicAdd(a.nuc_acc, t);
-    }
-  }
-}
-
-// At most 32 CTAs stride over the blocks (a launch that finds nothing to do
-// then holds few SMs); one CTA per block when the certified paths are off.
-__global__ void __launch_bounds__(kEigThreads)
-eig_fallback_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace ws, int nblocks) {
-  for (int b = blockIdx.x; b < nblocks; b += gridDim.x) {
-    if (ws.k[b] >= 0) continue;
-    eig_fallback_block(a, Gall, ws, b);
-    __syncthreads();
-  }
-}
-
-size_t fallback_smem_bytes(int nn) {
-  return sizeof(float) * ((((size_t)nn * (nn + 1) / 2 + 3) & ~(size_t)3) + 9 * kEigMax +
-                          4 * kEigThreads + 64);
 }
 
 // Z' = (C V_f) V_f^T, W' = 2 Z' - A for blocks of rank k <= kRowK: one warp
@@ -605,7 +528,7 @@ rebuild_kernel(ScaleLaunch a, const float* __restrict__ Yall, size_t ystride,
 }  // namespace
 
 static size_t y_stride(int nn) {
-  const size_t a = (size_t)nn * nn, b = (size_t)(kLzMaxJ + 2 * kLzMaxK) * nn;
+  const size_t a = (size_t)nn * nn, b = (size_t)(kLzMaxJ + 2 * kEigK) * nn;
   return ((a > b ? a : b) + 63) & ~(size_t)63;
 }
 
@@ -618,7 +541,7 @@ size_t big_workspace_bytes(int M, int N, int m, int n) {
   if (d.chunks > 1) bytes += sizeof(float) * (size_t)d.nblocks * d.chunks * d.ntiles * kTile * kTile;
   bytes += sizeof(float) * (size_t)d.nblocks * y_stride(d.nn);  // Y
   bytes += sizeof(int) * (size_t)d.nblocks;                      // k
-  bytes += sizeof(float) * (size_t)d.nblocks * kLzMaxK * d.nn;   // warm
+  bytes += sizeof(float) * (size_t)d.nblocks * kEigK * d.nn;   // warm
   bytes += sizeof(int) * (size_t)d.nblocks;                      // kwarm
   bytes += 8 * 256;  // alignment slack for the carve below
   return bytes;
@@ -646,7 +569,7 @@ BigWorkspace carve_big_workspace(void* base, int M, int N, int m, int n) {
   w.k = (int*)p;
   p = align256(p + sizeof(int) * (size_t)d.nblocks);
   w.warm = (float*)p;
-  p = align256(p + sizeof(float) * (size_t)d.nblocks * kLzMaxK * d.nn);
+  p = align256(p + sizeof(float) * (size_t)d.nblocks * kEigK * d.nn);
   w.kwarm = (int*)p;
   return w;
 }
@@ -677,9 +600,7 @@ cudaError_t configure_big_kernels() {
   cudaError_t e = cudaFuncSetAttribute(eig_big_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)eig_smem_bytes(kEigMax));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(eig_fallback_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)fallback_smem_bytes(kEigMax));
-  if (e != cudaSuccess) return e;
+  if (cudaError_t e3 = configure_tridiag()) return e3;
   e = cudaFuncSetAttribute(rebuild_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            100 * 1024);
   if (e != cudaSuccess) return e;
@@ -723,12 +644,10 @@ cudaError_t launch_big(const ScaleLaunch& s, const BigWorkspace& ws, cudaStream_
   eig_big_kernel<<<d.nblocks, kEigThreads, eig_smem_bytes(d.nn), st>>>(s, ws.G, ws);
   PROF_AFTER()
   PROF_BEFORE(KK_EIG_FALLBACK)
-  // up to 32 CTAs stride over the blocks: enough for scales where many
-  // blocks need the Householder path (blocks of rank above 8, or with an
-  // eigenvalue just below tau^2), few idle SMs where almost none do
-  const int fb_grid = s.skip_bound ? (d.nblocks < 32 ? d.nblocks : 32) : d.nblocks;
-  eig_fallback_kernel<<<fb_grid, kEigThreads, fallback_smem_bytes(d.nn), st>>>(s, ws.G, ws,
-                                                                               d.nblocks);
+  // up to 64 CTAs stride over the blocks: enough for scales where many blocks
+  // need the Householder path, few idle SMs where almost none do
+  const int fb_groups = s.skip_bound ? (d.nblocks < 32 ? d.nblocks : 32) : d.nblocks;
+  if (cudaError_t e_ = launch_tridiag(s, ws, d.nblocks, fb_groups, st)) return e_;
   PROF_AFTER()
   const int rs = kRebElems / d.nn;
   const int slabs = (d.mm + rs - 1) / rs;

@@ -32,7 +32,9 @@
 namespace msllr {
 
 constexpr int kLzMaxJ = 32;  // Lanczos steps
-constexpr int kLzMaxK = 8;   // Ritz pairs kept (above 0.95 tau^2)
+// Ritz pairs kept (above 0.95 tau^2): 8 for blocks up to 64 wide, 16 above,
+// where the alternative is a 3 ms Householder reduction (256 wide)
+constexpr int lz_maxk(int nmax) { return nmax > 64 ? 16 : 8; }
 
 // FP32 flops of the eigen-solve steps, each counted at its algorithmic cost
 // (a multiply-add is 2 flops); the kernels add them up per block so that the
@@ -42,7 +44,7 @@ __device__ __forceinline__ double fl_chol(int n) { return (double)n * n * n / 3.
 // J Lanczos steps (matrix-vector product plus two Gram-Schmidt passes over
 // j + 1 vectors), U = Q_J Y, W = G U for 8 vectors, B = U^T W
 __device__ __forceinline__ double fl_lanczos(int n, int J, int ku) {
-  return 2.0 * n * n * J + 4.0 * n * J * (J + 1) + 2.0 * n * J * ku + 16.0 * n * n + 16.0 * n * ku;
+  return 2.0 * n * n * J + 4.0 * n * J * (J + 1) + 2.0 * n * J * ku + 2.0 * n * n * ((ku + 7) & ~7) + 16.0 * n * ku;
 }
 // the rank-2k deflation G - U What^T - What U^T on the lower triangle
 __device__ __forceinline__ double fl_deflate(int n, int ku) { return 2.0 * ku * n * n; }
@@ -60,7 +62,7 @@ __host__ __device__ constexpr int lz_ldq(int n) {
 
 // shared scratch (floats) of the certificate step of lanczos_candidates
 __host__ __device__ constexpr int lz_cert_floats(int nmax, int nt) {
-  return 16 * nmax + regchol_scratch_floats(nmax, nt);
+  return 2 * lz_maxk(nmax) * nmax + regchol_scratch_floats(nmax, nt);
 }
 
 // Shared-memory scratch of the Lanczos path.
@@ -70,17 +72,17 @@ struct LzScratch {
   float* alpha;  // [kLzMaxJ]
   float* beta;   // [kLzMaxJ]
   float* h;      // [2 * kLzMaxJ + 8] projection coefficients (two passes)
-  float* ty;     // [jcap * kLzMaxK] eigenvectors of T_J (row i, column q)
-  float* lu;     // [4 * jcap * kLzMaxK] inverse-iteration LU factors
-  unsigned* piv; // [2 * kLzMaxK] pivot bits
-  float* Bm;     // [kLzMaxK * kLzMaxK] U^T G U
+  float* ty;     // [jcap * K] eigenvectors of T_J (row i, column q), K = lz_maxk
+  float* lu;     // [4 * jcap * K] inverse-iteration LU factors
+  unsigned* piv; // [2 * K] pivot bits
+  float* Bm;     // [K * K] U^T G U
   int jcap;      // row capacity of ty / lu (>= Lanczos steps)
 };
 
 // floats of LzScratch for a given n capacity and J capacity
 __host__ __device__ constexpr int lz_scratch_floats(int nmax, int jcap) {
-  return 2 * nmax + 2 * kLzMaxJ + (2 * kLzMaxJ + 8) + jcap * kLzMaxK + 4 * jcap * kLzMaxK +
-         2 * kLzMaxK + kLzMaxK * kLzMaxK;
+  return 2 * nmax + 2 * kLzMaxJ + (2 * kLzMaxJ + 8) + 5 * jcap * lz_maxk(nmax) +
+         2 * lz_maxk(nmax) + lz_maxk(nmax) * lz_maxk(nmax);
 }
 
 template <int NT>
@@ -91,9 +93,10 @@ __device__ void lz_bind(LzScratch& z, float* base, int nmax, int jcap) {
   z.beta = z.alpha + kLzMaxJ;
   z.h = z.beta + kLzMaxJ;
   z.ty = z.h + 2 * kLzMaxJ + 8;
-  z.lu = z.ty + jcap * kLzMaxK;
-  z.piv = reinterpret_cast<unsigned*>(z.lu + 4 * jcap * kLzMaxK);
-  z.Bm = reinterpret_cast<float*>(z.piv + 2 * kLzMaxK);
+  const int K = lz_maxk(nmax);
+  z.lu = z.ty + jcap * K;
+  z.piv = reinterpret_cast<unsigned*>(z.lu + 4 * jcap * K);
+  z.Bm = reinterpret_cast<float*>(z.piv + 2 * K);
   z.jcap = jcap;
 }
 
@@ -294,12 +297,12 @@ __device__ float lz_project(float* w, const float* Q, int ldq, int n, int nq, fl
 
 // Inverse iteration on T (s.d, s.e, size J) for the k shifts s.shf[0..k),
 // one thread per target, LU factors in shared memory; eigenvectors into ty
-// (row i, column q, stride kLzMaxK), orthonormalised inside clusters.
-template <int NT>
+// (row i, column q, stride K), orthonormalised inside clusters.
+template <int NT, int K>
 __device__ void lz_tri_vectors(int J, int k, float tnorm, EigScratch& s, LzScratch& z) {
   const int tid = threadIdx.x;
   const float tiny = FLT_EPSILON * tnorm;
-  constexpr int ST = kLzMaxK;
+  constexpr int ST = K;
   float* dd = z.lu;
   float* du = dd + z.jcap * ST;
   float* du2 = du + z.jcap * ST;
@@ -376,8 +379,8 @@ __device__ void lz_tri_vectors(int J, int k, float tnorm, EigScratch& s, LzScrat
 }
 
 // Ritz values of T_J above thr (descending) into s.lam and their vectors
-// into z.ty.  Returns the count (a count above kLzMaxK means "too many").
-template <int NT>
+// into z.ty.  Returns the count (a count above K means "too many").
+template <int NT, int K>
 __device__ int lz_ritz(int J, float thr, EigScratch& s, LzScratch& z, float* tnorm_out) {
   const int tid = threadIdx.x;
   for (int i = tid; i < J; i += NT) {
@@ -388,8 +391,8 @@ __device__ int lz_ritz(int J, float thr, EigScratch& s, LzScratch& z, float* tno
   float tn = 0.f;
   const int k = top_eigenvalues<NT>(J, thr, s, &tn);
   *tnorm_out = tn;
-  if (k == 0 || k > kLzMaxK) return k;
-  lz_tri_vectors<NT>(J, k, tn, s, z);
+  if (k == 0 || k > K) return k;
+  lz_tri_vectors<NT, K>(J, k, tn, s, z);
   return k;
 }
 
@@ -409,7 +412,7 @@ __device__ float gershgorin_lower(S A, int n, float* ones, float* sums, float* r
 //  Gs  G in lower storage, read only (the Lanczos operator).
 //  Q   shared scratch of jmax * lz_ldq<NMAX>(n) floats (column j at
 //      Q + j * lz_ldq<NMAX>(n)), jmax <= n.
-//  U   receives the kept Ritz vectors (kLzMaxK * n floats, column-major,
+//  U   receives the kept Ritz vectors (lz_maxk(NMAX) * n floats, column-major,
 //      any memory).
 //  warm / kwarm: previous Ritz vectors (column-major n x kwarm) or kwarm = 0.
 //  gbound: an upper bound of ||G||_2.
@@ -418,11 +421,11 @@ __device__ float gershgorin_lower(S A, int n, float* ones, float* sums, float* r
 // Steps 1-3 and the set-up of step 4.  On success returns k >= 0 (pairs
 // above thr) with s.lam[0..k), the vectors in U's columns 0..k-1 (U holds
 // ku >= k kept pairs, *ku_out = ku), U and What = W - U sym(B) / 2 staged at
-// panel and panel + 8 n8 (n8 = roundup(n, 8)) and the certificate shift
+// panel and panel + K n8 (n8 = roundup(n, 8), K = lz_maxk(NMAX)) and the certificate shift
 // in *c0_out (and, if J_out is given, the Lanczos steps run in *J_out):
 // the pairs are certified iff
-//   regchol_pd<NT, NMAX>(G, n, *c0_out, true, panel, panel + 8 n8, ku,
-//                        panel + 16 n8, red)
+//   regchol_pd<NT, NMAX>(G, n, *c0_out, true, panel, panel + K n8, ku,
+//                        panel + 2 K n8, red)
 // holds (one call site per kernel keeps the code size and the register
 // allocation of that routine in one place).  Returns -1 when the caller
 // must fall back.  G is never modified.
@@ -432,7 +435,7 @@ __device__ int lanczos_candidates(SG Gs, int n, float thr, float gbound, float* 
                                   uint32_t seed, EigScratch& s, LzScratch& z, float* panel,
                                   int* ku_out, float* c0_out, int slot = -1,
                                   int* J_out = nullptr) {
-  constexpr int NW = NT / 32;
+  constexpr int NW = NT / 32, K = lz_maxk(NMAX);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   PHASE_INIT();
   const float thr_keep = 0.95f * thr;  // pairs kept in U (deflated)
@@ -488,64 +491,76 @@ __device__ int lanczos_candidates(SG Gs, int n, float thr, float gbound, float* 
     PHASE(slot, 10);
     if (J >= jmin && ((J - jmin) % 4 == 0 || J == jmax)) {
       // converged when every kept Ritz pair has |beta_J * y_{J-1}| small
-      k = lz_ritz<NT>(J, thr_keep, s, z, &tn);
+      k = lz_ritz<NT, K>(J, thr_keep, s, z, &tn);
       PHASE(slot, 11);
-      if (k > kLzMaxK) {
+      if (k > K) {
       if (J_out) *J_out = J;
       return -1;
     }
       bool conv = true;
       const float bJ = z.beta[J - 1];
+      // (many pairs: each adds its share of the error)
+      const float tol = k > 8 ? 3e-6f : 1e-5f;
       for (int q = 0; q < k; ++q)
-        if (fabsf(bJ * z.ty[(J - 1) * kLzMaxK + q]) > 1e-5f * fmaxf(s.lam[0], thr)) conv = false;
+        if (fabsf(bJ * z.ty[(J - 1) * K + q]) > tol * fmaxf(s.lam[0], thr)) conv = false;
       if (conv) break;
       k = -1;
     }
   }
   if (k < 0) {
-    k = lz_ritz<NT>(J, thr_keep, s, z, &tn);
-    if (k > kLzMaxK) {
+    k = lz_ritz<NT, K>(J, thr_keep, s, z, &tn);
+    if (k > K) {
       if (J_out) *J_out = J;
       return -1;
     }
   }
   const int ku = k;
-  // U = Q_J Y (n x ku) into the caller's U and, row-major n x 8 with zero
-  // columns beyond ku, into X8 (shared; Q may alias the panel, so the values
-  // wait in registers for the barrier)
+  // U = Q_J Y (n x ku) into the caller's U and, as K / 8 row-major n x 8
+  // arrays with zero columns beyond ku, into X8 (shared; Q may alias the
+  // panel, so the values wait in registers for the barrier)
+  constexpr int H = K / 8, PER = (8 * NMAX + NT - 1) / NT;
   static_assert(8 * NMAX <= 4 * NT, "staging split");
-  float* X8 = panel + 16 * NMAX;
-  float* Y8 = panel + 24 * NMAX;
-  float uv[4];
+  float* X8 = panel;
+  float* Y8 = panel + K * NMAX;
+  const int n8 = (n + 7) & ~7;
+  float uv[H][PER];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int e = tid + i * NT, r = e >> 3, q = e & 7;
-    float v = 0.f;
-    if (r < n && q < ku)
-      for (int jj = 0; jj < J; ++jj) v = fmaf(Q[jj * ldq + r], z.ty[jj * kLzMaxK + q], v);
-    uv[i] = v;
-  }
+  for (int h = 0; h < H; ++h)
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int e = tid + i * NT, r = e >> 3, q = 8 * h + (e & 7);
+      float v = 0.f;
+      if (r < n && q < ku)
+        for (int jj = 0; jj < J; ++jj) v = fmaf(Q[jj * ldq + r], z.ty[jj * K + q], v);
+      uv[h][i] = v;
+    }
   __syncthreads();
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int e = tid + i * NT, r = e >> 3, q = e & 7;
-    if (r < n) {
-      X8[e] = uv[i];
-      if (q < ku) U[(size_t)q * n + r] = uv[i];
+  for (int h = 0; h < H; ++h)
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int e = tid + i * NT, r = e >> 3, q = 8 * h + (e & 7);
+      if (r < n) {
+        X8[h * 8 * NMAX + e] = uv[h][i];
+        if (q < ku) U[(size_t)q * n + r] = uv[h][i];
+      }
     }
-  }
   __syncthreads();
   PHASE(slot, 12);
-  // W = G U (all columns in one pass over G), B = U^T W, rho
-  symm_rows8<NT, NMAX>(Gs, n, X8, Y8);
-  for (int pr = warp; pr < ku; pr += NW) {
+  // W = G U (eight columns per pass over G), B = U^T W, rho
+  const int nh = (ku + 7) >> 3;
+  for (int h = 0; h < nh; ++h) symm_rows8<NT, NMAX>(Gs, n, X8 + h * 8 * NMAX, Y8 + h * 8 * NMAX);
+  for (int pr = warp; pr < ku * nh; pr += NW) {
+    const int p = pr % ku, h = pr / ku;
+    const float* Xp = X8 + (p >> 3) * 8 * NMAX + (p & 7);
+    const float* Yh = Y8 + h * 8 * NMAX;
     float d[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) d[q] = 0.f;
     for (int r = lane; r < n; r += 32) {
-      const float x = X8[r * 8 + pr];
-      const float4 y0 = *reinterpret_cast<const float4*>(Y8 + r * 8);
-      const float4 y1 = *reinterpret_cast<const float4*>(Y8 + r * 8 + 4);
+      const float x = Xp[r * 8];
+      const float4 y0 = *reinterpret_cast<const float4*>(Yh + r * 8);
+      const float4 y1 = *reinterpret_cast<const float4*>(Yh + r * 8 + 4);
       d[0] = fmaf(x, y0.x, d[0]);
       d[1] = fmaf(x, y0.y, d[1]);
       d[2] = fmaf(x, y0.z, d[2]);
@@ -558,54 +573,68 @@ __device__ int lanczos_candidates(SG Gs, int n, float thr, float gbound, float* 
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const float t = warp_sum(d[q]);
-      if (lane == 0 && q < ku) z.Bm[pr * kLzMaxK + q] = t;
+      if (lane == 0 && 8 * h + q < ku) z.Bm[p * K + 8 * h + q] = t;
     }
   }
   __syncthreads();
   part = 0.f;
-  for (int e = tid; e < 8 * n; e += NT) {
-    const int q = e & 7;
-    if (q < ku) {
-      const float rr = Y8[e] - z.Bm[q * kLzMaxK + q] * X8[e];
-      part = fmaf(rr, rr, part);
+  for (int h = 0; h < nh; ++h)
+    for (int e = tid; e < 8 * n; e += NT) {
+      const int q = 8 * h + (e & 7);
+      if (q < ku) {
+        const float rr = Y8[h * 8 * NMAX + e] - z.Bm[q * K + q] * X8[h * 8 * NMAX + e];
+        part = fmaf(rr, rr, part);
+      }
     }
-  }
   const float rho = sqrtf(block_sum<NT>(part, s.red));
   PHASE(slot, 13);
   // kept pairs: Rayleigh quotients, count above thr; pairs above thr first
   int kk = 0;
   for (int q = 0; q < ku; ++q) {
-    const float th = z.Bm[q * kLzMaxK + q];
+    const float th = z.Bm[q * K + q];
     kk += th > thr;
-    if (q > 0 && th > thr && !(z.Bm[(q - 1) * kLzMaxK + (q - 1)] > thr)) {
+    if (q > 0 && th > thr && !(z.Bm[(q - 1) * K + (q - 1)] > thr)) {
       if (J_out) *J_out = J;
       return -1;
     }
   }
   const float c0 = thr - 2.f * rho - 8.f * (float)(ku + 1) * FLT_EPSILON * gbound;
   if (!(c0 > 0.f)) {
-      if (J_out) *J_out = J;
-      return -1;
+    if (J_out) *J_out = J;
+    return -1;
+  }
+  // P G P = G - U What^T - What U^T with What = W - U sym(B) / 2, staged in
+  // shared memory for the register Cholesky of (c I - P G P): column-major
+  // over X8 and Y8, so the values wait in registers
+  float wv[H][PER];
+#pragma unroll
+  for (int h = 0; h < H; ++h)
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int e = tid + i * NT, r = e >> 3, q = 8 * h + (e & 7);
+      float w = 0.f;
+      if (r < n && q < ku) {
+        w = Y8[h * 8 * NMAX + e];
+        for (int p = 0; p < ku; ++p)
+          w = fmaf(-0.25f * (z.Bm[p * K + q] + z.Bm[q * K + p]),
+                   X8[(p >> 3) * 8 * NMAX + r * 8 + (p & 7)], w);
+      }
+      wv[h][i] = w;
     }
   __syncthreads();
-  if (tid < ku) s.lam[tid] = z.Bm[tid * kLzMaxK + tid];
-  // P G P = G - U What^T - What U^T with What = W - U sym(B) / 2, staged in
-  // shared memory for the register Cholesky of (c I - P G P)
-  const int n8 = (n + 7) & ~7;
+  if (tid < ku) s.lam[tid] = z.Bm[tid * K + tid];
   float* U8 = panel;
-  float* W8 = panel + 8 * n8;
-  for (int e = tid; e < ku * n8; e += NT) {
-    const int q = e / n8, r = e - q * n8;
-    float u = 0.f, w = 0.f;
-    if (r < n) {
-      u = X8[r * 8 + q];
-      w = Y8[r * 8 + q];
-      for (int p = 0; p < ku; ++p)
-        w = fmaf(-0.25f * (z.Bm[p * kLzMaxK + q] + z.Bm[q * kLzMaxK + p]), X8[r * 8 + p], w);
+  float* W8 = panel + K * n8;
+#pragma unroll
+  for (int h = 0; h < H; ++h)
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int e = tid + i * NT, r = e >> 3, q = 8 * h + (e & 7);
+      if (r < n8 && q < ku) {
+        U8[q * n8 + r] = r < n ? uv[h][i] : 0.f;
+        W8[q * n8 + r] = wv[h][i];
+      }
     }
-    U8[e] = u;
-    W8[e] = w;
-  }
   __syncthreads();
   PHASE(slot, 11);
   *ku_out = ku;

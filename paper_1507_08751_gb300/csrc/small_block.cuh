@@ -51,7 +51,7 @@ struct SmallLayout {
     oL = al(oG + nn * (nn + 1));
     oQ = al(oL + lz_cert_floats(NMAX, NT));
     oU = kLz ? oQ + lz_ldq<NMAX>(NMAX) * JCAP : oQ;
-    oZ = kLz ? oU + NMAX * kLzMaxK : oU;
+    oZ = kLz ? oU + NMAX * lz_maxk(NMAX) : oU;
     oEnd = kLz ? al(oZ + lz_scratch_floats(NMAX, JCAP)) : oQ;
     oP = mm * nn <= nn * (nn + 1) ? oG : oEnd;
     total = oP == oG ? oEnd : oEnd + mm * nn;
@@ -59,7 +59,7 @@ struct SmallLayout {
 };
 static_assert(16 * 16 <= lz_cert_floats(16, 32), "Y alias (16)");
 static_assert(32 * 32 <= lz_cert_floats(32, 64), "Y alias (32)");
-static_assert(64 * 64 <= lz_cert_floats(64, 128) + 65 * 32 + 64 * kLzMaxK, "Y alias (64)");
+static_assert(64 * 64 <= lz_cert_floats(64, 128) + 65 * 32 + 64 * lz_maxk(64), "Y alias (64)");
 
 // Block b of the scale by the calling CTA (NT threads, dynamic shared memory
 // `sm` laid out by SmallLayout<NT, NMAX>); `a2(off, row, col)` gives the
@@ -97,7 +97,7 @@ __device__ __forceinline__ void small_block_svt(const ScaleLaunch& a, int b, flo
   s.xs = s.hi + NT;
   s.cnt = reinterpret_cast<int*>(s.xs + NT);
   s.red = reinterpret_cast<float*>(s.cnt + NT);
-  // Lanczos region: Q (lz_ldq x JCAP), U (NMAX x kLzMaxK); none for blocks
+  // Lanczos region: Q (lz_ldq x JCAP), U (NMAX x lz_maxk); none for blocks
   // of width <= 16, which skip Lanczos (kAttempts == 1)
   constexpr int kAttempts = SmallLayout<NT, NMAX>::kLz ? 2 : 1;
   constexpr int JCAP = SmallLayout<NT, NMAX>::JCAP;
@@ -219,7 +219,8 @@ __device__ __forceinline__ void small_block_svt(const ScaleLaunch& a, int b, flo
     }
     fl += (float)fl_chol(nn);
     const bool pd = regchol_pd<NT, NMAX>(LowerFull{G, ldg}, nn, c0, attempt == 1, panel,
-                                         panel + 8 * n8, attempt == 1 ? ku : 0, panel + 16 * n8,
+                                         panel + lz_maxk(NMAX) * n8, attempt == 1 ? ku : 0,
+                                         panel + 2 * lz_maxk(NMAX) * n8,
                                          s.red, attempt == 1 ? 5 + SLOT : -1);
     __syncthreads();
     PHASE(SLOT, 8 + attempt);

@@ -1,0 +1,65 @@
+"""Block SVT of blocks whose thresholded rank runs through the limits of the
+eigen paths (8 pairs up to 64 wide, 16 pairs up to 256 wide), against the FP64
+oracle, through the C ABI."""
+
+import numpy as np
+import pytest
+
+import oracle as O
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-4
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1507_08751_gb300 import binding as B
+    c = B.Context(0)
+    yield c
+    c.close()
+
+
+def _blocks(seed, M, N, m, n, ranks, tau):
+    """Dense noise well below tau plus, per block, the given rank of terms with
+    singular values between 1.3 and 6 tau."""
+    rng = np.random.default_rng(seed)
+    A = 0.3 * tau / (np.sqrt(m) + np.sqrt(n)) * rng.standard_normal((M, N))
+    i = 0
+    for p in range(M // m):
+        for q in range(N // n):
+            r = min(ranks[i % len(ranks)], m, n)
+            i += 1
+            if r:
+                u, _ = np.linalg.qr(rng.standard_normal((m, r)))
+                v, _ = np.linalg.qr(rng.standard_normal((n, r)))
+                s = tau * np.exp(rng.uniform(np.log(1.3), np.log(6.0), r))
+                A[p * m:(p + 1) * m, q * n:(q + 1) * n] += (u * s) @ v.T
+    return A.astype(np.float32)
+
+
+@pytest.mark.parametrize("m,n", [(17, 17), (33, 40), (48, 64), (64, 64), (120, 60), (65, 65),
+                                 (100, 130), (129, 128), (250, 200), (256, 256), (700, 256)])
+def test_ranks_around_the_limits(ctx, m, n):
+    ranks = (0, 1, 7, 8, 9, 12, 15, 16, 17, 24)
+    M, N, tau = 5 * m, 2 * n, 20.0
+    A = _blocks(m * 1000 + n, M, N, m, n, ranks, tau)
+    Z = torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")
+    rank = torch.empty((10,), dtype=torch.int32, device="cuda")
+    ctx.msllr_blocksvt(torch.from_numpy(A).cuda(), Z, m, n, tau, (0, 0), rank_out=rank)
+    torch.cuda.synchronize()
+    want = O.block_svt(A.astype(np.float64), m, n, tau)
+    got = Z.cpu().numpy().astype(np.float64)
+    assert np.linalg.norm(got - want) <= TOL * np.linalg.norm(want)
+    B = A.astype(np.float64).reshape(5, m, 2, n).transpose(0, 2, 1, 3).reshape(-1, m, n)
+    s = np.linalg.svd(B, compute_uv=False)
+    near = (np.abs(s - tau) <= 1e-4 * np.maximum(s[:, :1], tau)).any(axis=1)
+    assert np.all((rank.cpu().numpy() == (s > tau).sum(axis=1)) | near)
+    # block by block, so that a weak block's error is not hidden by a strong one
+    for b in range(10):
+        p, q = divmod(b, 2)
+        sl = np.s_[p * m:(p + 1) * m, q * n:(q + 1) * n]
+        assert np.linalg.norm(got[sl] - want[sl]) <= TOL * max(np.linalg.norm(want[sl]), tau)
