@@ -190,6 +190,10 @@ cudaError_t launch_gram_tc(const ScaleLaunch& s, float* G, float* part, int chun
 // MSLLR_GRAM_FP32=1: the FP32 CUDA-core Gram kernels instead (comparisons)
 bool gram_fp32_forced();
 
+// Eigenpairs of blocks up to 256 wide (k_eig.cu): kernel attributes, launch.
+cudaError_t configure_eig();
+cudaError_t launch_eig(const ScaleLaunch& s, const BigWorkspace& ws, int nblocks, cudaStream_t st);
+
 // The Householder path of blocks up to 256 wide (k_tridiag.cu): kernel
 // attributes, and the launch over the blocks with ws.k < 0 (`groups` clusters
 // stride over them).

@@ -3,9 +3,9 @@
 //   1. gram_tiles: G_b = C_b^T C_b for every block, tiled 64x64 over the
 //      lower triangle and split over row chunks (partial sums reduced in a
 //      fixed order, so results are deterministic), stored packed;
-//   2. eig_big: one CTA per block -- skip bound (Sec. 8), certified zero
-//      rank or certified Lanczos eigenpairs of G_b (lanczos.cuh,
-//      regchol.cuh), output V_b diag(sqrt(f));
+//   2. eig (k_eig.cu): a cluster per block -- skip bound (Sec. 8), certified
+//      zero rank or certified Lanczos eigenpairs of G_b, output V_b
+//      diag(sqrt(f));
 //   3. tridiag (k_tridiag.cu): the Householder path for the blocks step 2
 //      could not certify;
 //   4. rebuild: Z'_b = (C_b V_f) V_f^T, scattered through Shift_{-s}, with
@@ -22,16 +22,11 @@
 
 namespace msllr {
 
-cudaError_t set_phase_buffer_big(unsigned long long* p) {
-  return cudaMemcpyToSymbol(g_phase_acc, &p, sizeof(p));
-}
-
 namespace {
 
 constexpr int kTile = 64;       // Gram tile
 constexpr int kChunk = 256;     // rows of C per Gram partial sum
 constexpr int kGramThreads = 256;
-constexpr int kEigThreads = 512;
 constexpr int kEigMax = 256;
 constexpr int kEigK = lz_maxk(kEigMax);  // Ritz pairs kept per block
 constexpr int kRebThreads = 256;
@@ -166,199 +161,6 @@ gram_reduce_kernel(const float* __restrict__ part, float* __restrict__ G, int nn
     for (int c = 0; c < chunks; ++c)
       s += part[(((size_t)b * chunks + c) * ntiles + t) * (kTile * kTile) + e];
     if (j <= i) G[(size_t)b * nn * nn + (size_t)i * (i + 1) / 2 + j] = s;
-  }
-}
-
-// panel region: Lanczos Q (kLzMaxJ x n), or the certificate's staging and
-// Cholesky scratch, or the V_f staging
-constexpr int kEigPanelFloats = (lz_cert_floats(kEigMax, kEigThreads) > kLzMaxJ * kEigMax)
-                                    ? lz_cert_floats(kEigMax, kEigThreads)
-                                    : kLzMaxJ * kEigMax;
-
-size_t eig_smem_bytes(int nn) {
-  return sizeof(float) * ((((size_t)nn * (nn + 1) / 2 + 3) & ~(size_t)3) + kEigPanelFloats +
-                          9 * kEigMax + 4 * kEigThreads + 64 + lz_scratch_floats(kEigMax, kLzMaxJ));
-}
-
-// Up to three power steps from a pseudo-random vector: true when the
-// Rayleigh quotient (a lower bound of lambda_max(G)) exceeds `thr`.  Called
-// with thr = kZeroTry tau^2: a block whose quotient comes that close to
-// tau^2 goes straight to the Lanczos path, because its zero-rank
-// certificate would most likely fail, and a failed Cholesky costs as much
-// as a successful one (the decision only routes work; the certificates
-// decide the result).
-constexpr float kZeroTry = 0.85f;
-template <class S>
-__device__ bool power_above(S G, int n, float thr, EigScratch& s, LzScratch& z, int* steps) {
-  constexpr int NT = kEigThreads;
-  const int tid = threadIdx.x;
-  float part = 0.f;
-  for (int e = tid; e < n; e += NT) {
-    const float v = lz_hash(0xC0FFEEu, e) + 1.5f;
-    z.x[e] = v;
-    part = fmaf(v, v, part);
-  }
-  float nrm = sqrtf(block_sum<NT>(part, s.red));
-  float rq = 0.f;
-  *steps = 0;
-  for (int it = 0; it < 3; ++it) {
-    *steps = it + 1;
-    for (int e = tid; e < n; e += NT) z.x[e] /= nrm;
-    __syncthreads();
-    symv_rows<NT, kEigMax>(G, n, z.x, z.w);
-    float p1 = 0.f, p2 = 0.f;
-    for (int e = tid; e < n; e += NT) {
-      p1 = fmaf(z.x[e], z.w[e], p1);
-      p2 = fmaf(z.w[e], z.w[e], p2);
-    }
-    rq = block_sum<NT>(p1, s.red);
-    nrm = sqrtf(block_sum<NT>(p2, s.red));
-    if (rq > thr || !(nrm > 0.f)) break;
-    for (int e = tid; e < n; e += NT) z.x[e] = z.w[e];
-    __syncthreads();
-  }
-  return rq > thr;
-}
-
-__global__ void __launch_bounds__(kEigThreads)
-eig_big_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace ws) {
-  extern __shared__ float sm[];
-  constexpr int NT = kEigThreads, NMAX = kEigMax;
-  const int b = blockIdx.x, tid = threadIdx.x;
-  const int nn = a.m >= a.n ? a.n : a.m;
-  const float* Gg = Gall + (size_t)b * nn * nn;
-  float* Y = ws.Y + (size_t)b * ws.ystride;
-  float* Gp = sm;
-  float* panel = Gp + (((nn * (nn + 1)) / 2 + 3) & ~3);  // kEigPanelFloats, 16-byte aligned
-  float* scr = panel + kEigPanelFloats;
-  EigScratch s;
-  s.d = scr;
-  s.e = s.d + NMAX;
-  s.e2 = s.e + NMAX;
-  s.beta = s.e2 + NMAX;
-  s.vbuf = s.beta + NMAX;
-  s.pbuf = s.vbuf + NMAX;
-  s.lam = s.pbuf + NMAX;
-  s.shf = s.lam + NMAX;
-  s.clus = reinterpret_cast<int*>(s.shf + NMAX);
-  s.lo = reinterpret_cast<float*>(s.clus + NMAX);
-  s.hi = s.lo + NT;
-  s.xs = s.hi + NT;
-  s.cnt = reinterpret_cast<int*>(s.xs + NT);
-  s.red = reinterpret_cast<float*>(s.cnt + NT);
-  LzScratch z;
-  // Lanczos Q shares the panel region with the certificate scratch; they
-  // are never live together
-  float* Qs = panel;
-  lz_bind<NT>(z, s.red + 64, NMAX, kLzMaxJ);
-  PHASE_INIT();
-  LowerPacked Gacc{Gp};
-  // G arrives packed (lower triangle, row by row): a straight copy
-  auto load_g = [&]() {
-    const int ntri = nn * (nn + 1) / 2;
-    if ((ntri & 3) == 0 && ((reinterpret_cast<uintptr_t>(Gg) & 15) == 0)) {
-      const float4* src = reinterpret_cast<const float4*>(Gg);
-      float4* dst = reinterpret_cast<float4*>(Gp);
-      for (int e = tid; e < ntri / 4; e += NT) dst[e] = src[e];
-    } else {
-      for (int e = tid; e < ntri; e += NT) Gp[e] = Gg[e];
-    }
-    __syncthreads();
-  };
-  load_g();
-  PHASE(3, 0);
-  const float thr = a.tau * a.tau;
-  // trace and Gershgorin bounds of lambda_max(G)
-  float tr = 0.f;
-  for (int i = tid; i < nn; i += NT) tr += Gacc.at(i, i);
-  tr = block_sum<NT>(tr, s.red);
-  const float rs = gershgorin_lower<NT, NMAX>(Gacc, nn, z.x, z.w, s.red);
-  const float gbound = fminf(tr, rs);
-  double fl = nn + fl_symv(nn);  // trace, Gershgorin row sums
-  const bool full = (a.m == launch_rows(a) && a.n == a.N);
-  const int kwarm = (a.warm_start && (full || !a.shift)) ? min(ws.kwarm[b], kEigK) : 0;
-  bool skipped = false, lanczos_ok = false;
-  int k = -1, ku = 0;
-  // Two certificates share one Cholesky call site: attempt 0 tests
-  // lambda_max(G) < tau^2 (zero rank), attempt 1 certifies the Lanczos pairs
-  // by the deflated matrix.
-  const int n8 = (nn + 7) & ~7;
-  float* U = Y;
-  for (int attempt = 0; attempt < 2 && k < 0 && a.skip_bound; ++attempt) {
-    float c0;
-    int kk = 0;
-    if (attempt == 0) {
-      if (gbound <= thr) {
-        skipped = true;
-        k = 0;
-        break;
-      }
-      if (kwarm > 0) continue;
-      int psteps = 0;
-      const bool above = power_above(Gacc, nn, kZeroTry * thr, s, z, &psteps);
-      fl += psteps * (fl_symv(nn) + 4.0 * nn);
-      if (above) continue;
-      // certified lambda_max(G) < tau^2 by Cholesky of (tau^2 - margin) I - G
-      c0 = thr - (float)n8 * (float)n8 * FLT_EPSILON * (thr + gbound);
-      if (!(c0 > 0.f)) continue;
-      PHASE(3, 6);
-    } else {
-      PHASE(3, 1);
-      const float* warm = ws.warm + (size_t)b * kEigK * nn;
-      int J = 0;
-      kk = lanczos_candidates<NT, NMAX>(Gacc, nn, thr, gbound, Qs,
-                                                        min(nn, kLzMaxJ), U, warm, kwarm,
-                                                        0x1234567u + 977u * job_block(a, b), s, z, panel, &ku,
-                                                        &c0, 4, &J);
-      fl += fl_lanczos(nn, J, ku);
-      PHASE(3, 5);
-      if (kk < 0) break;
-      fl += fl_deflate(nn, ku);
-    }
-    fl += fl_chol(nn);
-    const bool pd = regchol_pd<NT, NMAX>(Gacc, nn, c0, attempt == 1, panel, panel + kEigK * n8,
-                                         attempt == 1 ? ku : 0, panel + 2 * kEigK * n8, s.red,
-                                         3 + attempt);
-    PHASE(3, 7 + attempt);
-    if (pd) {
-      k = kk;
-      skipped = attempt == 0;
-      lanczos_ok = attempt == 1;
-    }
-  }
-  if (lanczos_ok) {
-    // keep the Ritz vectors for the next call's warm start
-    float* wdst = ws.warm + (size_t)b * kEigK * nn;
-    for (int e = tid; e < nn * ku; e += NT) wdst[e] = U[e];
-    if (tid == 0) ws.kwarm[b] = ku;
-    // V_f (row-major, ld nn) for the rebuild, staged through shared memory
-    for (int e = tid; e < nn * k; e += NT) panel[e] = U[e];
-    __syncthreads();
-    for (int e = tid; e < nn * k; e += NT) {
-      const int i = e / k, q = e - i * k;
-      const float sig = sqrtf(s.lam[q]);
-      Y[(size_t)i * nn + q] = panel[(size_t)q * nn + i] * sqrtf(fmaxf(1.f - a.tau / sig, 0.f));
-    }
-  }
-  if (tid == 0) {
-    if (a.cnt) atomicAdd(a.cnt + 5, (unsigned long long)fl);
-    // k < 0: not settled here; tridiag_kernel takes the block
-    ws.k[b] = k;
-    if (k < 0) {
-      if (ws.kwarm) ws.kwarm[b] = 0;
-    } else {
-      if (a.rank_out) a.rank_out[b] = k;
-      if (a.cnt) {
-        if (skipped) atomicAdd(a.cnt, 1ull);
-        if (k == 0) atomicAdd(a.cnt + 1, 1ull);
-        if (lanczos_ok) atomicAdd(a.cnt + 2, 1ull);
-      }
-      if (a.nuc_acc && k > 0) {
-        double t = 0.0;
-        for (int q = 0; q < k; ++q) t += (double)fmaxf(sqrtf(s.lam[q]) - a.tau, 0.f);
-        atomicAdd(a.nuc_acc, t);
-      }
-    }
   }
 }
 
@@ -597,11 +399,9 @@ cudaError_t configure_big_kernels() {
   if (cudaError_t e0 = configure_gram_tc()) return e0;
   if (cudaError_t e1 = configure_cert()) return e1;
   if (cudaError_t e2 = configure_subspace()) return e2;
-  cudaError_t e = cudaFuncSetAttribute(eig_big_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)eig_smem_bytes(kEigMax));
-  if (e != cudaSuccess) return e;
+  if (cudaError_t e4 = configure_eig()) return e4;
   if (cudaError_t e3 = configure_tridiag()) return e3;
-  e = cudaFuncSetAttribute(rebuild_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(rebuild_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            100 * 1024);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(rebuild_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -641,7 +441,7 @@ cudaError_t launch_big(const ScaleLaunch& s, const BigWorkspace& ws, cudaStream_
   if (after_gram)
     if (cudaError_t e_ = cudaEventRecord(after_gram, st)) return e_;
   PROF_BEFORE(KK_EIG)
-  eig_big_kernel<<<d.nblocks, kEigThreads, eig_smem_bytes(d.nn), st>>>(s, ws.G, ws);
+  if (cudaError_t e_ = launch_eig(s, ws, d.nblocks, st)) return e_;
   PROF_AFTER()
   PROF_BEFORE(KK_EIG_FALLBACK)
   // up to 64 CTAs stride over the blocks: enough for scales where many blocks
