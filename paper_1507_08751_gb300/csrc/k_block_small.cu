@@ -22,7 +22,7 @@ cudaError_t set_phase_buffer_small(unsigned long long* p) {
 namespace {
 
 template <int NT, int NMAX, bool ST>
-__global__ void __launch_bounds__(NT, NT == 32 ? 24 : (NT == 128 ? 3 : 1))
+__global__ void __launch_bounds__(NT, NT == 32 ? 24 : (NT == 128 ? 3 : 8))
 blocksvt_small_kernel(ScaleLaunch a) {
   extern __shared__ float sm[];
   small_block_svt<NT, NMAX, ST>(a, (int)blockIdx.x, sm, A2Global{a.A2});

@@ -86,23 +86,6 @@ __device__ __forceinline__ uint64_t e_desc(uint32_t saddr) {
          ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
 
-// the sum over a warp's lanes of eight values (one per row of the warp): row
-// 4 bit4 + 2 bit3 + bit2 of the lane, in all four lanes that agree on them
-__device__ __forceinline__ float sum8(float p[8], int lane) {
-#pragma unroll
-  for (int o = 16, h = 4; o >= 4; o >>= 1, h >>= 1) {
-    const bool up = lane & o;
-#pragma unroll
-    for (int i = 0; i < h; ++i) {
-      const float keep = up ? p[i + h] : p[i], give = up ? p[i] : p[i + h];
-      p[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-    }
-  }
-  p[0] += __shfl_xor_sync(0xffffffffu, p[0], 2);
-  p[0] += __shfl_xor_sync(0xffffffffu, p[0], 1);
-  return p[0];
-}
-
 // The distributed matrix of one block.
 template <int CL>
 struct RegGram {
@@ -309,147 +292,6 @@ __device__ __forceinline__ bool eig_power_cert(const RegGram<CL>& g, unsigned ch
       if (tid == 0 && err) atomicOr(err, 1);
     }
   }
-}
-
-// Ritz values of T_J above thr (descending, at most K) into lam and their
-// vectors into z.ty, a warp per pair: count and multisection on Sturm counts
-// (32 points a round), then two steps of inverse iteration in lane 0, as
-// top_eigenvalues and lz_tri_vectors do with CTA barriers.  Returns the count
-// (above K: nothing else is set).  d, e2: J shared floats each.
-template <int K>
-__device__ __forceinline__ int eig_ritz(int J, float thr, const LzScratch& z, float* d, float* e2,
-                                        float* lam, float* shf, int* clus, float* red) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  static_assert(kENW >= K, "a warp per pair");
-  __syncthreads();
-  // norm and bounds, in every warp (J <= 32)
-  const float ai = lane < J ? z.alpha[lane] : 0.f;
-  const float bi = lane < J - 1 ? z.beta[lane] : 0.f;
-  const float bm = __shfl_up_sync(0xffffffffu, bi, 1);
-  const float rad = fabsf(bi) + (lane > 0 ? fabsf(bm) : 0.f);
-  const float gup = warp_max(lane < J ? ai + rad : -FLT_MAX);
-  const float tn = warp_max(lane < J ? fabsf(ai) + rad : -FLT_MAX);
-  const float pivmin = FLT_MIN * fmaxf(1.f, warp_max(bi * bi));
-  if (warp == 0 && lane < J) {
-    d[lane] = ai;
-    e2[lane] = bi * bi;
-  }
-  __syncthreads();
-  const int k = J - sturm_below(d, e2, J, thr, pivmin);
-  if (k <= 0 || k > K) return k < 0 ? 0 : k;
-  if (warp < k) {
-    const int target = J - 1 - warp;  // ascending index of the eigenvalue sought
-    float lo = thr, hi = gup + 4.f * FLT_EPSILON * fmaxf(fabsf(gup), tn) + pivmin;
-    const float tol = 2.f * FLT_EPSILON * tn;
-    for (int round = 0; round < 64; ++round) {
-      if (!(hi - lo > fmaxf(tol, 2.f * FLT_EPSILON * fmaxf(fabsf(lo), fabsf(hi))))) break;
-      const float x = lo + (hi - lo) * ((float)(lane + 1) / 33.f);
-      const unsigned above =
-          __ballot_sync(0xffffffffu, sturm_below(d, e2, J, x, pivmin) > target);
-      // counts grow with x: the first point above the target brackets it
-      float nlo = lo, nhi = hi;
-      if (above == 0u) {
-        nlo = __shfl_sync(0xffffffffu, x, 31);
-      } else {
-        const int f = __ffs(above) - 1;
-        nhi = __shfl_sync(0xffffffffu, x, f);
-        if (f > 0) nlo = __shfl_sync(0xffffffffu, x, f - 1);
-      }
-      lo = fminf(nlo, nhi);
-      hi = nhi;
-    }
-    if (lane == 0) lam[warp] = 0.5f * (lo + hi);
-  }
-  __syncthreads();
-  // inverse-iteration shifts kept apart, clusters of close eigenvalues
-  if (tid == 0) {
-    shf[0] = lam[0];
-    clus[0] = 0;
-    for (int j = 1; j < k; ++j) {
-      shf[j] = fminf(lam[j], shf[j - 1] - 10.f * FLT_EPSILON * tn);
-      clus[j] = (lam[j - 1] - lam[j] <= 1e-3f * tn) ? clus[j - 1] : j;
-    }
-  }
-  __syncthreads();
-  bool grouped = false;
-  for (int j = 1; j < k; ++j) grouped = grouped || clus[j] != j;
-  const float tiny = FLT_EPSILON * tn;
-  float* dd = z.lu + warp;
-  float* du = dd + z.jcap * K;
-  float* du2 = du + z.jcap * K;
-  float* dl = du2 + z.jcap * K;
-  float* y = z.ty + warp;
-  unsigned bits = 0u;
-  for (int pass = 0; pass < 2; ++pass) {
-    if (warp < k && lane == 0) {
-      if (pass == 0) {
-        // pivoted LU of T - shift I, tiny pivots replaced by +-tiny
-        const float shift = shf[warp];
-        float di = d[0] - shift, ui = J > 1 ? z.beta[0] : 0.f;
-        for (int i = 0; i < J - 1; ++i) {
-          const float li = z.beta[i], dn = d[i + 1] - shift, un = i < J - 2 ? z.beta[i + 1] : 0.f;
-          float f, p;
-          if (fabsf(di) >= fabsf(li)) {
-            p = (di == 0.f) ? tiny : di;
-            f = li / p;
-            du[i * K] = ui;
-            du2[i * K] = 0.f;
-            di = dn - f * ui;
-            ui = un;
-          } else {
-            f = di / li;
-            p = li;
-            du[i * K] = dn;
-            du2[i * K] = un;
-            di = ui - f * dn;
-            ui = -f * un;
-            bits |= 1u << i;
-          }
-          dl[i * K] = f;
-          // (the reciprocal pivot: the solves multiply)
-          dd[i * K] = 1.f / (fabsf(p) < tiny ? (p < 0.f ? -tiny : tiny) : p);
-          y[i * K] = tiny * lz_hash(977u + warp, i);
-        }
-        dd[(J - 1) * K] = 1.f / (fabsf(di) < tiny ? (di < 0.f ? -tiny : tiny) : di);
-        y[(J - 1) * K] = tiny * lz_hash(977u + warp, J - 1);
-      } else {
-        for (int i = 0; i < J; ++i) y[i * K] *= tiny;
-      }
-      float a = y[0];
-      for (int i = 0; i < J - 1; ++i) {
-        const float b = y[(i + 1) * K], f = dl[i * K];
-        if ((bits >> i) & 1u) {
-          y[i * K] = b;
-          a = a - f * b;
-        } else {
-          y[i * K] = a;
-          a = b - f * a;
-        }
-      }
-      float y1 = a * dd[(J - 1) * K], y2 = 0.f;
-      y[(J - 1) * K] = y1;
-      for (int i = J - 2; i >= 0; --i) {
-        const float u2 = i < J - 2 ? du2[i * K] : 0.f;
-        const float v = (y[i * K] - du[i * K] * y1 - u2 * y2) * dd[i * K];
-        y[i * K] = v;
-        y2 = y1;
-        y1 = v;
-      }
-    }
-    __syncwarp();
-    if (warp < k) {
-      // unit length (a lane per entry)
-      const float v = lane < J ? y[lane * K] : 0.f;
-      const float ss = warp_sum(v * v);
-      if (lane < J) y[lane * K] = v * (ss > 0.f ? rsqrtf(ss) : 0.f);
-    }
-    __syncthreads();
-    if (grouped) {
-      cluster_mgs<kENT>(z.ty, K, J, k, clus, red);
-      __syncthreads();
-    }
-  }
-  return k;
 }
 
 // Power steps route only: a block whose Rayleigh quotient comes this close
@@ -679,7 +521,7 @@ eig_cluster_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace w
         PHASE(4, 10);
         if (J >= jmin && ((J - jmin) % 4 == 0 || J == jmax)) {
           // converged when every kept Ritz pair has |beta_J y_{J-1}| small
-          kr = eig_ritz<K>(J, thr_keep, z, s.d, s.e2, s.lam, s.shf, s.clus, s.red);
+          kr = lz_ritz<NT, K>(J, thr_keep, z, s);
           PHASE(4, 11);
           if (kr > K) {
             many = true;
@@ -697,7 +539,7 @@ eig_cluster_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace w
       }
       __syncthreads();
       if (kr < 0 && !many) {
-        kr = eig_ritz<K>(J, thr_keep, z, s.d, s.e2, s.lam, s.shf, s.clus, s.red);
+        kr = lz_ritz<NT, K>(J, thr_keep, z, s);
         many = kr > K;
       }
       fl += fl_lanczos(n, J, many ? 0 : kr);

@@ -23,8 +23,6 @@
 
 #include <float.h>
 
-#include <type_traits>
-
 #include "common.cuh"
 #include "regchol.cuh"
 #include "symeig.cuh"
@@ -74,7 +72,6 @@ struct LzScratch {
   float* h;      // [2 * kLzMaxJ + 8] projection coefficients (two passes)
   float* ty;     // [jcap * K] eigenvectors of T_J (row i, column q), K = lz_maxk
   float* lu;     // [4 * jcap * K] inverse-iteration LU factors
-  unsigned* piv; // [2 * K] pivot bits
   float* Bm;     // [K * K] U^T G U
   int jcap;      // row capacity of ty / lu (>= Lanczos steps)
 };
@@ -82,7 +79,7 @@ struct LzScratch {
 // floats of LzScratch for a given n capacity and J capacity
 __host__ __device__ constexpr int lz_scratch_floats(int nmax, int jcap) {
   return 2 * nmax + 2 * kLzMaxJ + (2 * kLzMaxJ + 8) + 5 * jcap * lz_maxk(nmax) +
-         2 * lz_maxk(nmax) + lz_maxk(nmax) * lz_maxk(nmax);
+         lz_maxk(nmax) * lz_maxk(nmax);
 }
 
 template <int NT>
@@ -95,8 +92,7 @@ __device__ void lz_bind(LzScratch& z, float* base, int nmax, int jcap) {
   z.ty = z.h + 2 * kLzMaxJ + 8;
   const int K = lz_maxk(nmax);
   z.lu = z.ty + jcap * K;
-  z.piv = reinterpret_cast<unsigned*>(z.lu + 4 * jcap * K);
-  z.Bm = reinterpret_cast<float*>(z.piv + 2 * K);
+  z.Bm = z.lu + 4 * jcap * K;
   z.jcap = jcap;
 }
 
@@ -110,364 +106,362 @@ __device__ __forceinline__ float lz_hash(uint32_t seed, int i) {
   return (float)(h >> 8) * (2.f / 16777216.f) - 1.f;
 }
 
-// y = G x with TPR threads per row (G symmetric in lower storage, n <= NMAX,
-// x and y shared, y must not alias x).  Each thread walks its part of row r
-// in two ranges, G(r, c) for c <= r and G(c, r) above, so every element of
-// the row is read once and the only reduction is a shuffle inside the TPR
-// lanes of the row.  Ends with a CTA barrier.
-template <int NT, int NMAX, bool ABS = false, class S>
-__device__ void symv_rows(S G, int n, const float* x, float* y) {
-  constexpr int TPR = (NT / NMAX >= 2) ? 2 : 1;
-  const int tid = threadIdx.x, p = tid % TPR;
-  if constexpr (std::is_same<S, LowerPacked>::value && NT == 512) {
-    // packed storage: warp w takes rows 32 (w & 7) + lane and half (w >> 3)
-    // of the columns.  All lanes of a warp walk the same column c, so the
-    // loads T(r) + c (c <= r) and T(c) + r (c > r), T(i) = i (i + 1) / 2,
-    // hit distinct banks, and x[c] is a broadcast.  Left of the warp's row
-    // band the row part is contiguous, right of it the column part advances
-    // by c + 1; only the 32 columns of the band need both forms.
-    const float* g = G.g;
-    const int lane = tid & 31, warp = tid >> 5;
-    const int b0 = 32 * (warp & 7), half = warp >> 3;
-    const int r = b0 + lane;
-    const int cs = (n + 1) >> 1;
-    const int c_lo = half ? cs : 0, c_hi = half ? n : cs;
-    float acc = 0.f;
-    if (b0 < n) {
-      const int rr = r < n ? r : n - 1;  // lanes past n compute a dummy row
-      const int tr = (rr * (rr + 1)) / 2;
-      // four accumulators, so that four loads and FMAs are in flight
-      float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-      int c = c_lo;
-      const int e1 = min(c_hi, b0);
-      for (; c + 3 < e1; c += 4) {
-        a0 = fmaf(ABS ? fabsf(g[tr + c]) : g[tr + c], x[c], a0);
-        a1 = fmaf(ABS ? fabsf(g[tr + c + 1]) : g[tr + c + 1], x[c + 1], a1);
-        a2 = fmaf(ABS ? fabsf(g[tr + c + 2]) : g[tr + c + 2], x[c + 2], a2);
-        a3 = fmaf(ABS ? fabsf(g[tr + c + 3]) : g[tr + c + 3], x[c + 3], a3);
-      }
-      for (; c < e1; ++c) a0 = fmaf(ABS ? fabsf(g[tr + c]) : g[tr + c], x[c], a0);
-      const int e2 = min(c_hi, b0 + 32);
-      for (; c < e2; ++c) {
-        const int idx = c <= rr ? tr + c : (c * (c + 1)) / 2 + rr;
-        a1 = fmaf(ABS ? fabsf(g[idx]) : g[idx], x[c], a1);
-      }
-      int idx = (c * (c + 1)) / 2 + rr;
-      for (; c + 3 < c_hi; c += 4) {
-        const int i1 = idx + c + 1;
-        const int i2 = i1 + c + 2;
-        const int i3 = i2 + c + 3;
-        a0 = fmaf(ABS ? fabsf(g[idx]) : g[idx], x[c], a0);
-        a1 = fmaf(ABS ? fabsf(g[i1]) : g[i1], x[c + 1], a1);
-        a2 = fmaf(ABS ? fabsf(g[i2]) : g[i2], x[c + 2], a2);
-        a3 = fmaf(ABS ? fabsf(g[i3]) : g[i3], x[c + 3], a3);
-        idx = i3 + c + 4;
-      }
-      for (; c < c_hi; ++c) {
-        a0 = fmaf(ABS ? fabsf(g[idx]) : g[idx], x[c], a0);
-        idx += c + 1;
-      }
-      acc = (a0 + a1) + (a2 + a3);
-    }
-    if (half && r < n) y[r] = acc;
-    __syncthreads();
-    if (!half && r < n) y[r] += acc;
-  } else {
-    // the row loop is uniform across the CTA so that every lane reaches the
-    // shuffle below
-    for (int r0 = 0; r0 < n; r0 += NT / TPR) {
-      const int r = r0 + tid / TPR;
-      float a0 = 0.f, a1 = 0.f;
-      if (r < n) {
-        int c = p;
-        for (; c + TPR <= r; c += 2 * TPR) {
-          const float g0 = G.at(r, c), g1 = G.at(r, c + TPR);
-          a0 = fmaf(ABS ? fabsf(g0) : g0, x[c], a0);
-          a1 = fmaf(ABS ? fabsf(g1) : g1, x[c + TPR], a1);
-        }
-        if (c <= r) {
-          const float g = G.at(r, c);
-          a0 = fmaf(ABS ? fabsf(g) : g, x[c], a0);
-          c += TPR;
-        }
-        for (; c + TPR < n; c += 2 * TPR) {
-          const float g0 = G.at(c, r), g1 = G.at(c + TPR, r);
-          a0 = fmaf(ABS ? fabsf(g0) : g0, x[c], a0);
-          a1 = fmaf(ABS ? fabsf(g1) : g1, x[c + TPR], a1);
-        }
-        if (c < n) {
-          const float g = G.at(c, r);
-          a0 = fmaf(ABS ? fabsf(g) : g, x[c], a0);
-        }
-      }
-      float acc = a0 + a1;
-      if constexpr (TPR == 2) acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-      if (p == 0 && r < n) y[r] = acc;
-    }
-  }
-  __syncthreads();
-}
-
-// Y = G X for 8 vectors at once (X, Y shared, n x 8 row-major, 16-byte
-// aligned): every element of G is read once per row walk for all 8
-// products.  Same row split as symv_rows; ends with a CTA barrier.
-template <int NT, int NMAX, class S>
-__device__ void symm_rows8(S G, int n, const float* X, float* Yo) {
-  constexpr int TPR = (NT / NMAX >= 2) ? 2 : 1;
-  const int tid = threadIdx.x, p = tid % TPR;
-  for (int r0 = 0; r0 < n; r0 += NT / TPR) {
-    const int r = r0 + tid / TPR;
-    float acc[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = 0.f;
-    if (r < n) {
-      for (int c = p; c < n; c += TPR) {
-        const float g = c <= r ? G.at(r, c) : G.at(c, r);
-        const float4 x0 = *reinterpret_cast<const float4*>(X + c * 8);
-        const float4 x1 = *reinterpret_cast<const float4*>(X + c * 8 + 4);
-        acc[0] = fmaf(g, x0.x, acc[0]);
-        acc[1] = fmaf(g, x0.y, acc[1]);
-        acc[2] = fmaf(g, x0.z, acc[2]);
-        acc[3] = fmaf(g, x0.w, acc[3]);
-        acc[4] = fmaf(g, x1.x, acc[4]);
-        acc[5] = fmaf(g, x1.y, acc[5]);
-        acc[6] = fmaf(g, x1.z, acc[6]);
-        acc[7] = fmaf(g, x1.w, acc[7]);
-      }
-    }
-    if constexpr (TPR == 2) {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], 1);
-    }
-    if (p == 0 && r < n) {
-      *reinterpret_cast<float4*>(Yo + r * 8) = make_float4(acc[0], acc[1], acc[2], acc[3]);
-      *reinterpret_cast<float4*>(Yo + r * 8 + 4) = make_float4(acc[4], acc[5], acc[6], acc[7]);
-    }
-  }
-  __syncthreads();
-}
-
-// w <- (I - Q Q^T) w twice (classical Gram-Schmidt, two passes) over Q's
-// columns 0..nq-1 (column i at Q + i*ldq, shared).  h1 and h2 receive the
-// two passes' coefficients; returns ||w||^2 after the second pass.  Small
-// n: one thread per coefficient with four partial sums (ldq = n + 1 keeps
-// the threads on distinct banks); large n: one warp per coefficient.
-template <int NT, int NMAX>
-__device__ float lz_project(float* w, const float* Q, int ldq, int n, int nq, float* h1,
-                            float* h2, float* red) {
+// Ritz values of T_J above thr (descending, at most K) into lam and their
+// vectors into z.ty, a warp per pair: count and multisection on Sturm counts
+// (32 points a round), then two steps of inverse iteration in its lane 0 (the
+// approximate division only perturbs the factors by an ulp or two, which the
+// second step corrects).
+// Returns the count (above K: nothing else is set).  Uses s.d, s.e2, s.lam,
+// s.shf, s.clus (J entries) and s.red.
+template <int NT, int K>
+__device__ __forceinline__ int lz_ritz(int J, float thr, const LzScratch& z, EigScratch& s) {
   constexpr int NW = NT / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  float part = 0.f;
-#pragma unroll
-  for (int pass = 0; pass < 2; ++pass) {
-    float* h = pass == 0 ? h1 : h2;
-    if constexpr (NMAX <= 64) {
-      for (int i = tid; i < nq; i += NT) {
-        const float* qi = Q + i * ldq;
-        float d0 = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;
-        int e = 0;
-        for (; e + 3 < n; e += 4) {
-          d0 = fmaf(qi[e], w[e], d0);
-          d1 = fmaf(qi[e + 1], w[e + 1], d1);
-          d2 = fmaf(qi[e + 2], w[e + 2], d2);
-          d3 = fmaf(qi[e + 3], w[e + 3], d3);
-        }
-        for (; e < n; ++e) d0 = fmaf(qi[e], w[e], d0);
-        h[i] = (d0 + d1) + (d2 + d3);
-      }
-    } else {
-      for (int i = warp; i < nq; i += NW) {
-        float d = 0.f;
-        for (int e = lane; e < n; e += 32) d = fmaf(Q[i * ldq + e], w[e], d);
-        d = warp_sum(d);
-        if (lane == 0) h[i] = d;
-      }
-    }
-    __syncthreads();
-    for (int e = tid; e < n; e += NT) {
-      float v = w[e];
-      for (int i = 0; i < nq; ++i) v = fmaf(-h[i], Q[i * ldq + e], v);
-      w[e] = v;
-      if (pass == 1) part = fmaf(v, v, part);
-    }
-    __syncthreads();
-  }
-  return block_sum<NT>(part, red);
-}
-
-// Inverse iteration on T (s.d, s.e, size J) for the k shifts s.shf[0..k),
-// one thread per target, LU factors in shared memory; eigenvectors into ty
-// (row i, column q, stride K), orthonormalised inside clusters.
-template <int NT, int K>
-__device__ void lz_tri_vectors(int J, int k, float tnorm, EigScratch& s, LzScratch& z) {
-  const int tid = threadIdx.x;
-  const float tiny = FLT_EPSILON * tnorm;
-  constexpr int ST = K;
-  float* dd = z.lu;
-  float* du = dd + z.jcap * ST;
-  float* du2 = du + z.jcap * ST;
-  float* dl = du2 + z.jcap * ST;
-  for (int pass = 0; pass < 2; ++pass) {
-    if (tid < k) {
-      const int q = tid;
-      if (pass == 0) {
-        const float shift = s.shf[q];
-        for (int i = 0; i < J; ++i) dd[i * ST + q] = s.d[i] - shift;
-        for (int i = 0; i < J - 1; ++i) {
-          du[i * ST + q] = s.e[i];
-          dl[i * ST + q] = s.e[i];
-          du2[i * ST + q] = 0.f;
-        }
-        unsigned bits[2] = {0u, 0u};
-        for (int i = 0; i < J - 1; ++i) {
-          const float di = dd[i * ST + q], li = dl[i * ST + q];
-          if (fabsf(di) >= fabsf(li)) {
-            const float dv = (di == 0.f) ? tiny : di;
-            dd[i * ST + q] = dv;
-            const float f = li / dv;
-            dl[i * ST + q] = f;
-            dd[(i + 1) * ST + q] -= f * du[i * ST + q];
-          } else {
-            const float f = di / li;
-            dd[i * ST + q] = li;
-            dl[i * ST + q] = f;
-            const float t = du[i * ST + q];
-            du[i * ST + q] = dd[(i + 1) * ST + q];
-            dd[(i + 1) * ST + q] = t - f * dd[(i + 1) * ST + q];
-            if (i < J - 2) {
-              du2[i * ST + q] = du[(i + 1) * ST + q];
-              du[(i + 1) * ST + q] = -f * du[(i + 1) * ST + q];
-            }
-            bits[i >> 5] |= 1u << (i & 31);
-          }
-        }
-        for (int i = 0; i < J; ++i) {
-          const float v = dd[i * ST + q];
-          if (fabsf(v) < tiny) dd[i * ST + q] = v < 0.f ? -tiny : tiny;
-        }
-        z.piv[2 * q] = bits[0];
-        z.piv[2 * q + 1] = bits[1];
-        for (int i = 0; i < J; ++i) z.ty[i * ST + q] = tiny * lz_hash(977u + q, i);
-      } else {
-        for (int i = 0; i < J; ++i) z.ty[i * ST + q] *= tiny;
-      }
-      // solve (T - shift I) y = y
-      const unsigned b0 = z.piv[2 * q], b1 = z.piv[2 * q + 1];
-      float* y = z.ty + q;
-      for (int i = 0; i < J - 1; ++i) {
-        const float a = y[i * ST], b = y[(i + 1) * ST];
-        const bool pv = (i < 32) ? ((b0 >> i) & 1u) : ((b1 >> (i - 32)) & 1u);
-        if (pv) {
-          y[i * ST] = b;
-          y[(i + 1) * ST] = a - dl[i * ST + q] * b;
-        } else {
-          y[(i + 1) * ST] = b - dl[i * ST + q] * a;
-        }
-      }
-      y[(J - 1) * ST] /= dd[(J - 1) * ST + q];
-      if (J > 1)
-        y[(J - 2) * ST] = (y[(J - 2) * ST] - du[(J - 2) * ST + q] * y[(J - 1) * ST]) / dd[(J - 2) * ST + q];
-      for (int i = J - 3; i >= 0; --i)
-        y[i * ST] = (y[i * ST] - du[i * ST + q] * y[(i + 1) * ST] - du2[i * ST + q] * y[(i + 2) * ST]) /
-                    dd[i * ST + q];
-      normalize_column(y, ST, J);
-    }
-    __syncthreads();
-    cluster_mgs<NT>(z.ty, ST, J, k, s.clus, s.red);
-    __syncthreads();
-  }
-}
-
-// Ritz values of T_J above thr (descending) into s.lam and their vectors
-// into z.ty.  Returns the count (a count above K means "too many").
-template <int NT, int K>
-__device__ int lz_ritz(int J, float thr, EigScratch& s, LzScratch& z, float* tnorm_out) {
-  const int tid = threadIdx.x;
-  for (int i = tid; i < J; i += NT) {
-    s.d[i] = z.alpha[i];
-    s.e[i] = (i < J - 1) ? z.beta[i] : 0.f;
+  float *d = s.d, *e2 = s.e2, *lam = s.lam, *shf = s.shf;
+  int* clus = s.clus;
+  __syncthreads();
+  // norm and bounds, in every warp (J <= 32)
+  const float ai = lane < J ? z.alpha[lane] : 0.f;
+  const float bi = lane < J - 1 ? z.beta[lane] : 0.f;
+  const float bm = __shfl_up_sync(0xffffffffu, bi, 1);
+  const float rad = fabsf(bi) + (lane > 0 ? fabsf(bm) : 0.f);
+  const float gup = warp_max(lane < J ? ai + rad : -FLT_MAX);
+  const float tn = warp_max(lane < J ? fabsf(ai) + rad : -FLT_MAX);
+  const float pivmin = FLT_MIN * fmaxf(1.f, warp_max(bi * bi));
+  if (warp == 0 && lane < J) {
+    d[lane] = ai;
+    e2[lane] = bi * bi;
   }
   __syncthreads();
-  float tn = 0.f;
-  const int k = top_eigenvalues<NT>(J, thr, s, &tn);
-  *tnorm_out = tn;
-  if (k == 0 || k > K) return k;
-  lz_tri_vectors<NT, K>(J, k, tn, s, z);
+  const int k = J - sturm_below(d, e2, J, thr, pivmin);
+  if (k <= 0 || k > K) return k < 0 ? 0 : k;
+  for (int q = warp; q < k; q += NW) {
+    const int target = J - 1 - q;  // ascending index of the eigenvalue sought
+    float lo = thr, hi = gup + 4.f * FLT_EPSILON * fmaxf(fabsf(gup), tn) + pivmin;
+    const float tol = 2.f * FLT_EPSILON * tn;
+    for (int round = 0; round < 64; ++round) {
+      if (!(hi - lo > fmaxf(tol, 2.f * FLT_EPSILON * fmaxf(fabsf(lo), fabsf(hi))))) break;
+      const float x = lo + (hi - lo) * ((float)(lane + 1) / 33.f);
+      const unsigned above =
+          __ballot_sync(0xffffffffu, sturm_below(d, e2, J, x, pivmin) > target);
+      // counts grow with x: the first point above the target brackets it
+      float nlo = lo, nhi = hi;
+      if (above == 0u) {
+        nlo = __shfl_sync(0xffffffffu, x, 31);
+      } else {
+        const int f = __ffs(above) - 1;
+        nhi = __shfl_sync(0xffffffffu, x, f);
+        if (f > 0) nlo = __shfl_sync(0xffffffffu, x, f - 1);
+      }
+      lo = fminf(nlo, nhi);
+      hi = nhi;
+    }
+    if (lane == 0) lam[q] = 0.5f * (lo + hi);
+  }
+  __syncthreads();
+  // inverse-iteration shifts kept apart, clusters of close eigenvalues
+  if (tid == 0) {
+    shf[0] = lam[0];
+    clus[0] = 0;
+    for (int j = 1; j < k; ++j) {
+      shf[j] = fminf(lam[j], shf[j - 1] - 10.f * FLT_EPSILON * tn);
+      clus[j] = (lam[j - 1] - lam[j] <= 1e-3f * tn) ? clus[j - 1] : j;
+    }
+  }
+  __syncthreads();
+  bool grouped = false;
+  for (int j = 1; j < k; ++j) grouped = grouped || clus[j] != j;
+  const float tiny = FLT_EPSILON * tn;
+  constexpr int PQ = (K + NW - 1) / NW;  // pairs per warp, at most
+  unsigned pbits[PQ] = {};
+  for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll
+    for (int w = 0; w < PQ; ++w) {
+    const int q = warp + w * NW;
+    float* dd = z.lu + q;
+    float* du = dd + z.jcap * K;
+    float* du2 = du + z.jcap * K;
+    float* dl = du2 + z.jcap * K;
+    float* y = z.ty + q;
+    unsigned bits = pbits[w];
+    // deterministic pseudo-random start vector of size ~eps |T|
+    if (pass == 0 && q < k && lane < J) y[lane * K] = tiny * lz_hash(977u + q, lane);
+    if (pass == 1 && q < k && lane < J) y[lane * K] *= tiny;
+    __syncwarp();
+    if (q < k && lane == 0) {
+      if (pass == 0) {
+        // pivoted LU of T - shift I, tiny pivots replaced by +-tiny
+        const float shift = shf[q];
+        float di = d[0] - shift, ui = J > 1 ? z.beta[0] : 0.f;
+        for (int i = 0; i < J - 1; ++i) {
+          const float li = z.beta[i], dn = d[i + 1] - shift, un = i < J - 2 ? z.beta[i + 1] : 0.f;
+          float f, p;
+          if (fabsf(di) >= fabsf(li)) {
+            p = (di == 0.f) ? tiny : di;
+            f = __fdividef(li, p);
+            du[i * K] = ui;
+            du2[i * K] = 0.f;
+            di = dn - f * ui;
+            ui = un;
+          } else {
+            f = __fdividef(di, li);
+            p = li;
+            du[i * K] = dn;
+            du2[i * K] = un;
+            di = ui - f * dn;
+            ui = -f * un;
+            bits |= 1u << i;
+          }
+          dl[i * K] = f;
+          // (the reciprocal pivot: the solves multiply)
+          dd[i * K] = __fdividef(1.f, fabsf(p) < tiny ? (p < 0.f ? -tiny : tiny) : p);
+        }
+        dd[(J - 1) * K] = __fdividef(1.f, fabsf(di) < tiny ? (di < 0.f ? -tiny : tiny) : di);
+      }
+      float a = y[0];
+      for (int i = 0; i < J - 1; ++i) {
+        const float b = y[(i + 1) * K], f = dl[i * K];
+        if ((bits >> i) & 1u) {
+          y[i * K] = b;
+          a = a - f * b;
+        } else {
+          y[i * K] = a;
+          a = b - f * a;
+        }
+      }
+      float y1 = a * dd[(J - 1) * K], y2 = 0.f;
+      y[(J - 1) * K] = y1;
+      for (int i = J - 2; i >= 0; --i) {
+        const float u2 = i < J - 2 ? du2[i * K] : 0.f;
+        const float v = (y[i * K] - du[i * K] * y1 - u2 * y2) * dd[i * K];
+        y[i * K] = v;
+        y2 = y1;
+        y1 = v;
+      }
+    }
+    pbits[w] = bits;
+    __syncwarp();
+    if (q < k) {
+      // unit length (a lane per entry)
+      const float v = lane < J ? y[lane * K] : 0.f;
+      const float ss = warp_sum(v * v);
+      if (lane < J) y[lane * K] = v * (ss > 0.f ? rsqrtf(ss) : 0.f);
+    }
+    }
+    __syncthreads();
+    if (grouped) {
+      cluster_mgs<NT>(z.ty, K, J, k, clus, s.red);
+      __syncthreads();
+    }
+  }
   return k;
 }
 
-// Gershgorin bound max_i sum_j |A_ij| of a symmetric matrix in lower storage:
-// the row sums are |A| times a vector of ones.
-template <int NT, int NMAX, class S>
-__device__ float gershgorin_lower(S A, int n, float* ones, float* sums, float* red) {
-  for (int e = threadIdx.x; e < n; e += NT) ones[e] = 1.f;
-  __syncthreads();
-  symv_rows<NT, NMAX, true>(A, n, ones, sums);
-  float m = 0.f;
-  for (int e = threadIdx.x; e < n; e += NT) m = fmaxf(m, sums[e]);
-  return block_max<NT>(m, red);
+// the sum over a warp's lanes of eight values (one per row of the warp): row
+// 4 bit4 + 2 bit3 + bit2 of the lane, in all four lanes that agree on them
+__device__ __forceinline__ float sum8(float p[8], int lane) {
+#pragma unroll
+  for (int o = 16, h = 4; o >= 4; o >>= 1, h >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const float keep = up ? p[i + h] : p[i], give = up ? p[i] : p[i + h];
+      p[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  p[0] += __shfl_xor_sync(0xffffffffu, p[0], 2);
+  p[0] += __shfl_xor_sync(0xffffffffu, p[0], 1);
+  return p[0];
 }
 
-// The whole Lanczos + certificate path.
-//  Gs  G in lower storage, read only (the Lanczos operator).
-//  Q   shared scratch of jmax * lz_ldq<NMAX>(n) floats (column j at
-//      Q + j * lz_ldq<NMAX>(n)), jmax <= n.
-//  U   receives the kept Ritz vectors (lz_maxk(NMAX) * n floats, column-major,
-//      any memory).
-//  warm / kwarm: previous Ritz vectors (column-major n x kwarm) or kwarm = 0.
+// The Gram matrix of a narrow block (order n <= NMAX) in the registers of a
+// CTA of NMAX / 16 warps: warp w holds rows 16 w .., lane l the columns l,
+// l + 32.  A product is 16 NMAX / 32 multiply-adds per thread and a
+// 16-shuffle multi-reduction; from shared memory with a thread or two per row
+// it took ten times as long (2.8k -> 0.25k cycles at n = 64).
+template <int NT, int NMAX>
+struct SmallGram {
+  static constexpr int RW = 16, NC = NMAX >= 32 ? NMAX / 32 : 1, NW = NT / 32;
+  static_assert(NW * RW == NMAX, "16 rows per warp");
+  float A[RW][NC];
+  int n, lane, warp;
+  template <class S>
+  __device__ __forceinline__ void load(S G, int n_) {
+    n = n_;
+    lane = threadIdx.x & 31;
+    warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < RW; ++i)
+#pragma unroll
+      for (int k = 0; k < NC; ++k) {
+        const int r = RW * warp + i, c = lane + 32 * k;
+        const int hi = max(r, c), lo = min(r, c);
+        A[i][k] = hi < n ? G.at(hi, lo) : 0.f;
+      }
+  }
+  // the sums over the lanes of the warp's 16 row values: row 8 bit4 + 4 bit3
+  // + 2 bit2 + bit1 of the lane
+  __device__ __forceinline__ float sum16(float p[RW]) const {
+#pragma unroll
+    for (int o = 16, h = 8; o >= 2; o >>= 1, h >>= 1) {
+      const bool up = lane & o;
+#pragma unroll
+      for (int i = 0; i < h; ++i) {
+        const float keep = up ? p[i + h] : p[i], give = up ? p[i] : p[i + h];
+        p[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      }
+    }
+    return p[0] + __shfl_xor_sync(0xffffffffu, p[0], 1);
+  }
+  __device__ __forceinline__ int sum_row() const {
+    return RW * warp + ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 +
+           ((lane >> 1) & 1);
+  }
+  // y (n shared entries) = A x, x in registers (entry lane + 32 k, zero from n
+  // on); the caller's barrier publishes y
+  __device__ __forceinline__ void mul(const float x[NC], float* y) const {
+    float p[RW];
+#pragma unroll
+    for (int i = 0; i < RW; ++i) p[i] = 0.f;
+#pragma unroll
+    for (int k = 0; k < NC; ++k)
+#pragma unroll
+      for (int i = 0; i < RW; ++i) p[i] = fmaf(A[i][k], x[k], p[i]);
+    const float t = sum16(p);
+    const int r = sum_row();
+    if ((lane & 1) == 0 && r < n) y[r] = t;
+  }
+  // entries of a shared n-vector for mul
+  __device__ __forceinline__ void vec(const float* x, float v[NC]) const {
+#pragma unroll
+    for (int k = 0; k < NC; ++k) v[k] = lane + 32 * k < n ? x[lane + 32 * k] : 0.f;
+  }
+  // Gershgorin bound max_i sum_j |A_ij| of the warp's rows (every lane)
+  __device__ __forceinline__ float row_bound() const {
+    float p[RW];
+#pragma unroll
+    for (int i = 0; i < RW; ++i) {
+      p[i] = 0.f;
+#pragma unroll
+      for (int k = 0; k < NC; ++k) p[i] += fabsf(A[i][k]);
+    }
+    return warp_max(sum16(p));
+  }
+  // dot product of two n-vectors, the same in every warp
+  __device__ __forceinline__ float dot(const float* x, const float* y) const {
+    float t = 0.f;
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      const int c = lane + 32 * k;
+      if (c < n) t = fmaf(x[c], y[c], t);
+    }
+    return warp_sum(t);
+  }
+};
+
+// w <- (I - Q Q^T) w twice over nq basis vectors (vector i at Q + i ldq), all
+// in the calling warp: w in registers, eight basis vectors at a time with one
+// multi-reduction.  Every warp of the CTA does the same, so no barrier is
+// needed.  Adds the coefficients of vector nq - 1 to *alpha; returns |w|^2.
+template <int NT, int NMAX>
+__device__ __forceinline__ float lz_project(const SmallGram<NT, NMAX>& g,
+                                            float w[SmallGram<NT, NMAX>::NC], const float* Q,
+                                            int ldq, int nq, float* alpha) {
+  constexpr int NC = SmallGram<NT, NMAX>::NC;
+#pragma unroll 1
+  for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll 1
+    for (int i0 = 0; i0 < nq; i0 += 8) {
+      float q[8][NC], p[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        p[u] = 0.f;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+          q[u][k] = (i0 + u < nq && g.lane + 32 * k < g.n) ? Q[(i0 + u) * ldq + g.lane + 32 * k] : 0.f;
+          p[u] = fmaf(q[u][k], w[k], p[u]);
+        }
+      }
+      const float t = sum8(p, g.lane);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const float h = __shfl_sync(0xffffffffu, t, u << 2);
+        if (i0 + u == nq - 1) *alpha += h;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) w[k] = fmaf(-h, q[u][k], w[k]);
+      }
+    }
+  }
+  float t = 0.f;
+#pragma unroll
+  for (int k = 0; k < NC; ++k) t = fmaf(w[k], w[k], t);
+  return warp_sum(t);
+}
+
+// Steps 1-3 of the Lanczos path of a narrow block and the set-up of step 4.
+//  g   G in registers.
+//  Q   shared scratch of jmax vectors, ldq apart (every warp writes the same
+//      values and each lane reads only its own entries of it).
+//  U   receives the kept Ritz vectors (lz_maxk(NMAX) * n shared floats,
+//      column-major).
 //  gbound: an upper bound of ||G||_2.
-//  panel: lz_cert_floats(NMAX, NT) floats of 16-byte aligned shared
-//      scratch for the certificate (may alias Q and the symv scratch).
-// Steps 1-3 and the set-up of step 4.  On success returns k >= 0 (pairs
-// above thr) with s.lam[0..k), the vectors in U's columns 0..k-1 (U holds
-// ku >= k kept pairs, *ku_out = ku), U and What = W - U sym(B) / 2 staged at
-// panel and panel + K n8 (n8 = roundup(n, 8), K = lz_maxk(NMAX)) and the certificate shift
-// in *c0_out (and, if J_out is given, the Lanczos steps run in *J_out):
+//  panel: lz_cert_floats(NMAX, NT) floats of 16-byte aligned shared scratch
+//      for the certificate (apart from Q and U).
+// On success returns k >= 0 (pairs above thr) with s.lam[0..k), the vectors
+// in U's columns 0..k-1 (U holds ku >= k kept pairs, *ku_out = ku), U and
+// What = W - U sym(B) / 2 staged column-major at panel and panel + K n8 (n8 =
+// roundup(n, 8), K = lz_maxk(NMAX)) and the certificate shift in *c0_out:
 // the pairs are certified iff
 //   regchol_pd<NT, NMAX>(G, n, *c0_out, true, panel, panel + K n8, ku,
 //                        panel + 2 K n8, red)
-// holds (one call site per kernel keeps the code size and the register
-// allocation of that routine in one place).  Returns -1 when the caller
-// must fall back.  G is never modified.
-template <int NT, int NMAX, class SG>
-__device__ int lanczos_candidates(SG Gs, int n, float thr, float gbound, float* Q, int jmax,
-                                  float* U, const float* warm, int kwarm,
-                                  uint32_t seed, EigScratch& s, LzScratch& z, float* panel,
-                                  int* ku_out, float* c0_out, int slot = -1,
-                                  int* J_out = nullptr) {
+// holds.  Returns -1 when the caller must fall back.  *J_out: steps run.
+template <int NT, int NMAX>
+__device__ int lanczos_candidates(const SmallGram<NT, NMAX>& g, float thr, float gbound, float* Q,
+                                  int ldq, int jmax, float* U, uint32_t seed, EigScratch& s,
+                                  LzScratch& z, float* panel, int* ku_out, float* c0_out, int slot,
+                                  int* J_out) {
   constexpr int NW = NT / 32, K = lz_maxk(NMAX);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = g.lane, warp = g.warp, n = g.n;
   PHASE_INIT();
   const float thr_keep = 0.95f * thr;  // pairs kept in U (deflated)
-
-  // start vector
-  float part = 0.f;
-  for (int e = tid; e < n; e += NT) {
-    float v = 0.f;
-    for (int i = 0; i < kwarm; ++i) v += warm[(size_t)i * n + e] * (1.f + 0.25f * i);
-    v += 1e-3f * lz_hash(seed, e);
-    z.x[e] = v;
-    part = fmaf(v, v, part);
+  // the vectors of a step live in every warp's registers (entry lane + 32 k);
+  // only G q passes through shared memory, two buffers in turn
+  constexpr int NC = SmallGram<NT, NMAX>::NC;
+  float q[NC], w[NC];
+  auto store_q = [&](int j) {
+#pragma unroll
+    for (int k = 0; k < NC; ++k)
+      if (lane + 32 * k < n) Q[j * ldq + lane + 32 * k] = q[k];
+  };
+  {
+    float t = 0.f;
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      q[k] = lane + 32 * k < n ? 1e-3f * lz_hash(seed, lane + 32 * k) : 0.f;
+      t = fmaf(q[k], q[k], t);
+    }
+    const float inrm = 1.f / sqrtf(warp_sum(t));
+#pragma unroll
+    for (int k = 0; k < NC; ++k) q[k] *= inrm;
+    store_q(0);
   }
-  const float inrm = 1.f / sqrtf(block_sum<NT>(part, s.red));
-  const int ldq = lz_ldq<NMAX>(n);
-  for (int e = tid; e < n; e += NT) Q[e] = z.x[e] * inrm;
-  __syncthreads();
-  const int jmin = min(jmax, kwarm > 0 ? kwarm + 3 : 8);
+  const int jmin = min(jmax, 8);
   int J = 0, k = -1;
-  float tn = 0.f;
   uint32_t restart = 1;
   PHASE(slot, 6);
   for (int j = 0; j < jmax; ++j) {
     // w = G q_j, then w <- w - Q_j Q_j^T w twice: alpha_j is the q_j
     // coefficient of the two passes, beta_j = ||w|| (full reorthogonalisation)
-    symv_rows<NT, NMAX>(Gs, n, Q + (size_t)j * ldq, z.w);
+    float* y = (j & 1) ? z.w : z.x;
+    g.mul(q, y);
+    __syncthreads();
+    g.vec(y, w);
     PHASE(slot, 7);
-    float b = sqrtf(lz_project<NT, NMAX>(z.w, Q, ldq, n, j + 1, z.h, z.h + kLzMaxJ, s.red));
-    const float a = z.h[j] + z.h[kLzMaxJ + j];
+    float al = 0.f;
+    float b = sqrtf(lz_project(g, w, Q, ldq, j + 1, &al));
     PHASE(slot, 9);
     if (tid == 0) {
-      z.alpha[j] = a;
+      z.alpha[j] = al;
       z.beta[j] = b;
     }
     J = j + 1;
@@ -476,170 +470,111 @@ __device__ int lanczos_candidates(SG Gs, int n, float thr, float gbound, float* 
       if (!(b > 1e-5f * gbound)) {
         // breakdown: an invariant subspace was found; continue from a random
         // direction orthogonal to it
-        for (int e = tid; e < n; e += NT) z.w[e] = lz_hash(seed + 7919u * restart, e);
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+          w[c] = lane + 32 * c < n ? lz_hash(seed + 7919u * restart, lane + 32 * c) : 0.f;
         ++restart;
-        __syncthreads();
-        const float bn = sqrtf(lz_project<NT, NMAX>(z.w, Q, ldq, n, j + 1, z.h, z.h + kLzMaxJ, s.red));
+        const float bn = sqrtf(lz_project(g, w, Q, ldq, j + 1, &al));
         if (!(bn > 0.f)) break;
         if (tid == 0) z.beta[j] = 0.f;
         b = bn;
       }
       const float ib = 1.f / b;
-      for (int e = tid; e < n; e += NT) Q[(size_t)(j + 1) * ldq + e] = z.w[e] * ib;
-      __syncthreads();
+#pragma unroll
+      for (int c = 0; c < NC; ++c) q[c] = w[c] * ib;
+      store_q(j + 1);
     }
     PHASE(slot, 10);
     if (J >= jmin && ((J - jmin) % 4 == 0 || J == jmax)) {
       // converged when every kept Ritz pair has |beta_J * y_{J-1}| small
-      k = lz_ritz<NT, K>(J, thr_keep, s, z, &tn);
+      k = lz_ritz<NT, K>(J, thr_keep, z, s);
       PHASE(slot, 11);
       if (k > K) {
-      if (J_out) *J_out = J;
-      return -1;
-    }
+        *J_out = J;
+        return -1;
+      }
       bool conv = true;
       const float bJ = z.beta[J - 1];
-      // (many pairs: each adds its share of the error)
-      const float tol = k > 8 ? 3e-6f : 1e-5f;
       for (int q = 0; q < k; ++q)
-        if (fabsf(bJ * z.ty[(J - 1) * K + q]) > tol * fmaxf(s.lam[0], thr)) conv = false;
+        if (fabsf(bJ * z.ty[(J - 1) * K + q]) > 1e-5f * fmaxf(s.lam[0], thr)) conv = false;
       if (conv) break;
       k = -1;
     }
   }
+  *J_out = J;
   if (k < 0) {
-    k = lz_ritz<NT, K>(J, thr_keep, s, z, &tn);
-    if (k > K) {
-      if (J_out) *J_out = J;
-      return -1;
-    }
+    k = lz_ritz<NT, K>(J, thr_keep, z, s);
+    if (k > K) return -1;
   }
-  const int ku = k;
-  // U = Q_J Y (n x ku) into the caller's U and, as K / 8 row-major n x 8
-  // arrays with zero columns beyond ku, into X8 (shared; Q may alias the
-  // panel, so the values wait in registers for the barrier)
-  constexpr int H = K / 8, PER = (8 * NMAX + NT - 1) / NT;
-  static_assert(8 * NMAX <= 4 * NT, "staging split");
-  float* X8 = panel;
-  float* Y8 = panel + K * NMAX;
-  const int n8 = (n + 7) & ~7;
-  float uv[H][PER];
-#pragma unroll
-  for (int h = 0; h < H; ++h)
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-      const int e = tid + i * NT, r = e >> 3, q = 8 * h + (e & 7);
-      float v = 0.f;
-      if (r < n && q < ku)
-        for (int jj = 0; jj < J; ++jj) v = fmaf(Q[jj * ldq + r], z.ty[jj * K + q], v);
-      uv[h][i] = v;
-    }
-  __syncthreads();
-#pragma unroll
-  for (int h = 0; h < H; ++h)
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-      const int e = tid + i * NT, r = e >> 3, q = 8 * h + (e & 7);
-      if (r < n) {
-        X8[h * 8 * NMAX + e] = uv[h][i];
-        if (q < ku) U[(size_t)q * n + r] = uv[h][i];
-      }
-    }
-  __syncthreads();
-  PHASE(slot, 12);
-  // W = G U (eight columns per pass over G), B = U^T W, rho
-  const int nh = (ku + 7) >> 3;
-  for (int h = 0; h < nh; ++h) symm_rows8<NT, NMAX>(Gs, n, X8 + h * 8 * NMAX, Y8 + h * 8 * NMAX);
-  for (int pr = warp; pr < ku * nh; pr += NW) {
-    const int p = pr % ku, h = pr / ku;
-    const float* Xp = X8 + (p >> 3) * 8 * NMAX + (p & 7);
-    const float* Yh = Y8 + h * 8 * NMAX;
-    float d[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) d[q] = 0.f;
-    for (int r = lane; r < n; r += 32) {
-      const float x = Xp[r * 8];
-      const float4 y0 = *reinterpret_cast<const float4*>(Yh + r * 8);
-      const float4 y1 = *reinterpret_cast<const float4*>(Yh + r * 8 + 4);
-      d[0] = fmaf(x, y0.x, d[0]);
-      d[1] = fmaf(x, y0.y, d[1]);
-      d[2] = fmaf(x, y0.z, d[2]);
-      d[3] = fmaf(x, y0.w, d[3]);
-      d[4] = fmaf(x, y1.x, d[4]);
-      d[5] = fmaf(x, y1.y, d[5]);
-      d[6] = fmaf(x, y1.z, d[6]);
-      d[7] = fmaf(x, y1.w, d[7]);
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const float t = warp_sum(d[q]);
-      if (lane == 0 && 8 * h + q < ku) z.Bm[p * K + 8 * h + q] = t;
-    }
-  }
-  __syncthreads();
-  part = 0.f;
-  for (int h = 0; h < nh; ++h)
-    for (int e = tid; e < 8 * n; e += NT) {
-      const int q = 8 * h + (e & 7);
-      if (q < ku) {
-        const float rr = Y8[h * 8 * NMAX + e] - z.Bm[q * K + q] * X8[h * 8 * NMAX + e];
-        part = fmaf(rr, rr, part);
-      }
-    }
-  const float rho = sqrtf(block_sum<NT>(part, s.red));
-  PHASE(slot, 13);
-  // kept pairs: Rayleigh quotients, count above thr; pairs above thr first
-  int kk = 0;
-  for (int q = 0; q < ku; ++q) {
-    const float th = z.Bm[q * K + q];
-    kk += th > thr;
-    if (q > 0 && th > thr && !(z.Bm[(q - 1) * K + (q - 1)] > thr)) {
-      if (J_out) *J_out = J;
-      return -1;
-    }
-  }
-  const float c0 = thr - 2.f * rho - 8.f * (float)(ku + 1) * FLT_EPSILON * gbound;
-  if (!(c0 > 0.f)) {
-    if (J_out) *J_out = J;
-    return -1;
-  }
-  // P G P = G - U What^T - What U^T with What = W - U sym(B) / 2, staged in
-  // shared memory for the register Cholesky of (c I - P G P): column-major
-  // over X8 and Y8, so the values wait in registers
-  float wv[H][PER];
-#pragma unroll
-  for (int h = 0; h < H; ++h)
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-      const int e = tid + i * NT, r = e >> 3, q = 8 * h + (e & 7);
-      float w = 0.f;
-      if (r < n && q < ku) {
-        w = Y8[h * 8 * NMAX + e];
-        for (int p = 0; p < ku; ++p)
-          w = fmaf(-0.25f * (z.Bm[p * K + q] + z.Bm[q * K + p]),
-                   X8[(p >> 3) * 8 * NMAX + r * 8 + (p & 7)], w);
-      }
-      wv[h][i] = w;
-    }
-  __syncthreads();
-  if (tid < ku) s.lam[tid] = z.Bm[tid * K + tid];
+  const int ku = k, n8 = (n + 7) & ~7;
   float* U8 = panel;
   float* W8 = panel + K * n8;
-#pragma unroll
-  for (int h = 0; h < H; ++h)
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-      const int e = tid + i * NT, r = e >> 3, q = 8 * h + (e & 7);
-      if (r < n8 && q < ku) {
-        U8[q * n8 + r] = r < n ? uv[h][i] : 0.f;
-        W8[q * n8 + r] = wv[h][i];
-      }
+  // U = Q_J Y; W = G U
+  for (int e = tid; e < ku * n8; e += NT) {
+    const int q = e / n8, r = e - q * n8;
+    float v = 0.f;
+    if (r < n) {
+      for (int j = 0; j < J; ++j) v = fmaf(Q[j * ldq + r], z.ty[j * K + q], v);
+      U[q * n + r] = v;
     }
+    U8[e] = v;
+    W8[e] = 0.f;
+  }
+  __syncthreads();
+  PHASE(slot, 12);
+  for (int p = 0; p < ku; ++p) {
+    g.vec(U8 + p * n8, q);
+    g.mul(q, W8 + p * n8);
+  }
+  __syncthreads();
+  // B = U^T W, residuals |W_q - B_qq U_q|^2: a warp per row of B
+  for (int p = warp; p < ku; p += NW) {
+    float bpp = 0.f;
+    for (int q = 0; q < ku; ++q) {
+      const float t = g.dot(U8 + p * n8, W8 + q * n8);
+      if (q == p) bpp = t;
+      if (lane == 0) z.Bm[p * K + q] = t;
+    }
+    float rr = 0.f;
+    for (int r = lane; r < n; r += 32) {
+      const float d = W8[p * n8 + r] - bpp * U8[p * n8 + r];
+      rr = fmaf(d, d, rr);
+    }
+    rr = warp_sum(rr);
+    if (lane == 0) z.h[p] = rr;
+  }
+  __syncthreads();
+  PHASE(slot, 13);
+  // kept pairs: Rayleigh quotients, count above thr; pairs above thr first
+  float rho = 0.f;
+  int kk = 0;
+  for (int q = 0; q < ku; ++q) {
+    rho += z.h[q];
+    const float th = z.Bm[q * K + q];
+    kk += th > thr;
+    if (q > 0 && th > thr && !(z.Bm[(q - 1) * K + (q - 1)] > thr)) return -1;
+  }
+  rho = sqrtf(rho);
+  const float c0 = thr - 2.f * rho - 8.f * (float)(ku + 1) * FLT_EPSILON * gbound;
+  if (!(c0 > 0.f)) return -1;
+  if (tid < ku) s.lam[tid] = z.Bm[tid * K + tid];
+  // What = W - U sym(B) / 2 in place: a thread owns a row
+  for (int r = tid; r < n; r += NT) {
+    float u[K];
+#pragma unroll
+    for (int p = 0; p < K; ++p) u[p] = p < ku ? U8[p * n8 + r] : 0.f;
+    for (int q = 0; q < ku; ++q) {
+      float w = W8[q * n8 + r];
+#pragma unroll
+      for (int p = 0; p < K; ++p)
+        if (p < ku) w = fmaf(-0.25f * (z.Bm[p * K + q] + z.Bm[q * K + p]), u[p], w);
+      W8[q * n8 + r] = w;
+    }
+  }
   __syncthreads();
   PHASE(slot, 11);
   *ku_out = ku;
   *c0_out = c0;
-  if (J_out) *J_out = J;
   return kk;
 }
 

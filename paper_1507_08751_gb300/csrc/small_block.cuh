@@ -106,16 +106,34 @@ __device__ __forceinline__ void small_block_svt(const ScaleLaunch& a, int b, flo
   LzScratch z;
   lz_bind<NT>(z, sm + lay.oZ, NMAX, JCAP);
 
-  // gather A = A1 + A2 on the shifted grid; ||C||_F^2
+  // gather A = A1 + A2 on the shifted grid; ||C||_F^2.  Element e is (e / n, e
+  // mod n): the quotient by a float product (exact below 2^13 elements)
   const int melem = a.m * a.n;
+  const float rcp_n = 1.f / (float)a.n;
+  auto row_of = [&](int e) { return __float2int_rz(((float)e + 0.5f) * rcp_n); };
   float fro = 0.f;
-#pragma unroll 8
-  for (int e = tid; e < melem; e += NT) {
-    const int r = e / a.n, c = e - r * a.n;
-    const size_t off = g.offset(r, c);
-    const float v = a.A1[off] + a2(off, r, c);
-    C[g.cidx(r, c, ldc)] = v;
-    fro = fmaf(v, v, fro);
+  constexpr int GU = 8;  // loads in flight per thread and half of A
+  for (int e0 = tid; e0 < melem; e0 += GU * NT) {
+    float x[GU], y[GU];
+#pragma unroll
+    for (int u = 0; u < GU; ++u) {
+      const int e = e0 + u * NT;
+      const bool in = e < melem;
+      const int r = in ? row_of(e) : 0, c = in ? e - r * a.n : 0;
+      const size_t off = g.offset(r, c);
+      x[u] = in ? a.A1[off] : 0.f;
+      y[u] = in ? a2(off, r, c) : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < GU; ++u) {
+      const int e = e0 + u * NT;
+      if (e < melem) {
+        const int r = row_of(e), c = e - r * a.n;
+        const float v = x[u] + y[u];
+        C[g.cidx(r, c, ldc)] = v;
+        fro = fmaf(v, v, fro);
+      }
+    }
   }
   fro = block_sum<NT>(fro, s.red);
   if constexpr (NT == 32) __syncwarp();
@@ -127,10 +145,53 @@ __device__ __forceinline__ void small_block_svt(const ScaleLaunch& a, int b, flo
   bool skipped = false;
   float gbound = fro;  // trace(G) >= lambda_max(G)
   float fl = 0.f;      // flops of the steps run (see fl_symv in lanczos.cuh)
+  SmallGram<NT, NMAX> gr;  // G in registers
   if (a.skip_bound && fro <= thr) skipped = true;
   if (!skipped) {
     fl += (float)(mm * nn * (nn + 1));  // lower triangle of G
-    if ((nn & 3) == 0) {
+    const int t8 = nn >> 3, tiles8 = t8 * (t8 + 1) / 2;
+    if ((nn & 7) == 0 && NT >= 64 && 2 * tiles8 <= NT) {
+      // 8x8 register tiles of the lower triangle, the rows of C split over
+      // two lanes: per row two 128-bit loads for the tile's rows and two for
+      // its columns, 64 FMAs (4x4 tiles were bound by their shared-memory
+      // reads and took two rounds of threads at 64 wide: 8.5k cycles, here 4k)
+      const int t = tid >> 1, half = tid & 1;
+      const bool on = t < tiles8;
+      const int ta = on ? tri_row(t) : 0, tb = on ? t - (ta * (ta + 1)) / 2 : 0;
+      float acc[8][8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int v = 0; v < 8; ++v) acc[u][v] = 0.f;
+      if (on) {
+        const float* ci = C + 8 * ta;
+        const float* cj = C + 8 * tb;
+#pragma unroll 2
+        for (int r = half; r < mm; r += 2) {
+          const float4 x0 = *reinterpret_cast<const float4*>(ci + r * ldc);
+          const float4 x1 = *reinterpret_cast<const float4*>(ci + r * ldc + 4);
+          const float4 y0 = *reinterpret_cast<const float4*>(cj + r * ldc);
+          const float4 y1 = *reinterpret_cast<const float4*>(cj + r * ldc + 4);
+          const float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+          const float yv[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+#pragma unroll
+            for (int v = 0; v < 8; ++v) acc[u][v] = fmaf(xv[u], yv[v], acc[u][v]);
+        }
+      }
+      // the two halves' sums: each lane finishes four of the tile's rows
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {
+          const float keep = half ? acc[u + 4][v] : acc[u][v];
+          const float give = half ? acc[u][v] : acc[u + 4][v];
+          const float w = keep + __shfl_xor_sync(0xffffffffu, give, 1);
+          const int i = 8 * ta + 4 * half + u, j = 8 * tb + v;
+          if (on && j <= i) G[i * ldg + j] = w;
+        }
+    } else if ((nn & 3) == 0) {
       // 4x4 register tiles of the lower triangle: per row of C one 128-bit
       // load for the tile's rows and one for its columns, 16 FMAs
       const int nt = nn >> 2, ntiles = nt * (nt + 1) / 2;
@@ -175,15 +236,15 @@ __device__ __forceinline__ void small_block_svt(const ScaleLaunch& a, int b, flo
     PHASE(SLOT, 1);
     if (a.skip_bound) {
       // Gershgorin: sigma_max^2 = lambda_max(G) <= max_i sum_j |G_ij|
-      float rs = 0.f;
-      for (int i = tid; i < nn; i += NT) {
-        float t = 0.f;
-        for (int j = 0; j <= i; ++j) t += fabsf(G[i * ldg + j]);
-        for (int j = i + 1; j < nn; ++j) t += fabsf(G[j * ldg + i]);
-        rs = fmaxf(rs, t);
+      float rs;
+      gr.load(LowerFull{G, ldg}, nn);
+      rs = gr.row_bound();
+      if constexpr (NT > 32) {
+        if ((tid & 31) == 0) s.red[tid >> 5] = rs;
+        __syncthreads();
+        for (int w = 0; w < NT / 32; ++w) rs = fmaxf(rs, s.red[w]);
+        __syncthreads();
       }
-      rs = block_max<NT>(rs, s.red);
-      if constexpr (NT == 32) __syncwarp();
       gbound = fminf(gbound, rs);
       fl += (float)fl_symv(nn);
       if (rs <= thr) {
@@ -208,10 +269,9 @@ __device__ __forceinline__ void small_block_svt(const ScaleLaunch& a, int b, flo
       if (!(c_skip > 0.f)) continue;
     } else if constexpr (kAttempts == 2) {
       int J = 0;
-      kk = lanczos_candidates<NT, NMAX>(LowerFull{G, ldg}, nn, thr, gbound, Qs,
-                                        nn < JCAP ? nn : JCAP, Us, nullptr, 0,
-                                        0x51ED27u + 131u * job_block(a, b), s, z, panel, &ku, &c0,
-                                        5 + SLOT, &J);
+      kk = lanczos_candidates(gr, thr, gbound, Qs, lz_ldq<NMAX>(nn), nn < JCAP ? nn : JCAP, Us,
+                              0x51ED27u + 131u * job_block(a, b), s, z, panel, &ku, &c0, 5 + SLOT,
+                              &J);
       fl += (float)fl_lanczos(nn, J, ku);
       PHASE(SLOT, 10);
       if (kk < 0) break;
@@ -244,8 +304,9 @@ __device__ __forceinline__ void small_block_svt(const ScaleLaunch& a, int b, flo
   }
   const bool transposed = g.transposed();
   if (k == 0) {
+#pragma unroll 8
     for (int e = tid; e < melem; e += NT) {
-      const int r = e / a.n, c = e - r * a.n;
+      const int r = row_of(e), c = e - r * a.n;
       const size_t off = g.offset(r, c);
       a.Zout[off] = 0.f;
       if (a.Wout) a.Wout[off] = -C[g.cidx(r, c, ldc)];
@@ -275,21 +336,56 @@ __device__ __forceinline__ void small_block_svt(const ScaleLaunch& a, int b, flo
   __syncthreads();
   // P = C V diag(f)   (mm x k, row stride nn)
   for (int e = tid; e < mm * k; e += NT) {
-    const int i = e / k, q = e - i * k;
-    float acc = 0.f;
-    for (int c = 0; c < nn; ++c) acc = fmaf(C[i * ldc + c], Vb[c * vsc + q * vsq], acc);
-    P[i * nn + q] = acc * s.xs[q];
+    const int q = e / mm, i = e - q * mm;
+    const float* ci = C + i * ldc;
+    const float* vq = Vb + q * vsq;
+    float t0 = 0.f, t1 = 0.f, t2 = 0.f, t3 = 0.f;
+    int c = 0;
+    // (thread i starts at column i, so that the rows' reads meet no bank twice)
+    const int c0 = i % nn;
+    for (; c + 3 < nn; c += 4) {
+      int x0 = c0 + c, x1 = x0 + 1, x2 = x0 + 2, x3 = x0 + 3;
+      if (x0 >= nn) x0 -= nn;
+      if (x1 >= nn) x1 -= nn;
+      if (x2 >= nn) x2 -= nn;
+      if (x3 >= nn) x3 -= nn;
+      t0 = fmaf(ci[x0], vq[x0 * vsc], t0);
+      t1 = fmaf(ci[x1], vq[x1 * vsc], t1);
+      t2 = fmaf(ci[x2], vq[x2 * vsc], t2);
+      t3 = fmaf(ci[x3], vq[x3 * vsc], t3);
+    }
+    for (; c < nn; ++c) {
+      int x0 = c0 + c;
+      if (x0 >= nn) x0 -= nn;
+      t0 = fmaf(ci[x0], vq[x0 * vsc], t0);
+    }
+    P[i * nn + q] = ((t0 + t1) + (t2 + t3)) * s.xs[q];
   }
   __syncthreads();
   // Z' = P V^T, scattered through Shift_{-s}; W' = 2 Z' - A
-  for (int e = tid; e < melem; e += NT) {
-    const int r = e / a.n, c = e - r * a.n;
-    const int i = transposed ? c : r, col = transposed ? r : c;
-    float z = 0.f;
-    for (int q = 0; q < k; ++q) z = fmaf(P[i * nn + q], Vb[col * vsc + q * vsq], z);
-    const size_t off = g.offset(r, c);
-    a.Zout[off] = z;
-    if (a.Wout) a.Wout[off] = 2.f * z - C[i * ldc + col];
+  constexpr int SU = 8;  // elements per thread and round
+  for (int e0 = tid; e0 < melem; e0 += SU * NT) {
+    float zz[SU];
+    int ii[SU], cc[SU];
+#pragma unroll
+    for (int u = 0; u < SU; ++u) {
+      const int e = min(e0 + u * NT, melem - 1);
+      const int r = row_of(e), c = e - r * a.n;
+      ii[u] = transposed ? c : r;
+      cc[u] = transposed ? r : c;
+      zz[u] = 0.f;
+    }
+    for (int q = 0; q < k; ++q)
+#pragma unroll
+      for (int u = 0; u < SU; ++u)
+        zz[u] = fmaf(P[ii[u] * nn + q], Vb[cc[u] * vsc + q * vsq], zz[u]);
+#pragma unroll
+    for (int u = 0; u < SU; ++u)
+      if (e0 + u * NT < melem) {
+        const size_t off = transposed ? g.offset(cc[u], ii[u]) : g.offset(ii[u], cc[u]);
+        a.Zout[off] = zz[u];
+        if (a.Wout) a.Wout[off] = 2.f * zz[u] - C[ii[u] * ldc + cc[u]];
+      }
   }
   PHASE(SLOT, 6);
   if (tid == 0) {
