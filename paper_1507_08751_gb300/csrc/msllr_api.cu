@@ -75,8 +75,9 @@ struct msllr_ctx {
   void* io = nullptr;
   size_t io_bytes = 0;
   // small device scalars
-  int* d_small = nullptr;          // [0] iter, [1..2] cur shift, [3] nonfinite flag, [4..5] tmp shift,
-                                   // [6] device wait timeout flag
+  int* d_small = nullptr;          // [0] iter, [1..2] cur shift, [3] nonfinite flag, [4..5] a zero
+                                   // shift, [6] device wait timeout flag
+  int* h_flag = nullptr;           // pinned copy of the timeout flag
   double* d_acc = nullptr;         // [0..MAX) nuc per scale, [MAX] primal residual^2
   double* d_noise = nullptr;       // [MAX] noise-scale ||A||_F^2 scratch
   unsigned long long* d_cnt = nullptr;  // [2*MAX]
@@ -291,7 +292,9 @@ int msllr_create(msllr_ctx** out, int device, size_t hbm_budget_bytes, void* cud
       cudaMalloc(&ctx->d_acc, (MSLLR_MAX_SCALES + 8) * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&ctx->d_noise, MSLLR_MAX_SCALES * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&ctx->d_cnt, 8 * MSLLR_MAX_SCALES * sizeof(unsigned long long)) != cudaSuccess ||
-      cudaMalloc(&ctx->d_shift, 2 * sizeof(int)) != cudaSuccess)
+      cudaMalloc(&ctx->d_shift, 2 * sizeof(int)) != cudaSuccess ||
+      cudaMemsetAsync(ctx->d_small, 0, 64 * sizeof(int), ctx->stream) != cudaSuccess ||
+      cudaMallocHost(&ctx->h_flag, sizeof(int)) != cudaSuccess)
     return bail(fail(ctx, MSLLR_ENOMEM, "cudaMalloc of context scalars"));
   ctx->shift_cap = 1;
   *out = ctx;
@@ -334,6 +337,7 @@ int msllr_destroy(msllr_ctx* ctx) {
     set_phase_buffer_warp(nullptr);
     cudaFree(ctx->d_phase);
   }
+  if (ctx->h_flag) cudaFreeHost(ctx->h_flag);
   if (ctx->d_small) cudaFree(ctx->d_small);
   if (ctx->d_acc) cudaFree(ctx->d_acc);
   if (ctx->d_noise) cudaFree(ctx->d_noise);
@@ -392,7 +396,12 @@ int msllr_blocksvt(msllr_ctx* ctx, const float* A, float* Z, int M, int N, int l
   const size_t big = big_workspace_bytes(M, N, bm, bn);
   if (int r = ensure_ws(ctx, align_up(big) + 256)) return r;
   const int sh[2] = {((shift_r % M) + M) % M, ((shift_c % N) + N) % N};
-  CK(cudaMemcpyAsync(ctx->d_small + 4, sh, sizeof(sh), cudaMemcpyHostToDevice, ctx->stream));
+  // The shift goes with the launch (added to a device shift that stays zero)
+  // and the timeout flag, through pinned memory, only where a tensor-core
+  // wait can set it: three copies and a memset less for the narrow blocks,
+  // whose whole call they halve.
+  const ScalePath path = choose_path(bm, bn);
+  const bool waits = path == ScalePath::Big || path == ScalePath::Huge;
   ScaleLaunch s{};
   s.A1 = A;
   s.A2 = nullptr;
@@ -404,20 +413,23 @@ int msllr_blocksvt(msllr_ctx* ctx, const float* A, float* Z, int M, int N, int l
   s.m = bm;
   s.n = bn;
   s.shift = ctx->d_small + 4;
+  s.shift_add_r = sh[0];
+  s.shift_add_c = sh[1];
   s.tau = (float)tau;
   s.skip_bound = 1;
   s.rank_out = block_rank_out;
   s.norm_acc = ctx->d_noise;
   s.err = ctx->d_small + 6;
   BigWorkspace w = carve_big_workspace(ctx->ws, M, N, bm, bn);
-  CK(cudaMemsetAsync(ctx->d_small + 6, 0, sizeof(int), ctx->stream));
+  if (waits) CK(cudaMemsetAsync(ctx->d_small + 6, 0, sizeof(int), ctx->stream));
   CK(reset_warm_start(w, M, N, bm, bn, ctx->stream));
   CK(launch_scale(s, w, ctx->stream, nullptr));
-  int timed_out = 0;
-  CK(cudaMemcpyAsync(&timed_out, ctx->d_small + 6, sizeof(int), cudaMemcpyDeviceToHost,
-                     ctx->stream));
+  if (waits)
+    CK(cudaMemcpyAsync(ctx->h_flag, ctx->d_small + 6, sizeof(int), cudaMemcpyDeviceToHost,
+                       ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
-  if (timed_out) return fail(ctx, MSLLR_ECUDA, "a tensor-core wait timed out on the device");
+  if (waits && *ctx->h_flag)
+    return fail(ctx, MSLLR_ECUDA, "a tensor-core wait timed out on the device");
   return MSLLR_OK;
 }
 
