@@ -1,7 +1,7 @@
 // Block SVT of narrow blocks (min(m, n) <= 16, max(m, n) <= 32): one warp
-// per block (warp_block.cuh), one warp per CTA -- eq:bsvt under the Sec. 9
-// shift.
-#include "warp_block.cuh"
+// per block (warp_block.cuh), or several blocks per warp up to 8 x 16
+// (pack_block.cuh), one warp per CTA -- eq:bsvt under the Sec. 9 shift.
+#include "pack_block.cuh"
 
 namespace msllr {
 
@@ -24,6 +24,23 @@ blocksvt_warp_kernel(ScaleLaunch a, int nblocks) {
   warp_block_svt<RPL, ST, NP>(a, b, vsh[wid], A2Global{a.A2});
 }
 
+// W lanes and R rows per lane for a block, 32 / W blocks per warp
+template <int W, int R, bool ST>
+__global__ void __launch_bounds__(kWT, R <= 8 ? 32 : 16)
+blocksvt_pack_kernel(ScaleLaunch a, int nblocks) {
+  __shared__ float vs[32 * W];
+  const int b = blockIdx.x * (32 / W) + (threadIdx.x & 31) / W;
+  const bool on = b < nblocks;
+  pack_block_svt<W, R, ST>(a, on ? b : nblocks - 1, on, vs, A2Global{a.A2});
+}
+
+template <int W, int R>
+void launch_pack(const ScaleLaunch& s, int nblocks, cudaStream_t st) {
+  const int per = 32 / W, grid = (nblocks + per - 1) / per;
+  if (s.fw || s.rows) blocksvt_pack_kernel<W, R, true><<<grid, kWT, 0, st>>>(s, nblocks);
+  else blocksvt_pack_kernel<W, R, false><<<grid, kWT, 0, st>>>(s, nblocks);
+}
+
 }  // namespace
 
 bool warp_path(int m, int n) {
@@ -39,7 +56,16 @@ cudaError_t launch_warp(const ScaleLaunch& s, cudaStream_t st, Prof* prof) {
     if (cudaError_t e = prof->before(st, KK_FUSED)) return e;
   const int nn = s.m < s.n ? s.m : s.n;
   const bool gen = s.fw || s.rows, w16 = nn >= 15;
-  if (mm <= 16) {
+  if (const int w = pack_lanes(s.m, s.n)) {
+    const int r = pack_rows(s.m, s.n);
+    if (w == 4) {
+      if (r == 4) launch_pack<4, 4>(s, nblocks, st);
+      else launch_pack<4, 8>(s, nblocks, st);
+    } else {
+      if (r == 8) launch_pack<8, 8>(s, nblocks, st);
+      else launch_pack<8, 16>(s, nblocks, st);
+    }
+  } else if (mm <= 16) {
     if (w16) {
       if (gen) blocksvt_warp_kernel<8, true, 16><<<grid, kWT, 0, st>>>(s, nblocks);
       else blocksvt_warp_kernel<8, false, 16><<<grid, kWT, 0, st>>>(s, nblocks);

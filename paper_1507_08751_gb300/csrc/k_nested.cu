@@ -10,6 +10,7 @@
 //      the same tile,
 // each with the same arithmetic as its own per-scale kernel, so the outputs
 // equal the separate kernels' bit for bit; R is read once instead of twice.
+#include "pack_block.cuh"
 #include "small_block.cuh"
 
 namespace msllr {
@@ -27,6 +28,19 @@ struct A2Tile {
     return t[(r0 + row) * ld + (c0 + col)];
   }
 };
+
+// the fine blocks by the packed path: 32 / W per warp
+template <int W, int R, class F>
+__device__ __forceinline__ void nested_pack(const ScaleLaunch& fine, int count, float* vs, const F& at) {
+  const int warp = threadIdx.x >> 5, per = 32 / W, grp = (threadIdx.x & 31) / W;
+  for (int u0 = warp * per; u0 < count; u0 += (kNT / 32) * per) {
+    const int u = u0 + grp;
+    const bool on = u < count;
+    A2Tile t;
+    const int bf = at(on ? u : count - 1, t);
+    pack_block_svt<W, R, false>(fine, bf, on, vs, t);
+  }
+}
 
 // NP: the fine blocks' fixed rotation order (16 for blocks 15 or 16 wide)
 template <int NP>
@@ -52,10 +66,24 @@ nested_kernel(ScaleLaunch fine, ScaleLaunch coarse) {
   const int fm = fine.m, fn = fine.n;
   const int pi = m / fm, qi = n / fn, nbn_fine = fine.N / fn;
   const int warp = threadIdx.x >> 5;
-  for (int u = warp; u < pi * qi; u += kNT / 32) {
+  auto at = [&](int u, A2Tile& t) {
     const int du = u / qi, dv = u - du * qi;
-    const int bf = (g.p * pi + du) * nbn_fine + (g.q * qi + dv);
-    warp_block_svt<8, false, NP>(fine, bf, vs[warp], A2Tile{Rt, ldr, du * fm, dv * fn});
+    t = A2Tile{Rt, ldr, du * fm, dv * fn};
+    return (g.p * pi + du) * nbn_fine + (g.q * qi + dv);
+  };
+  const int lanes = NP == 16 ? 0 : pack_lanes(fm, fn), rows = pack_rows(fm, fn);
+  if (lanes == 4) {
+    if (rows == 4) nested_pack<4, 4>(fine, pi * qi, &vs[warp][0][0], at);
+    else nested_pack<4, 8>(fine, pi * qi, &vs[warp][0][0], at);
+  } else if (lanes == 8) {
+    if (rows == 8) nested_pack<8, 8>(fine, pi * qi, &vs[warp][0][0], at);
+    else nested_pack<8, 16>(fine, pi * qi, &vs[warp][0][0], at);
+  } else {
+    for (int u = warp; u < pi * qi; u += kNT / 32) {
+      A2Tile t;
+      const int bf = at(u, t);
+      warp_block_svt<8, false, NP>(fine, bf, vs[warp], t);
+    }
   }
   __syncthreads();
   // the coarse block: its gather reads the tile before its Gram phase
