@@ -222,36 +222,103 @@ __device__ __forceinline__ void cta_add_d(double v, double* acc, double* sred) {
   __syncthreads();
 }
 
+// Sum of squares of differences of FP32 values.  EXACT false: FP64 throughout.
+// EXACT true: the difference a - b as the unevaluated FP32 pair (s, e) of
+// Knuth's two-sum, its square and the running sum as FP32 pairs (two-product
+// by fma; relative error 2^-46), added to the FP64 total every kFold terms.
+// The FP64 pipe is the bound otherwise (seven conversions, differences and
+// products per entry: 5.5 ms at 8192 x 8192 x 6); with some hundred terms per
+// thread the fewer FP64 additions also make the error bound smaller than that
+// of adding every term to the FP64 total (n 2^-53).
+constexpr int kFold = 8;
+template <bool EXACT>
+struct SqDiff {
+  double total = 0.0;
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float a, float b) {
+    if constexpr (EXACT) {
+      const float s = a - b, bb = s - a;
+      const float e = (a - (s - bb)) + (-b - bb);
+      const float p = s * s;
+      if (!(p <= 1e35f && (p >= 1e-24f || s == 0.f))) {
+        // the square or its rounding leaves the FP32 range
+        const double d = (double)a - (double)b;
+        total += d * d;
+        return;
+      }
+      const float q = fmaf(2.f * s, e, fmaf(s, s, -p));
+      const float t = hi + p, tb = t - hi;
+      lo += ((hi - (t - tb)) + (p - tb)) + q;
+      hi = t;
+    } else {
+      const double d = (double)a - (double)b;
+      total += d * d;
+    }
+  }
+  __device__ __forceinline__ void fold() {
+    if constexpr (EXACT) {
+      total += (double)hi + (double)lo;
+      hi = lo = 0.f;
+    }
+  }
+};
+
 // X_i = W_i + R (the X-update of eq:admm on the final state), U_i = Z_i - W_i,
-// and in FP64 sum over i of ||X_i - Z_i||^2 (primal residual) into
-// pres_acc[0] and, with `dual`, sum of ||Z_i - Z_i^prev||^2 into
-// pres_acc[1], where X_out holds the previous iteration's Z on entry.
+// and sum over i of ||X_i - Z_i||^2 (primal residual) into pres_acc[0] and,
+// with `dual`, sum of ||Z_i - Z_i^prev||^2 into pres_acc[1], where X_out holds
+// the previous iteration's Z on entry.
+template <bool EXACT, int V>  // V: entries per thread and step (1 or 4)
 __global__ void __launch_bounds__(kEwThreads)
 finalize_kernel(const float* __restrict__ W, const float* __restrict__ Z,
                 const float* __restrict__ R, float* X_out, float* __restrict__ U_out,
                 double* pres_acc, int dual, int L, size_t MN) {
   __shared__ double sred[kEwThreads / 32];
   const size_t stride = (size_t)gridDim.x * blockDim.x;
-  double acc = 0.0, accd = 0.0;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < MN; i += stride) {
-    const float r = R[i];
+  SqDiff<EXACT> acc, accd;
+  const size_t n = MN / V;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    float r[V];
+    if constexpr (V == 4) *reinterpret_cast<float4*>(r) = reinterpret_cast<const float4*>(R)[i];
+    else r[0] = R[i];
     for (int j = 0; j < L; ++j) {
-      const size_t o = (size_t)j * MN + i;
-      const float w = W[o], z = Z[o];
-      const float x = w + r;
-      if (dual) {
-        const double dz = (double)z - (double)X_out[o];
-        accd += dz * dz;
+      const size_t o = (size_t)j * MN + i * V;
+      float w[V], z[V], x[V], zp[V] = {};
+      if constexpr (V == 4) {
+        *reinterpret_cast<float4*>(w) = *reinterpret_cast<const float4*>(W + o);
+        *reinterpret_cast<float4*>(z) = *reinterpret_cast<const float4*>(Z + o);
+        if (dual) *reinterpret_cast<float4*>(zp) = *reinterpret_cast<const float4*>(X_out + o);
+      } else {
+        w[0] = W[o];
+        z[0] = Z[o];
+        if (dual) zp[0] = X_out[o];
       }
-      X_out[o] = x;
-      if (U_out) U_out[o] = z - w;
-      const double dxz = (double)x - (double)z;
-      acc += dxz * dxz;
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        x[v] = w[v] + r[v];
+        if (dual) accd.add(z[v], zp[v]);
+        acc.add(x[v], z[v]);
+      }
+      static_assert(V <= kFold && kFold % V == 0, "terms between folds");
+      if (((j + 1) * V) % kFold == 0) {
+        acc.fold();
+        accd.fold();
+      }
+      if constexpr (V == 4) {
+        *reinterpret_cast<float4*>(X_out + o) = *reinterpret_cast<const float4*>(x);
+        if (U_out)
+          *reinterpret_cast<float4*>(U_out + o) =
+              make_float4(z[0] - w[0], z[1] - w[1], z[2] - w[2], z[3] - w[3]);
+      } else {
+        X_out[o] = x[0];
+        if (U_out) U_out[o] = z[0] - w[0];
+      }
     }
+    acc.fold();
+    accd.fold();
   }
   if (pres_acc) {
-    cta_add_d(acc, pres_acc, sred);
-    if (dual) cta_add_d(accd, pres_acc + 1, sred);
+    cta_add_d(acc.total, pres_acc, sred);
+    if (dual) cta_add_d(accd.total, pres_acc + 1, sred);
   }
 }
 
@@ -447,8 +514,16 @@ cudaError_t launch_finalize(const float* W, const float* Z, const float* R, floa
                             float* U_out, double* pres_acc, bool dual, int L, size_t MN,
                             cudaStream_t st, Prof* prof) {
   MISC_BEFORE()
-  finalize_kernel<<<ew_grid(MN), kEwThreads, 0, st>>>(W, Z, R, X_out, U_out, pres_acc, dual ? 1 : 0,
-                                                      L, MN);
+  const int grid = ew_grid(MN), d = dual ? 1 : 0;
+  const bool vec = (MN & 3) == 0 && ((((uintptr_t)W) | ((uintptr_t)Z) | ((uintptr_t)R) |
+                                      ((uintptr_t)X_out) | ((uintptr_t)U_out)) & 15) == 0;
+  // the FP32-pair sums from 128 terms per thread on (see SqDiff)
+  if (vec && MN * L >= (size_t)grid * kEwThreads * 128)
+    finalize_kernel<true, 4><<<grid, kEwThreads, 0, st>>>(W, Z, R, X_out, U_out, pres_acc, d, L, MN);
+  else if (vec)
+    finalize_kernel<false, 4><<<grid, kEwThreads, 0, st>>>(W, Z, R, X_out, U_out, pres_acc, d, L, MN);
+  else
+    finalize_kernel<false, 1><<<grid, kEwThreads, 0, st>>>(W, Z, R, X_out, U_out, pres_acc, d, L, MN);
   MISC_AFTER()
   return cudaGetLastError();
 }
