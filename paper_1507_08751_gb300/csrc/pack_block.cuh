@@ -121,7 +121,11 @@ __device__ __forceinline__ void pack_block_svt(const ScaleLaunch& a, int b, bool
 #pragma unroll
       for (int i = 0; i < R; ++i) al = fmaf(y[i], y[i], al);
       const float small = group_sum<W>(al <= thr ? al : 0.f);
-      const float skip = (a.skip_bound && small <= 0.9999f * thr) ? thr : -1.f;
+      float large = al <= thr ? FLT_MAX : al;
+#pragma unroll
+      for (int o = W / 2; o > 0; o >>= 1) large = fminf(large, __shfl_xor_sync(kFull, large, o));
+      const float skip =
+          (a.skip_bound && small <= 0.9999f * thr && small <= kSkipRatio * large) ? thr : -1.f;
       bool rotated = false;
 #pragma unroll 1
       for (int rd = 0; rd < np - 1; ++rd) {

@@ -46,7 +46,10 @@ constexpr int kWT = 32;
 constexpr int kWarps = kWT / 32;
 constexpr float kRotTol = 2e-6f;    // rotate columns p, q while |c_p . c_q| > tol ||c_p|| ||c_q||
 constexpr float kTinyCol = 1e-13f;  // squared norm of a numerically zero column, relative to ||C||_F^2
-constexpr int kMaxSweeps = 12;
+constexpr int kMaxSweeps = 16;
+// pairs of small columns are left alone while their squares sum to at most
+// this fraction of the smallest large column's (the convergence factor)
+constexpr float kSkipRatio = 0.4f;
 constexpr unsigned kFull = 0xffffffffu;
 
 // Block b of the scale by the calling warp.  RPL: rows of C per lane
@@ -167,10 +170,15 @@ __device__ __forceinline__ void warp_block_svt(const ScaleLaunch& a, int b, floa
       // columns need no rotation: the block is settled once the columns above
       // tau are orthogonal to each other and to these.  A rotation of a
       // large and a small column only shrinks the small one, so the sum, taken
-      // here, holds for the whole sweep.  Blocks of few terms then settle in 3
-      // sweeps instead of 7 or 8.
+      // here, holds for the whole sweep.  Blocks of few terms then settle in 4
+      // or 5 sweeps instead of 7 or 8.  The convergence is only linear, by a
+      // factor of about the ratio of the small columns' squares to the
+      // smallest large column's, so where that is above kSkipRatio every pair
+      // is rotated.
       const float small = warp_sum((h == 0 && al <= thr) ? al : 0.f);
-      const float skip = (a.skip_bound && small <= 0.9999f * thr) ? thr : -1.f;
+      const float large = -warp_max(al <= thr ? -FLT_MAX : -al);
+      const float skip =
+          (a.skip_bound && small <= 0.9999f * thr && small <= kSkipRatio * large) ? thr : -1.f;
       bool rotated = false;
 #pragma unroll 1
       for (int rd = 0; rd < np - 1; ++rd) {

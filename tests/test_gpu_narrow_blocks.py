@@ -64,3 +64,24 @@ def test_narrow_blocks_match_oracle(ctx, m, n):
             p, q = divmod(b, bn)
             blk = np.s_[p * m:(p + 1) * m, q * n:(q + 1) * n]
             assert np.linalg.norm(got[blk] - want[blk]) <= 1e-5 * max(s[b, 0], tau)
+
+
+@pytest.mark.parametrize("n", [4, 8, 16])
+def test_narrow_blocks_with_pairs_on_both_sides_of_tau(ctx, n):
+    """Singular values 1.04 and 0.946 tau and small ones: rotations that leave
+    the columns below tau alone converge slowly here, the result must not
+    depend on it.  Bar per block as above, halved: 5e-6."""
+    rng = np.random.default_rng(n)
+    nb, tau = 2048, 3.0
+    s = np.full(n, 0.03)
+    s[:4] = (1.043, 0.9458, 0.1926, 0.0669)
+    U, _ = np.linalg.qr(rng.standard_normal((nb, n, n)))
+    V, _ = np.linalg.qr(rng.standard_normal((nb, n, n)))
+    A = ((U * (s * tau)) @ V.transpose(0, 2, 1)).astype(np.float32)
+    Z = torch.empty((nb * n, n), dtype=torch.float32, device="cuda")
+    ctx.msllr_blocksvt(torch.from_numpy(A.reshape(nb * n, n)).cuda(), Z, n, n, tau, (0, 0))
+    torch.cuda.synchronize()
+    u, sv, vt = np.linalg.svd(A.astype(np.float64))
+    want = (u * np.maximum(sv - tau, 0.0)[:, None, :]) @ vt
+    err = np.linalg.norm(Z.cpu().numpy().astype(np.float64).reshape(nb, n, n) - want, axis=(1, 2))
+    assert np.all(err <= 5e-6 * sv[:, 0])
