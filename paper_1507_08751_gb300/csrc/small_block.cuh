@@ -10,6 +10,8 @@
 
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "internal.h"
 #include "lanczos.cuh"
@@ -18,6 +20,13 @@
 
 namespace msllr {
 namespace {
+
+__device__ __forceinline__ void copy4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
 
 // row index i of packed lower-triangle position e (e = i(i+1)/2 + j, j <= i)
 __device__ __forceinline__ int tri_row(int e) {
@@ -112,26 +121,57 @@ __device__ __forceinline__ void small_block_svt(const ScaleLaunch& a, int b, flo
   const float rcp_n = 1.f / (float)a.n;
   auto row_of = [&](int e) { return __float2int_rz(((float)e + 0.5f) * rcp_n); };
   float fro = 0.f;
-  constexpr int GU = 8;  // loads in flight per thread and half of A
-  for (int e0 = tid; e0 < melem; e0 += GU * NT) {
-    float x[GU], y[GU];
-#pragma unroll
-    for (int u = 0; u < GU; ++u) {
-      const int e = e0 + u * NT;
-      const bool in = e < melem;
-      const int r = in ? row_of(e) : 0, c = in ? e - r * a.n : 0;
-      const size_t off = g.offset(r, c);
-      x[u] = in ? a.A1[off] : 0.f;
-      y[u] = in ? a2(off, r, c) : 0.f;
-    }
-#pragma unroll
-    for (int u = 0; u < GU; ++u) {
-      const int e = e0 + u * NT;
-      if (e < melem) {
+  bool gathered = false;
+  if constexpr (std::is_same<SRC, A2Global>::value && NT >= 64) {
+    // asynchronous copies: every element of both halves in flight at once (a
+    // block's gather is latency: four rounds of eight register loads took
+    // 10-14k cycles, one round takes one latency); the second half waits in
+    // G's place
+    if (mm * nn <= nn * ldg) {
+      gathered = true;
+      for (int e = tid; e < melem; e += NT) {
         const int r = row_of(e), c = e - r * a.n;
-        const float v = x[u] + y[u];
-        C[g.cidx(r, c, ldc)] = v;
+        const size_t off = g.offset(r, c);
+        const int ci = g.cidx(r, c, ldc);
+        copy4(C + ci, a.A1 + off);
+        if (a2.p) copy4(G + ci, a2.p + off);
+      }
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      // (a thread reads back its own copies)
+      for (int e = tid; e < melem; e += NT) {
+        const int r = row_of(e), c = e - r * a.n;
+        const int ci = g.cidx(r, c, ldc);
+        float v = C[ci];
+        if (a2.p) {
+          v += G[ci];
+          C[ci] = v;
+        }
         fro = fmaf(v, v, fro);
+      }
+    }
+  }
+  if (!gathered) {
+    constexpr int GU = 8;  // loads in flight per thread and half of A
+    for (int e0 = tid; e0 < melem; e0 += GU * NT) {
+      float x[GU], y[GU];
+  #pragma unroll
+      for (int u = 0; u < GU; ++u) {
+        const int e = e0 + u * NT;
+        const bool in = e < melem;
+        const int r = in ? row_of(e) : 0, c = in ? e - r * a.n : 0;
+        const size_t off = g.offset(r, c);
+        x[u] = in ? a.A1[off] : 0.f;
+        y[u] = in ? a2(off, r, c) : 0.f;
+      }
+  #pragma unroll
+      for (int u = 0; u < GU; ++u) {
+        const int e = e0 + u * NT;
+        if (e < melem) {
+          const int r = row_of(e), c = e - r * a.n;
+          const float v = x[u] + y[u];
+          C[g.cidx(r, c, ldc)] = v;
+          fro = fmaf(v, v, fro);
+        }
       }
     }
   }
