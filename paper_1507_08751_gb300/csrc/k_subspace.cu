@@ -81,7 +81,11 @@ __device__ __forceinline__ void cp_wait() {
 // 8 x 8 register tiles (lane: rows lr + 8 i, columns 8 lc ..), which balances
 // its shared-memory reads (16 x 128 bits per 4 columns of G) with its 256
 // multiply-adds; the warps of a row half split each chunk's columns, and
-// their sums are added pairwise in a fixed order.
+// their sums are added pairwise in a fixed order.  MANY: compact code for
+// launches that fill the chip (its instruction fetch limits the unrolled form
+// there: 16 blocks 512 wide 6 % slower; a lone 1024-wide block is 3 % faster
+// with it).
+template <bool MANY>
 __device__ void sub_gv(const float* __restrict__ Gr, const float* V, int np, int rp, float* pipe,
                        float* Ws) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -119,7 +123,7 @@ __device__ void sub_gv(const float* __restrict__ Gr, const float* V, int np, int
     const float* Vs = Gs + rp * kSLdG;
     for (int k4 = split; k4 < kSKC / 4; k4 += ns) {
       const float* gp = Gs + (row0 + lr) * kSLdG + 4 * k4;
-#pragma unroll
+#pragma unroll(MANY ? 1 : 2)
       for (int k2 = 0; k2 < 4; k2 += 2) {
         float2 g[8];
 #pragma unroll
@@ -567,6 +571,7 @@ __device__ __forceinline__ bool sub_active(const HugeBlock& h) {
 
 // Every step of every round for the blocks of a scale, a cluster per block.
 // `first`: steps of the first round (later rounds: 4 and 8).
+template <bool MANY>
 __global__ void __launch_bounds__(kSNT)
 subspace_cluster_kernel(const float* __restrict__ G, float* V, float* __restrict__ U,
                         float* __restrict__ GU, int nn, int np, float thr, int first,
@@ -589,7 +594,7 @@ subspace_cluster_kernel(const float* __restrict__ G, float* V, float* __restrict
   bool failed = false, conv = false;
   for (int rd = 0; rd < 3 && !conv && !failed; ++rd) {
     for (int st = 0; st < rounds[rd] && !failed; ++st) {
-      sub_gv(Gr, Vb, np, rp, m.pipe, m.Ws);
+      sub_gv<MANY>(Gr, Vb, np, rp, m.pipe, m.Ws);
       // the third pass brings V to working precision for the Ritz problem;
       // between steps a well-conditioned basis of the same span is enough
       failed = !sub_orth(cl, m, rp, r0, nn, b, mu, st + 1 < rounds[rd] ? 2 : 3);
@@ -598,7 +603,7 @@ subspace_cluster_kernel(const float* __restrict__ G, float* V, float* __restrict
       cl.sync();  // the new V is visible to the cluster
     }
     if (failed) break;
-    sub_gv(Gr, Vb, np, rp, m.pipe, m.Ws);
+    sub_gv<MANY>(Gr, Vb, np, rp, m.pipe, m.Ws);
     conv = sub_ritz(cl, m, rp, U + uo, GU + uo, thr, h);
     if (!conv) {
       for (int e = tid; e < rp * kHP; e += kSNT)
@@ -618,7 +623,7 @@ subspace_gv_kernel(const float* __restrict__ G, const float* __restrict__ V, flo
   const int b = blockIdx.y, r0 = blockIdx.x * 64, tid = threadIdx.x;
   if (!sub_active(hb[b])) return;
   float* Ws = sm + sub_pipe_floats(64);
-  sub_gv(G + (size_t)b * np * np + (size_t)r0 * np, V + (size_t)b * np * kHP, np, 64, sm, Ws);
+  sub_gv<true>(G + (size_t)b * np * np + (size_t)r0 * np, V + (size_t)b * np * kHP, np, 64, sm, Ws);
   float* Wb = W + ((size_t)b * np + r0) * kHP;
   for (int e = tid; e < 64 * kHP; e += kSNT) Wb[e] = Ws[(e >> 5) * kSLd + (e & 31)];
 }
@@ -712,7 +717,8 @@ cudaError_t sub_launch(K k, int CL, int B, int rows, cudaStream_t st, A... args)
 }  // namespace
 
 cudaError_t configure_subspace() {
-  if (cudaError_t e = sub_attributes(subspace_cluster_kernel, kSMaxRows)) return e;
+  if (cudaError_t e = sub_attributes(subspace_cluster_kernel<false>, kSMaxRows)) return e;
+  if (cudaError_t e = sub_attributes(subspace_cluster_kernel<true>, kSMaxRows)) return e;
   if (cudaError_t e = sub_attributes(subspace_phase_kernel, kSPhaseRows)) return e;
   if (cudaError_t e = cudaFuncSetAttribute(subspace_gv_kernel,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -730,12 +736,17 @@ cudaError_t launch_subspace(const float* G, float* V, float* W, float* U, float*
     if (cudaError_t e = launch()) return e;
     return prof ? prof->after(st) : cudaSuccess;
   };
-  // 8 CTAs up to 512 wide, 16 above; 32 to 128 rows a CTA
-  const int CL = np <= 512 ? 8 : 16;
+  // 8 CTAs per block up to 512 wide, 16 above (32 to 128 rows a CTA), where a
+  // lone block's latency counts; 8 up to 1024 wide when the blocks fill the
+  // chip anyway (64 blocks of 1024: 3.4 -> 2.3 ms)
+  const bool many = 16 * B > sm_count();
+  const int CL = np <= 512 || (many && np <= 8 * kSMaxRows) ? 8 : 16;
   if (np / CL <= kSMaxRows)
     return timed([&] {
-      return sub_launch(subspace_cluster_kernel, CL, B, np / CL, st, G, V, U, GU, nn, np, thr, first,
-                        hb);
+      return many ? sub_launch(subspace_cluster_kernel<true>, CL, B, np / CL, st, G, V, U, GU, nn, np,
+                               thr, first, hb)
+                  : sub_launch(subspace_cluster_kernel<false>, CL, B, np / CL, st, G, V, U, GU, nn, np,
+                               thr, first, hb);
     });
   auto gv = [&] {
     subspace_gv_kernel<<<dim3(np / 64, B), kSNT, sub_smem_bytes(64), st>>>(G, V, W, np, hb);
