@@ -530,7 +530,7 @@ eig_cluster_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace w
           bool conv = true;
           const float bJ = z.beta[J - 1];
           // (many pairs: each adds its share of the error)
-          const float tol = kr > 8 ? 3e-6f : 1e-5f;
+          const float tol = kr > 8 ? 1e-6f : 1e-5f;
           for (int q = 0; q < kr; ++q)
             if (fabsf(bJ * z.ty[(J - 1) * K + q]) > tol * fmaxf(s.lam[0], thr)) conv = false;
           if (conv) break;
@@ -540,7 +540,9 @@ eig_cluster_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace w
       __syncthreads();
       if (kr < 0 && !many) {
         kr = lz_ritz<NT, K>(J, thr_keep, z, s);
-        many = kr > K;
+        // pairs that jmax steps did not settle go to the Householder path
+        // (the certificate alone admits a residual of some per cent of tau^2)
+        many = kr > K || (J == jmax && J < n && kr > 0);
       }
       fl += fl_lanczos(n, J, many ? 0 : kr);
       PHASE(3, 1);

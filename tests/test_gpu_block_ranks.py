@@ -63,3 +63,30 @@ def test_ranks_around_the_limits(ctx, m, n):
         p, q = divmod(b, 2)
         sl = np.s_[p * m:(p + 1) * m, q * n:(q + 1) * n]
         assert np.linalg.norm(got[sl] - want[sl]) <= TOL * max(np.linalg.norm(want[sl]), tau)
+
+
+@pytest.mark.parametrize("m,n,above", [(176, 176, 6), (300, 176, 12), (130, 240, 14), (256, 256, 10),
+                                       (120, 100, 9)])
+def test_pairs_above_a_crowd_below_tau(ctx, m, n, above):
+    """Singular values that crowd just below tau (0.9 .. 0.999 tau) under some
+    from 1.002 to 2 tau: slow to converge, must not be taken unconverged.  Bar:
+    2e-5 of tau per block entry norm -- the FP32 Gram matrix moves an
+    eigenvalue by about n eps lambda_1 = 1e-4 tau^2 at most, a few per cent of
+    that in the mean."""
+    rng = np.random.default_rng(m + n)
+    k, tau = min(m, n), 30.0
+    s = np.concatenate([np.linspace(2.0, 1.002, above), np.linspace(0.999, 0.9, k - above)]) * tau
+    blocks = []
+    for _ in range(4):
+        U, _ = np.linalg.qr(rng.standard_normal((m, k)))
+        V, _ = np.linalg.qr(rng.standard_normal((n, k)))
+        blocks.append((U * s) @ V.T)
+    A = np.concatenate(blocks).astype(np.float32)
+    Z = torch.empty(A.shape, dtype=torch.float32, device="cuda")
+    ctx.msllr_blocksvt(torch.from_numpy(A).cuda(), Z, m, n, tau, (0, 0))
+    torch.cuda.synchronize()
+    want = O.block_svt(A.astype(np.float64), m, n, tau)
+    got = Z.cpu().numpy().astype(np.float64)
+    for b in range(4):
+        sl = np.s_[b * m:(b + 1) * m]
+        assert np.linalg.norm(got[sl] - want[sl]) <= 2e-5 * tau
