@@ -139,10 +139,10 @@ def peaks(n_sm):
     return p
 
 
-# DRAM bytes (read + write) per launch of a kernel, from one ncu capture of
+# DRAM bytes (read + write) per launch of a kernel, from an ncu capture of
 # the kernel as it stands (key: kernel kind and scale); kernels not listed
 # report traffic null.
-NCU_TRAFFIC_BYTES = {"eig_big[scale 3: 256x256]": 8777984}
+NCU_TRAFFIC_BYTES = {}
 ITERS_OF = {}
 
 
@@ -171,26 +171,17 @@ def kernel_roofline(stats, scales, M, N, pk):
                 "unit": "TFLOP/s", "frac": round(ach / pk["fp32_tflops"], 4), "traffic": None,
                 "peak_src": pk["fp32_src"]}
     elif kind == "subspace":
-        # W = G V launches read G (4 nn^2 bytes per block); per iteration the
-        # wide path launches sum(steps) + 3 of them among 5 sum(steps) + 3
-        # subspace launches (steps 2 or 6, 6, 12).  Every launch is counted
-        # as active: an upper bound when blocks converge in an early round.
+        # every product W = G V reads G (4 nn^2 bytes per block): the first
+        # round's steps (2 with a basis carried over, else 6) and the one
+        # before its Ritz test, over the iteration's launches (one up to 2048
+        # wide); later rounds come on top
         full = (m, nsz) == (M, N)
-        steps = (2 if full else 6) + 6 + 12
-        per = (steps + 3) / (5 * steps + 3) * 4 * nn * nn * nblocks
+        per_iter_launches = n / max(1, ITERS_OF.get("cur", 1))
+        per = ((2 if full else 6) + 1) * 4 * nn * nn * nblocks / per_iter_launches
         ach = per / avg_s / 1e9
         roof = {"bound": "hbm", "achieved": round(ach, 1), "peak": pk["hbm_gbs"], "unit": "GB/s",
                 "frac": round(ach / pk["hbm_gbs"], 4), "traffic": None,
-                "peak_src": pk["src"], "note": "G V launches counted as all active (upper bound)"}
-    elif kind == "certificate":
-        # tiled Cholesky of an nn x nn matrix per block: nn^3 / 3 flop per
-        # iteration, over all of that iteration's panel and update launches
-        per_iter_launches = n / max(1, ITERS_OF.get("cur", 1))
-        flops = nblocks * nn ** 3 / 3 / per_iter_launches
-        ach = flops / avg_s / 1e12
-        roof = {"bound": "alu", "achieved": round(ach, 4), "peak": round(pk["fp32_tflops"], 1),
-                "unit": "TFLOP/s", "frac": round(ach / pk["fp32_tflops"], 5), "traffic": None,
-                "peak_src": pk["fp32_src"]}
+                "peak_src": pk["src"], "note": "products of the first round only (lower bound)"}
     elif kind in ("eig_big", "eig_fallback"):
         # flops of the steps the kernel ran (counted on the device over every
         # launch of the profiled job), per launch

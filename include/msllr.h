@@ -52,7 +52,7 @@ typedef enum msllr_status {
  * kernels (finiteness check, state init, X/U output), 9 wide-block
  * Householder fallback (blocks the certified paths did not settle),
  * 10 subspace iteration of blocks wider than 256 (G V, orthonormalisation,
- * Rayleigh-Ritz), 11 their tiled Cholesky certificate. */
+ * Rayleigh-Ritz), 11 their certificate (repeated squaring). */
 #define MSLLR_KERNEL_KINDS 12
 
 /* Widest block (min(m_i, n_i)) the block-SVT kernels accept; the full-matrix
@@ -69,7 +69,8 @@ typedef struct msllr_ctx msllr_ctx;
 typedef struct msllr_params {
   int skip_bound;    /* 1 (default): certified shortcuts -- skip a block whose
                         upper bound on sigma_max is <= tau (Sec. 8: trace,
-                        Gershgorin, or a Cholesky of tau^2 I - G), and for
+                        Gershgorin, or a certificate that
+                        lambda_max(G) < tau^2), and for
                         wide blocks find the pairs above tau by certified
                         Lanczos before falling back to Householder.
                         0: every block takes the full Householder
@@ -181,7 +182,7 @@ typedef struct msllr_stats {
   long long blocks_uncertified[MSLLR_MAX_SCALES];
   /* FP32 flops of the block eigen-solve steps that ran, each step counted
    * at its algorithmic cost (a multiply-add is 2 flops): zero-rank and
-   * deflated Cholesky certificates n^3/3, Lanczos and power steps,
+   * deflated certificates n^3/3 (a Cholesky factorisation's), Lanczos and power steps,
    * Householder tridiagonalisation 4n^3/3.  `flops`: the fused narrow-block
    * kernel (its Gram and rebuild included) or the wide-block eigen kernel;
    * `flops_fallback`: the wide-block Householder fallback kernel.  Blocks up

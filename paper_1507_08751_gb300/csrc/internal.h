@@ -53,17 +53,20 @@ __host__ __device__ __forceinline__ int job_block(const ScaleLaunch& s, int b) {
   return s.rows ? b % ((s.rows / s.m) * (s.N / s.n)) : b;
 }
 
+constexpr int kBigWarm = 8;  // Ritz vectors kept per block for the warm start
+
 // Device workspace needed by the wide-block path for one scale.
 struct BigWorkspace {
   float* G;      // nblocks * nn * nn; block b at b * nn * nn, lower triangle packed row by row
   float* part;   // nblocks * chunks * ntiles * 64 * 64 (when chunks > 1)
   float* Y;      // nblocks * ystride: eigenvectors / Lanczos scratch per block
   int* k;        // nblocks
-  float* warm;   // nblocks * 8 * nn: previous Ritz vectors (warm start)
+  float* warm;   // nblocks * kBigWarm * nn: previous Ritz vectors (warm start)
   int* kwarm;    // nblocks: how many of them (0 = none)
   size_t ystride;
   // blocks wider than 256 (k_block_huge.cu): G is a full square there
   void* Ma;      // nblocks * np * np FP16, np = nn rounded up to 64: certificate matrices
+                 // (over part, which is free once G is formed, as far as they fit)
   void* Mb;
   double* fpart; // nblocks * tiles: their F-norm partials
   float* tstat;  // nblocks * ntiles * 2: per-tile diagonal sums, sums of squares

@@ -28,7 +28,6 @@ constexpr int kTile = 64;       // Gram tile
 constexpr int kChunk = 256;     // rows of C per Gram partial sum
 constexpr int kGramThreads = 256;
 constexpr int kEigMax = 256;
-constexpr int kEigK = lz_maxk(kEigMax);  // Ritz pairs kept per block
 constexpr int kRebThreads = 256;
 constexpr int kRebElems = 4096;  // rows-per-slab * nn
 constexpr int kKC = 16;          // eigenvectors per rebuild step
@@ -329,10 +328,8 @@ rebuild_kernel(ScaleLaunch a, const float* __restrict__ Yall, size_t ystride,
 
 }  // namespace
 
-static size_t y_stride(int nn) {
-  const size_t a = (size_t)nn * nn, b = (size_t)(kLzMaxJ + 2 * kEigK) * nn;
-  return ((a > b ? a : b) + 63) & ~(size_t)63;
-}
+// the thresholded eigenvectors of a block: nn x k, k <= nn
+static size_t y_stride(int nn) { return ((size_t)nn * nn + 63) & ~(size_t)63; }
 
 size_t big_workspace_bytes(int M, int N, int m, int n) {
   if (choose_path(m, n) == ScalePath::Huge) return huge_workspace_bytes(M, N, m, n);
@@ -343,7 +340,7 @@ size_t big_workspace_bytes(int M, int N, int m, int n) {
   if (d.chunks > 1) bytes += sizeof(float) * (size_t)d.nblocks * d.chunks * d.ntiles * kTile * kTile;
   bytes += sizeof(float) * (size_t)d.nblocks * y_stride(d.nn);  // Y
   bytes += sizeof(int) * (size_t)d.nblocks;                      // k
-  bytes += sizeof(float) * (size_t)d.nblocks * kEigK * d.nn;   // warm
+  bytes += sizeof(float) * (size_t)d.nblocks * kBigWarm * d.nn;   // warm
   bytes += sizeof(int) * (size_t)d.nblocks;                      // kwarm
   bytes += 8 * 256;  // alignment slack for the carve below
   return bytes;
@@ -371,7 +368,7 @@ BigWorkspace carve_big_workspace(void* base, int M, int N, int m, int n) {
   w.k = (int*)p;
   p = align256(p + sizeof(int) * (size_t)d.nblocks);
   w.warm = (float*)p;
-  p = align256(p + sizeof(float) * (size_t)d.nblocks * kEigK * d.nn);
+  p = align256(p + sizeof(float) * (size_t)d.nblocks * kBigWarm * d.nn);
   w.kwarm = (int*)p;
   return w;
 }

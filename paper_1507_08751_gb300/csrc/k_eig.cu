@@ -404,8 +404,8 @@ eig_cluster_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace w
   const float gbound = fminf(tr, rs);
   double fl = n + fl_symv(n);
   const bool full = (a.m == launch_rows(a) && a.n == a.N);
-  const int kwarm = (a.warm_start && (full || !a.shift)) ? min(ws.kwarm[b], K) : 0;
-  const float* warm = ws.warm + (size_t)b * K * n;
+  const int kwarm = (a.warm_start && (full || !a.shift)) ? min(ws.kwarm[b], kBigWarm) : 0;
+  const float* warm = ws.warm + (size_t)b * kBigWarm * n;
   bool skipped = false, lanczos_ok = false;
   int k = -1, ku = 0;
   // FP16 of the register matrix / c into the own rows of M; the thread's part
@@ -638,12 +638,13 @@ eig_cluster_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace w
   }
   if (lanczos_ok && g.rank == 0) {
     // keep the Ritz vectors for the next call's warm start
-    float* wdst = ws.warm + (size_t)b * K * n;
-    for (int e = tid; e < n * ku; e += NT) {
+    const int kw = min(ku, kBigWarm);
+    float* wdst = ws.warm + (size_t)b * kBigWarm * n;
+    for (int e = tid; e < n * kw; e += NT) {
       const int q = e / n, r = e - q * n;
       wdst[e] = U[q * NV + r];
     }
-    if (tid == 0) ws.kwarm[b] = ku;
+    if (tid == 0) ws.kwarm[b] = kw;
     // V_f (row-major, ld n) for the rebuild
     float* Y = ws.Y + (size_t)b * ws.ystride;
     for (int e = tid; e < n * k; e += NT) {
