@@ -193,8 +193,9 @@ __device__ __forceinline__ void small_block_svt(const ScaleLaunch& a, int b, flo
     if ((nn & 7) == 0 && NT >= 64 && 2 * tiles8 <= NT) {
       // 8x8 register tiles of the lower triangle, the rows of C split over
       // two lanes: per row two 128-bit loads for the tile's rows and two for
-      // its columns, 64 FMAs (4x4 tiles were bound by their shared-memory
-      // reads and took two rounds of threads at 64 wide: 8.5k cycles, here 4k)
+      // its columns, 64 FMAs (half the shared-memory reads per FMA of the 4x4
+      // tiles below, and one round of threads at 64 wide: 6.6k cycles for a
+      // lone 64 x 64 block; 9k with three CTAs per SM, as before)
       const int t = tid >> 1, half = tid & 1;
       const bool on = t < tiles8;
       const int ta = on ? tri_row(t) : 0, tb = on ? t - (ta * (ta + 1)) / 2 : 0;
