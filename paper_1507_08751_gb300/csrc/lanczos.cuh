@@ -504,7 +504,10 @@ __device__ int lanczos_candidates(const SmallGram<NT, NMAX>& g, float thr, float
   *J_out = J;
   if (k < 0) {
     k = lz_ritz<NT, K>(J, thr_keep, z, s);
-    if (k > K) return -1;
+    // pairs that jmax < n steps did not settle are not taken: the certificate
+    // below admits any residual that leaves lambda_max(P G P) below tau^2 -
+    // 2 rho, up to some per cent of tau^2
+    if (k > K || (J == jmax && J < n && k > 0)) return -1;
   }
   const int ku = k, n8 = (n + 7) & ~7;
   float* U8 = panel;

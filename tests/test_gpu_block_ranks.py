@@ -90,3 +90,34 @@ def test_pairs_above_a_crowd_below_tau(ctx, m, n, above):
     for b in range(4):
         sl = np.s_[b * m:(b + 1) * m]
         assert np.linalg.norm(got[sl] - want[sl]) <= 2e-5 * tau
+
+
+@pytest.mark.parametrize("m,n", [(33, 33), (40, 40), (40, 100), (48, 64), (60, 60), (64, 64)])
+def test_narrow_pairs_above_a_crowd_below_tau(ctx, m, n):
+    """Blocks 33 to 64 wide with eight pairs from 1.002 to 1.03 tau over a crowd
+    from 0.77 to 0.96 tau, which 32 Lanczos steps do not settle from 40 wide
+    on.  Bar per block: settled pairs have residuals of at most 1e-5 lambda_1
+    each, so they are exact for a matrix within sqrt(2) sqrt(8) 1e-5 lambda_1
+    <= 4.3e-5 tau^2 of G (Frobenius), plus n eps lambda_1 <= 0.9e-5 tau^2 of
+    rounding in G; (1 - tau / sqrt(x))_+ has slope 1 / (2 tau^2) at most, so Z
+    is within sigma_1 5.2e-5 / 2 = 2.7e-5 tau: 4e-5 tau with the output's own
+    rounding."""
+    rng = np.random.default_rng(100 * m + n)
+    k, tau, nb = min(m, n), 30.0, 16
+    s = np.concatenate([np.linspace(1.03, 1.002, 8), np.linspace(0.96, 0.77, k - 8)]) * tau
+    blocks = []
+    for _ in range(nb):
+        U, _ = np.linalg.qr(rng.standard_normal((m, k)))
+        V, _ = np.linalg.qr(rng.standard_normal((n, k)))
+        blocks.append((U * s) @ V.T)
+    A = np.concatenate(blocks).astype(np.float32)
+    Z = torch.empty(A.shape, dtype=torch.float32, device="cuda")
+    rank = torch.empty((nb,), dtype=torch.int32, device="cuda")
+    ctx.msllr_blocksvt(torch.from_numpy(A).cuda(), Z, m, n, tau, (0, 0), rank_out=rank)
+    torch.cuda.synchronize()
+    want = O.block_svt(A.astype(np.float64), m, n, tau)
+    got = Z.cpu().numpy().astype(np.float64)
+    assert np.all(rank.cpu().numpy() == 8)
+    for b in range(nb):
+        sl = np.s_[b * m:(b + 1) * m]
+        assert np.linalg.norm(got[sl] - want[sl]) <= 4e-5 * tau
