@@ -176,9 +176,10 @@ typedef struct msllr_stats {
    * params->profile was set (else 0). */
   long long kernel_launches[MSLLR_KERNEL_KINDS][MSLLR_MAX_SCALES];
   double kernel_ms[MSLLR_KERNEL_KINDS][MSLLR_MAX_SCALES];
-  /* blocks wider than 256 whose certificate (no singular value above tau
-   * outside the kept Ritz pairs) failed at the last iteration; their
-   * thresholded rank is taken from the Ritz pairs.  0 in normal runs. */
+  /* blocks wider than 256 whose kept Ritz pairs had not converged after every
+   * round of the subspace iteration, or whose certificate (no singular value
+   * above tau outside the kept pairs) failed, at the last iteration; their
+   * output is formed from the Ritz pairs at hand.  0 in normal runs. */
   long long blocks_uncertified[MSLLR_MAX_SCALES];
   /* FP32 flops of the block eigen-solve steps that ran, each step counted
    * at its algorithmic cost (a multiply-add is 2 flops): zero-rank and

@@ -27,6 +27,7 @@ struct HugeBlock {
   int ku;        // kept Ritz pairs
   int k;         // pairs above tau
   int conv;      // Rayleigh-Ritz residual test passed
+  int over;      // more than kHK Ritz values above tau^2
   int orth_fail; // a CholQR factorisation broke down (basis restarted)
   int cert;      // kCert*
   int arrived;   // CTAs of the running certificate level that are done

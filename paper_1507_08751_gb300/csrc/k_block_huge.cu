@@ -21,7 +21,8 @@
 //   5. rebuild: Z'_b = (C_b V_f) V_f^T with V_f = U diag(sqrt(1 - tau/sigma))
 //      over the pairs above tau, scattered through Shift_{-s}, with the fused
 //      dual update W' = 2 Z' - A of eq:admm.
-// A block whose certificate fails keeps its Ritz pairs and is counted.
+// A block whose pairs do not converge in every round run, or whose certificate
+// fails, keeps its Ritz pairs and is counted.
 #include <float.h>
 #include <math.h>
 
@@ -242,6 +243,7 @@ huge_gram_finish_kernel(const float* __restrict__ part, float* __restrict__ G, f
     h.ku = 0;
     h.k = 0;
     h.conv = 0;
+    h.over = 0;
     h.cert = kCertOpen;
     h.arrived = 0;
     h.orth_fail = 0;
@@ -293,7 +295,9 @@ huge_rebuild_kernel(ScaleLaunch a, const float* __restrict__ U, int np,
     }
   if (blockIdx.x == 0 && tid == 0) {
     const bool skipped = h.status == kHsSkip;
-    const bool cert = skipped || (h.status == kHsIter && h.cert == kCertYes);
+    // certified: no other eigenvalue above tau^2, and the pairs kept have
+    // small residuals (the certificate alone says nothing about them)
+    const bool cert = skipped || (h.status == kHsIter && h.cert == kCertYes && h.conv);
     if (a.rank_out) a.rank_out[b] = k;
     if (a.cnt) {
       if (skipped) atomicAdd(a.cnt, 1ull);

@@ -64,6 +64,11 @@ size_t sub_smem_bytes(int rp) {
   return sizeof(float) *
          (size_t)(sub_pipe_floats(rp) + 2 * rp * kSLd + kHP * kHP + 3 * kSM + kHK * kHK);
 }
+// subspace_more_kernel: the phases' arrays, or G V of 64 rows and its result
+size_t sub_more_bytes(int rp) {
+  const size_t gv = sizeof(float) * (size_t)(sub_pipe_floats(64) + 64 * kSLd);
+  return gv > sub_smem_bytes(rp) ? gv : sub_smem_bytes(rp);
+}
 
 __device__ __forceinline__ void cp16(float* dst, const float* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
@@ -421,13 +426,14 @@ __device__ bool sub_orth(const cg::cluster_group& cl, const SubSmem& m, int rp, 
 // Rayleigh-Ritz with V in Xs and G V in Ws: T = V^T G V, its eigenpairs above
 // thr (at most kHK, largest first), the Ritz vectors U = V Q, G U, B = U^T G
 // U, the residuals and What = G U - U sym(B) / 2 (into GU).  Overwrites Xs.
-// Returns true (in every CTA) when the pairs have converged.
+// Returns true (in every CTA) when the pairs have converged; *over: more than
+// kHK Ritz values above thr, so that the block cannot be certified.
 __device__ bool sub_ritz(const cg::cluster_group& cl, const SubSmem& m, int rp, float* Ub, float* GUb,
-                         float thr, HugeBlock& h) {
+                         float thr, HugeBlock& h, bool* over) {
   const int tid = threadIdx.x, CL = (int)cl.num_blocks();
   __shared__ float rq[2 * kHK], red[kSNW][2 * kHK];
   __shared__ float2 cs[16];
-  __shared__ int sel[kHK], ku_s;
+  __shared__ int sel[kHK], nabove;
   float *Xs = m.Xs, *Ws = m.Ws, *P = m.P, *Sm = m.Sm, *Rm = m.Rm, *Qm = m.Qm, *Bm = m.Bm;
   const float gF = h.gF;
   sub_atb(Xs, Ws, rp, m.pipe, P);
@@ -452,10 +458,11 @@ __device__ bool sub_ritz(const cg::cluster_group& cl, const SubSmem& m, int rp, 
     }
     const unsigned above = __ballot_sync(0xffffffffu, th > thr);
     if (th > thr && rk < kHK) sel[rk] = tid;
-    if (tid == 0) ku_s = min(__popc(above), kHK);
+    if (tid == 0) nabove = __popc(above);
   }
   __syncthreads();
-  const int ku = ku_s;
+  const int ku = min(nabove, kHK);
+  *over = nabove > kHK;
   // U = V Q and G U = W Q, over V's rows in Xs: entries 0 .. 15 U, 16 .. 31 G
   // U (the 16 threads of a row are in one warp)
   {
@@ -560,6 +567,7 @@ __device__ bool sub_ritz(const cg::cluster_group& cl, const SubSmem& m, int rp, 
     h.ku = ku;
     h.k = k;
     h.conv = conv;
+    h.over = nabove > kHK;
   }
   cl.sync();  // the partial sums have been read
   return conv;
@@ -569,8 +577,18 @@ __device__ __forceinline__ bool sub_active(const HugeBlock& h) {
   return h.status == kHsIter && !h.conv && !h.orth_fail;
 }
 
+// Rounds of a block: `first`, 4 and 8 steps for every block, then up to
+// kSMoreRounds of 8 for blocks whose pairs have not converged and that can
+// still be certified.  128 further steps bring the residual of a pair down by
+// a factor of 1000 where the eigenvalue below the basis is 0.95 of the pair's;
+// what is slower is counted as uncertified.
+constexpr int kSRounds = 3;
+constexpr int kSMoreRounds = 16;
+__device__ __forceinline__ int sub_steps(int round, int first) {
+  return round == 0 ? first : round == 1 ? 4 : 8;
+}
+
 // Every step of every round for the blocks of a scale, a cluster per block.
-// `first`: steps of the first round (later rounds: 4 and 8).
 template <bool MANY>
 __global__ void __launch_bounds__(kSNT)
 subspace_cluster_kernel(const float* __restrict__ G, float* V, float* __restrict__ U,
@@ -590,21 +608,22 @@ subspace_cluster_kernel(const float* __restrict__ G, float* V, float* __restrict
   const float mu = 1e-4f * h.gF;
   for (int e = tid; e < rp * kHP; e += kSNT) m.Xs[(e >> 5) * kSLd + (e & 31)] = Vb[(size_t)r0 * kHP + e];
   __syncthreads();
-  const int rounds[3] = {first, 4, 8};
-  bool failed = false, conv = false;
-  for (int rd = 0; rd < 3 && !conv && !failed; ++rd) {
-    for (int st = 0; st < rounds[rd] && !failed; ++st) {
+  bool failed = false, conv = false, over = false;
+  for (int rd = 0; rd < kSRounds + kSMoreRounds && !conv && !failed; ++rd) {
+    if (rd >= kSRounds && over) break;
+    const int steps = sub_steps(rd, first);
+    for (int st = 0; st < steps && !failed; ++st) {
       sub_gv<MANY>(Gr, Vb, np, rp, m.pipe, m.Ws);
       // the third pass brings V to working precision for the Ritz problem;
       // between steps a well-conditioned basis of the same span is enough
-      failed = !sub_orth(cl, m, rp, r0, nn, b, mu, st + 1 < rounds[rd] ? 2 : 3);
+      failed = !sub_orth(cl, m, rp, r0, nn, b, mu, st + 1 < steps ? 2 : 3);
       for (int e = tid; e < rp * kHP; e += kSNT)
         Vb[(size_t)r0 * kHP + e] = m.Xs[(e >> 5) * kSLd + (e & 31)];
       cl.sync();  // the new V is visible to the cluster
     }
     if (failed) break;
     sub_gv<MANY>(Gr, Vb, np, rp, m.pipe, m.Ws);
-    conv = sub_ritz(cl, m, rp, U + uo, GU + uo, thr, h);
+    conv = sub_ritz(cl, m, rp, U + uo, GU + uo, thr, h, &over);
     if (!conv) {
       for (int e = tid; e < rp * kHP; e += kSNT)
         m.Xs[(e >> 5) * kSLd + (e & 31)] = Vb[(size_t)r0 * kHP + e];
@@ -629,11 +648,52 @@ subspace_gv_kernel(const float* __restrict__ G, const float* __restrict__ V, flo
 }
 
 // V = orth(W + mu V) (passes > 0), or the Rayleigh-Ritz test on V and W
-// (passes = 0), in one cluster per block.
+// (passes = 0), for the rows at Vr, Wr of a CTA.  False when the
+// orthonormalisation broke down or the pairs have not converged.
+__device__ bool sub_phase(const cg::cluster_group& cl, const SubSmem& m, int rp, int r0, float* Vr,
+                          const float* Wr, float* Ub, float* GUb, int nn, int b, float thr, int passes,
+                          HugeBlock& h, bool* over) {
+  const int tid = threadIdx.x;
+  for (int e = tid; e < rp * kHP; e += kSNT) {
+    const int o = (e >> 5) * kSLd + (e & 31);
+    m.Xs[o] = Vr[e];
+    m.Ws[o] = Wr[e];
+  }
+  __syncthreads();
+  if (passes == 0) return sub_ritz(cl, m, rp, Ub, GUb, thr, h, over);
+  const bool ok = sub_orth(cl, m, rp, r0, nn, b, 1e-4f * h.gF, passes);
+  for (int e = tid; e < rp * kHP; e += kSNT) Vr[e] = m.Xs[(e >> 5) * kSLd + (e & 31)];
+  cl.sync();  // the new V is visible to the cluster
+  return ok;
+}
+
+// One phase of the blocks that have not converged, a cluster per block.
 __global__ void __launch_bounds__(kSNT)
-subspace_phase_kernel(float* V, const float* __restrict__ W, float* __restrict__ U,
-                      float* __restrict__ GU, int nn, int np, float thr, int passes,
-                      HugeBlock* __restrict__ hb) {
+subspace_phase_kernel(float* V, const float* W, float* __restrict__ U, float* __restrict__ GU, int nn,
+                      int np, float thr, int passes, HugeBlock* __restrict__ hb) {
+  extern __shared__ __align__(16) float sm[];
+  const cg::cluster_group cl = cg::this_cluster();
+  const int CL = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int b = blockIdx.x / CL;
+  const int rp = np / CL, r0 = rank * rp;
+  HugeBlock& h = hb[b];
+  // (the state is written only after a later cluster barrier)
+  if (!sub_active(h)) return;
+  const size_t vo = ((size_t)b * np + r0) * kHP, uo = ((size_t)b * np + r0) * kHK;
+  bool over = false;
+  const bool ok = sub_phase(cl, SubSmem(sm, rp), rp, r0, V + vo, W + vo, U + uo, GU + uo, nn, b, thr,
+                            passes, h, &over);
+  if (passes > 0 && !ok && rank == 0 && threadIdx.x == 0) h.orth_fail = 1;
+  cl.sync();  // no CTA leaves while others read its shared memory
+}
+
+// The further rounds of a block, all steps in its cluster: G V of a CTA's rows
+// by 64 at a time (its scratch lies over the phases' arrays).  16 SMs read G
+// several times slower than the grid-wide launch, but blocks that get here
+// are rare and a launch with none of them costs its launch only.
+__global__ void __launch_bounds__(kSNT)
+subspace_more_kernel(const float* __restrict__ G, float* V, float* W, float* __restrict__ U,
+                     float* __restrict__ GU, int nn, int np, float thr, HugeBlock* __restrict__ hb) {
   extern __shared__ __align__(16) float sm[];
   const cg::cluster_group cl = cg::this_cluster();
   const int CL = (int)cl.num_blocks(), rank = (int)cl.block_rank();
@@ -641,29 +701,34 @@ subspace_phase_kernel(float* V, const float* __restrict__ W, float* __restrict__
   const int rp = np / CL, r0 = rank * rp;
   HugeBlock& h = hb[b];
   // (the state is written only after a later cluster barrier)
-  if (!sub_active(h)) return;
+  if (!sub_active(h) || h.over) return;
   const SubSmem m(sm, rp);
-  float* Vr = V + ((size_t)b * np + r0) * kHP;
-  const float* Wr = W + ((size_t)b * np + r0) * kHP;
-  for (int e = tid; e < rp * kHP; e += kSNT) {
-    const int o = (e >> 5) * kSLd + (e & 31);
-    m.Xs[o] = Vr[e];
-    m.Ws[o] = Wr[e];
+  const float* Gr = G + (size_t)b * np * np + (size_t)r0 * np;
+  const float* Vb = V + (size_t)b * np * kHP;
+  const size_t vo = ((size_t)b * np + r0) * kHP, uo = ((size_t)b * np + r0) * kHK;
+  float* Wc = sm + sub_pipe_floats(64);
+  bool ok = true, conv = false, over = false;
+  for (int rd = 0; rd < kSMoreRounds && ok && !conv && !over; ++rd) {
+    for (int st = 0; st <= 8 && ok; ++st) {
+      for (int c = 0; c < rp; c += 64) {
+        const int rows = min(64, rp - c);
+        sub_gv<true>(Gr + (size_t)c * np, Vb, np, rows, sm, Wc);
+        for (int e = tid; e < rows * kHP; e += kSNT)
+          W[vo + (size_t)c * kHP + e] = Wc[(e >> 5) * kSLd + (e & 31)];
+        __syncthreads();
+      }
+      const int passes = st < 8 ? (st + 1 < 8 ? 2 : 3) : 0;
+      const bool r = sub_phase(cl, m, rp, r0, V + vo, W + vo, U + uo, GU + uo, nn, b, thr, passes, h,
+                               &over);
+      if (passes > 0) ok = r;
+      else conv = r;
+    }
   }
-  __syncthreads();
-  if (passes > 0) {
-    const bool ok = sub_orth(cl, m, rp, r0, nn, b, 1e-4f * h.gF, passes);
-    for (int e = tid; e < rp * kHP; e += kSNT) Vr[e] = m.Xs[(e >> 5) * kSLd + (e & 31)];
-    cl.sync();
-    if (!ok && rank == 0 && tid == 0) h.orth_fail = 1;
-  } else {
-    const size_t uo = ((size_t)b * np + r0) * kHK;
-    sub_ritz(cl, m, rp, U + uo, GU + uo, thr, h);
-  }
+  if (!ok && rank == 0 && tid == 0) h.orth_fail = 1;
   cl.sync();  // no CTA leaves while others read its shared memory
 }
 
-constexpr int kSPhaseRows = 512;  // rows per CTA of subspace_phase_kernel, at most
+constexpr int kSPhaseRows = 512;  // rows per CTA of the phase kernels, at most
 
 // the widest cluster the device runs at the largest shared-memory size
 int widest_cluster() {
@@ -698,7 +763,7 @@ cudaError_t sub_attributes(K k, int rows) {
 }
 
 template <class K, class... A>
-cudaError_t sub_launch(K k, int CL, int B, int rows, cudaStream_t st, A... args) {
+cudaError_t sub_launch(K k, int CL, int B, size_t bytes, cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -707,7 +772,7 @@ cudaError_t sub_launch(K k, int CL, int B, int rows, cudaStream_t st, A... args)
   at[0].val.clusterDim.z = 1;
   cfg.gridDim = dim3(CL * B);
   cfg.blockDim = dim3(kSNT);
-  cfg.dynamicSmemBytes = sub_smem_bytes(rows);
+  cfg.dynamicSmemBytes = bytes;
   cfg.stream = st;
   cfg.attrs = at;
   cfg.numAttrs = 1;
@@ -720,6 +785,7 @@ cudaError_t configure_subspace() {
   if (cudaError_t e = sub_attributes(subspace_cluster_kernel<false>, kSMaxRows)) return e;
   if (cudaError_t e = sub_attributes(subspace_cluster_kernel<true>, kSMaxRows)) return e;
   if (cudaError_t e = sub_attributes(subspace_phase_kernel, kSPhaseRows)) return e;
+  if (cudaError_t e = sub_attributes(subspace_more_kernel, kSPhaseRows)) return e;
   if (cudaError_t e = cudaFuncSetAttribute(subspace_gv_kernel,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)sub_smem_bytes(64)))
@@ -741,30 +807,34 @@ cudaError_t launch_subspace(const float* G, float* V, float* W, float* U, float*
   // chip anyway (64 blocks of 1024: 3.4 -> 2.3 ms)
   const bool many = 16 * B > sm_count();
   const int CL = np <= 512 || (many && np <= 8 * kSMaxRows) ? 8 : 16;
+  const size_t bytes = sub_smem_bytes(np / CL);
   if (np / CL <= kSMaxRows)
     return timed([&] {
-      return many ? sub_launch(subspace_cluster_kernel<true>, CL, B, np / CL, st, G, V, U, GU, nn, np,
+      return many ? sub_launch(subspace_cluster_kernel<true>, CL, B, bytes, st, G, V, U, GU, nn, np,
                                thr, first, hb)
-                  : sub_launch(subspace_cluster_kernel<false>, CL, B, np / CL, st, G, V, U, GU, nn, np,
+                  : sub_launch(subspace_cluster_kernel<false>, CL, B, bytes, st, G, V, U, GU, nn, np,
                                thr, first, hb);
     });
   auto gv = [&] {
     subspace_gv_kernel<<<dim3(np / 64, B), kSNT, sub_smem_bytes(64), st>>>(G, V, W, np, hb);
     return cudaGetLastError();
   };
-  const int rounds[3] = {first, 4, 8};
-  for (int r = 0; r < 3; ++r) {
+  const int rounds[kSRounds] = {first, 4, 8};
+  for (int r = 0; r < kSRounds; ++r) {
     for (int i = 0; i <= rounds[r]; ++i) {
       if (cudaError_t e = timed(gv)) return e;
       const int passes = i < rounds[r] ? (i + 1 < rounds[r] ? 2 : 3) : 0;
       if (cudaError_t e = timed([&] {
-            return sub_launch(subspace_phase_kernel, 16, B, np / 16, st, V, W, U, GU, nn, np, thr,
+            return sub_launch(subspace_phase_kernel, 16, B, bytes, st, V, W, U, GU, nn, np, thr,
                               passes, hb);
           }))
         return e;
     }
   }
-  return cudaSuccess;
+  return timed([&] {
+    return sub_launch(subspace_more_kernel, 16, B, sub_more_bytes(np / 16), st, G, V, W, U, GU, nn, np, thr,
+                      hb);
+  });
 }
 
 }  // namespace msllr

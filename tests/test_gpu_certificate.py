@@ -61,3 +61,61 @@ def test_more_pairs_than_kept_is_not_certified(ctx, M, N):
     s = np.concatenate([np.linspace(200.0, 100.0, 20), np.full(50, 1.0)])
     _, st = _one_svt(ctx, _with_spectrum(M, M, N, s), 50.0)
     assert st["blocks_uncertified"][0] == 1
+
+
+def _cold_svts(ctx, blocks, tau):
+    """One iteration on a stack of blocks, moved so that the shifted grid meets
+    them: not the full matrix, so every block starts from the cold basis."""
+    from paper_1507_08751_gb300 import binding as B
+    A = np.concatenate(blocks)
+    sr, sc = (int(v) for v in B.msllr_shift_table(1, 1, *A.shape)[0])
+    X = torch.empty((1,) + A.shape, dtype=torch.float32, device="cuda")
+    Z = torch.empty_like(X)
+    Y = np.ascontiguousarray(np.roll(A, (sr, sc), (0, 1)), dtype=np.float32)
+    st = ctx.msllr_decompose(torch.from_numpy(Y).cuda(), [blocks[0].shape], X, lambdas=[tau], rho=1.0,
+                             iters=1, seed=1, Z_out=Z)
+    torch.cuda.synchronize()
+    got = np.roll(Z[0].cpu().numpy().astype(np.float64), (-sr, -sc), (0, 1))
+    return np.split(got, len(blocks)), st
+
+
+@pytest.mark.parametrize("M,N,above", [(257, 300, 8), (300, 300, 8), (512, 600, 12), (1030, 1030, 6),
+                                       (2100, 2100, 6)])
+def test_slow_pairs_above_a_crowd_below_tau(ctx, M, N, above):
+    """Pairs from 1.002 to 1.3 tau over a crowd from 0.88 to 0.93 tau: the basis
+    gains a factor of 0.87 a step for the weakest, some 50 steps in all.  A block whose pairs
+    have not converged must not count as certified.  Bar: converged pairs have
+    residuals of at most 3e-4 tau^2 each, so they are exact for a matrix within
+    sqrt(2 k) 3e-4 tau^2 of G; (1 - tau / sqrt(x))_+ has slope 1 / (2 tau^2) at
+    most, so Z is within 1.3 sqrt(2 k) 1.5e-4 tau, plus the same factor times
+    G's rounding, n eps lambda_1 <= 2e-7 n tau^2."""
+    n, tau = min(M, N), 50.0
+    s = np.concatenate([np.linspace(1.3, 1.002, above), np.linspace(0.93, 0.8835, n - above)]) * tau
+    rng = np.random.default_rng(M + N)
+    blocks, want = [], []
+    for _ in range(2):
+        U, _ = np.linalg.qr(rng.standard_normal((M, n)))
+        V, _ = np.linalg.qr(rng.standard_normal((N, n)))
+        blocks.append((U * s) @ V.T)
+        want.append((U * np.maximum(s - tau, 0.0)) @ V.T)
+    got, st = _cold_svts(ctx, blocks, tau)
+    assert st["blocks_uncertified"][0] == 0
+    assert st["blocks_lanczos"][0] == 2
+    bar = 1.3 * (np.sqrt(2 * above) * 1.5e-4 + 1e-7 * n) * tau
+    for g, w in zip(got, want):
+        assert np.linalg.norm(g - w) <= bar
+
+
+def test_pairs_slower_than_every_round_count_as_uncertified(ctx):
+    """Pairs at 1.002 tau over forty at 0.995 tau: 0.986 a step, not settled in
+    any number of steps that is run."""
+    n, tau = 320, 50.0
+    s = np.concatenate([np.full(4, 1.002), np.full(40, 0.995), np.full(n - 44, 0.3)]) * tau
+    rng = np.random.default_rng(n)
+    blocks = []
+    for _ in range(2):
+        U, _ = np.linalg.qr(rng.standard_normal((n, n)))
+        V, _ = np.linalg.qr(rng.standard_normal((n, n)))
+        blocks.append((U * s) @ V.T)
+    _, st = _cold_svts(ctx, blocks, tau)
+    assert st["blocks_uncertified"][0] == 2
