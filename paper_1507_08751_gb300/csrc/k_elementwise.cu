@@ -224,12 +224,15 @@ __device__ __forceinline__ void cta_add_d(double v, double* acc, double* sred) {
 
 // Sum of squares of differences of FP32 values.  EXACT false: FP64 throughout.
 // EXACT true: the difference a - b as the unevaluated FP32 pair (s, e) of
-// Knuth's two-sum, its square and the running sum as FP32 pairs (two-product
-// by fma; relative error 2^-46), added to the FP64 total every kFold terms.
+// Knuth's two-sum, its square (two-product by fma) and the running sum as
+// FP32 pairs, added to the FP64 total every kFold terms.  Every operation that
+// the error-free steps rest on is a rounded intrinsic, which the compiler does
+// not contract.  A term errs by at most 2^-46 of itself, a sum of kFold terms
+// by at most 75 x 2^-48 of it (the roundings of lo, whose entries reach 11 x
+// 2^-24 of the sum), 2.7e-13; measured on the 1024 x 1024 and 16384 x 256
+// jobs against long-double sums: 1e-15 and less, as with FP64 terms.
 // The FP64 pipe is the bound otherwise (seven conversions, differences and
-// products per entry: 5.5 ms at 8192 x 8192 x 6); with some hundred terms per
-// thread the fewer FP64 additions also make the error bound smaller than that
-// of adding every term to the FP64 total (n 2^-53).
+// products per entry: 5.5 ms at 8192 x 8192 x 6, 1.1 ms so).
 constexpr int kFold = 8;
 template <bool EXACT>
 struct SqDiff {
@@ -237,9 +240,9 @@ struct SqDiff {
   float hi = 0.f, lo = 0.f;
   __device__ __forceinline__ void add(float a, float b) {
     if constexpr (EXACT) {
-      const float s = a - b, bb = s - a;
-      const float e = (a - (s - bb)) + (-b - bb);
-      const float p = s * s;
+      const float s = __fsub_rn(a, b), bb = __fsub_rn(s, a);
+      const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(-b, bb));
+      const float p = __fmul_rn(s, s);
       if (!(p <= 1e35f && (p >= 1e-24f || s == 0.f))) {
         // the square or its rounding leaves the FP32 range
         const double d = (double)a - (double)b;
@@ -247,8 +250,9 @@ struct SqDiff {
         return;
       }
       const float q = fmaf(2.f * s, e, fmaf(s, s, -p));
-      const float t = hi + p, tb = t - hi;
-      lo += ((hi - (t - tb)) + (p - tb)) + q;
+      const float t = __fadd_rn(hi, p), tb = __fsub_rn(t, hi);
+      const float r = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, tb)), __fsub_rn(p, tb));
+      lo = __fadd_rn(lo, __fadd_rn(r, q));
       hi = t;
     } else {
       const double d = (double)a - (double)b;
@@ -517,7 +521,8 @@ cudaError_t launch_finalize(const float* W, const float* Z, const float* R, floa
   const int grid = ew_grid(MN), d = dual ? 1 : 0;
   const bool vec = (MN & 3) == 0 && ((((uintptr_t)W) | ((uintptr_t)Z) | ((uintptr_t)R) |
                                       ((uintptr_t)X_out) | ((uintptr_t)U_out)) & 15) == 0;
-  // the FP32-pair sums from 128 terms per thread on (see SqDiff)
+  // the FP32-pair sums from 128 terms per thread on, where the FP64 pipe and
+  // not the memory would be the bound
   if (vec && MN * L >= (size_t)grid * kEwThreads * 128)
     finalize_kernel<true, 4><<<grid, kEwThreads, 0, st>>>(W, Z, R, X_out, U_out, pres_acc, d, L, MN);
   else if (vec)
