@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 #include <float.h>
+#include <math.h>
 #include <stddef.h>
 
 #include "internal.h"
@@ -47,11 +48,14 @@ __device__ __forceinline__ void tile_of(int t, int* ta, int* tc) {
 // The bound the certificate has to prove: ||P G P||_2 < c shows, by Cauchy
 // interlacing, that G has at most ku eigenvalues above c (and the ku Ritz
 // values above tau^2 are lower bounds of ku eigenvalues), so exactly the kept
-// pairs lie above tau^2.  c = tau^2 less the rounding of forming X = P G P,
-// (2 ku + 4) eps (||G||_F + 2 sqrt(ku) ||What||_F), wsum = ||What||_F^2; the
+// pairs lie above tau^2.  c = tau^2 less the rounding of forming X = P G P
+// entry by entry as G - U What^T - What U^T: 2 ku multiply-adds, so an entry
+// errs by at most ku eps (|G| + 2 |U| |What|^T) of it.  gnorm bounds the
+// spectral norm of |G|: ||G||_F, its trace, or its largest row sum; that of
+// |U| |What|^T is at most sqrt(ku) ||What||_F, wsum = ||What||_F^2.  The
 // certificate accounts for its own rounding.
-__device__ __forceinline__ float cert_bound(float thr, float gF, int ku, float wsum) {
-  const float xf = gF + 2.f * sqrtf((float)ku) * sqrtf(wsum);
+__host__ __device__ __forceinline__ float cert_bound(float thr, float gnorm, int ku, float wsum) {
+  const float xf = gnorm + 2.f * sqrtf((float)ku) * sqrtf(wsum);
   return thr - 1.1f * FLT_EPSILON * (float)(2 * ku + 4) * xf;
 }
 

@@ -12,10 +12,13 @@
 // blocks are settled at k = 3 or 4, and the remaining launches return at
 // once.  The error terms are worst-case bounds from the norms computed on
 // the way:
-//   rounding to FP16   2^-11 ||.||_F + n 2^-25  (normal + subnormal entries)
+//   rounding to FP16   2^-11 ||.||_F + n 2^-25  (normal + subnormal entries;
+//     round to nearest errs by 2^-11 / (1 + 2^-11) at most, which leaves 2^-22
+//     for the FP32 scaling by 1 / c)
 //   accumulation       (n / 16 + 8) 2^-22 ||M_{k-1}||_F^2: every addition of
 //     the running FP32 sum (one per 16-wide MMA step) errs by at most 2^-22
-//     of sum_l |m_il m_jl| <= |m_i| |m_j| (truncating adders included)
+//     of sum_l |m_il m_jl| <= |m_i| |m_j| (truncating adders included; the
+//     tensor core's adder is not documented: this is an assumption)
 // They cost 0.5-1 % of c at n = 512-1024.
 //
 // Why not a Cholesky factorisation of c I - X: that is n/64 dependent panels

@@ -580,19 +580,22 @@ eig_cluster_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace w
         __syncthreads();
         // kept pairs: Rayleigh quotients, count above thr; pairs above thr
         // first
-        float rho = 0.f;
+        float rho = 0.f, wsum = 0.f;
         int kk = 0;
         bool ordered = true;
         for (int q = 0; q < ku; ++q) {
           rho += z.h[q];
           const float th = z.Bm[q * K + q];
+          wsum = fmaf(0.25f * th, th, wsum);
           kk += th > thr;
           if (q > 0 && th > thr && !(z.Bm[(q - 1) * K + (q - 1)] > thr)) ordered = false;
         }
         rho = sqrtf(rho);
-        // c0 as in lanczos.cuh; forming P G P adds (2 ku + 4) eps (||G||_F + 2
-        // ||U|| ||What||) <= 8 (ku + 1) eps gbound, already in it
-        const float c0 = thr - 2.f * rho - 8.f * (float)(ku + 1) * FLT_EPSILON * gbound;
+        // the pairs above tau^2 may be off by 2 rho (see lanczos.cuh).  gbound is
+        // the trace or the largest row sum; What_q = W_q - U sym(B)_q / 2 has
+        // half of W_q's part along U and the rest, so ||What||_F^2 <= sum
+        // theta_q^2 / 4 + rho^2
+        const float c0 = cert_bound(thr, gbound, ku, fmaf(rho, rho, wsum)) - 2.f * rho;
         if (ordered && c0 > 0.f) {
           // What = W - U sym(B) / 2 in place (a thread owns a row), then A <-
           // P G P = A - U What^T - What U^T
