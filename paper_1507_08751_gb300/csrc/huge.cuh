@@ -70,6 +70,25 @@ __device__ __forceinline__ float huge_hash(uint32_t a, uint32_t b) {
   return (float)(h >> 8) * (2.f / 16777216.f) - 1.f;
 }
 
+// How the subspace iteration of B blocks of order np (a multiple of 64) runs
+// on a device of `sms` multiprocessors whose clusters hold up to `widest`
+// CTAs (16, or 8 where the device has no room for 16).
+constexpr int kSMaxRows = 128;    // rows per CTA of the one-launch kernel, at most
+constexpr int kSPhaseRows = 512;  // rows per CTA of the phase kernels, at most
+struct SubspacePlan {
+  int cluster;  // CTAs per block; 0: the device cannot run blocks this wide
+  bool phases;  // a launch per phase instead of one for every step
+};
+inline SubspacePlan subspace_plan(int np, int B, int sms, int widest) {
+  // 8 CTAs per block up to 512 wide, 16 above (32 to 128 rows a CTA), where a
+  // lone block's latency counts; 8 up to 1024 wide when the blocks fill the
+  // chip anyway (64 blocks of 1024: 3.4 -> 2.3 ms)
+  const bool few = np <= 512 || (16 * B > sms && np <= 8 * kSMaxRows);
+  const int cl = few || widest < 16 ? 8 : 16;
+  if (np / cl <= kSMaxRows) return {cl, false};
+  return {np / cl <= kSPhaseRows ? cl : 0, true};
+}
+
 // Subspace iteration and Rayleigh-Ritz (k_subspace.cu): kernel attributes and
 // the launches (first: steps of the first round; W: workspace, np x kHP).
 cudaError_t configure_subspace();

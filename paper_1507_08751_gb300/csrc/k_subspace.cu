@@ -49,7 +49,7 @@ constexpr int kSStages = 3;
 constexpr int kSLdG = kSKC + 4;  // row stride of a G chunk (floats): 8 rows on distinct banks
 constexpr int kSLd = 36;       // row stride of X and W
 constexpr int kSM = kHP * 33;
-constexpr int kSMaxRows = 128;  // rows per CTA: two 64-row halves of 8 x 8 register tiles
+static_assert(kSMaxRows == 2 * 64, "two 64-row halves of 8 x 8 register tiles");
 
 // floats of one pipeline stage; between products the stages' space holds the
 // split sums of the products
@@ -728,8 +728,6 @@ subspace_more_kernel(const float* __restrict__ G, float* V, float* W, float* __r
   cl.sync();  // no CTA leaves while others read its shared memory
 }
 
-constexpr int kSPhaseRows = 512;  // rows per CTA of the phase kernels, at most
-
 // the widest cluster the device runs at the largest shared-memory size
 int widest_cluster() {
   static const int w = [] {
@@ -790,8 +788,8 @@ cudaError_t configure_subspace() {
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)sub_smem_bytes(64)))
     return e;
-  // 8192-wide blocks need the 16-CTA cluster
-  return widest_cluster() == 16 ? cudaSuccess : cudaErrorNotSupported;
+  widest_cluster();  // cached outside any stream capture
+  return cudaSuccess;
 }
 
 cudaError_t launch_subspace(const float* G, float* V, float* W, float* U, float* GU, int nn, int np,
@@ -802,13 +800,12 @@ cudaError_t launch_subspace(const float* G, float* V, float* W, float* U, float*
     if (cudaError_t e = launch()) return e;
     return prof ? prof->after(st) : cudaSuccess;
   };
-  // 8 CTAs per block up to 512 wide, 16 above (32 to 128 rows a CTA), where a
-  // lone block's latency counts; 8 up to 1024 wide when the blocks fill the
-  // chip anyway (64 blocks of 1024: 3.4 -> 2.3 ms)
   const bool many = 16 * B > sm_count();
-  const int CL = np <= 512 || (many && np <= 8 * kSMaxRows) ? 8 : 16;
+  const SubspacePlan plan = subspace_plan(np, B, sm_count(), widest_cluster());
+  const int CL = plan.cluster;
+  if (CL == 0) return cudaErrorNotSupported;
   const size_t bytes = sub_smem_bytes(np / CL);
-  if (np / CL <= kSMaxRows)
+  if (!plan.phases)
     return timed([&] {
       return many ? sub_launch(subspace_cluster_kernel<true>, CL, B, bytes, st, G, V, U, GU, nn, np,
                                thr, first, hb)
@@ -825,15 +822,15 @@ cudaError_t launch_subspace(const float* G, float* V, float* W, float* U, float*
       if (cudaError_t e = timed(gv)) return e;
       const int passes = i < rounds[r] ? (i + 1 < rounds[r] ? 2 : 3) : 0;
       if (cudaError_t e = timed([&] {
-            return sub_launch(subspace_phase_kernel, 16, B, bytes, st, V, W, U, GU, nn, np, thr,
+            return sub_launch(subspace_phase_kernel, CL, B, bytes, st, V, W, U, GU, nn, np, thr,
                               passes, hb);
           }))
         return e;
     }
   }
   return timed([&] {
-    return sub_launch(subspace_more_kernel, 16, B, sub_more_bytes(np / 16), st, G, V, W, U, GU, nn, np, thr,
-                      hb);
+    return sub_launch(subspace_more_kernel, CL, B, sub_more_bytes(np / CL), st, G, V, W, U, GU, nn, np,
+                      thr, hb);
   });
 }
 

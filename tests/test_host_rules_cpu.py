@@ -22,6 +22,11 @@ int main() {
       int ku;
       if (scanf("%f %f %d %f", &thr, &g, &ku, &w) != 4) return 1;
       printf("%.9g\n", cert_bound(thr, g, ku, w));
+    } else if (!strcmp(what, "plan")) {
+      int np, B, sms, widest;
+      if (scanf("%d %d %d %d", &np, &B, &sms, &widest) != 4) return 1;
+      const SubspacePlan p = subspace_plan(np, B, sms, widest);
+      printf("%d %d\n", p.cluster, (int)p.phases);
     }
   }
   return 0;
@@ -69,3 +74,24 @@ def test_certificate_bound_covers_forming_the_deflated_matrix(ask, n, ku):
             c = float(ask([f"bound {thr} {gnorm:.9g} {ku} {(W ** 2).sum():.9g}"])[0])
             # (2^-24: the bound itself is rounded to FP32)
             assert thr - c >= worst - 2.0 ** -24
+
+
+@pytest.mark.parametrize("blocks", [1, 9, 10, 64])
+def test_subspace_plan_needs_sixteen_ctas_above_4096_only(ask, blocks):
+    """Every order up to 8192 with clusters of 16, up to 4096 with clusters of 8;
+    rows per CTA within the kernels' limits, 16-CTA clusters only where the
+    device has them."""
+    orders = range(320, 8193, 64)
+    for widest in (16, 8):
+        got = ask([f"plan {o} {blocks} 152 {widest}" for o in orders])
+        assert len(got) == len(orders)
+        for o, line in zip(orders, got):
+            cluster, phases = (int(v) for v in line.split())
+            if widest == 8 and o > 4096:
+                assert cluster == 0
+                continue
+            assert cluster in (8, widest)
+            assert o % cluster == 0 and o // cluster <= (512 if phases else 128)
+            assert phases == (o > (2048 if widest == 16 else 1024))
+            if widest == 16 and blocks < 10:
+                assert cluster == (8 if o <= 512 else 16)
