@@ -70,9 +70,12 @@ __device__ __forceinline__ float huge_hash(uint32_t a, uint32_t b) {
   return (float)(h >> 8) * (2.f / 16777216.f) - 1.f;
 }
 
-// How the subspace iteration of B blocks of order np (a multiple of 64) runs
-// on a device of `sms` multiprocessors whose clusters hold up to `widest`
-// CTAs (16, or 8 where the device has no room for 16).
+// How the subspace iteration of blocks of order np (a multiple of 64), B of
+// them in a job, runs on a device of `sms` multiprocessors whose clusters hold
+// up to `widest` CTAs (16, or 8 where the device has no room for 16).  The
+// cluster size sets the order of the sums, so it depends on the job alone and
+// not on how many jobs share the launch: a batched job then sums as its solo
+// run does.
 constexpr int kSMaxRows = 128;    // rows per CTA of the one-launch kernel, at most
 constexpr int kSPhaseRows = 512;  // rows per CTA of the phase kernels, at most
 struct SubspacePlan {
@@ -92,8 +95,10 @@ inline SubspacePlan subspace_plan(int np, int B, int sms, int widest) {
 // Subspace iteration and Rayleigh-Ritz (k_subspace.cu): kernel attributes and
 // the launches (first: steps of the first round; W: workspace, np x kHP).
 cudaError_t configure_subspace();
+// The launches cover B blocks of jobs with `job_blocks` blocks each.
 cudaError_t launch_subspace(const float* G, float* V, float* W, float* U, float* GU, int nn, int np,
-                            float thr, int first, HugeBlock* hb, int B, cudaStream_t st, Prof* prof);
+                            float thr, int first, HugeBlock* hb, int B, int job_blocks, cudaStream_t st,
+                            Prof* prof);
 
 // Certificate workspace per block (bytes of one of the two FP16 matrices,
 // F-norm partials) and its launches: form plus kCertLevels squarings.

@@ -503,8 +503,9 @@ cudaError_t launch_huge(const ScaleLaunch& s, const BigWorkspace& ws, cudaStream
   // blocks whose Ritz residuals are still large
   const bool full = (s.m == launch_rows(s) && s.n == s.N);
   const bool warm = s.warm_start && (full || !s.shift);
+  const int job_blocks = (launch_rows(s) / s.m) * (s.N / s.n);
   if (cudaError_t e_ = launch_subspace(ws.G, ws.V, ws.Wv, ws.U, ws.GU, nn, np, thr, warm ? 2 : 6,
-                                       hb, B, st, prof))
+                                       hb, B, job_blocks, st, prof))
     return e_;
   if (cudaError_t e_ = launch_cert(ws.G, ws.U, ws.GU, ws.Ma, ws.Mb, ws.fpart, hb, nn, B, s.err, st,
                                    prof))

@@ -793,15 +793,16 @@ cudaError_t configure_subspace() {
 }
 
 cudaError_t launch_subspace(const float* G, float* V, float* W, float* U, float* GU, int nn, int np,
-                            float thr, int first, HugeBlock* hb, int B, cudaStream_t st, Prof* prof) {
+                            float thr, int first, HugeBlock* hb, int B, int job_blocks, cudaStream_t st,
+                            Prof* prof) {
   auto timed = [&](auto&& launch) -> cudaError_t {
     if (prof)
       if (cudaError_t e = prof->before(st, KK_SUBSPACE)) return e;
     if (cudaError_t e = launch()) return e;
     return prof ? prof->after(st) : cudaSuccess;
   };
-  const bool many = 16 * B > sm_count();
-  const SubspacePlan plan = subspace_plan(np, B, sm_count(), widest_cluster());
+  const bool many = 16 * B > sm_count();  // (the code's form: the same sums)
+  const SubspacePlan plan = subspace_plan(np, job_blocks, sm_count(), widest_cluster());
   const int CL = plan.cluster;
   if (CL == 0) return cudaErrorNotSupported;
   const size_t bytes = sub_smem_bytes(np / CL);
