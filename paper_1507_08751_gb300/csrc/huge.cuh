@@ -95,14 +95,16 @@ inline SubspacePlan subspace_plan(int np, int B, int sms, int widest) {
 // Subspace iteration and Rayleigh-Ritz (k_subspace.cu): kernel attributes and
 // the launches (first: steps of the first round; W: workspace, np x kHP).
 cudaError_t configure_subspace();
-// The launches cover B blocks of jobs with `job_blocks` blocks each.
+// The launches cover B blocks of jobs with `job_blocks` blocks each; W is used
+// only where subspace_phases(np).
+bool subspace_phases(int np);
 cudaError_t launch_subspace(const float* G, float* V, float* W, float* U, float* GU, int nn, int np,
                             float thr, int first, HugeBlock* hb, int B, int job_blocks, cudaStream_t st,
                             Prof* prof);
 
-// Certificate workspace per block (bytes of one of the two FP16 matrices,
-// F-norm partials) and its launches: form plus kCertLevels squarings.
-size_t cert_matrix_bytes(int nn);
+// Certificate workspace per block (F-norm partials; Ma and Mb hold np x np FP16
+// each) and its launches: form plus kCertLevels squarings.  Mb may be G's own
+// space: only the forming launch, which writes Ma, reads G.
 size_t cert_fpart_count(int nn);
 cudaError_t configure_cert();
 cudaError_t launch_cert(const float* G, const float* U, const float* Wh, void* Ma, void* Mb,

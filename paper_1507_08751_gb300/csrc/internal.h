@@ -65,13 +65,12 @@ struct BigWorkspace {
   int* kwarm;    // nblocks: how many of them (0 = none)
   size_t ystride;
   // blocks wider than 256 (k_block_huge.cu): G is a full square there
-  void* Ma;      // nblocks * np * np FP16, np = nn rounded up to 64: certificate matrices
-                 // (over part, which is free once G is formed, as far as they fit)
-  void* Mb;
+  void* Ma;      // nblocks * np * np FP16, np = nn rounded up to 64: certificate matrices,
+  void* Mb;      // over part and over G (free by then)
   double* fpart; // nblocks * tiles: their F-norm partials
   float* tstat;  // nblocks * ntiles * 2: per-tile diagonal sums, sums of squares
   float* V;      // nblocks * nn * 32: subspace basis (kept across calls)
-  float* Wv;     // nblocks * nn * 32: G V
+  float* Wv;     // nblocks * nn * 32: G V (null where the subspace steps are one launch)
   float* U;      // nblocks * nn * 16: Ritz vectors
   float* GU;     // nblocks * nn * 16: G U, then What
   void* hb;      // nblocks per-block states

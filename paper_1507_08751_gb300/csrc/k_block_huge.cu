@@ -401,23 +401,15 @@ huge_rebuild_kernel(ScaleLaunch a, const float* __restrict__ U, int np,
 
 static char* halign(char* p) { return (char*)(((uintptr_t)p + 255) & ~(uintptr_t)255); }
 
-// bytes of certificate matrices that do not fit over the Gram partials (which
-// hold one of the two at least: np (np + 64) / 2 floats per chunk)
-static size_t cert_own_bytes(const HugeDims& d) {
-  const size_t B = (size_t)d.nblocks, mb = B * cert_matrix_bytes(d.nn);
-  return sizeof(float) * B * d.chunks * d.ntiles * kHT * kHT >= 2 * mb ? 0 : mb;
-}
-
 size_t huge_workspace_bytes(int M, int N, int m, int n) {
   const HugeDims d = huge_dims(M, N, m, n);
   const size_t B = (size_t)d.nblocks, np = (size_t)d.T * kHT;
   size_t bytes = 0;
   bytes += sizeof(float) * B * d.chunks * d.ntiles * kHT * kHT;  // Gram partials
   bytes += sizeof(float) * B * np * np;                          // G
-  bytes += cert_own_bytes(d);                                    // certificate matrices
   bytes += sizeof(double) * B * cert_fpart_count(d.nn);
   bytes += 2 * sizeof(float) * B * d.ntiles;                     // tile sums
-  bytes += 2 * sizeof(float) * B * np * kHP;                     // V, W
+  bytes += (subspace_phases((int)np) ? 2 : 1) * sizeof(float) * B * np * kHP;  // V, W
   bytes += 2 * sizeof(float) * B * np * kHK;                     // U, What
   bytes += sizeof(HugeBlock) * B + sizeof(int) * B;
   bytes += 16 * 256;
@@ -437,15 +429,15 @@ BigWorkspace carve_huge_workspace(void* base, int M, int N, int m, int n) {
   };
   w.part = (float*)take(sizeof(float) * B * d.chunks * d.ntiles * kHT * kHT);
   w.G = (float*)take(sizeof(float) * B * np * np);
-  // the first certificate matrix lies over the Gram partials, the second too
-  // where they hold both (two row chunks or more)
-  const size_t mb = B * cert_matrix_bytes(d.nn), own = cert_own_bytes(d);
+  // the certificate matrices take no room of their own: the first lies over
+  // the Gram partials, which are summed by then (np (np + 64) / 2 floats per
+  // chunk), the second over G, which forming the first reads last
   w.Ma = w.part;
-  w.Mb = own ? take(own) : (void*)((char*)w.part + mb);
+  w.Mb = w.G;
   w.fpart = (double*)take(sizeof(double) * B * cert_fpart_count(d.nn));
   w.tstat = (float*)take(2 * sizeof(float) * B * d.ntiles);
   w.V = (float*)take(sizeof(float) * B * np * kHP);
-  w.Wv = (float*)take(sizeof(float) * B * np * kHP);
+  if (subspace_phases((int)np)) w.Wv = (float*)take(sizeof(float) * B * np * kHP);
   w.U = (float*)take(sizeof(float) * B * np * kHK);
   w.GU = (float*)take(sizeof(float) * B * np * kHK);
   w.hb = take(sizeof(HugeBlock) * B);

@@ -430,11 +430,6 @@ cudaError_t cert_map(CUtensorMap* map, __half* M, int np, int B) {
 
 }  // namespace
 
-size_t cert_matrix_bytes(int nn) {
-  const size_t np = (size_t)(nn + 63) & ~(size_t)63;
-  return np * np * sizeof(__half);
-}
-
 size_t cert_fpart_count(int nn) {
   const size_t t = ((size_t)nn + kFT - 1) / kFT;
   return t * (t + 1) / 2;

@@ -779,6 +779,9 @@ cudaError_t sub_launch(K k, int CL, int B, size_t bytes, cudaStream_t st, A... a
 
 }  // namespace
 
+// (any number of blocks: the plans differ up to 1024 wide only, in one launch)
+bool subspace_phases(int np) { return subspace_plan(np, 1, sm_count(), widest_cluster()).phases; }
+
 cudaError_t configure_subspace() {
   if (cudaError_t e = sub_attributes(subspace_cluster_kernel<false>, kSMaxRows)) return e;
   if (cudaError_t e = sub_attributes(subspace_cluster_kernel<true>, kSMaxRows)) return e;

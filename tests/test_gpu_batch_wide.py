@@ -31,3 +31,27 @@ def test_batched_wide_jobs_equal_their_solo_runs(n, jobs):
             torch.cuda.synchronize()
             assert torch.equal(X[:, j], Xs)
             assert Xs.abs().sum() > 0
+
+
+def test_blocks_just_above_256_fit_the_budget_they_always_had():
+    """102 blocks of 257 x 257 (one row chunk of the Gram sums each) within the
+    bytes that two FP32 matrices, the Gram partials and the bases take; first
+    and last block against FP64."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1507_08751_gb300 import binding as B
+    n, nb, tau = 257, 102, 40.0
+    M, N = n * nb // 2, 2 * n
+    tiles = 15
+    need = nb * (4 * tiles * 4096 + 8 * n * n + 8 * tiles + 8 * n * 32 + 12 * n * 16 + 104) + 4096
+    g = torch.Generator(device="cuda").manual_seed(7)
+    A = torch.randn((M, N), generator=g, device="cuda")
+    A += torch.randn((M, 2), generator=g, device="cuda") @ torch.randn((2, N), generator=g, device="cuda")
+    Z = torch.empty_like(A)
+    with B.Context(0, (need + 255) // 256 * 256 + 256) as ctx:
+        ctx.msllr_blocksvt(A, Z, n, n, tau, (0, 0))
+    torch.cuda.synchronize()
+    for sl in (np.s_[:n, :n], np.s_[M - n:, n:]):
+        U, s, Vt = np.linalg.svd(A[sl].double().cpu().numpy(), full_matrices=False)
+        want = (U * np.maximum(s - tau, 0.0)) @ Vt
+        assert np.linalg.norm(Z[sl].double().cpu().numpy() - want) <= 1e-4 * np.linalg.norm(want)
