@@ -182,9 +182,18 @@ def kernel_roofline(stats, scales, M, N, pk):
         roof = {"bound": "hbm", "achieved": round(ach, 1), "peak": pk["hbm_gbs"], "unit": "GB/s",
                 "frac": round(ach / pk["hbm_gbs"], 4), "traffic": None,
                 "peak_src": pk["src"], "note": "products of the first round only (lower bound)"}
+    elif kind == "certificate":
+        # one squaring (lower triangle, nn^3 flop per block) an iteration, over
+        # that iteration's launches: a block settles after one to eight
+        per_iter_launches = n / max(1, ITERS_OF.get("cur", 1))
+        ach = nblocks * nn ** 3 / per_iter_launches / avg_s / 1e12
+        roof = {"bound": "tensor", "achieved": round(ach, 3), "peak": pk["bf16_tflops"],
+                "unit": "TFLOP/s", "frac": round(ach / pk["bf16_tflops"], 5), "traffic": None,
+                "peak_src": pk["src"], "note": "one FP16 squaring counted (lower bound)"}
     elif kind in ("eig_big", "eig_fallback"):
-        # flops of the steps the kernel ran (counted on the device over every
-        # launch of the profiled job), per launch
+        # FP32 flops of the steps the kernel ran (counted on the device over
+        # every launch of the profiled job; its certificates run on the tensor
+        # cores and are not among them), per launch
         key = "flops" if kind == "eig_big" else "flops_fallback"
         flops = stats[key][i] / n
         ach = flops / avg_s / 1e12

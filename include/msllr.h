@@ -182,8 +182,9 @@ typedef struct msllr_stats {
    * output is formed from the Ritz pairs at hand.  0 in normal runs. */
   long long blocks_uncertified[MSLLR_MAX_SCALES];
   /* FP32 flops of the block eigen-solve steps that ran, each step counted
-   * at its algorithmic cost (a multiply-add is 2 flops): zero-rank and
-   * deflated certificates n^3/3 (a Cholesky factorisation's), Lanczos and power steps,
+   * at its algorithmic cost (a multiply-add is 2 flops): certificates of
+   * blocks up to 64 wide n^3/3 (wider ones run on the tensor cores and are not
+   * counted), deflation, Lanczos and power steps,
    * Householder tridiagonalisation 4n^3/3.  `flops`: the fused narrow-block
    * kernel (its Gram and rebuild included) or the wide-block eigen kernel;
    * `flops_fallback`: the wide-block Householder fallback kernel.  Blocks up

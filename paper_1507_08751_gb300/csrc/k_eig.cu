@@ -461,7 +461,6 @@ eig_cluster_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace w
           skipped = true;
           k = 0;
         }
-        fl += fl_chol(n);
         PHASE(3, 7);
       }
       g.barrier();
@@ -628,7 +627,7 @@ eig_cluster_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace w
             }
           }
           const float f2 = stage(c0);
-          fl += fl_deflate(n, ku) + fl_chol(n);
+          fl += fl_deflate(n, ku);
           PHASE(3, 5);
           if (eig_power_cert<CL>(g, M, tmem, bar, phase, f2, n, fx, s.red, a.err)) {
             k = kk;

@@ -121,3 +121,14 @@ def test_narrow_pairs_above_a_crowd_below_tau(ctx, m, n):
     for b in range(nb):
         sl = np.s_[b * m:(b + 1) * m]
         assert np.linalg.norm(got[sl] - want[sl]) <= 4e-5 * tau
+
+
+def test_flops_of_a_certified_block_are_its_fp32_steps(ctx):
+    """A 256 x 256 noise block of rank 0 above tau: row sums and up to three
+    power steps in FP32; the certificate itself runs on the tensor cores."""
+    n, tau = 256, 40.0
+    A = torch.from_numpy(np.random.default_rng(3).standard_normal((n, n)).astype(np.float32)).cuda()
+    X = torch.empty((1, n, n), device="cuda")
+    st = ctx.msllr_decompose(A, [(n, n)], X, lambdas=[tau], iters=1, seed=1)
+    assert st["blocks_zero"][0] == 1 and st["blocks_householder"][0] == 0
+    assert 2 * n * n <= st["flops"][0] <= n + 2 * n * n + 3 * (2 * n * n + 4 * n)
