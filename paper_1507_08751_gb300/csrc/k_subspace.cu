@@ -557,15 +557,9 @@ __device__ bool sub_ritz(const cg::cluster_group& cl, const SubSmem& m, int rp, 
   for (int q = 0; q < ku; ++q)
     if (sqrtf(rq[q]) > fmaxf(3e-4f * thr, 4e-6f * th0)) conv = false;
   if (cl.block_rank() == 0 && tid == 0) {
-    int k = 0;
-    for (int q = 0; q < ku; ++q) {
-      const float th = Bm[q * kHK + q];
-      h.theta[q] = th;
-      k += th > thr;
-    }
+    for (int q = 0; q < ku; ++q) h.theta[q] = Bm[q * kHK + q];
     h.c = cert_bound(thr, gF, ku, wsum);
     h.ku = ku;
-    h.k = k;
     h.conv = conv;
     h.over = nabove > kHK;
   }
@@ -584,6 +578,36 @@ __device__ __forceinline__ bool sub_active(const HugeBlock& h) {
 // what is slower is counted as uncertified.
 constexpr int kSRounds = 3;
 constexpr int kSMoreRounds = 16;
+
+// The further rounds of a lone block; false when a factorisation broke down.
+// Not inlined: as more turns of the loop below they cost every block 0.8 %
+// (1024 wide: 383 us instead of 377 without a further round).
+__device__ __noinline__ bool sub_further(const float* Gr, float* Vb, float* Ub, float* GUb, int nn, int np,
+                                         float thr, int rp, int r0, int b, float* sm, HugeBlock& h) {
+  const cg::cluster_group cl = cg::this_cluster();
+  const SubSmem m(sm, rp);
+  const int tid = threadIdx.x;
+  const float mu = 1e-4f * h.gF;
+  bool over = false;
+  for (int rd = 0; rd < kSMoreRounds && !over; ++rd) {
+    for (int st = 0; st <= 8; ++st) {
+      sub_gv<false>(Gr, Vb, np, rp, m.pipe, m.Ws);
+      if (st < 8) {
+        const bool ok = sub_orth(cl, m, rp, r0, nn, b, mu, st + 1 < 8 ? 2 : 3);
+        for (int e = tid; e < rp * kHP; e += kSNT)
+          Vb[(size_t)r0 * kHP + e] = m.Xs[(e >> 5) * kSLd + (e & 31)];
+        cl.sync();  // the new V is visible to the cluster
+        if (!ok) return false;
+      } else {
+        if (sub_ritz(cl, m, rp, Ub, GUb, thr, h, &over)) return true;
+        for (int e = tid; e < rp * kHP; e += kSNT)
+          m.Xs[(e >> 5) * kSLd + (e & 31)] = Vb[(size_t)r0 * kHP + e];
+        __syncthreads();
+      }
+    }
+  }
+  return true;
+}
 
 // Every step of every round for the blocks of a scale, a cluster per block.
 template <bool MANY>
@@ -605,18 +629,15 @@ subspace_cluster_kernel(const float* __restrict__ G, float* V, float* __restrict
   const float mu = 1e-4f * h.gF;
   for (int e = tid; e < rp * kHP; e += kSNT) m.Xs[(e >> 5) * kSLd + (e & 31)] = Vb[(size_t)r0 * kHP + e];
   __syncthreads();
-  // (a table: with the steps by comparisons the 1024 x 1024 prox took 467 us
-  // instead of 464)
   const int rounds[kSRounds] = {first, 4, 8};
   bool failed = false, conv = false, over = false;
-  for (int rd = 0; rd < kSRounds + kSMoreRounds && !conv && !failed; ++rd) {
-    if (rd >= kSRounds && over) break;
-    const int steps = rounds[min(rd, kSRounds - 1)];
-    for (int st = 0; st < steps && !failed; ++st) {
+  int more = kSMoreRounds;
+  for (int rd = 0; rd < kSRounds && !conv && !failed; ++rd) {
+    for (int st = 0; st < rounds[rd] && !failed; ++st) {
       sub_gv<MANY>(Gr, Vb, np, rp, m.pipe, m.Ws);
       // the third pass brings V to working precision for the Ritz problem;
       // between steps a well-conditioned basis of the same span is enough
-      failed = !sub_orth(cl, m, rp, r0, nn, b, mu, st + 1 < steps ? 2 : 3);
+      failed = !sub_orth(cl, m, rp, r0, nn, b, mu, st + 1 < rounds[rd] ? 2 : 3);
       for (int e = tid; e < rp * kHP; e += kSNT)
         Vb[(size_t)r0 * kHP + e] = m.Xs[(e >> 5) * kSLd + (e & 31)];
       cl.sync();  // the new V is visible to the cluster
@@ -628,7 +649,14 @@ subspace_cluster_kernel(const float* __restrict__ G, float* V, float* __restrict
       for (int e = tid; e < rp * kHP; e += kSNT)
         m.Xs[(e >> 5) * kSLd + (e & 31)] = Vb[(size_t)r0 * kHP + e];
       __syncthreads();
+      // the last round again: here the call below would take the kernel from
+      // 128 registers to 221 (one CTA per SM, 16 blocks of 512: 279 -> 428 us)
+      if (MANY && rd == kSRounds - 1 && !over && more-- > 0) --rd;
     }
+  }
+  if constexpr (!MANY) {
+    if (!conv && !failed && !over)
+      failed = !sub_further(Gr, Vb, U + uo, GU + uo, nn, np, thr, rp, r0, b, sm, h);
   }
   if (failed && rank == 0 && tid == 0) h.orth_fail = 1;
   cl.sync();  // no CTA leaves while others read its shared memory

@@ -119,3 +119,22 @@ def test_pairs_slower_than_every_round_count_as_uncertified(ctx):
         blocks.append((U * s) @ V.T)
     _, st = _cold_svts(ctx, blocks, tau)
     assert st["blocks_uncertified"][0] == 2
+
+
+def test_slow_pairs_of_many_blocks(ctx):
+    """The further rounds in the form for launches that fill the chip: ten
+    blocks and more, as test_slow_pairs_above_a_crowd_below_tau."""
+    n, above, tau = 260, 6, 50.0
+    s = np.concatenate([np.linspace(1.3, 1.002, above), np.linspace(0.93, 0.8835, n - above)]) * tau
+    rng = np.random.default_rng(n)
+    blocks, want = [], []
+    for _ in range(12):
+        U, _ = np.linalg.qr(rng.standard_normal((n, n)))
+        V, _ = np.linalg.qr(rng.standard_normal((n, n)))
+        blocks.append((U * s) @ V.T)
+        want.append((U * np.maximum(s - tau, 0.0)) @ V.T)
+    got, st = _cold_svts(ctx, blocks, tau)
+    assert st["blocks_uncertified"][0] == 0
+    bar = 1.3 * (np.sqrt(2 * above) * 1.5e-4 + 1e-7 * n) * tau
+    for g, w in zip(got, want):
+        assert np.linalg.norm(g - w) <= bar
