@@ -56,10 +56,12 @@ typedef enum msllr_status {
 #define MSLLR_KERNEL_KINDS 12
 
 /* Widest block (min(m_i, n_i)) the block-SVT kernels accept; the full-matrix
- * scale obeys the same limit on min(M, N).  Blocks up to 256 wide are solved
- * by one CTA each; wider ones (e.g. the full-matrix scale of a 1024 x 1024
- * matrix) by certified subspace iteration spread over many CTAs, where a
- * block's thresholded rank is at most 16. */
+ * scale obeys the same limit on min(M, N).  Blocks up to 64 wide are solved
+ * by part of a warp up to one CTA each, up to 256 wide by a pair of CTAs (one
+ * up to 128); wider ones (e.g. the full-matrix scale of a 1024 x 1024 matrix)
+ * by certified subspace iteration spread over many CTAs, where a block's
+ * thresholded rank is at most 16.  Blocks wider than 4096 need a device that
+ * runs clusters of 16 CTAs. */
 #define MSLLR_MAX_BLOCK_WIDTH 8192
 
 typedef struct msllr_ctx msllr_ctx;
@@ -285,7 +287,10 @@ int msllr_decompose(msllr_ctx* ctx, const float* Y, int M, int N, int ld,
  * msllr_decompose with its own cycle-spin shift sequence (seeds[j], as
  * msllr_shift_table), run together so that every kernel launch of an
  * iteration covers the blocks of all jobs (one CUDA graph per iteration for
- * the whole batch).  Job j's result equals msllr_decompose of that job alone.
+ * the whole batch).  Job j's result equals msllr_decompose of that job alone
+ * (bit for bit; blocks wider than 256 to rounding where the batch is large
+ * enough that their Gram sums are split into fewer row chunks, from six
+ * 1024-wide blocks on).
  *  Y        device, the jobs stacked row-wise: batch x M rows of N, row
  *           stride ld (job j at Y + j M ld).
  *  seeds    host array of batch shift seeds.

@@ -1,5 +1,6 @@
-// Shared by the kernels of blocks wider than 256: the subspace iteration
-// (k_block_huge.cu) and the certificate (k_cert_tc.cu).
+// Shared by the kernels of blocks wider than 256: Gram and rebuild
+// (k_block_huge.cu), subspace iteration (k_subspace.cu) and certificate
+// (k_cert_tc.cu; its bound also by k_eig.cu).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -26,7 +27,6 @@ struct HugeBlock {
   float theta[kHK];
   int status;    // kHs*
   int ku;        // kept Ritz pairs
-  int k;         // pairs above tau
   int conv;      // Rayleigh-Ritz residual test passed
   int over;      // more than kHK Ritz values above tau^2
   int orth_fail; // a CholQR factorisation broke down (basis restarted)

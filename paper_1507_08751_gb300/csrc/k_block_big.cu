@@ -236,7 +236,7 @@ rebuild_rows_kernel(ScaleLaunch a, const float* __restrict__ Yall, size_t ystrid
 }
 
 // Z' = (C V_f) V_f^T for a slab of `rs` rows of C, W' = 2 Z' - A: blocks of
-// rank above kRowK (only the Householder path produces them).  The CTAs
+// rank above kRowK (Lanczos keeps up to 16 pairs, Householder any).  The CTAs
 // stride over the (slab, block) items, so that a launch with nothing to do
 // holds few SMs.
 template <bool ST>

@@ -6,14 +6,13 @@
 //   1. Gram: G_b = C_b^T C_b, 64x64 tiles of the lower triangle split over
 //      row chunks; the partial sums are added in a fixed order and G_b is
 //      stored as a full square (both triangles);
-//   2. subspace iteration on G_b with a basis of kP = 32 columns kept from
-//      the previous call (warm start): W = G V over row tiles, then one CTA
-//      per block orthonormalises W + mu V by shifted CholQR followed by two
-//      plain CholQR passes (Fukaya, Kannan, Nakatsukasa, Yamamoto, Yanagisawa,
-//      SIAM J. Sci. Comput. 2020);
-//   3. Rayleigh-Ritz on V^T G V (32 x 32, the tridiagonal solver of
-//      symeig.cuh) for the pairs above tau^2, their residuals and a
-//      convergence test; unconverged blocks get further rounds of steps;
+//   2. subspace iteration on G_b with a basis of kHP = 32 columns kept from
+//      the previous call (warm start), in one cluster launch up to 2048 wide
+//      (k_subspace.cu): W = G V, then W + mu V is orthonormalised by a shifted
+//      CholQR pass and one more, two before a test;
+//   3. Rayleigh-Ritz on V^T G V (32 x 32, parallel Jacobi) for the pairs above
+//      tau^2, their residuals and a convergence test; unconverged blocks get
+//      further rounds of steps;
 //   4. certificate: ||P G P||_2 < tau^2 with P = I - U U^T over the kept
 //      Ritz vectors, by repeated squaring on the tensor cores
 //      (k_cert_tc.cu); by Cauchy interlacing G then has no eigenvalue above
@@ -75,12 +74,10 @@ __device__ __forceinline__ float huge_load(const ScaleLaunch& a, size_t off) {
 // ---------------------------------------------------------------------------
 template <bool ST>
 __global__ void __launch_bounds__(kHThreads, 4)
-huge_gram_kernel(ScaleLaunch a, float* __restrict__ part, int chunk_rows, int chunks,
-                 const HugeBlock* __restrict__ hb) {
+huge_gram_kernel(ScaleLaunch a, float* __restrict__ part, int chunk_rows, int chunks) {
   __shared__ __align__(16) float As[32][kHT + 4];
   __shared__ __align__(16) float Bs[32][kHT + 4];
   const int t = blockIdx.x, chunk = blockIdx.y, b = blockIdx.z;
-  (void)hb;
   int ta, tc;
   tile_of(t, &ta, &tc);
   const BlockGeom g = block_geom_t<ST>(a, b);
@@ -133,7 +130,7 @@ huge_gram_kernel(ScaleLaunch a, float* __restrict__ part, int chunk_rows, int ch
 // order np (nn rounded up to the tile; the tiles are zero beyond nn), and per
 // tile: the diagonal sum and the sum of squares (off-diagonal tiles twice).
 // The mirrored tile goes through shared memory, so that both triangles are
-// written as row segments (1024 wide: 15 -> 6 us).  The CTA that finishes
+// written as row segments (1024 wide: 15 -> 10 us).  The CTA that finishes
 // a block last adds the tile sums in tile order to trace(G) and ||G||_F,
 // takes the zero-rank shortcut trace(G) <= tau^2 (the trace bounds
 // lambda_max) and resets the block's state (a launch of its own before).
@@ -241,7 +238,6 @@ huge_gram_finish_kernel(const float* __restrict__ part, float* __restrict__ G, f
     h.gF = (float)sqrt(qt);
     h.status = (h.trace <= thr) ? kHsSkip : kHsIter;
     h.ku = 0;
-    h.k = 0;
     h.conv = 0;
     h.over = 0;
     h.cert = kCertOpen;
@@ -479,10 +475,10 @@ cudaError_t launch_huge(const ScaleLaunch& s, const BigWorkspace& ws, cudaStream
       return e_;
   } else if (s.fw || s.rows)
     huge_gram_kernel<true><<<dim3(d.ntiles, d.chunks, B), kHThreads, 0, st>>>(s, ws.part, d.chunk_rows,
-                                                                      d.chunks, hb);
+                                                                              d.chunks);
   else
     huge_gram_kernel<false><<<dim3(d.ntiles, d.chunks, B), kHThreads, 0, st>>>(s, ws.part, d.chunk_rows,
-                                                                      d.chunks, hb);
+                                                                               d.chunks);
   PROF_AFTER()
   PROF_BEFORE(KK_GRAM_REDUCE)
   huge_gram_finish_kernel<<<dim3(d.ntiles, B), kHThreads, 0, st>>>(ws.part, ws.G, ws.tstat, np,

@@ -59,7 +59,7 @@ struct SmallLayout {
     oG = al(oS + 9 * NMAX + 4 * NT + 64);
     oL = al(oG + nn * (nn + 1));
     oQ = al(oL + lz_cert_floats(NMAX, NT));
-    oU = kLz ? oQ + lz_ldq<NMAX>(NMAX) * JCAP : oQ;
+    oU = kLz ? oQ + lz_ldq(NMAX) * JCAP : oQ;
     oZ = kLz ? oU + NMAX * lz_maxk(NMAX) : oU;
     oEnd = kLz ? al(oZ + lz_scratch_floats(NMAX, JCAP)) : oQ;
     oP = mm * nn <= nn * (nn + 1) ? oG : oEnd;
@@ -310,7 +310,7 @@ __device__ __forceinline__ void small_block_svt(const ScaleLaunch& a, int b, flo
       if (!(c_skip > 0.f)) continue;
     } else if constexpr (kAttempts == 2) {
       int J = 0;
-      kk = lanczos_candidates(gr, thr, gbound, Qs, lz_ldq<NMAX>(nn), nn < JCAP ? nn : JCAP, Us,
+      kk = lanczos_candidates(gr, thr, gbound, Qs, lz_ldq(nn), nn < JCAP ? nn : JCAP, Us,
                               0x51ED27u + 131u * job_block(a, b), s, z, panel, &ku, &c0, 5 + SLOT,
                               &J);
       fl += (float)fl_lanczos(nn, J, ku);

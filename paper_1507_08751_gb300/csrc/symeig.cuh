@@ -30,10 +30,6 @@ struct LowerFull {
   int ld;
   __device__ __forceinline__ float& at(int i, int k) const { return g[i * ld + k]; }
 };
-struct LowerPacked {
-  float* g;
-  __device__ __forceinline__ float& at(int i, int k) const { return g[((i * (i + 1)) >> 1) + k]; }
-};
 
 // Shared-memory scratch of the solver.  Arrays marked [n] hold NMAX floats,
 // those marked [NT] hold NT entries.
