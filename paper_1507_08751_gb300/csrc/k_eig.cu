@@ -500,7 +500,7 @@ eig_cluster_kernel(ScaleLaunch a, const float* __restrict__ Gall, BigWorkspace w
         J = j + 1;
         if (J == n) break;  // Q spans everything: T_J is similar to G
         if (J < jmax) {
-          if (!(bt > 1e-5f * gbound)) {
+          if (!(bt > kLzBreak * gbound)) {
             // breakdown: an invariant subspace was found; continue from a
             // random direction orthogonal to it
             __syncthreads();

@@ -30,6 +30,13 @@
 namespace msllr {
 
 constexpr int kLzMaxJ = 32;  // Lanczos steps
+// A coupling beta below this fraction of the norm bound counts as a breakdown
+// and is set to zero, which moves G by as much: the rounding level of G q (a
+// few eps).  At 1e-5 the neglected coupling showed in the result: blocks of rank
+// three (5, 3 and 2 tau) came out up to 8e-5 tau off, 4e-6 tau now.  A breakdown
+// that goes unnoticed does no harm: the next direction is rounding, made
+// orthogonal like any other.
+constexpr float kLzBreak = 3e-7f;
 // Ritz pairs kept (above 0.95 tau^2): 8 for blocks up to 64 wide, 16 above,
 // where the alternative, a Householder reduction, takes some 0.3 ms (256 wide)
 constexpr int lz_maxk(int nmax) { return nmax > 64 ? 16 : 8; }
@@ -463,7 +470,7 @@ __device__ int lanczos_candidates(const SmallGram<NT, NMAX>& g, float thr, float
     J = j + 1;
     if (J == n) break;  // Q spans everything: T_J is similar to G
     if (J < jmax) {
-      if (!(b > 1e-5f * gbound)) {
+      if (!(b > kLzBreak * gbound)) {
         // breakdown: an invariant subspace was found; continue from a random
         // direction orthogonal to it
 #pragma unroll

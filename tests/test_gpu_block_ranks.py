@@ -132,3 +132,33 @@ def test_flops_of_a_certified_block_are_its_fp32_steps(ctx):
     st = ctx.msllr_decompose(A, [(n, n)], X, lambdas=[tau], iters=1, seed=1)
     assert st["blocks_zero"][0] == 1 and st["blocks_householder"][0] == 0
     assert 2 * n * n <= st["flops"][0] <= n + 2 * n * n + 3 * (2 * n * n + 4 * n)
+
+
+@pytest.mark.parametrize("m,n,kind", [(16, 1024, "full"), (20, 512, "full"), (33, 33, "three"),
+                                      (64, 64, "three"), (64, 100, "three"), (100, 100, "three"),
+                                      (200, 200, "three")])
+def test_what_a_lanczos_breakdown_neglects_is_rounding(ctx, m, n, kind):
+    """Blocks whose Krylov space ends after three steps (exact rank three), or is
+    used up entirely (14 pairs over two or more equal small values): a coupling
+    that the steps neglect must be at rounding level.  Both paths work on the
+    same Gram matrix, so the bar is three times the Householder path's own error
+    (skip_bound = 0) plus 1e-6 sigma_1 for the rounding of the vectors."""
+    from paper_1507_08751_gb300 import binding as B
+    k, tau = min(m, n), 10.0
+    s = (np.concatenate([np.linspace(6.0, 1.3, 14), np.full(k - 14, 0.2)]) if kind == "full"
+         else np.concatenate([[5.0, 3.0, 2.0], np.zeros(k - 3)])) * tau
+    for seed in range(12):
+        rng = np.random.default_rng(1000 * m + seed)
+        U, _ = np.linalg.qr(rng.standard_normal((m, k)))
+        V, _ = np.linalg.qr(rng.standard_normal((n, k)))
+        want = (U * np.maximum(s - tau, 0.0)) @ V.T
+        Y = torch.from_numpy(((U * s) @ V.T).astype(np.float32)).cuda()
+        err = []
+        for skip in (0, 1):
+            p = B.msllr_params_default()
+            p.skip_bound = skip
+            X = torch.empty((1, m, n), device="cuda")
+            Z = torch.empty_like(X)
+            ctx.msllr_decompose(Y, [(m, n)], X, lambdas=[tau], iters=1, seed=1, Z_out=Z, params=p)
+            err.append(np.linalg.norm(Z[0].double().cpu().numpy() - want))
+        assert err[1] <= 3.0 * err[0] + 1e-6 * s[0]
