@@ -434,6 +434,7 @@ __device__ bool sub_ritz(const cg::cluster_group& cl, const SubSmem& m, int rp, 
   __shared__ float rq[2 * kHK], red[kSNW][2 * kHK];
   __shared__ float2 cs[16];
   __shared__ int sel[kHK], nabove;
+  __shared__ float qn[kHP];
   float *Xs = m.Xs, *Ws = m.Ws, *P = m.P, *Sm = m.Sm, *Rm = m.Rm, *Qm = m.Qm, *Bm = m.Bm;
   const float gF = h.gF;
   sub_atb(Xs, Ws, rp, m.pipe, P);
@@ -458,6 +459,11 @@ __device__ bool sub_ritz(const cg::cluster_group& cl, const SubSmem& m, int rp, 
     }
     const unsigned above = __ballot_sync(0xffffffffu, th > thr);
     if (th > thr && rk < kHK) sel[rk] = tid;
+    // some two hundred rotations leave the columns of Q 1e-6 off unit length
+    float n2 = 0.f;
+#pragma unroll 8
+    for (int a = 0; a < kHP; ++a) n2 = fmaf(Qm[a * 33 + tid], Qm[a * 33 + tid], n2);
+    qn[tid] = fmaf(-0.5f, n2, 1.5f);
     if (tid == 0) nabove = __popc(above);
   }
   __syncthreads();
@@ -468,6 +474,7 @@ __device__ bool sub_ritz(const cg::cluster_group& cl, const SubSmem& m, int rp, 
   {
     const int q = tid & 15;
     const int cq = q < ku ? sel[q] : 0;
+    const float cn = qn[cq];
     for (int r = tid >> 4; r < rp; r += kSNT / 16) {
       float u = 0.f, g = 0.f;
 #pragma unroll
@@ -483,8 +490,8 @@ __device__ bool sub_ritz(const cg::cluster_group& cl, const SubSmem& m, int rp, 
         }
       }
       __syncwarp();
-      Xs[r * kSLd + q] = q < ku ? u : 0.f;
-      Xs[r * kSLd + kHK + q] = q < ku ? g : 0.f;
+      Xs[r * kSLd + q] = q < ku ? u * cn : 0.f;
+      Xs[r * kSLd + kHK + q] = q < ku ? g * cn : 0.f;
     }
   }
   __syncthreads();

@@ -138,3 +138,25 @@ def test_slow_pairs_of_many_blocks(ctx):
     bar = 1.3 * (np.sqrt(2 * above) * 1.5e-4 + 1e-7 * n) * tau
     for g, w in zip(got, want):
         assert np.linalg.norm(g - w) <= bar
+
+
+@pytest.mark.parametrize("M,N", [(257, 257), (320, 300), (512, 512), (1024, 1024)])
+def test_many_pairs_are_as_accurate_as_few(ctx, M, N):
+    """Fourteen pairs from 1.3 to 6 tau: the rotations of the 32 x 32 Ritz problem
+    must not leave the vectors off unit length.  Bar per block: 8 eps ||Z||_F --
+    two eps for the length of u on either side of the product, as much again
+    for the rounding of G (an eigenvalue's counts half in sigma) and of the
+    products."""
+    n, tau = min(M, N), 10.0
+    s = np.concatenate([np.linspace(6.0, 1.3, 14), np.full(n - 14, 0.2)]) * tau
+    rng = np.random.default_rng(M + N)
+    blocks, want = [], []
+    for _ in range(4):
+        U, _ = np.linalg.qr(rng.standard_normal((M, n)))
+        V, _ = np.linalg.qr(rng.standard_normal((N, n)))
+        blocks.append((U * s) @ V.T)
+        want.append((U * np.maximum(s - tau, 0.0)) @ V.T)
+    got, st = _cold_svts(ctx, blocks, tau)
+    assert st["blocks_uncertified"][0] == 0
+    for g, w in zip(got, want):
+        assert np.linalg.norm(g - w) <= 8 * 2.0 ** -23 * np.linalg.norm(w)
