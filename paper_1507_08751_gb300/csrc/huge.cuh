@@ -28,7 +28,8 @@ struct HugeBlock {
   int status;    // kHs*
   int ku;        // kept Ritz pairs
   int conv;      // Rayleigh-Ritz residual test passed
-  int over;      // more than kHK Ritz values above tau^2
+  int stop;      // further rounds would not bring the pairs to convergence
+  float worst;   // largest residual of the pairs relative to its bar
   int orth_fail; // a CholQR factorisation broke down (basis restarted)
   int cert;      // kCert*
   int arrived;   // CTAs of the running certificate level that are done

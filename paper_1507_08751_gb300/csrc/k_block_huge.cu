@@ -239,7 +239,8 @@ huge_gram_finish_kernel(const float* __restrict__ part, float* __restrict__ G, f
     h.status = (h.trace <= thr) ? kHsSkip : kHsIter;
     h.ku = 0;
     h.conv = 0;
-    h.over = 0;
+    h.stop = 0;
+    h.worst = 0.f;
     h.cert = kCertOpen;
     h.arrived = 0;
     h.orth_fail = 0;

@@ -423,13 +423,27 @@ __device__ bool sub_orth(const cg::cluster_group& cl, const SubSmem& m, int rp, 
   return true;
 }
 
+// Rounds of a block: `first`, 4 and 8 steps for every block, then up to
+// kSMoreRounds of 8 for blocks whose pairs have not converged but will at the
+// rate seen so far.  128 further steps bring the residual of a pair down by a
+// factor of 1000 where the eigenvalue below the basis is 0.95 of the pair's;
+// what is slower is counted as uncertified.
+constexpr int kSRounds = 3;
+constexpr int kSMoreRounds = 16;
+static_assert((kSMoreRounds & (kSMoreRounds - 1)) == 0, "a power of two (sub_ritz)");
+
 // Rayleigh-Ritz with V in Xs and G V in Ws: T = V^T G V, its eigenpairs above
 // thr (at most kHK, largest first), the Ritz vectors U = V Q, G U, B = U^T G
 // U, the residuals and What = G U - U sym(B) / 2 (into GU).  Overwrites Xs.
-// Returns true (in every CTA) when the pairs have converged; *over: more than
-// kHK Ritz values above thr, so that the block cannot be certified.
+// Returns true (in every CTA) when the pairs have converged.  `t`: the block's
+// previous test on entry, this one on return.
+struct SubTest {
+  float worst;  // largest residual relative to its bar (0: no test yet)
+  int ku;       // pairs
+  bool stop;    // no further rounds: they would not bring it to convergence
+};
 __device__ bool sub_ritz(const cg::cluster_group& cl, const SubSmem& m, int rp, float* Ub, float* GUb,
-                         float thr, HugeBlock& h, bool* over) {
+                         float thr, HugeBlock& h, SubTest& t) {
   const int tid = threadIdx.x, CL = (int)cl.num_blocks();
   __shared__ float rq[2 * kHK], red[kSNW][2 * kHK];
   __shared__ float2 cs[16];
@@ -468,7 +482,6 @@ __device__ bool sub_ritz(const cg::cluster_group& cl, const SubSmem& m, int rp, 
   }
   __syncthreads();
   const int ku = min(nabove, kHK);
-  *over = nabove > kHK;
   // U = V Q and G U = W Q, over V's rows in Xs: entries 0 .. 15 U, 16 .. 31 G
   // U (the 16 threads of a row are in one warp)
   {
@@ -561,14 +574,32 @@ __device__ bool sub_ritz(const cg::cluster_group& cl, const SubSmem& m, int rp, 
     th0 = fmaxf(th0, Bm[q * kHK + q]);
     wsum += rq[kHK + q];
   }
-  for (int q = 0; q < ku; ++q)
-    if (sqrtf(rq[q]) > fmaxf(3e-4f * thr, 4e-6f * th0)) conv = false;
+  const float bar = fmaxf(3e-4f * thr, 4e-6f * th0);
+  float worst = 0.f;
+  for (int q = 0; q < ku; ++q) {
+    const float res = sqrtf(rq[q]);
+    if (res > bar) conv = false;
+    worst = fmaxf(worst, res);
+  }
+  worst /= bar;
+  // more than kHK Ritz values above tau^2 are never certified; and at the rate
+  // of the last eight steps kSMoreRounds rounds of eight have to be enough (a
+  // new pair has no rate yet)
+  bool stop = nabove > kHK;
+  if (ku == t.ku && t.worst > 0.f) {
+    float rate = worst / t.worst;
+#pragma unroll
+    for (int i = 1; i < kSMoreRounds; i *= 2) rate *= rate;
+    stop = stop || worst * rate > 1.f;
+  }
+  t = SubTest{worst, ku, stop};
   if (cl.block_rank() == 0 && tid == 0) {
     for (int q = 0; q < ku; ++q) h.theta[q] = Bm[q * kHK + q];
     h.c = cert_bound(thr, gF, ku, wsum);
     h.ku = ku;
     h.conv = conv;
-    h.over = nabove > kHK;
+    h.worst = worst;
+    h.stop = stop;
   }
   cl.sync();  // the partial sums have been read
   return conv;
@@ -578,25 +609,17 @@ __device__ __forceinline__ bool sub_active(const HugeBlock& h) {
   return h.status == kHsIter && !h.conv && !h.orth_fail;
 }
 
-// Rounds of a block: `first`, 4 and 8 steps for every block, then up to
-// kSMoreRounds of 8 for blocks whose pairs have not converged and that can
-// still be certified.  128 further steps bring the residual of a pair down by
-// a factor of 1000 where the eigenvalue below the basis is 0.95 of the pair's;
-// what is slower is counted as uncertified.
-constexpr int kSRounds = 3;
-constexpr int kSMoreRounds = 16;
-
 // The further rounds of a lone block; false when a factorisation broke down.
 // Not inlined: as more turns of the loop below they cost every block 0.8 %
 // (1024 wide: 383 us instead of 377 without a further round).
 __device__ __noinline__ bool sub_further(const float* Gr, float* Vb, float* Ub, float* GUb, int nn, int np,
-                                         float thr, int rp, int r0, int b, float* sm, HugeBlock& h) {
+                                         float thr, int rp, int r0, int b, float* sm, HugeBlock& h,
+                                         SubTest t) {
   const cg::cluster_group cl = cg::this_cluster();
   const SubSmem m(sm, rp);
   const int tid = threadIdx.x;
   const float mu = 1e-4f * h.gF;
-  bool over = false;
-  for (int rd = 0; rd < kSMoreRounds && !over; ++rd) {
+  for (int rd = 0; rd < kSMoreRounds && !t.stop; ++rd) {
     for (int st = 0; st <= 8; ++st) {
       sub_gv<false>(Gr, Vb, np, rp, m.pipe, m.Ws);
       if (st < 8) {
@@ -606,7 +629,7 @@ __device__ __noinline__ bool sub_further(const float* Gr, float* Vb, float* Ub, 
         cl.sync();  // the new V is visible to the cluster
         if (!ok) return false;
       } else {
-        if (sub_ritz(cl, m, rp, Ub, GUb, thr, h, &over)) return true;
+        if (sub_ritz(cl, m, rp, Ub, GUb, thr, h, t)) return true;
         for (int e = tid; e < rp * kHP; e += kSNT)
           m.Xs[(e >> 5) * kSLd + (e & 31)] = Vb[(size_t)r0 * kHP + e];
         __syncthreads();
@@ -637,7 +660,8 @@ subspace_cluster_kernel(const float* __restrict__ G, float* V, float* __restrict
   for (int e = tid; e < rp * kHP; e += kSNT) m.Xs[(e >> 5) * kSLd + (e & 31)] = Vb[(size_t)r0 * kHP + e];
   __syncthreads();
   const int rounds[kSRounds] = {first, 4, 8};
-  bool failed = false, conv = false, over = false;
+  bool failed = false, conv = false;
+  SubTest t{0.f, -1, false};
   int more = kSMoreRounds;
   for (int rd = 0; rd < kSRounds && !conv && !failed; ++rd) {
     for (int st = 0; st < rounds[rd] && !failed; ++st) {
@@ -651,19 +675,19 @@ subspace_cluster_kernel(const float* __restrict__ G, float* V, float* __restrict
     }
     if (failed) break;
     sub_gv<MANY>(Gr, Vb, np, rp, m.pipe, m.Ws);
-    conv = sub_ritz(cl, m, rp, U + uo, GU + uo, thr, h, &over);
+    conv = sub_ritz(cl, m, rp, U + uo, GU + uo, thr, h, t);
     if (!conv) {
       for (int e = tid; e < rp * kHP; e += kSNT)
         m.Xs[(e >> 5) * kSLd + (e & 31)] = Vb[(size_t)r0 * kHP + e];
       __syncthreads();
       // the last round again: here the call below would take the kernel from
       // 128 registers to 221 (one CTA per SM, 16 blocks of 512: 279 -> 428 us)
-      if (MANY && rd == kSRounds - 1 && !over && more-- > 0) --rd;
+      if (MANY && rd == kSRounds - 1 && !t.stop && more-- > 0) --rd;
     }
   }
   if constexpr (!MANY) {
-    if (!conv && !failed && !over)
-      failed = !sub_further(Gr, Vb, U + uo, GU + uo, nn, np, thr, rp, r0, b, sm, h);
+    if (!conv && !failed && !t.stop)
+      failed = !sub_further(Gr, Vb, U + uo, GU + uo, nn, np, thr, rp, r0, b, sm, h, t);
   }
   if (failed && rank == 0 && tid == 0) h.orth_fail = 1;
   cl.sync();  // no CTA leaves while others read its shared memory
@@ -687,7 +711,7 @@ subspace_gv_kernel(const float* __restrict__ G, const float* __restrict__ V, flo
 // orthonormalisation broke down or the pairs have not converged.
 __device__ bool sub_phase(const cg::cluster_group& cl, const SubSmem& m, int rp, int r0, float* Vr,
                           const float* Wr, float* Ub, float* GUb, int nn, int b, float thr, int passes,
-                          HugeBlock& h, bool* over) {
+                          HugeBlock& h, SubTest& t) {
   const int tid = threadIdx.x;
   for (int e = tid; e < rp * kHP; e += kSNT) {
     const int o = (e >> 5) * kSLd + (e & 31);
@@ -695,7 +719,7 @@ __device__ bool sub_phase(const cg::cluster_group& cl, const SubSmem& m, int rp,
     m.Ws[o] = Wr[e];
   }
   __syncthreads();
-  if (passes == 0) return sub_ritz(cl, m, rp, Ub, GUb, thr, h, over);
+  if (passes == 0) return sub_ritz(cl, m, rp, Ub, GUb, thr, h, t);
   const bool ok = sub_orth(cl, m, rp, r0, nn, b, 1e-4f * h.gF, passes);
   for (int e = tid; e < rp * kHP; e += kSNT) Vr[e] = m.Xs[(e >> 5) * kSLd + (e & 31)];
   cl.sync();  // the new V is visible to the cluster
@@ -715,9 +739,9 @@ subspace_phase_kernel(float* V, const float* W, float* __restrict__ U, float* __
   // (the state is written only after a later cluster barrier)
   if (!sub_active(h)) return;
   const size_t vo = ((size_t)b * np + r0) * kHP, uo = ((size_t)b * np + r0) * kHK;
-  bool over = false;
+  SubTest t{h.worst, h.ku, false};
   const bool ok = sub_phase(cl, SubSmem(sm, rp), rp, r0, V + vo, W + vo, U + uo, GU + uo, nn, b, thr,
-                            passes, h, &over);
+                            passes, h, t);
   if (passes > 0 && !ok && rank == 0 && threadIdx.x == 0) h.orth_fail = 1;
   cl.sync();  // no CTA leaves while others read its shared memory
 }
@@ -736,14 +760,15 @@ subspace_more_kernel(const float* __restrict__ G, float* V, float* W, float* __r
   const int rp = np / CL, r0 = rank * rp;
   HugeBlock& h = hb[b];
   // (the state is written only after a later cluster barrier)
-  if (!sub_active(h) || h.over) return;
+  if (!sub_active(h) || h.stop) return;
   const SubSmem m(sm, rp);
   const float* Gr = G + (size_t)b * np * np + (size_t)r0 * np;
   const float* Vb = V + (size_t)b * np * kHP;
   const size_t vo = ((size_t)b * np + r0) * kHP, uo = ((size_t)b * np + r0) * kHK;
   float* Wc = sm + sub_pipe_floats(64);
-  bool ok = true, conv = false, over = false;
-  for (int rd = 0; rd < kSMoreRounds && ok && !conv && !over; ++rd) {
+  bool ok = true, conv = false;
+  SubTest t{h.worst, h.ku, false};
+  for (int rd = 0; rd < kSMoreRounds && ok && !conv && !t.stop; ++rd) {
     for (int st = 0; st <= 8 && ok; ++st) {
       for (int c = 0; c < rp; c += 64) {
         const int rows = min(64, rp - c);
@@ -754,7 +779,7 @@ subspace_more_kernel(const float* __restrict__ G, float* V, float* W, float* __r
       }
       const int passes = st < 8 ? (st + 1 < 8 ? 2 : 3) : 0;
       const bool r = sub_phase(cl, m, rp, r0, V + vo, W + vo, U + uo, GU + uo, nn, b, thr, passes, h,
-                               &over);
+                               t);
       if (passes > 0) ok = r;
       else conv = r;
     }
